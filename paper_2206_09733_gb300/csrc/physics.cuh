@@ -19,7 +19,54 @@ namespace hs3d {
 template <typename R>
 struct Prim {
     R rho, v1, v2, v3, p, E;   // E = rho e, the conserved total energy
+    R ir;                      // FP64 path: 1/rho (the FP32 functions do not read it)
 };
+
+// FP64 reciprocal, reciprocal square root and square root.  The FP64 pipe
+// (2 FMA per clock and SM, 1/64 of the FP32 rate) bounds every FP64 kernel, so
+// what counts is the number of FP64 instructions: the seed comes from the
+// hardware's approximate instruction (on another pipe; about 20 bits) and is
+// carried to full precision by one third-order Newton-type step,
+//   1/x:        e = 1 - x y,    y (1 + e + e^2)            (error e^3)
+//   x^(-1/2):   e = 1 - x y^2,  y (1 + e/2 + 3 e^2/8)      (error ~ e^3)
+// (the leading terms of the binomial series of 1/(1-e) and (1-e)^(-1/2)):
+// 3 and 5 FP64 instructions for a result within about one unit in the last
+// place.  The range test is on the integer pipe; zero, negative, subnormal,
+// huge, infinite and NaN arguments take the IEEE operation out of line.
+__device__ __noinline__ inline double rcp_ieee(double x) { return 1.0 / x; }
+__device__ __noinline__ inline double rsqrt_ieee(double x) { return 1.0 / sqrt(x); }
+__device__ __noinline__ inline double sqrt_ieee(double x) { return sqrt(x); }
+
+__device__ __forceinline__ double rcp_fast(double x)
+{
+    if (((unsigned)__double2hiint(x) & 0x7fffffffu) - 0x00200000u >= 0x7fa00000u) return rcp_ieee(x);
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    double e = fma(-x, y, 1.0);
+    e = fma(e, e, e);
+    return fma(y, e, y);
+}
+
+__device__ __forceinline__ double rsqrt_step(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x * y, y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ bool sqrt_plain(double x)
+{
+    return (unsigned)__double2hiint(x) - 0x00200000u < 0x7fa00000u;
+}
+__device__ __forceinline__ double rsqrt_fast(double x) { return sqrt_plain(x) ? rsqrt_step(x) : rsqrt_ieee(x); }
+__device__ __forceinline__ double sqrt_fast(double x) { return sqrt_plain(x) ? x * rsqrt_step(x) : sqrt_ieee(x); }
+
+// sqrt(x) in the arithmetic type.
+__device__ __forceinline__ double sqrt_(double x) { return sqrt_fast(x); }
+__device__ __forceinline__ float sqrt_(float x) { return sqrt(x); }
+// a / b: FP64 as a times rcp_fast(b).
+__device__ __forceinline__ double div_(double a, double b) { return a * rcp_fast(b); }
+__device__ __forceinline__ float div_(float a, float b) { return a / b; }
 
 // FP64 -> FP32 with round-to-nearest-even, on the integer pipe.  On this GPU
 // every FP64-pipe instruction (conversions included) costs as much issue
@@ -86,9 +133,10 @@ __device__ __forceinline__ Prim<R> prim_from_u(const double u[5], R gm1);
 template <>
 __device__ __forceinline__ Prim<double> prim_from_u<double>(const double u[5], double gm1)
 {
-    double ir = 1.0 / u[0];
+    double ir = rcp_fast(u[0]);
     double v1 = u[1] * ir, v2 = u[2] * ir, v3 = u[3] * ir;
     Prim<double> q;
+    q.ir = ir;
     q.rho = u[0];
     q.v1 = v1;
     q.v2 = v2;
@@ -119,13 +167,6 @@ __device__ __forceinline__ Prim<float> prim_from_u<float>(const double u[5], flo
     const float uf[5] = {d2f_rn(u[0]), d2f_rn(u[1]), d2f_rn(u[2]), d2f_rn(u[3]), d2f_rn(u[4])};
     return prim_from_f(uf, gm1);
 }
-
-template <typename R>
-__device__ __forceinline__ R rsqrt_(R x);
-template <>
-__device__ __forceinline__ double rsqrt_<double>(double x) { return 1.0 / sqrt(x); }
-template <>
-__device__ __forceinline__ float rsqrt_<float>(float x) { return rsqrtf(x); }
 
 template <typename R>
 __device__ __forceinline__ R log_(R x);
@@ -170,6 +211,20 @@ __device__ __forceinline__ void visc_flux(const Prim<R> &q, const R G[12], R mu,
     f[4] = q.v1 * s1 + q.v2 * s2 + q.v3 * s3 + kappa * (G[9] * a1 + G[10] * a2 + G[11] * a3);
 }
 
+// Speed of sound and total enthalpy of a state.
+template <typename R>
+__device__ __forceinline__ R sound_speed(const Prim<R> &q, R gamma)
+{
+    if constexpr (sizeof(R) == 8) return sqrt_(gamma * q.p * q.ir);
+    else return sqrt(gamma * q.p / q.rho);
+}
+template <typename R>
+__device__ __forceinline__ R enthalpy(const Prim<R> &q, R E)
+{
+    if constexpr (sizeof(R) == 8) return (E + q.p) * q.ir;
+    else return (E + q.p) / q.rho;
+}
+
 // Lax-Friedrichs flux times the face scale s = |Sn|, Sn the scaled normal
 // pointing from L to R:  s [ (F_L + F_R).n/2 - lambda (u_R - u_L)/2 ],
 // lambda = max(|v_L.n| + c_L, |v_R.n| + c_R).
@@ -177,12 +232,12 @@ template <typename R>
 __device__ __forceinline__ void flux_lf(const Prim<R> &L, const R uL[5], const Prim<R> &Rr, const R uR[5], R gamma,
                                         R s1, R s2, R s3, R f[5])
 {
-    R s = sqrt(s1 * s1 + s2 * s2 + s3 * s3);
+    R s = sqrt_(s1 * s1 + s2 * s2 + s3 * s3);
     R fl[5], fr[5];
     euler_flux(L, uL[4], s1, s2, s3, fl);
     euler_flux(Rr, uR[4], s1, s2, s3, fr);
-    R vnL = fabs(L.v1 * s1 + L.v2 * s2 + L.v3 * s3) + s * sqrt(gamma * L.p / L.rho);
-    R vnR = fabs(Rr.v1 * s1 + Rr.v2 * s2 + Rr.v3 * s3) + s * sqrt(gamma * Rr.p / Rr.rho);
+    R vnL = fabs(L.v1 * s1 + L.v2 * s2 + L.v3 * s3) + s * sound_speed(L, gamma);
+    R vnR = fabs(Rr.v1 * s1 + Rr.v2 * s2 + Rr.v3 * s3) + s * sound_speed(Rr, gamma);
     R lam = fmax(vnL, vnR);    // = s * lambda
 #pragma unroll
     for (int v = 0; v < 5; ++v) f[v] = (R)0.5 * (fl[v] + fr[v]) - (R)0.5 * lam * (uR[v] - uL[v]);
@@ -194,15 +249,27 @@ template <typename R>
 __device__ __forceinline__ void flux_rusanov(const Prim<R> &L, const R uL[5], const Prim<R> &Rr, const R uR[5],
                                              R gamma, R s1, R s2, R s3, R f[5])
 {
-    R s = sqrt(s1 * s1 + s2 * s2 + s3 * s3);
+    R s = sqrt_(s1 * s1 + s2 * s2 + s3 * s3);
     R fl[5], fr[5];
     euler_flux(L, uL[4], s1, s2, s3, fl);
     euler_flux(Rr, uR[4], s1, s2, s3, fr);
     R vn = fmax(fabs(L.v1 * s1 + L.v2 * s2 + L.v3 * s3), fabs(Rr.v1 * s1 + Rr.v2 * s2 + Rr.v3 * s3));
-    R c = fmax(sqrt(gamma * L.p / L.rho), sqrt(gamma * Rr.p / Rr.rho));
+    R c = fmax(sound_speed(L, gamma), sound_speed(Rr, gamma));
     R lam = vn + s * c;        // = s * lambda
 #pragma unroll
     for (int v = 0; v < 5; ++v) f[v] = (R)0.5 * (fl[v] + fr[v]) - (R)0.5 * lam * (uR[v] - uL[v]);
+}
+
+// sqrt(s2) and its reciprocal.
+__device__ __forceinline__ void norm_and_inverse(double s2, double &s, double &is)
+{
+    is = rsqrt_fast(s2);
+    s = s2 * is;
+}
+__device__ __forceinline__ void norm_and_inverse(float s2, float &s, float &is)
+{
+    s = sqrt(s2);
+    is = 1.0f / s;
 }
 
 // Roe flux times the face scale (Roe 1981, sqrt(rho)-weighted averages, no
@@ -213,23 +280,32 @@ template <typename R>
 __device__ __forceinline__ void flux_roe(const Prim<R> &L, const R uL[5], const Prim<R> &Rr, const R uR[5], R gamma,
                                          R s1, R s2, R s3, R f[5], R zvel = (R)1)
 {
-    R s = sqrt(s1 * s1 + s2 * s2 + s3 * s3);
-    R is = (R)1 / s;
+    R s, is;
+    norm_and_inverse(s1 * s1 + s2 * s2 + s3 * s3, s, is);
     R n1 = s1 * is, n2 = s2 * is, n3 = s3 * is;
     R fl[5], fr[5];
     euler_flux(L, uL[4], s1, s2, s3, fl);
     euler_flux(Rr, uR[4], s1, s2, s3, fr);
-    R sl = sqrt(L.rho), sr = sqrt(Rr.rho);
-    R iw = (R)1 / (sl + sr);
-    R HL = (uL[4] + L.p) / L.rho, HR = (uR[4] + Rr.p) / Rr.rho;
+    R sl = sqrt_(L.rho), sr = sqrt_(Rr.rho);
+    R iw;
+    if constexpr (sizeof(R) == 8) iw = rcp_fast(sl + sr);
+    else iw = (R)1 / (sl + sr);
+    R HL = enthalpy(L, uL[4]), HR = enthalpy(Rr, uR[4]);
     R vt1 = (sl * L.v1 + sr * Rr.v1) * iw;
     R vt2 = (sl * L.v2 + sr * Rr.v2) * iw;
     R vt3 = (sl * L.v3 + sr * Rr.v3) * iw;
     R Ht = (sl * HL + sr * HR) * iw;
     R q2 = vt1 * vt1 + vt2 * vt2 + vt3 * vt3;
     R c2 = (gamma - (R)1) * (Ht - (R)0.5 * q2);
-    R ct = sqrt(c2);
-    R ic2 = (R)1 / c2;
+    R ct, ic2;
+    if constexpr (sizeof(R) == 8) {
+        double ict;
+        norm_and_inverse(c2, ct, ict);
+        ic2 = ict * ict;
+    } else {
+        ct = sqrt(c2);
+        ic2 = (R)1 / c2;
+    }
     R rt = sl * sr;
     R vnt = vt1 * n1 + vt2 * n2 + vt3 * n3;
     R dr = Rr.rho - L.rho, dp = Rr.p - L.p;
@@ -264,9 +340,9 @@ template <typename R>
 __device__ __forceinline__ void flux_ldroe(const Prim<R> &L, const R uL[5], const Prim<R> &Rr, const R uR[5], R gamma,
                                            R s1, R s2, R s3, R f[5])
 {
-    const R mL = (L.v1 * L.v1 + L.v2 * L.v2 + L.v3 * L.v3) * L.rho / (gamma * L.p);
-    const R mR = (Rr.v1 * Rr.v1 + Rr.v2 * Rr.v2 + Rr.v3 * Rr.v3) * Rr.rho / (gamma * Rr.p);
-    const R z = fmin((R)1, sqrt(fmax(mL, mR)));
+    const R mL = div_((L.v1 * L.v1 + L.v2 * L.v2 + L.v3 * L.v3) * L.rho, gamma * L.p);
+    const R mR = div_((Rr.v1 * Rr.v1 + Rr.v2 * Rr.v2 + Rr.v3 * Rr.v3) * Rr.rho, gamma * Rr.p);
+    const R z = fmin((R)1, sqrt_(fmax(mL, mR)));
     flux_roe(L, uL, Rr, uR, gamma, s1, s2, s3, f, z);
 }
 
@@ -284,7 +360,7 @@ struct LogMeanEps<float> {
 template <typename R>
 __device__ __forceinline__ R rcp_(R x);
 template <>
-__device__ __forceinline__ double rcp_<double>(double x) { return 1.0 / x; }
+__device__ __forceinline__ double rcp_<double>(double x) { return rcp_fast(x); }
 // FP32: the hardware approximate reciprocal (at most 2 ulp, no IEEE fix-up
 // path), well inside the rounding the FP32 flux arithmetic makes anyway.
 template <>
@@ -304,10 +380,64 @@ __device__ __forceinline__ ECNode<R> ec_node(const Prim<R> &q)
     z.v1 = q.v1;
     z.v2 = q.v2;
     z.v3 = q.v3;
-    z.beta = q.rho / ((R)2 * q.p);
+    z.beta = div_(q.rho, (R)2 * q.p);
     z.lrho = log_(q.rho);
     z.lbeta = log_(z.beta);
     return z;
+}
+
+// F = ln(a/b) (a+b) / (2(a-b)) for u = ((a-b)/(a+b))^2 beyond the short series
+// of ec_pair64: 1 + u/3 + u^2/5 + ... to u^10/21 below u = 0.04 (a/b < 1.5; the
+// first term left out is below 2e-17), the logarithm above.  Few pairs of a
+// resolved flow come here, so no logarithm is computed per node.
+__device__ __forceinline__ double logmean_F(double a, double b, double f, double u)
+{
+    if (u < 0.04) {
+        double F = 1.0 / 21.0;
+        F = fma(F, u, 1.0 / 19.0);
+        F = fma(F, u, 1.0 / 17.0);
+        F = fma(F, u, 1.0 / 15.0);
+        F = fma(F, u, 1.0 / 13.0);
+        F = fma(F, u, 1.0 / 11.0);
+        F = fma(F, u, 1.0 / 9.0);
+        F = fma(F, u, 1.0 / 7.0);
+        F = fma(F, u, 1.0 / 5.0);
+        F = fma(F, u, 1.0 / 3.0);
+        return fma(F, u, 1.0);
+    }
+    return log(a / b) / (2.0 * f);
+}
+
+// Chandrashekar's flux in FP64 from the per-node inputs (rho, v/2, 2 beta =
+// rho/p, |v|^2/4): the means {v} and {|v|^2}/2 are plain sums, the means'
+// factors sit in the constants, and 1/(rho_L + rho_R), 1/(beta_L + beta_R)
+// come from one reciprocal: 48 FP64 instructions for a pair on the short
+// series (u < 1e-4, first term left out below 1.2e-17) against 72 with
+// per-node logarithms, full means and an IEEE division.
+__device__ __forceinline__ void ec_pair64(const double *L, const double *Rr, double hg, double a1, double a2,
+                                          double a3, double f[5])
+{
+    const double srho = L[0] + Rr[0], sb2 = L[4] + Rr[4];
+    const double inv = rcp_fast(srho * sb2);
+    const double irho = sb2 * inv, ib2 = srho * inv;   // 1/(rho_L + rho_R), 1/(2(beta_L + beta_R))
+    const double fr = (L[0] - Rr[0]) * irho, ur = fr * fr;
+    const double fb = (L[4] - Rr[4]) * ib2, ub = fb * fb;
+    double rho_ln, hib;   // rho^, hg/beta^
+    if (ur < LogMeanEps<double>::v)
+        rho_ln = srho * fma(-ur, fma(ur, fma(ur, 22.0 / 945.0, 2.0 / 45.0), 1.0 / 6.0), 0.5);
+    else
+        rho_ln = 0.5 * srho * rcp_fast(logmean_F(L[0], Rr[0], fr, ur));
+    const double q = (4.0 * hg) * ib2;
+    if (ub < LogMeanEps<double>::v) hib = q * fma(ub, fma(ub, fma(ub, 1.0 / 7.0, 0.2), 1.0 / 3.0), 1.0);
+    else hib = q * logmean_F(L[4], Rr[4], fb, ub);
+    const double m1 = L[1] + Rr[1], m2 = L[2] + Rr[2], m3 = L[3] + Rr[3];
+    const double pt = srho * ib2;
+    const double fm = rho_ln * (m1 * a1 + m2 * a2 + m3 * a3);
+    f[0] = fm;
+    f[1] = fm * m1 + pt * a1;
+    f[2] = fm * m2 + pt * a2;
+    f[3] = fm * m3 + pt * a3;
+    f[4] = fm * (hib - (L[5] + Rr[5])) + m1 * f[1] + m2 * f[2] + m3 * f[3];
 }
 
 // Chandrashekar's entropy-conservative, kinetic-energy-preserving flux dotted
@@ -322,20 +452,20 @@ __device__ __forceinline__ ECNode<R> ec_node(const Prim<R> &q)
 // 44u^3/945), for 1/beta^ directly as 2F/(a+b).  Only the two reciprocals
 // 1/(rho_L+rho_R) and 1/(beta_L+beta_R) are needed on that branch;
 // hg = 1/(2(gamma-1)).
+// (FP64: ec_pair64 below, the same flux with no logarithms per node.)
 template <typename R>
 __device__ __forceinline__ void flux_ec(const ECNode<R> &L, const ECNode<R> &Rr, R hg, R a1, R a2, R a3, R f[5])
 {
-    const R srho = L.rho + Rr.rho, sbeta = L.beta + Rr.beta;
-    R irho, ibeta;
     if constexpr (sizeof(R) == 8) {
-        // FP64: one division for both reciprocals (the FP64 pipe bounds this path)
-        const R inv = (R)1 / (srho * sbeta);
-        irho = sbeta * inv;
-        ibeta = srho * inv;
-    } else {
-        irho = rcp_(srho);
-        ibeta = rcp_(sbeta);
+        const double zl[6] = {L.rho, 0.5 * L.v1, 0.5 * L.v2, 0.5 * L.v3, 2.0 * L.beta,
+                              0.25 * (L.v1 * L.v1 + L.v2 * L.v2 + L.v3 * L.v3)};
+        const double zr[6] = {Rr.rho, 0.5 * Rr.v1, 0.5 * Rr.v2, 0.5 * Rr.v3, 2.0 * Rr.beta,
+                              0.25 * (Rr.v1 * Rr.v1 + Rr.v2 * Rr.v2 + Rr.v3 * Rr.v3)};
+        ec_pair64(zl, zr, hg, a1, a2, a3, f);
+        return;
     }
+    const R srho = L.rho + Rr.rho, sbeta = L.beta + Rr.beta;
+    const R irho = rcp_(srho), ibeta = rcp_(sbeta);
     const R dr = L.rho - Rr.rho;
     const R fr = dr * irho, ur = fr * fr;
     R rho_ln;
@@ -371,7 +501,7 @@ __device__ __forceinline__ R ln_mean(R a, R b, R la, R lb)
     const R s = a + b, d = a - b, fr = d * rcp_(s), u = fr * fr;
     if (u < LogMeanEps<R>::v)
         return (R)0.5 * s * ((R)1 - u * ((R)(1.0 / 3.0) + u * ((R)(4.0 / 45.0) + u * (R)(44.0 / 945.0))));
-    return d / (la - lb);
+    return div_(d, la - lb);
 }
 
 template <typename R>
@@ -379,7 +509,7 @@ __device__ __forceinline__ R inv_ln_mean(R a, R b, R la, R lb)
 {
     const R s = a + b, d = a - b, is = rcp_(s), fr = d * is, u = fr * fr;
     if (u < LogMeanEps<R>::v) return (R)2 * is * ((R)1 + u * ((R)(1.0 / 3.0) + u * ((R)0.2 + u * (R)(1.0 / 7.0))));
-    return (la - lb) / d;
+    return div_(la - lb, d);
 }
 
 // Entropy-stable flux with matrix dissipation (Winters, Derigs, Gassner and
@@ -400,7 +530,7 @@ __device__ __forceinline__ void flux_matrix(const Prim<R> &L, const Prim<R> &Rr,
 {
     const ECNode<R> zl = ec_node(L), zr = ec_node(Rr);
     flux_ec(zl, zr, hg, s1, s2, s3, f);
-    const R s = sqrt(s1 * s1 + s2 * s2 + s3 * s3);
+    const R s = sqrt_(s1 * s1 + s2 * s2 + s3 * s3);
     const R is = rcp_(s);
     const R n1 = s1 * is, n2 = s2 * is, n3 = s3 * is;
     const R rho_h = ln_mean(zl.rho, zr.rho, zl.lrho, zr.lrho);
@@ -409,7 +539,7 @@ __device__ __forceinline__ void flux_matrix(const Prim<R> &L, const Prim<R> &Rr,
     const R v1 = (R)0.5 * (L.v1 + Rr.v1), v2 = (R)0.5 * (L.v2 + Rr.v2), v3 = (R)0.5 * (L.v3 + Rr.v3);
     const R qL = L.v1 * L.v1 + L.v2 * L.v2 + L.v3 * L.v3, qR = Rr.v1 * Rr.v1 + Rr.v2 * Rr.v2 + Rr.v3 * Rr.v3;
     const R v2h = (R)2 * (v1 * v1 + v2 * v2 + v3 * v3) - (R)0.5 * (qL + qR);
-    const R a_h = sqrt(gamma * p_h / rho_h);
+    const R a_h = sqrt_(div_(gamma * p_h, rho_h));
     const R h_h = gamma * hg * ib_ln + (R)0.5 * v2h;
     const R vn = v1 * n1 + v2 * n2 + v3 * n3;
     // [[w]]: (gamma-1) [[ln rho]] + [[ln beta]] enters w_0 through 2 hg = 1/(gamma-1)
@@ -424,7 +554,7 @@ __device__ __forceinline__ void flux_matrix(const Prim<R> &L, const Prim<R> &Rr,
     const R c1 = dw[0] + r1[1] * dw[1] + r1[2] * dw[2] + r1[3] * dw[3] + r1[4] * dw[4];
     const R c5 = dw[0] + r5[1] * dw[1] + r5[2] * dw[2] + r5[3] * dw[3] + r5[4] * dw[4];
     const R c2 = dw[0] + v1 * dw[1] + v2 * dw[2] + v3 * dw[3] + (R)0.5 * v2h * dw[4];
-    const R T15 = rho_h / ((R)2 * gamma), T2 = rho_h * (gamma - (R)1) / gamma;
+    const R T15 = div_(rho_h, (R)2 * gamma), T2 = div_(rho_h * (gamma - (R)1), gamma);
     const R k1 = fabs(vn - a_h) * T15 * c1, k5 = fabs(vn + a_h) * T15 * c5;
     const R l2 = fabs(vn);
     const R k2 = l2 * T2 * c2;
@@ -465,7 +595,7 @@ __device__ __forceinline__ void split_node(const Prim<R> &q, R z[kSplitSlots])
         z[5] = c.lrho;
         z[6] = c.lbeta;
     } else if constexpr (FORM == HS3D_VOL_IR) {
-        const R z1 = sqrt(q.rho / q.p), z5 = sqrt(q.rho * q.p);
+        const R z1 = sqrt_(div_(q.rho, q.p)), z5 = sqrt_(q.rho * q.p);
         z[0] = z1;
         z[1] = z1 * q.v1;
         z[2] = z1 * q.v2;
@@ -550,7 +680,7 @@ __device__ __forceinline__ void flux_ir(const R *L, const R *Rr, R gamma, R hg, 
     const R p1 = z5a * iz1a;
     const R ig = rcp_(gamma);
     const R p2 = h * ((gamma + (R)1) * ig) * z5ln * iz1ln + h * ((gamma - (R)1) * ig) * p1;
-    const R hh = (R)2 * hg * gamma * p2 / rho + h * (v1 * v1 + v2 * v2 + v3 * v3);
+    const R hh = div_((R)2 * hg * gamma * p2, rho) + h * (v1 * v1 + v2 * v2 + v3 * v3);
     const R m = rho * (v1 * a1 + v2 * a2 + v3 * a3);
     f[0] = m;
     f[1] = m * v1 + p1 * a1;
@@ -572,6 +702,85 @@ __device__ __forceinline__ void split_pair(const R *L, const R *Rr, R gamma, R h
         flux_ir(L, Rr, gamma, hg, a1, a2, a3, f);
     } else {
         flux_avg_product<FORM>(L, Rr, a1, a2, a3, f);
+    }
+}
+
+// ------------------------------------------------------------------ split forms in FP64
+//
+// Per-node inputs scaled by powers of two (exact), so that the arithmetic
+// means of a pair are plain sums:
+//   EC         rho, v/2, rho/p, |v|^2/4                 (ec_pair64)
+//   KG         rho/2, v/2, p/2, e/2
+//   PIROZZOLI  rho/2, v/2, p/2, h/2
+//   DUCROS     rho/2, v/2, p/2, (rho e + p)/2
+//   MORINISHI  rho/2, v/2, p/2, |v|^2/4
+//   IR         as split_node
+template <int FORM>
+constexpr int split_slots64()
+{
+    return FORM == HS3D_VOL_IR ? 7 : 6;
+}
+
+template <int FORM>
+__device__ __forceinline__ void split_node64(const Prim<double> &q, double *z)
+{
+    if constexpr (FORM == HS3D_VOL_IR) {
+        split_node<FORM>(q, z);
+    } else {
+        z[1] = 0.5 * q.v1;
+        z[2] = 0.5 * q.v2;
+        z[3] = 0.5 * q.v3;
+        if constexpr (FORM == HS3D_VOL_EC) {
+            z[0] = q.rho;
+            z[4] = div_(q.rho, q.p);
+            z[5] = z[1] * z[1] + z[2] * z[2] + z[3] * z[3];
+        } else {
+            z[0] = 0.5 * q.rho;
+            z[4] = 0.5 * q.p;
+            if constexpr (FORM == HS3D_VOL_KG) z[5] = 0.5 * (q.E * q.ir);
+            else if constexpr (FORM == HS3D_VOL_PIROZZOLI) z[5] = 0.5 * ((q.E + q.p) * q.ir);
+            else if constexpr (FORM == HS3D_VOL_DUCROS) z[5] = 0.5 * (q.E + q.p);
+            else z[5] = z[1] * z[1] + z[2] * z[2] + z[3] * z[3];
+        }
+    }
+}
+
+template <int FORM>
+__device__ __forceinline__ void split_pair64(const double *L, const double *Rr, double gamma, double hg, double a1,
+                                             double a2, double a3, double f[5])
+{
+    if constexpr (FORM == HS3D_VOL_EC) {
+        ec_pair64(L, Rr, hg, a1, a2, a3, f);
+    } else if constexpr (FORM == HS3D_VOL_IR) {
+        flux_ir(L, Rr, gamma, hg, a1, a2, a3, f);
+    } else {
+        const double p = L[4] + Rr[4];
+        const double m1 = L[1] + Rr[1], m2 = L[2] + Rr[2], m3 = L[3] + Rr[3];
+        if constexpr (FORM == HS3D_VOL_MORINISHI) {
+            const double vaL = L[1] * a1 + L[2] * a2 + L[3] * a3, vaR = Rr[1] * a1 + Rr[2] * a2 + Rr[3] * a3;
+            const double m = 2.0 * (L[0] * vaL + Rr[0] * vaR);
+            f[0] = m;
+            f[1] = m * m1 + p * a1;
+            f[2] = m * m2 + p * a2;
+            f[3] = m * m3 + p * a3;
+            f[4] = m * (L[5] + Rr[5]) + (2.0 + 4.0 * hg) * (L[4] * vaL + Rr[4] * vaR);
+        } else {
+            const double va = m1 * a1 + m2 * a2 + m3 * a3;
+            const double m = (L[0] + Rr[0]) * va, w = L[5] + Rr[5];
+            f[0] = m;
+            if constexpr (FORM == HS3D_VOL_DUCROS) {
+                const double va2 = 2.0 * va;
+                f[1] = (L[0] * L[1] + Rr[0] * Rr[1]) * va2 + p * a1;
+                f[2] = (L[0] * L[2] + Rr[0] * Rr[2]) * va2 + p * a2;
+                f[3] = (L[0] * L[3] + Rr[0] * Rr[3]) * va2 + p * a3;
+                f[4] = w * va;
+            } else {
+                f[1] = m * m1 + p * a1;
+                f[2] = m * m2 + p * a2;
+                f[3] = m * m3 + p * a3;
+                f[4] = FORM == HS3D_VOL_KG ? m * w + p * va : m * w;
+            }
+        }
     }
 }
 

@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(256) k_lambda(const __grid_constant__ Batch b,
         if (!(q.rho > (R)0) || !(q.p > (R)0)) {
             it.clk->bad = 1;
         } else {
-            const R c = sqrt(P.gamma * q.p / q.rho);
+            const R c = sound_speed(q, P.gamma);
             const R *JA = lambda_metric<R>(it) + (size_t)e * 9 * n3 + p;
             R iJ;
             if constexpr (sizeof(R) == 8) iJ = it.invJ[(size_t)e * n3 + p];
@@ -75,12 +75,22 @@ __global__ void __launch_bounds__(256) k_lambda(const __grid_constant__ Batch b,
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 const R a1 = JA[(d * 3) * n3], a2 = JA[(d * 3 + 1) * n3], a3 = JA[(d * 3 + 2) * n3];
-                const R an = sqrt(a1 * a1 + a2 * a2 + a3 * a3);
-                sc += (fabs(a1 * q.v1 + a2 * q.v2 + a3 * q.v3) + c * an) * iJ;
-                sv += (an * iJ) * (an * iJ);
+                const R s2 = a1 * a1 + a2 * a2 + a3 * a3, an = sqrt_(s2);
+                if constexpr (sizeof(R) == 8) {
+                    sc += fabs(a1 * q.v1 + a2 * q.v2 + a3 * q.v3) + c * an;
+                    sv += s2;
+                } else {
+                    sc += (fabs(a1 * q.v1 + a2 * q.v2 + a3 * q.v3) + c * an) * iJ;
+                    sv += (an * iJ) * (an * iJ);
+                }
             }
-            lc = widen<R>(sc);
-            if (ns) lv = widen<R>(P.mu * sv / q.rho);
+            if constexpr (sizeof(R) == 8) {
+                lc = sc * iJ;
+                if (ns) lv = P.mu * sv * (iJ * iJ) * q.ir;
+            } else {
+                lc = widen<R>(sc);
+                if (ns) lv = widen<R>(P.mu * sv / q.rho);
+            }
             active = true;
         }
     }
