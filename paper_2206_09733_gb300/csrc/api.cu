@@ -86,7 +86,7 @@ size_t mesh_bytes(int N, long long E, int nodes)
     size_t scratch = sizeof(double) * (3 * (size_t)E * 5 * n2 + (size_t)E * 12 * n3);
     // Gauss-Legendre meshes hold Gauss-Lobatto temporaries while they are built
     size_t build = (nodes == HS3D_NODES_GAUSS) ? sizeof(double) * ((size_t)E * 21 * n3 + 9 * (size_t)E * n2) : 0;
-    return geo + scratch + build + sizeof(Clock) + 4096 * 7 * sizeof(double);
+    return geo + scratch + build + sizeof(Clock) + 7 * kDiagMaxBlocks * sizeof(double);
 }
 
 hs3d_status check_mesh_cfg(const hs3d_mesh *m, const hs3d_solver_cfg *c)
@@ -118,7 +118,7 @@ static hs3d_status mesh_alloc(hs3d_mesh *m)
         {(void **)&m->fstar, sizeof(double) * 3 * E * 5 * n2},
         {(void **)&m->grad, sizeof(double) * E * 12 * n3},
         {(void **)&m->clk, sizeof(Clock)},
-        {(void **)&m->diag_partials, sizeof(double) * 4096 * 7},
+        {(void **)&m->diag_partials, sizeof(double) * 7 * kDiagMaxBlocks},
     };
     for (auto &a : allocs) {
         if (a.bytes == 0) continue;
@@ -549,9 +549,8 @@ hs3d_status hs3d_diagnostics(const hs3d_mesh *m, const hs3d_solver_cfg *c, const
     hs3d_status st = check_ptr(u, "u");
     if (st == HS3D_OK && !out) st = fail(HS3D_ERR_INVALID, "out is NULL");
     if (st != HS3D_OK) return st;
-    Item it = make_item(m, c, u, nullptr, nullptr);
-    int nb = diagnostics_blocks(m->N, m->E);
-    cudaError_t e = launch_diagnostics(m->N, it, dudt, m->diag_partials, nb, out, (cudaStream_t)stream);
+    cudaError_t e = launch_diagnostics(m->N, m->nodes, m->E, c ? c->gamma : 1.4, m->J, u, dudt, m->diag_partials, out,
+                                       (cudaStream_t)stream);
     return e == cudaSuccess ? HS3D_OK : cuda_fail(e, "diagnostics launch");
 }
 

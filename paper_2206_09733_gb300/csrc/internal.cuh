@@ -447,9 +447,15 @@ cudaError_t launch_metric_lo(const double *Ja, const float *Jaf, float *Jalo, lo
 // Low-storage RK schemes (HS3D_TIME_*): stage count and the stage's (A_k, B_k).
 int rk_stages(int scheme);
 void rk_coeffs(int scheme, int k, double *A, double *B);
-cudaError_t launch_diagnostics(int N, const Item &it, const double *dudt, double *partials, int nblocks, double *out,
-                               cudaStream_t s);
-int diagnostics_blocks(int N, int E);
+// Quadrature diagnostics of E elements of degree N on the given node family:
+// J [E][n3], u and (or NULL) dudt [E][5][n3], partials at least
+// kDiagMaxBlocks x 7 doubles, out 7 doubles (all device).
+constexpr int kDiagMaxBlocks = 8 * 152;
+struct DiagWeights {
+    double w[kMaxn];
+};
+cudaError_t launch_diagnostics(int N, int nodes, long long E, double gamma, const double *J, const double *u,
+                               const double *dudt, double *partials, double *out, cudaStream_t s);
 
 // One-time per-N set-up that must not happen inside a stream capture
 // (shared-memory attributes, operator tables).

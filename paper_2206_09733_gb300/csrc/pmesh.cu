@@ -558,9 +558,8 @@ hs3d_status hs3d_pmesh_diagnostics(const hs3d_pmesh *pm, const hs3d_solver_cfg *
     }
     for (size_t k = 0; k < pm->b.size() && e == cudaSuccess; ++k) {
         const auto &bk = pm->b[k];
-        const Item it = make_item(bk.m, c, u + bk.base, nullptr, nullptr);
-        e = launch_diagnostics(bk.N, it, dudt ? dudt + bk.base : nullptr, bk.m->diag_partials,
-                               diagnostics_blocks(bk.N, bk.E), pm->diag_tmp + 7 * k, s);
+        e = launch_diagnostics(bk.N, HS3D_NODES_LOBATTO, bk.E, c->gamma, bk.m->J, u + bk.base,
+                               dudt ? dudt + bk.base : nullptr, bk.m->diag_partials, pm->diag_tmp + 7 * k, s);
     }
     if (e == cudaSuccess) {
         k_pdiag_sum<<<1, 1, 0, s>>>(pm->diag_tmp, (int)pm->b.size(), out);

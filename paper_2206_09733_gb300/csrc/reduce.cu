@@ -229,96 +229,100 @@ cudaError_t launch_dt_finalize(int N, const Batch &b, int mode, int slot, cudaSt
 
 // ------------------------------------------------------------------ diagnostics
 
+// One block per 256 nodes until every SM has eight (small meshes: a node's
+// entropy variables are a long serial FP64 chain, two logarithms among it, so
+// a thread takes one node and the chains run side by side), from there a
+// fixed grid whose threads walk on.  Residual and sums of 4^3 elements of
+// N = 3: 100 -> 35 us against blocks of 2048 nodes (two blocks, 73 us).
 constexpr int kDiagThreads = 256;
 
-int diagnostics_blocks(int N, int E)
+int diagnostics_blocks(int N, long long E)
 {
-    long long total = (long long)E * (N + 1) * (N + 1) * (N + 1);
-    long long blocks = (total + kDiagThreads * 8 - 1) / (kDiagThreads * 8);
-    if (blocks > 4096) blocks = 4096;
-    if (blocks < 1) blocks = 1;
-    return (int)blocks;
+    const long long total = E * (N + 1) * (N + 1) * (N + 1);
+    const long long blocks = (total + kDiagThreads - 1) / kDiagThreads;
+    return (int)(blocks > kDiagMaxBlocks ? kDiagMaxBlocks : blocks < 1 ? 1 : blocks);
 }
 
-// Fixed-order block reduction of 7 values per thread.
-__device__ void block_sum7(double v[7], double *sm)
-{
-    for (int k = 0; k < 7; ++k) sm[k * kDiagThreads + threadIdx.x] = v[k];
-    __syncthreads();
-    for (int w = kDiagThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int k = 0; k < 7; ++k) sm[k * kDiagThreads + threadIdx.x] += sm[k * kDiagThreads + threadIdx.x + w];
-        __syncthreads();
-    }
-    for (int k = 0; k < 7; ++k) v[k] = sm[k * kDiagThreads];
-}
-
-__global__ void __launch_bounds__(kDiagThreads) k_diag_partial(int n, Item it, const double *__restrict__ dudt,
-                                                                const Ops *__restrict__ ops, double *partials)
+// Per-block sums to partials[k][block], k < 7: warp k sums quantity k of the
+// block's 256 threads (eight values per lane, then a shuffle tree).
+__global__ void __launch_bounds__(kDiagThreads) k_diag_partial(int n, long long total, double g, const DiagWeights W,
+                                                               const double *__restrict__ J,
+                                                               const double *__restrict__ ua,
+                                                               const double *__restrict__ dudt,
+                                                               double *__restrict__ partials)
 {
     __shared__ double sm[7 * kDiagThreads];
     const int n3 = n * n * n;
-    const long long total = (long long)it.E * n3;
-    const long long per = (total + gridDim.x - 1) / gridDim.x;
-    const long long begin = blockIdx.x * per, end = min(total, begin + per);
     double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    const double g = it.gamma;
-    for (long long t = begin + threadIdx.x; t < end; t += blockDim.x) {
+    for (long long t = (long long)blockIdx.x * kDiagThreads + threadIdx.x; t < total;
+         t += (long long)gridDim.x * kDiagThreads) {
         const long long e = t / n3;
         const int p = (int)(t - e * n3);
         const int i = p % n, j = (p / n) % n, k = p / (n * n);
-        const double wq = it.J[e * n3 + p] * ops->w[i] * ops->w[j] * ops->w[k];
-        const double *U = it.u + e * 5 * n3 + p;
+        const double wq = J[t] * W.w[i] * W.w[j] * W.w[k];
+        const double *U = ua + e * 5 * n3 + p;
+        double u[5];
+#pragma unroll
+        for (int v = 0; v < 5; ++v) u[v] = U[v * n3];
         if (dudt) {
             const double *R = dudt + e * 5 * n3 + p;
-            double u[5], r[5];
+            double r[5];
+#pragma unroll
+            for (int v = 0; v < 5; ++v) r[v] = R[v * n3];
+            const Prim<double> q = prim_from_u<double>(u, g - 1.0);
+            const double vv = q.v1 * q.v1 + q.v2 * q.v2 + q.v3 * q.v3;
+            const double s = log(q.p) - g * log(q.rho);
+            const double rp = (g - 1.0) * div_(q.rho, q.p);
+            const double w[5] = {g - s - 0.5 * rp * vv, rp * q.v1, rp * q.v2, rp * q.v3, -rp};
+#pragma unroll
             for (int v = 0; v < 5; ++v) {
-                u[v] = U[v * n3];
-                r[v] = R[v * n3];
                 acc[v] += wq * r[v];
-            }
-            double ir = 1.0 / u[0];
-            double v1 = u[1] * ir, v2 = u[2] * ir, v3 = u[3] * ir;
-            double vv = v1 * v1 + v2 * v2 + v3 * v3;
-            double pr = (g - 1.0) * (u[4] - 0.5 * u[0] * vv);
-            double s = log(pr) - g * log(u[0]);
-            double rp = (g - 1.0) * u[0] / pr;
-            double w[5] = {g - s - 0.5 * rp * vv, rp * v1, rp * v2, rp * v3, -rp};
-            for (int v = 0; v < 5; ++v) {
-                double tv = wq * w[v] * r[v];
+                const double tv = wq * w[v] * r[v];
                 acc[5] += tv;
                 acc[6] += fabs(tv);
             }
         } else {
-            for (int v = 0; v < 5; ++v) acc[v] += wq * U[v * n3];
+#pragma unroll
+            for (int v = 0; v < 5; ++v) acc[v] += wq * u[v];
         }
     }
-    block_sum7(acc, sm);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 7; ++k) partials[blockIdx.x * 7 + k] = acc[k];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) sm[k * kDiagThreads + threadIdx.x] = acc[k];
+    __syncthreads();
+    const int col = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (col >= 7) return;
+    double a = 0.0;
+#pragma unroll
+    for (int j = 0; j < kDiagThreads / 32; ++j) a += sm[col * kDiagThreads + 32 * j + lane];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
+    if (lane == 0) partials[(size_t)col * gridDim.x + blockIdx.x] = a;
 }
 
-__global__ void __launch_bounds__(kDiagThreads) k_diag_final(const double *partials, int nblocks, double *out)
+// out[k] = sum of partials[k][.] in a fixed order, one warp per quantity.
+__global__ void __launch_bounds__(7 * 32) k_diag_final(const double *partials, int nblocks, double *out)
 {
-    __shared__ double sm[7 * kDiagThreads];
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-        for (int k = 0; k < 7; ++k) acc[k] += partials[b * 7 + k];
-    block_sum7(acc, sm);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 7; ++k) out[k] = acc[k];
+    pdl_wait();
+    const int col = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double a = 0.0;
+    for (int b = lane; b < nblocks; b += 32) a += partials[(size_t)col * nblocks + b];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
+    if (lane == 0) out[col] = a;
 }
 
-cudaError_t launch_diagnostics(int N, const Item &it, const double *dudt, double *partials, int nblocks, double *out,
-                               cudaStream_t s)
+cudaError_t launch_diagnostics(int N, int nodes, long long E, double gamma, const double *J, const double *u,
+                               const double *dudt, double *partials, double *out, cudaStream_t s)
 {
-    const Ops *ops = device_ops(N, it.gauss ? HS3D_NODES_GAUSS : HS3D_NODES_LOBATTO);
-    if (!ops) return cudaErrorMemoryAllocation;
-    k_diag_partial<<<nblocks, kDiagThreads, 0, s>>>(N + 1, it, dudt, ops, partials);
-    cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess) return err;
-    k_diag_final<<<1, kDiagThreads, 0, s>>>(partials, nblocks, out);
-    return cudaGetLastError();
+    DiagWeights W{};
+    const Ops &o = host_ops(N, nodes);
+    for (int k = 0; k <= N; ++k) W.w[k] = o.w[k];
+    const int nblocks = diagnostics_blocks(N, E);
+    k_diag_partial<<<nblocks, kDiagThreads, 0, s>>>(N + 1, E * (N + 1) * (N + 1) * (N + 1), gamma, W, J, u, dudt,
+                                                    partials);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = launch_pdl(k_diag_final, 1, 7 * 32, 0, s, partials, nblocks, out);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace hs3d
