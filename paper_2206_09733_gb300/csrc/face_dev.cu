@@ -266,10 +266,12 @@ __global__ void __launch_bounds__(256, 4) k_face_dev(const __grid_constant__ Bat
 }
 
 template <int N, bool NS, bool TWO>
-static cudaError_t face_dev_launch3(int flux, const Batch &b, unsigned blocks, cudaStream_t s)
+static cudaError_t face_dev_launch3(int flux, const Batch &b, long long total, cudaStream_t s)
 {
-    const unsigned grid = b.persistent ? persistent_grid(k_face_dev<N, NS, TWO>, 256, 0, blocks) : blocks;
-    return launch_pdl(k_face_dev<N, NS, TWO>, grid, 256, 0, s, b, flux);
+    const int threads = spread_threads(total);
+    const unsigned blocks = (unsigned)((total + threads - 1) / threads);
+    const unsigned grid = b.persistent ? persistent_grid(k_face_dev<N, NS, TWO>, threads, 0, blocks) : blocks;
+    return launch_pdl(k_face_dev<N, NS, TWO>, grid, threads, 0, s, b, flux);
 }
 
 template <int N>
@@ -278,11 +280,10 @@ static cudaError_t face_dev_launch(int physics, int flux, const Batch &b, cudaSt
     constexpr int n2 = (N + 1) * (N + 1);
     const long long total = b.total_faces * n2;
     if (total == 0) return cudaSuccess;
-    const unsigned blocks = (unsigned)((total + 255) / 256);
     const bool two = (flux == HS3D_FLUX_EC || flux == HS3D_FLUX_MATRIX);
     if (physics == HS3D_NS)
-        return two ? face_dev_launch3<N, true, true>(flux, b, blocks, s) : face_dev_launch3<N, true, false>(flux, b, blocks, s);
-    return two ? face_dev_launch3<N, false, true>(flux, b, blocks, s) : face_dev_launch3<N, false, false>(flux, b, blocks, s);
+        return two ? face_dev_launch3<N, true, true>(flux, b, total, s) : face_dev_launch3<N, true, false>(flux, b, total, s);
+    return two ? face_dev_launch3<N, false, true>(flux, b, total, s) : face_dev_launch3<N, false, false>(flux, b, total, s);
 }
 
 cudaError_t launch_face_dev(int N, int physics, int flux, const Batch &b, cudaStream_t s)

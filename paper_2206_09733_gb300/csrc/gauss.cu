@@ -472,17 +472,18 @@ static cudaError_t face_gauss(int physics, int flux, const Batch &b, cudaStream_
     if (total == 0) return cudaSuccess;
     const Ops *ops = device_ops(N, HS3D_NODES_GAUSS);
     if (!ops) return cudaErrorMemoryAllocation;
-    const unsigned blocks = (unsigned)((total + 255) / 256);
-    if (physics == HS3D_NS) k_face_gauss<N, R, true><<<blocks, 256, 0, s>>>(b, ops, flux);
-    else k_face_gauss<N, R, false><<<blocks, 256, 0, s>>>(b, ops, flux);
+    const int threads = spread_threads(total);
+    const unsigned blocks = (unsigned)((total + threads - 1) / threads);
+    if (physics == HS3D_NS) k_face_gauss<N, R, true><<<blocks, threads, 0, s>>>(b, ops, flux);
+    else k_face_gauss<N, R, false><<<blocks, threads, 0, s>>>(b, ops, flux);
     return cudaGetLastError();
 }
 
 template <int N>
-static int gauss_epb(int prec, int which)
+static int gauss_epb(int prec, int which, long long elems)
 {
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
-    int epb = elems_per_block_p(N, prec, which);
+    int epb = spread_elems(elems_per_block_p(N, prec, which), elems);
     if (epb * n3 > gauss_threads<N>()) epb = gauss_threads<N>() / n3;
     return epb < 1 ? 1 : epb;
 }
@@ -492,7 +493,7 @@ static cudaError_t grad_gauss(const Batch &b, cudaStream_t s)
 {
     constexpr int n = N + 1, n3 = n * n * n;
     if (b.total_elems == 0) return cudaSuccess;
-    const int epb = gauss_epb<N>(sizeof(R) == 4 ? HS3D_MIXED32 : HS3D_FP64, 0);
+    const int epb = gauss_epb<N>(sizeof(R) == 4 ? HS3D_MIXED32 : HS3D_FP64, 0, b.total_elems);
     const size_t smem = sizeof(R) * (((n * n + 1) & ~1) + (size_t)epb * grad_gauss_per_elem<N>());
     const unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);
     const Ops *ops = device_ops(N, HS3D_NODES_GAUSS);
@@ -506,7 +507,7 @@ static cudaError_t volume_gauss(const Batch &b, int stage, double rkA, double rk
 {
     constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
     if (b.total_elems == 0) return cudaSuccess;
-    const int epb = gauss_epb<N>(sizeof(R) == 4 ? HS3D_MIXED32 : HS3D_FP64, 1);
+    const int epb = gauss_epb<N>(sizeof(R) == 4 ? HS3D_MIXED32 : HS3D_FP64, 1, b.total_elems);
     const size_t smem = sizeof(R) * (((n * n + 1) & ~1) + (size_t)epb * (15 * n3 + 30 * n2));
     const unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);
     const Ops *ops = device_ops(N, HS3D_NODES_GAUSS);

@@ -256,7 +256,7 @@ static cudaError_t grad_dev_launch(const Batch &b, cudaStream_t s)
 {
     constexpr int n = N + 1, n3 = n * n * n;
     if (b.total_elems == 0) return cudaSuccess;
-    int epb = elems_per_block_p(N, HS3D_MIXED32, 0);
+    int epb = spread_elems(elems_per_block_p(N, HS3D_MIXED32, 0), b.total_elems);
     if (epb * n3 > grad_dev_threads<N>()) epb = grad_dev_threads<N>() / n3;
     const int threads = epb * n3;
     const size_t smem = sizeof(float) * (((n * n + 3) & ~3) + (size_t)epb * grad_dev_per_elem<N>());

@@ -166,12 +166,13 @@ cudaError_t launch_lambda(int N, int prec, int physics, const Batch &b, int slot
     int n3 = (N + 1) * (N + 1) * (N + 1);
     long long total = b.total_elems * n3;
     if (total == 0) return cudaSuccess;
-    unsigned blocks = (unsigned)((total + 255) / 256);
+    const int threads = spread_threads(total);
+    unsigned blocks = (unsigned)((total + threads - 1) / threads);
     int ns = physics == HS3D_NS;
 #define HS3D_LAM(K)                                                                                 \
     case K:                                                                                         \
-        if (prec == HS3D_FP64) k_lambda<K, double><<<blocks, 256, 0, s>>>(b, ns, slot);             \
-        else k_lambda<K, float><<<blocks, 256, 0, s>>>(b, ns, slot);                                \
+        if (prec == HS3D_FP64) k_lambda<K, double><<<blocks, threads, 0, s>>>(b, ns, slot);         \
+        else k_lambda<K, float><<<blocks, threads, 0, s>>>(b, ns, slot);                            \
         break;
     switch (N) {
         HS3D_LAM(1) HS3D_LAM(2) HS3D_LAM(3) HS3D_LAM(4) HS3D_LAM(5) HS3D_LAM(6) HS3D_LAM(7)

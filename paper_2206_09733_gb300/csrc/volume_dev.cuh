@@ -788,7 +788,7 @@ template <int N, bool NS, int FORM>
 static cudaError_t vol_dev_launch2(const Batch &b, int stage, double rkA, double rkB, int lam_slot, cudaStream_t s)
 {
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
-    int epb = elems_per_block_p(N, HS3D_MIXED32, 1);
+    int epb = spread_elems(elems_per_block_p(N, HS3D_MIXED32, 1), b.total_elems);
     if (epb * n3 > dev_threads<N>()) epb = dev_threads<N>() / n3;
     if (epb < 1) epb = 1;
     const int threads = ((epb * n3) + 31) & ~31;
