@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kAFaceThreads) k_amortar(const AFace *__restri
                                                            const MortarOps *__restrict__ mo, APhys P,
                                                            double *__restrict__ out)
 {
-    constexpr int NV = (MODE == 1 && NS) ? 17 : 5;   // conservative state (+ 12 gradients) per trace point
+    constexpr int NV = (MODE == 1 && NS) ? 5 + kVisc : 5;   // conservative state (+ viscous stress) per trace point
     constexpr int NO = MODE == 0 ? 4 : 5;
     __shared__ double tr[2][NV][kAFaceThreads];
     __shared__ double sn[2][3][kAFaceThreads];
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(kAFaceThreads) k_amortar(const AFace *__restri
             const int n3 = sh[k].n3;
             for (int v = 0; v < 5; ++v) tr[k][v][p] = u[5 * nb + (size_t)v * n3 + node];
             if constexpr (MODE == 1 && NS)
-                for (int q = 0; q < 12; ++q) tr[k][5 + q][p] = grad[12 * nb + (size_t)q * n3 + node];
+                for (int q = 0; q < kVisc; ++q) tr[k][5 + q][p] = grad[kVisc * nb + (size_t)q * n3 + node];
             if constexpr (MODE == 1)
                 for (int c = 0; c < 3; ++c) sn[k][c][p] = Jaall[9 * nb + (size_t)(d * 3 + c) * n3 + node];
         }
@@ -333,8 +333,8 @@ __global__ void __launch_bounds__(kAFaceThreads) k_amortar(const AFace *__restri
             if constexpr (NS) {
                 double fl[5], fr[5];
                 const Prim<double> pL = mortar_prim(w[0], P.gm1), pR = mortar_prim(w[1], P.gm1);
-                visc_flux(pL, &w[0][5], P.mu, P.kappa, s3[0], s3[1], s3[2], fl);
-                visc_flux(pR, &w[1][5], P.mu, P.kappa, s3[0], s3[1], s3[2], fr);
+                visc_flux(pL, &w[0][5], s3[0], s3[1], s3[2], fl);
+                visc_flux(pR, &w[1][5], s3[0], s3[1], s3[2], fr);
                 for (int v = 1; v < 5; ++v) fs[v] -= 0.5 * (fl[v] + fr[v]);
             }
             for (int v = 0; v < 5; ++v) fm[v][p] = fs[v];
@@ -367,7 +367,8 @@ __global__ void __launch_bounds__(kAFaceThreads) k_amortar(const AFace *__restri
 // ------------------------------------------------------------------ BR1 gradients
 
 // J grad q_c = sum_d D_d (Ja^d_c q) + sum_faces (q*_e - q_in) (+-Ja^d_c)/w_end,
-// q = (v1, v2, v3, T), q*_e from the mortar kernel; grad [12][n3] at 12 noff[e].
+// q = (v1, v2, v3, T), q*_e from the mortar kernel, stored as viscous stress and
+// heat flux [kVisc][n3] at kVisc noff[e].
 __global__ void __launch_bounds__(512) k_agrad(const int *__restrict__ elems, const int *__restrict__ P3, const long long *__restrict__ noff,
                         const long long *__restrict__ fnoff, const AOps *__restrict__ ops,
                         const double *__restrict__ u, const double *__restrict__ Jaall,
@@ -394,38 +395,31 @@ __global__ void __launch_bounds__(512) k_agrad(const int *__restrict__ elems, co
     }
     __syncthreads();
     if (!live) return;
-    double G[12];
-    for (int v = 0; v < 4; ++v)
-        for (int c = 0; c < 3; ++c) {
-            double acc = 0.0;
-            for (int d = 0; d < 3; ++d) {
-                const int nd = s.n[d], st = astride(s, d);
-                const double *Drow = ops->D[nd - 1] + ijk[d] * nd;
-                const int base = p - ijk[d] * st;
-                const double *Jc = sJ + (d * 3 + c) * n3, *qv = sq + v * n3;
-                for (int m = 0; m < nd; ++m) acc += Drow[m] * (Jc[base + m * st] * qv[base + m * st]);
-            }
-            G[v * 3 + c] = acc;
-        }
+    double G[kVisc] = {};
     for (int d = 0; d < 3; ++d) {
-        for (int side = -1; side <= 1; side += 2) {
-            const int at = side > 0 ? s.n[d] - 1 : 0;
-            if (ijk[d] != at) continue;
-            int d0, d1;
-            aface_dirs(d, d0, d1);
-            const int f2 = s.n[d0] * s.n[d1];
-            const int slot = 2 * d + (side > 0 ? 1 : 0);
-            const double *qs = qhat + (size_t)4 * fnoff[6 * e + slot] + ijk[d0] + s.n[d0] * ijk[d1];
-            const double iw = ops->iw0[s.n[d] - 1];
-            for (int v = 0; v < 4; ++v) {
-                const double jump = qs[(size_t)v * f2] - qp[v];
-                for (int c = 0; c < 3; ++c) G[v * 3 + c] += jump * side * sJ[(d * 3 + c) * n3 + p] * iw;
-            }
+        const int nd = s.n[d], st = astride(s, d), i = ijk[d];
+        const double *Drow = ops->D[nd - 1] + i * nd;
+        const int base = p - i * st;
+        const double *J1 = sJ + d * 3 * n3, *J2 = J1 + n3, *J3 = J2 + n3;
+        for (int m = 0; m < nd; ++m) {
+            const int pm = base + m * st;
+            const double Dm = Drow[m];
+            stress_add(G, Dm * J1[pm], Dm * J2[pm], Dm * J3[pm], sq[pm], sq[n3 + pm], sq[2 * n3 + pm], sq[3 * n3 + pm]);
         }
+        if (i != 0 && i != nd - 1) continue;
+        int d0, d1;
+        aface_dirs(d, d0, d1);
+        const int f2 = s.n[d0] * s.n[d1];
+        const int slot = 2 * d + (i != 0 ? 1 : 0);
+        const double *qs = qhat + (size_t)4 * fnoff[6 * e + slot] + ijk[d0] + s.n[d0] * ijk[d1];
+        const double iw = i != 0 ? ops->iw0[nd - 1] : -ops->iw0[nd - 1];
+        stress_add(G, iw * J1[p], iw * J2[p], iw * J3[p], qs[0] - qp[0], qs[f2] - qp[1], qs[2 * f2] - qp[2],
+                   qs[3 * f2] - qp[3]);
     }
-    const double iJ = invJall[nb + p];
-    double *Gout = gradall + 12 * nb + p;
-    for (int k = 0; k < 12; ++k) Gout[(size_t)k * n3] = G[k] * iJ;
+    double t[kVisc];
+    stress_of(G, invJall[nb + p], P.mu, P.kappa, t);
+    double *Gout = gradall + kVisc * nb + p;
+    for (int k = 0; k < kVisc; ++k) Gout[(size_t)k * n3] = t[k];
 }
 
 // ------------------------------------------------------------------ volume + surface + RK
@@ -458,7 +452,7 @@ __global__ void __launch_bounds__(512) k_avol(const int *__restrict__ elems, con
     const long long nb = noff[e];
     const double *Ja = Jaall + 9 * nb;
     int ijk[3] = {0, 0, 0};
-    double w[5] = {0, 0, 0, 0, 0}, G[12] = {};
+    double w[5] = {0, 0, 0, 0, 0}, G[kVisc] = {};
     Prim<double> q{};
     if (live) {
         ijk[0] = p % s.n[0];
@@ -467,7 +461,7 @@ __global__ void __launch_bounds__(512) k_avol(const int *__restrict__ elems, con
         for (int v = 0; v < 5; ++v) w[v] = u[5 * nb + (size_t)v * n3 + p];
         q = prim_from_u<double>(w, P.gm1);
         if (NS)
-            for (int k = 0; k < 12; ++k) G[k] = gradall[12 * nb + (size_t)k * n3 + p];
+            for (int k = 0; k < kVisc; ++k) G[k] = gradall[kVisc * nb + (size_t)k * n3 + p];
         if constexpr (!STD) {
             double z[kSplitSlots];
             split_node<FORM>(q, z);
@@ -482,7 +476,7 @@ __global__ void __launch_bounds__(512) k_avol(const int *__restrict__ elems, con
             for (int c = 0; c < 3; ++c) a[c] = Ja[(size_t)(d * 3 + c) * n3 + p];
             double fe[5], fv[5] = {0, 0, 0, 0, 0};
             euler_flux(q, q.E, a[0], a[1], a[2], fe);
-            if (NS) visc_flux(q, G, P.mu, P.kappa, a[0], a[1], a[2], fv);
+            if (NS) visc_flux(q, G, a[0], a[1], a[2], fv);
             for (int v = 0; v < 5; ++v) own[d][v] = fe[v] - fv[v];
         }
         __syncthreads();   // the previous direction's shared values are consumed
@@ -493,7 +487,7 @@ __global__ void __launch_bounds__(512) k_avol(const int *__restrict__ elems, con
                 for (int c = 0; c < 3; ++c) sA[c * n3 + p] = a[c];
                 if (NS) {
                     double fv[5];
-                    visc_flux(q, G, P.mu, P.kappa, a[0], a[1], a[2], fv);
+                    visc_flux(q, G, a[0], a[1], a[2], fv);
                     for (int v = 1; v < 5; ++v) sV[(v - 1) * n3 + p] = fv[v];
                 }
             }
@@ -921,7 +915,7 @@ hs3d_status aniso_build(const hs3d_mesh_desc *desc, const int *degree3, AnisoMes
         {(void **)&a->Ja, sizeof(double) * 9 * nodes},
         {(void **)&a->J, sizeof(double) * nodes},
         {(void **)&a->invJ, sizeof(double) * nodes},
-        {(void **)&a->grad, sizeof(double) * 12 * nodes},
+        {(void **)&a->grad, sizeof(double) * kVisc * nodes},
         {(void **)&a->fstar, sizeof(double) * 5 * fnodes},
         {(void **)&a->qhat, sizeof(double) * 4 * fnodes},
         {(void **)&a->diag_part, sizeof(double) * 7 * E},

@@ -76,6 +76,11 @@ hs3d_status validate_desc(const hs3d_mesh_desc *d)
     return HS3D_OK;
 }
 
+// Values per node of the gradient scratch (doubles): the Gauss-Legendre kernels
+// keep the twelve gradients, the others (in FP32 also the mortar path's twelve
+// fit) the stress and heat flux.
+static int grad_values(int nodes) { return nodes == HS3D_NODES_GAUSS ? 12 : kVisc; }
+
 size_t mesh_bytes(int N, long long E, int nodes)
 {
     long long n = N + 1, n2 = n * n, n3 = n2 * n;
@@ -83,7 +88,7 @@ size_t mesh_bytes(int N, long long E, int nodes)
     size_t geo = sizeof(double) * (size_t)E * n3 * (3 + 9 + 1 + 1) +
                  sizeof(float) * (size_t)E * n3 * (19 + (nodes == HS3D_NODES_GAUSS ? 5 : 0)) +
                  (sizeof(double) + sizeof(float)) * 3 * (size_t)E * 3 * n2;
-    size_t scratch = sizeof(double) * (3 * (size_t)E * 5 * n2 + (size_t)E * 12 * n3);
+    size_t scratch = sizeof(double) * (3 * (size_t)E * 5 * n2 + (size_t)E * grad_values(nodes) * n3);
     // Gauss-Legendre meshes hold Gauss-Lobatto temporaries while they are built
     size_t build = (nodes == HS3D_NODES_GAUSS) ? sizeof(double) * ((size_t)E * 21 * n3 + 9 * (size_t)E * n2) : 0;
     return geo + scratch + build + sizeof(Clock) + 7 * kDiagMaxBlocks * sizeof(double);
@@ -116,7 +121,7 @@ static hs3d_status mesh_alloc(hs3d_mesh *m)
         {(void **)&m->fnf, sizeof(float) * 3 * E * 3 * n2},
         {(void **)&m->anc, (size_t)112 * E},
         {(void **)&m->fstar, sizeof(double) * 3 * E * 5 * n2},
-        {(void **)&m->grad, sizeof(double) * E * 12 * n3},
+        {(void **)&m->grad, sizeof(double) * E * grad_values(m->nodes) * n3},
         {(void **)&m->clk, sizeof(Clock)},
         {(void **)&m->diag_partials, sizeof(double) * 7 * kDiagMaxBlocks},
     };

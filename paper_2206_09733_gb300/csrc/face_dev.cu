@@ -226,17 +226,17 @@ __device__ __forceinline__ void face_dev_point(const Batch &b, int flux, long lo
         }
     }
     if (NS) {
-        const float *GLp = (const float *)it.grad + (size_t)eL * 12 * n3 + pL;
-        const float *GRp = (const float *)it.grad + (size_t)eR * 12 * n3 + pR;
-        float gl[12], gr[12];
+        const float *GLp = (const float *)it.grad + (size_t)eL * kVisc * n3 + pL;
+        const float *GRp = (const float *)it.grad + (size_t)eR * kVisc * n3 + pR;
+        float gl[kVisc], gr[kVisc];
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
+        for (int k = 0; k < kVisc; ++k) {
             gl[k] = GLp[k * n3];
             gr[k] = GRp[k * n3];
         }
         float vl[5], vr[5];
-        visc_flux(qL, gl, it.muf, it.kappaf, s1, s2, s3, vl);
-        visc_flux(qR, gr, it.muf, it.kappaf, s1, s2, s3, vr);
+        visc_flux(qL, gl, s1, s2, s3, vl);
+        visc_flux(qR, gr, s1, s2, s3, vr);
 #pragma unroll
         for (int v = 1; v < 5; ++v) {
             const float h = 0.5f * (vr[v] - vl[v]);

@@ -11,7 +11,8 @@
 //
 // k_grad: BR1 gradients of q = (v1, v2, v3, T), T = p/rho (Bassi & Rebay 1997):
 //   J grad q_c = sum_d D_d (Ja^d_c q) + sum_faces (1/w_end) (q* - q_in) (+-Ja^d_c),
-//   q* = (q_in + q_out)/2.  Element per thread group, node per thread.
+//   q* = (q_in + q_out)/2, stored as viscous stress and heat flux (kVisc
+// values per node).  Element per thread group, node per thread.
 //
 // Both are bound by the FP64 pipe, so they are written for few FP64
 // instructions per warp: one reciprocal per state (rcp_fast, shared by
@@ -72,12 +73,12 @@ __global__ void __launch_bounds__(kFaceThreads) k_face(const __grid_constant__ B
     }
     const double *Fn = it.fn + (size_t)f * 3 * n2 + ab;
     const double s1 = Fn[0], s2 = Fn[n2], s3 = Fn[2 * n2];
-    double gl[12], gr[12];
+    double gl[kVisc], gr[kVisc];
     if (NS) {
-        const double *GL = (const double *)it.grad + (size_t)eL * 12 * n3 + pL;
-        const double *GR = (const double *)it.grad + (size_t)eR * 12 * n3 + pR;
+        const double *GL = (const double *)it.grad + (size_t)eL * kVisc * n3 + pL;
+        const double *GR = (const double *)it.grad + (size_t)eR * kVisc * n3 + pR;
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
+        for (int k = 0; k < kVisc; ++k) {
             gl[k] = GL[k * n3];
             gr[k] = GR[k * n3];
         }
@@ -92,8 +93,8 @@ __global__ void __launch_bounds__(kFaceThreads) k_face(const __grid_constant__ B
     else flux_roe(qL, uL, qR, uR, P.gamma, s1, s2, s3, fs);
     if (NS) {
         double fl[5], fr[5];
-        visc_flux(qL, gl, P.mu, P.kappa, s1, s2, s3, fl);
-        visc_flux(qR, gr, P.mu, P.kappa, s1, s2, s3, fr);
+        visc_flux(qL, gl, s1, s2, s3, fl);
+        visc_flux(qR, gr, s1, s2, s3, fr);
 #pragma unroll
         for (int v = 1; v < 5; ++v) fs[v] -= 0.5 * (fl[v] + fr[v]);
     }
@@ -154,7 +155,6 @@ __global__ void __launch_bounds__(grad_threads<N>()) k_grad(const __grid_constan
     double *q = sE + (size_t)le * PER_ELEM;
     double *ja = q + 4 * n3;
     double *qn = ja + 9 * n3;
-    double qin[4];
     if (valid) {
         const Item &it = *itp;
         const double gm1 = it.gm1;
@@ -205,6 +205,7 @@ __global__ void __launch_bounds__(grad_threads<N>()) k_grad(const __grid_constan
                 for (int v = 0; v < 4; ++v) qn[(slot * 4 + v) * n2 + ab] = g4[v];
             }
         }
+        double qin[4];
         grad_vars(uo, gm1, qin);
 #pragma unroll
         for (int v = 0; v < 4; ++v) q[v * n3 + p] = qin[v];
@@ -212,54 +213,40 @@ __global__ void __launch_bounds__(grad_threads<N>()) k_grad(const __grid_constan
     __syncthreads();
     if (!valid) return;
     const int ijk[3] = {p % n, (p / n) % n, p / n2};
-    double acc[12];
+    double acc[kVisc];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = 0.0;
+    for (int k = 0; k < kVisc; ++k) acc[k] = 0.0;
+    // D_ii is zero inside and -+1/(2w) at the two ends, where the BR1 lift
+    // +-(1/w)(q_out - q_in)/2 Ja turns the diagonal term D_ii Ja q_in into
+    // D_ii Ja q_out: no separate lift
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
+        const int i = ijk[d];
         const int stride = (d == 0) ? 1 : (d == 1) ? n : n2;
-        const int base = p - ijk[d] * stride;
-        const double *Drow = sD + ijk[d] * n;
+        const int base = p - i * stride;
+        const double *Drow = sD + i * n;
+        const double *J1 = ja + d * 3 * n3, *J2 = J1 + n3, *J3 = J2 + n3;
 #pragma unroll
-        for (int m = 0; m < n; ++m) {
+        for (int k = 1; k < n; ++k) {
+            const int m = (i + k < n) ? i + k : i + k - n;
             const int pm = base + m * stride;
             const double Dm = Drow[m];
-            const double a1 = Dm * ja[(d * 3 + 0) * n3 + pm], a2 = Dm * ja[(d * 3 + 1) * n3 + pm],
-                         a3 = Dm * ja[(d * 3 + 2) * n3 + pm];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const double qv = q[v * n3 + pm];
-                acc[v * 3 + 0] += a1 * qv;
-                acc[v * 3 + 1] += a2 * qv;
-                acc[v * 3 + 2] += a3 * qv;
-            }
+            stress_add(acc, Dm * J1[pm], Dm * J2[pm], Dm * J3[pm], q[pm], q[n3 + pm], q[2 * n3 + pm], q[3 * n3 + pm]);
+        }
+        if (i == 0 || i == N) {
+            const int ta = (d == 0) ? ijk[1] : ijk[0];
+            const int tb = (d == 2) ? ijk[1] : ijk[2];
+            const double *Q = qn + (2 * d + (i == N ? 1 : 0)) * 4 * n2 + ta + n * tb;
+            const double Dm = Drow[i];
+            stress_add(acc, Dm * J1[p], Dm * J2[p], Dm * J3[p], Q[0], Q[n2], Q[2 * n2], Q[3 * n2]);
         }
     }
-    // surface lifting of the BR1 jumps (q* - q_in) = (q_out - q_in)/2
     const Item &it = *itp;
-    const double hw = 0.5 * ops->iw0;
+    double t[kVisc];
+    stress_of(acc, it.invJ[(size_t)e * n3 + p], it.mu, it.kappa, t);
+    double *G = (double *)it.grad + (size_t)e * kVisc * n3 + p;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        if (ijk[d] != 0 && ijk[d] != N) continue;
-        const int ta = (d == 0) ? ijk[1] : ijk[0];
-        const int tb = (d == 2) ? ijk[1] : ijk[2];
-        const bool plus = ijk[d] == N;
-        const double sw = plus ? hw : -hw;
-        const double *Q = qn + (2 * d + (plus ? 1 : 0)) * 4 * n2 + ta + n * tb;
-        const double a1 = sw * ja[(d * 3 + 0) * n3 + p], a2 = sw * ja[(d * 3 + 1) * n3 + p],
-                     a3 = sw * ja[(d * 3 + 2) * n3 + p];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const double j = Q[v * n2] - qin[v];
-            acc[v * 3 + 0] += j * a1;
-            acc[v * 3 + 1] += j * a2;
-            acc[v * 3 + 2] += j * a3;
-        }
-    }
-    const double ij = it.invJ[(size_t)e * n3 + p];
-    double *G = (double *)it.grad + (size_t)e * 12 * n3 + p;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) G[k * n3] = acc[k] * ij;
+    for (int k = 0; k < kVisc; ++k) G[k * n3] = t[k];
 }
 
 // ------------------------------------------------------------------ launchers

@@ -141,8 +141,8 @@ __global__ void __launch_bounds__(256) k_face_gauss(const __grid_constant__ Batc
             }
         }
         R fl[5], fr[5];
-        visc_flux(qL, gl, P.mu, P.kappa, s1, s2, s3, fl);
-        visc_flux(qR, gr, P.mu, P.kappa, s1, s2, s3, fr);
+        visc_flux_grad(qL, gl, P.mu, P.kappa, s1, s2, s3, fl);
+        visc_flux_grad(qR, gr, P.mu, P.kappa, s1, s2, s3, fr);
 #pragma unroll
         for (int v = 1; v < 5; ++v) fs[v] -= (R)0.5 * (fl[v] + fr[v]);
     }
@@ -396,7 +396,7 @@ k_volume_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int
         for (int d = 0; d < 3; ++d) {
             R fe[5], fv[5] = {(R)0, (R)0, (R)0, (R)0, (R)0};
             euler_flux(q, q.E, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fe);
-            if (NS) visc_flux(q, G, P.mu, P.kappa, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fv);
+            if (NS) visc_flux_grad(q, G, P.mu, P.kappa, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fv);
 #pragma unroll
             for (int v = 0; v < 5; ++v) S[(d * 5 + v) * n3 + p] = NS ? fe[v] - fv[v] : fe[v];
         }

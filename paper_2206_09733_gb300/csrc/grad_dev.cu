@@ -56,7 +56,7 @@ __device__ __forceinline__ void grad_dev_vars(const Dev &d, const Anchor &A, flo
 
 // One tile (epb elements) of the gradient kernel; returns true on the thread
 // that initialised its element's bulk-copy barrier.
-template <int N>
+template <int N, bool MORT>
 __device__ __forceinline__ bool grad_dev_tile(const Batch &b, const Ops *__restrict__ ops, long long tile,
                                               unsigned long long *bulk_bar)
 {
@@ -67,7 +67,8 @@ __device__ __forceinline__ bool grad_dev_tile(const Batch &b, const Ops *__restr
     float *sD = (float *)smem_raw;
     float *sE = sD + ((n * n + 3) & ~3);
     const int epb = blockDim.x / n3;
-    for (int t = threadIdx.x; t < n * n; t += blockDim.x) sD[t] = ops->Df[t];
+    for (int t = threadIdx.x; t < n * n; t += blockDim.x) sD[t] = (!MORT && t % (n + 1) == 0) ? 0.0f : ops->Df[t];
+    const float dend = ops->Df[n * n - 1];
     const int le = threadIdx.x / n3, p = threadIdx.x - le * n3;
     const long long ge = tile * epb + le;
     bool valid = ge < b.total_elems;
@@ -106,7 +107,7 @@ __device__ __forceinline__ bool grad_dev_tile(const Batch &b, const Ops *__restr
         const float Tb = A.p * __fdividef(1.0f, A.rho);
         const float rT = fmaf(-Tb, A.rho, A.p);
         constexpr int IT = (6 * n2 + n3 - 1) / n3;
-        if (it.face6) {
+        if constexpr (MORT) {
             // 2 q*_e - q_in from the mortar kernel, full FP32 values -> deviations
 #pragma unroll
             for (int k = 0; k < IT; ++k) {
@@ -159,66 +160,103 @@ __device__ __forceinline__ bool grad_dev_tile(const Batch &b, const Ops *__restr
     }
     __syncthreads();
     if (!valid) return armed;
+    bool landed = true;
     if constexpr (BULK) {
         if (!mbar_wait(bulk_bar + le, 0, kBulkWaitPolls)) {
             // a wait that ran out of polls poisons the gradients and flags the solve
-#pragma unroll
-            for (int v = 0; v < 4; ++v) qin[v] = NAN;
+            landed = false;
             if (itp->clk) itp->clk->bad = 2;
         }
     }
     const int ijk[3] = {p % n, (p / n) % n, p / n2};
-    float acc[12];
+    const Item &it = *itp;
+    if constexpr (MORT) {
+        // the twelve gradients, every rounding as the mortar path's FP32 fluxes
+        // expect it (visc_flux_grad)
+        if (!landed) qin[0] = qin[1] = qin[2] = qin[3] = NAN;
+        float acc[12];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = 0.0f;
+        for (int k = 0; k < 12; ++k) acc[k] = 0.0f;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int stride = (d == 0) ? 1 : (d == 1) ? n : n2;
+            const int base = p - ijk[d] * stride;
+            const float *Drow = sD + ijk[d] * n;
+#pragma unroll
+            for (int m = 0; m < n; ++m) {
+                const int pm = base + m * stride;
+                const float Dm = Drow[m];
+                const float a1 = Dm * ja[(d * 3 + 0) * n3 + pm], a2 = Dm * ja[(d * 3 + 1) * n3 + pm],
+                            a3 = Dm * ja[(d * 3 + 2) * n3 + pm];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const float qv = q[v * n3 + pm];
+                    acc[v * 3 + 0] += a1 * qv;
+                    acc[v * 3 + 1] += a2 * qv;
+                    acc[v * 3 + 2] += a3 * qv;
+                }
+            }
+        }
+        // surface lifting of the BR1 jumps (q* - q_in) = (q_out - q_in)/2
+        const float iw = ops->iw0f;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int ta = (d == 0) ? ijk[1] : ijk[0];
+            const int tb = (d == 2) ? ijk[1] : ijk[2];
+            const int ab = ta + n * tb;
+#pragma unroll
+            for (int plus = 0; plus < 2; ++plus) {
+                if (ijk[d] != (plus ? N : 0)) continue;
+                const float sg = plus ? 1.0f : -1.0f;
+                const float n1 = sg * ja[(d * 3 + 0) * n3 + p], n2_ = sg * ja[(d * 3 + 1) * n3 + p],
+                            n3_ = sg * ja[(d * 3 + 2) * n3 + p];
+                const int slot = 2 * d + plus;
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const float j = 0.5f * (qn[(slot * 4 + v) * n2 + ab] - qin[v]) * iw;
+                    acc[v * 3 + 0] += j * n1;
+                    acc[v * 3 + 1] += j * n2_;
+                    acc[v * 3 + 2] += j * n3_;
+                }
+            }
+        }
+        const float ij = it.invJf[(size_t)e * n3 + p];
+        float *G = (float *)it.grad + (size_t)e * 12 * n3 + p;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) G[k * n3] = acc[k] * ij;
+        return armed;
+    }
+    float acc[kVisc];
+#pragma unroll
+    for (int k = 0; k < kVisc; ++k) acc[k] = 0.0f;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
+        const int i = ijk[d];
         const int stride = (d == 0) ? 1 : (d == 1) ? n : n2;
-        const int base = p - ijk[d] * stride;
-        const float *Drow = sD + ijk[d] * n;
+        const int base = p - i * stride;
+        const float *Drow = sD + i * n;
+        const float *J1 = ja + d * 3 * n3, *J2 = J1 + n3, *J3 = J2 + n3;
 #pragma unroll
         for (int m = 0; m < n; ++m) {
             const int pm = base + m * stride;
             const float Dm = Drow[m];
-            const float a1 = Dm * ja[(d * 3 + 0) * n3 + pm], a2 = Dm * ja[(d * 3 + 1) * n3 + pm],
-                        a3 = Dm * ja[(d * 3 + 2) * n3 + pm];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const float qv = q[v * n3 + pm];
-                acc[v * 3 + 0] += a1 * qv;
-                acc[v * 3 + 1] += a2 * qv;
-                acc[v * 3 + 2] += a3 * qv;
-            }
+            stress_add(acc, Dm * J1[pm], Dm * J2[pm], Dm * J3[pm], q[pm], q[n3 + pm], q[2 * n3 + pm], q[3 * n3 + pm]);
+        }
+        // the two ends: D_ii Ja q_in + (+-1/w)(q_out - q_in)/2 Ja = D_ii Ja q_out,
+        // D_ii = +-1/(2w) (sD holds zero on the diagonal)
+        if (i == 0 || i == N) {
+            const int ta = (d == 0) ? ijk[1] : ijk[0];
+            const int tb = (d == 2) ? ijk[1] : ijk[2];
+            const float *Q = qn + (2 * d + (i == N ? 1 : 0)) * 4 * n2 + ta + n * tb;
+            const float Dm = i == N ? dend : -dend;
+            stress_add(acc, Dm * J1[p], Dm * J2[p], Dm * J3[p], Q[0], Q[n2], Q[2 * n2], Q[3 * n2]);
         }
     }
-    // surface lifting of the BR1 jumps (q* - q_in) = (q_out - q_in)/2
-    const Item &it = *itp;
-    const float iw = ops->iw0f;
+    float tau[kVisc];
+    stress_of(acc, landed ? it.invJf[(size_t)e * n3 + p] : NAN, it.muf, it.kappaf, tau);
+    float *G = (float *)it.grad + (size_t)e * kVisc * n3 + p;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const int ta = (d == 0) ? ijk[1] : ijk[0];
-        const int tb = (d == 2) ? ijk[1] : ijk[2];
-        const int ab = ta + n * tb;
-#pragma unroll
-        for (int plus = 0; plus < 2; ++plus) {
-            if (ijk[d] != (plus ? N : 0)) continue;
-            const float sg = plus ? 1.0f : -1.0f;
-            const float n1 = sg * ja[(d * 3 + 0) * n3 + p], n2_ = sg * ja[(d * 3 + 1) * n3 + p],
-                        n3_ = sg * ja[(d * 3 + 2) * n3 + p];
-            const int slot = 2 * d + plus;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const float j = 0.5f * (qn[(slot * 4 + v) * n2 + ab] - qin[v]) * iw;
-                acc[v * 3 + 0] += j * n1;
-                acc[v * 3 + 1] += j * n2_;
-                acc[v * 3 + 2] += j * n3_;
-            }
-        }
-    }
-    const float ij = it.invJf[(size_t)e * n3 + p];
-    float *G = (float *)it.grad + (size_t)e * 12 * n3 + p;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) G[k * n3] = acc[k] * ij;
+    for (int k = 0; k < kVisc; ++k) G[k * n3] = tau[k];
     return armed;
 }
 
@@ -226,12 +264,12 @@ template <int N>
 __device__ __noinline__ bool grad_dev_tile_call(const Batch &b, const Ops *__restrict__ ops, long long tile,
                                                 unsigned long long *bulk_bar)
 {
-    return grad_dev_tile<N>(b, ops, tile, bulk_bar);
+    return grad_dev_tile<N, false>(b, ops, tile, bulk_bar);
 }
 
 // The gradient kernel: a CTA per tile, or (PERSIST, Batch::persistent) a
 // persistent grid walking the tiles (as k_volume_dev).
-template <int N, bool PERSIST>
+template <int N, bool PERSIST, bool MORT = false>
 __global__ void __launch_bounds__(grad_dev_threads<N>()) k_grad_dev(const __grid_constant__ Batch b,
                                                                     const Ops *__restrict__ ops, long long ntiles)
 {
@@ -240,7 +278,7 @@ __global__ void __launch_bounds__(grad_dev_threads<N>()) k_grad_dev(const __grid
     constexpr bool BULK = ((N + 1) % 2 == 0);
     __shared__ unsigned long long bulk_bar[BULK ? 256 / (n3 < 256 ? n3 : 256) : 1];
     if constexpr (!PERSIST) {
-        grad_dev_tile<N>(b, ops, blockIdx.x, bulk_bar);
+        grad_dev_tile<N, MORT>(b, ops, blockIdx.x, bulk_bar);
     } else {
         for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
             const bool armed = grad_dev_tile_call<N>(b, ops, tile, bulk_bar);
@@ -264,7 +302,9 @@ static cudaError_t grad_dev_launch(const Batch &b, cudaStream_t s)
     const Ops *ops = device_ops(N);
     if (!ops) return cudaErrorMemoryAllocation;
     cudaError_t e;
-    if (b.persistent) {
+    if (b.mortar) {
+        e = launch_pdl(k_grad_dev<N, false, true>, blocks, threads, smem, s, b, ops, (long long)blocks);
+    } else if (b.persistent) {
         const unsigned grid = persistent_grid(k_grad_dev<N, true>, threads, smem, blocks);
         e = launch_pdl(k_grad_dev<N, true>, grid, threads, smem, s, b, ops, (long long)blocks);
     } else {
@@ -274,13 +314,13 @@ static cudaError_t grad_dev_launch(const Batch &b, cudaStream_t s)
     return cudaGetLastError();
 }
 
-template <int N, bool PERSIST>
+template <int N, bool PERSIST, bool MORT>
 static cudaError_t grad_dev_prep_one()
 {
     cudaError_t e =
-        cudaFuncSetAttribute(k_grad_dev<N, PERSIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(k_grad_dev<N, PERSIST, MORT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_grad_dev<N, PERSIST>, cudaFuncAttributePreferredSharedMemoryCarveout,
+        e = cudaFuncSetAttribute(k_grad_dev<N, PERSIST, MORT>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  cudaSharedmemCarveoutMaxShared);
     return e;
 }
@@ -288,8 +328,9 @@ static cudaError_t grad_dev_prep_one()
 template <int N>
 static cudaError_t grad_dev_prep()
 {
-    cudaError_t e = grad_dev_prep_one<N, false>();
-    if (e == cudaSuccess) e = grad_dev_prep_one<N, true>();
+    cudaError_t e = grad_dev_prep_one<N, false, false>();
+    if (e == cudaSuccess) e = grad_dev_prep_one<N, true, false>();
+    if (e == cudaSuccess) e = grad_dev_prep_one<N, false, true>();
     return e;
 }
 

@@ -11,7 +11,8 @@
 //                                              from element e on its +d face
 //   fstar       R      [3(d)][E][5][n2]        numerical flux minus viscous flux, times
 //                                              the face scale, for face (d, e)
-//   grad        R      [E][12][n3]             BR1 gradients of (v1,v2,v3,T), [v*3 + c]
+//   grad        R      [E][kVisc][n3]          viscous stress and heat flux of the BR1 gradients
+//                                              (Gauss nodes, FP32 mortar path: the 12 gradients)
 // Face f = d*E + e is the face between element e and its +d neighbour.
 #pragma once
 
@@ -24,6 +25,8 @@ namespace hs3d {
 
 constexpr int kMaxN = 7;
 constexpr int kMaxn = kMaxN + 1;
+// Viscous values per node: six stresses and three heat fluxes.
+constexpr int kVisc = 9;
 
 __host__ __device__ constexpr bool is_standard(int form) { return form == HS3D_VOL_STANDARD; }
 
@@ -62,7 +65,7 @@ struct Item {
     double *g;
     double *out;            // residual output (residual mode)
     void *fstar;            // R [3][E][5][n2] (face6: [6][E][5][n2], see below)
-    void *grad;             // R [E][12][n3]
+    void *grad;             // R [E][kVisc][n3]: stress and heat flux (visc_flux in physics.cuh)
     // face6 != 0 (one degree bucket of a mesh with per-element degrees): the
     // element's six face fluxes are its own blocks fstar[slot][e], slot 2d
     // the -d face and 2d+1 the +d face, each already projected onto this

@@ -175,10 +175,24 @@ __device__ __forceinline__ int mortar_face_node(int n, int d, int end, int ta, i
 //           to each side's qhat6 block;
 //   MODE 1: face fluxes (5 values) to each side's fstar block (both oriented
 //           along +d).
+// Viscous values per trace point: stress and heat flux in FP64, the twelve
+// gradients on the FP32 path (see visc_flux_grad).
+template <typename R>
+constexpr int mortar_grads()
+{
+    return sizeof(R) == 8 ? kVisc : 12;
+}
+template <typename R>
+__device__ __forceinline__ void mortar_visc(const Prim<R> &q, const R *t, const MortarPhys<R> &P, R s1, R s2, R s3, R f[5])
+{
+    if constexpr (sizeof(R) == 8) visc_flux(q, t, s1, s2, s3, f);
+    else visc_flux_grad(q, t, P.mu, P.kappa, s1, s2, s3, f);
+}
+
 template <typename R, bool NS, int MODE, int NM>
 struct MortarShape {
     static constexpr int nM = NM + 1, P = nM * nM;
-    static constexpr int NV = (MODE == 1 && NS) ? 17 : 5;         // values per trace point
+    static constexpr int NV = (MODE == 1 && NS) ? 5 + mortar_grads<R>() : 5;         // values per trace point
     static constexpr int TARGET = 128;                             // threads per CTA aimed at
     static constexpr int FPC = TARGET / P >= 1 ? TARGET / P : 1;  // faces per CTA
     static constexpr int THREADS = FPC * P;
@@ -237,9 +251,9 @@ k_mortar(const MortarFace *__restrict__ faces, int nfaces, const MortarSide *__r
                     for (int v = 0; v < 5; ++v) dst[v * P] = src[(size_t)v * n3];
                 }
                 if constexpr (MODE == 1 && NS) {
-                    const R *G = (const R *)SD.grad + (size_t)le * 12 * n3 + node;
+                    const R *G = (const R *)SD.grad + (size_t)le * mortar_grads<R>() * n3 + node;
 #pragma unroll
-                    for (int k = 0; k < 12; ++k) dst[(5 + k) * P] = G[(size_t)k * n3];
+                    for (int k = 0; k < mortar_grads<R>(); ++k) dst[(5 + k) * P] = G[(size_t)k * n3];
                 }
             }
         }
@@ -313,8 +327,8 @@ k_mortar(const MortarFace *__restrict__ faces, int nfaces, const MortarSide *__r
             if constexpr (NS) {
                 R fl[5], fr[5];
                 const Prim<R> pL = mortar_prim(w[0], Ph.gm1), pR = mortar_prim(w[1], Ph.gm1);
-                visc_flux(pL, &w[0][5], Ph.mu, Ph.kappa, s1, s2, s3, fl);
-                visc_flux(pR, &w[1][5], Ph.mu, Ph.kappa, s1, s2, s3, fr);
+                mortar_visc(pL, &w[0][5], Ph, s1, s2, s3, fl);
+                mortar_visc(pR, &w[1][5], Ph, s1, s2, s3, fr);
 #pragma unroll
                 for (int v = 1; v < 5; ++v) fs[v] -= (R)0.5 * (fl[v] + fr[v]);
             }
@@ -395,7 +409,7 @@ __global__ void __launch_bounds__(128) k_mortar_conf(const MortarFace *__restric
 {
     constexpr int n = N + 1, P = n * n, n3 = P * n;
     constexpr int FPC = 128 / P >= 1 ? 128 / P : 1;
-    constexpr int NV = (MODE == 1 && NS) ? 17 : 5;
+    constexpr int NV = (MODE == 1 && NS) ? 5 + mortar_grads<R>() : 5;
     const int q = threadIdx.x / P, p = threadIdx.x - q * P;
     const int f = blockIdx.x * FPC + q;
     if (q >= FPC || f >= nfaces) return;
@@ -418,9 +432,9 @@ __global__ void __launch_bounds__(128) k_mortar_conf(const MortarFace *__restric
             for (int v = 0; v < 5; ++v) w[s][v] = src[(size_t)v * n3];
         }
         if constexpr (MODE == 1 && NS) {
-            const R *G = (const R *)SD.grad + (size_t)le * 12 * n3 + node;
+            const R *G = (const R *)SD.grad + (size_t)le * mortar_grads<R>() * n3 + node;
 #pragma unroll
-            for (int k = 0; k < 12; ++k) w[s][5 + k] = G[(size_t)k * n3];
+            for (int k = 0; k < mortar_grads<R>(); ++k) w[s][5 + k] = G[(size_t)k * n3];
         }
     }
     if constexpr (MODE == 0) {
@@ -446,8 +460,8 @@ __global__ void __launch_bounds__(128) k_mortar_conf(const MortarFace *__restric
         if constexpr (NS) {
             R fl[5], fr[5];
             const Prim<R> pL = mortar_prim(w[0], Ph.gm1), pR = mortar_prim(w[1], Ph.gm1);
-            visc_flux(pL, &w[0][5], Ph.mu, Ph.kappa, s1, s2, s3, fl);
-            visc_flux(pR, &w[1][5], Ph.mu, Ph.kappa, s1, s2, s3, fr);
+            mortar_visc(pL, &w[0][5], Ph, s1, s2, s3, fl);
+            mortar_visc(pR, &w[1][5], Ph, s1, s2, s3, fr);
 #pragma unroll
             for (int v = 1; v < 5; ++v) fs[v] -= (R)0.5 * (fl[v] + fr[v]);
         }

@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/hs3d.h"
+#include "internal.cuh"
 
 namespace hs3d {
 
@@ -45,6 +46,15 @@ __device__ __forceinline__ double rcp_fast(double x)
     double e = fma(-x, y, 1.0);
     e = fma(e, e, e);
     return fma(y, e, y);
+}
+
+// One second-order step: about 40 bits (no range test: the caller's value is
+// used only where the argument is a plain number).
+__device__ __forceinline__ double rcp_newton(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return fma(y, fma(-x, y, 1.0), y);
 }
 
 __device__ __forceinline__ double rsqrt_step(double x)
@@ -188,10 +198,65 @@ __device__ __forceinline__ void euler_flux(const Prim<R> &q, R E, R a1, R a2, R 
     f[4] = (E + q.p) * va;
 }
 
-// Viscous flux dotted with a.  G[v*3 + c] = d q_v / d x_c for q = (v1,v2,v3,T).
+// Viscous stress and heat flux, kVisc values per node: t11, t22, t33, t12,
+// t13, t23 of tau = mu (grad v + grad v^T) - 2/3 mu I div v, then
+// kappa grad T.  The viscous fluxes read nothing else of the twelve BR1
+// gradients, so the gradient kernels store these nine (a quarter less to write
+// and to read in the face and element kernels, and mu, kappa and the symmetric
+// sums are applied once per node instead of at every use).
+// Adds a_c q_v, q = (v1, v2, v3, T), to the nine sums the stress needs:
+// d1 v1, d2 v2, d3 v3, d1 v2 + d2 v1, d1 v3 + d3 v1, d2 v3 + d3 v2, d1 T, d2 T, d3 T.
 template <typename R>
-__device__ __forceinline__ void visc_flux(const Prim<R> &q, const R G[12], R mu, R kappa, R a1, R a2, R a3,
-                                          R f[5])
+__device__ __forceinline__ void stress_add(R acc[kVisc], R a1, R a2, R a3, R q1, R q2, R q3, R T)
+{
+    acc[0] += a1 * q1;
+    acc[1] += a2 * q2;
+    acc[2] += a3 * q3;
+    acc[3] += a2 * q1;
+    acc[3] += a1 * q2;
+    acc[4] += a3 * q1;
+    acc[4] += a1 * q3;
+    acc[5] += a3 * q2;
+    acc[5] += a2 * q3;
+    acc[6] += a1 * T;
+    acc[7] += a2 * T;
+    acc[8] += a3 * T;
+}
+
+// Stress and heat flux from the sums times s (1/J).
+template <typename R>
+__device__ __forceinline__ void stress_of(const R acc[kVisc], R s, R mu, R kappa, R t[kVisc])
+{
+    const R m = mu * s, k = kappa * s;
+    const R l = (R)(2.0 / 3.0) * (acc[0] + acc[1] + acc[2]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        t[c] = m * ((R)2 * acc[c] - l);
+        t[3 + c] = m * acc[3 + c];
+        t[6 + c] = k * acc[6 + c];
+    }
+}
+
+// Viscous flux dotted with a from the stress and heat flux t.
+template <typename R>
+__device__ __forceinline__ void visc_flux(const Prim<R> &q, const R t[kVisc], R a1, R a2, R a3, R f[5])
+{
+    R s1 = t[0] * a1 + t[3] * a2 + t[4] * a3;
+    R s2 = t[3] * a1 + t[1] * a2 + t[5] * a3;
+    R s3 = t[4] * a1 + t[5] * a2 + t[2] * a3;
+    f[0] = (R)0;
+    f[1] = s1;
+    f[2] = s2;
+    f[3] = s3;
+    f[4] = q.v1 * s1 + q.v2 * s2 + q.v3 * s3 + (t[6] * a1 + t[7] * a2 + t[8] * a3);
+}
+
+// The same from the twelve gradients G[v*3 + c] = d q_v / d x_c, q = (v1, v2,
+// v3, T): the Gauss-Legendre kernels and the FP32 mortar path, which form F*
+// minus the own flux from full FP32 values and so keep every rounding.
+template <typename R>
+__device__ __forceinline__ void visc_flux_grad(const Prim<R> &q, const R G[12], R mu, R kappa, R a1, R a2, R a3,
+                                               R f[5])
 {
     R div = G[0] + G[4] + G[8];
     R l = (R)(2.0 / 3.0) * mu * div;
@@ -386,7 +451,7 @@ __device__ __forceinline__ ECNode<R> ec_node(const Prim<R> &q)
     return z;
 }
 
-// F = ln(a/b) (a+b) / (2(a-b)) for u = ((a-b)/(a+b))^2 beyond the short series
+// F = ln(a/b) (a+b) / (2(a-b)) for f = (a-b)/(a+b), u = f^2 beyond the short series
 // of ec_pair64: 1 + u/3 + u^2/5 + ... to u^10/21 below u = 0.04 (a/b < 1.5; the
 // first term left out is below 2e-17), the logarithm above.  Few pairs of a
 // resolved flow come here, so no logarithm is computed per node.
@@ -408,36 +473,46 @@ __device__ __forceinline__ double logmean_F(double a, double b, double f, double
     return log(a / b) / (2.0 * f);
 }
 
+// Logarithmic mean of a, b > 0 beyond the short series.
+__device__ __forceinline__ double logmean_far(double a, double b)
+{
+    const double s = a + b, f = (a - b) * rcp_fast(s);
+    return 0.5 * s * rcp_fast(logmean_F(a, b, f, f * f));
+}
+
 // Chandrashekar's flux in FP64 from the per-node inputs (rho, v/2, 2 beta =
-// rho/p, |v|^2/4): the means {v} and {|v|^2}/2 are plain sums, the means'
-// factors sit in the constants, and 1/(rho_L + rho_R), 1/(beta_L + beta_R)
-// come from one reciprocal: 48 FP64 instructions for a pair on the short
-// series (u < 1e-4, first term left out below 1.2e-17) against 72 with
-// per-node logarithms, full means and an IEEE division.
+// rho/p): the mean {v} is a plain sum, the means' factors sit in the
+// constants, and with |v_L|^2 + |v_R|^2 = |v_L + v_R|^2 - 2 v_L.v_R the
+// energy is f_E = f_rho (hg/beta^ + v_L.v_R/2) + p~ {v}.a: 47 FP64
+// instructions for a pair on the short series (u < 1e-4, first term left out
+// below 1.2e-17) against 72 with per-node logarithms, full means and an IEEE
+// division.
 __device__ __forceinline__ void ec_pair64(const double *L, const double *Rr, double hg, double a1, double a2,
                                           double a3, double f[5])
 {
     const double srho = L[0] + Rr[0], sb2 = L[4] + Rr[4];
-    const double inv = rcp_fast(srho * sb2);
-    const double irho = sb2 * inv, ib2 = srho * inv;   // 1/(rho_L + rho_R), 1/(2(beta_L + beta_R))
-    const double fr = (L[0] - Rr[0]) * irho, ur = fr * fr;
+    // 1/(rho_L + rho_R) enters the short series only through u < 1e-4, where
+    // the seed's 40 bits after one Newton step are enough (an error of 1e-12 u/3)
+    const double ib2 = rcp_fast(sb2);   // 1/(2(beta_L + beta_R))
+    const double fr = (L[0] - Rr[0]) * rcp_newton(srho), ur = fr * fr;
     const double fb = (L[4] - Rr[4]) * ib2, ub = fb * fb;
     double rho_ln, hib;   // rho^, hg/beta^
     if (ur < LogMeanEps<double>::v)
         rho_ln = srho * fma(-ur, fma(ur, fma(ur, 22.0 / 945.0, 2.0 / 45.0), 1.0 / 6.0), 0.5);
     else
-        rho_ln = 0.5 * srho * rcp_fast(logmean_F(L[0], Rr[0], fr, ur));
+        rho_ln = logmean_far(L[0], Rr[0]);
     const double q = (4.0 * hg) * ib2;
     if (ub < LogMeanEps<double>::v) hib = q * fma(ub, fma(ub, fma(ub, 1.0 / 7.0, 0.2), 1.0 / 3.0), 1.0);
     else hib = q * logmean_F(L[4], Rr[4], fb, ub);
     const double m1 = L[1] + Rr[1], m2 = L[2] + Rr[2], m3 = L[3] + Rr[3];
     const double pt = srho * ib2;
-    const double fm = rho_ln * (m1 * a1 + m2 * a2 + m3 * a3);
+    const double va = m1 * a1 + m2 * a2 + m3 * a3;
+    const double fm = rho_ln * va;
     f[0] = fm;
     f[1] = fm * m1 + pt * a1;
     f[2] = fm * m2 + pt * a2;
     f[3] = fm * m3 + pt * a3;
-    f[4] = fm * (hib - (L[5] + Rr[5])) + m1 * f[1] + m2 * f[2] + m3 * f[3];
+    f[4] = fm * fma(2.0, L[1] * Rr[1] + L[2] * Rr[2] + L[3] * Rr[3], hib) + pt * va;
 }
 
 // Chandrashekar's entropy-conservative, kinetic-energy-preserving flux dotted
@@ -457,10 +532,8 @@ template <typename R>
 __device__ __forceinline__ void flux_ec(const ECNode<R> &L, const ECNode<R> &Rr, R hg, R a1, R a2, R a3, R f[5])
 {
     if constexpr (sizeof(R) == 8) {
-        const double zl[6] = {L.rho, 0.5 * L.v1, 0.5 * L.v2, 0.5 * L.v3, 2.0 * L.beta,
-                              0.25 * (L.v1 * L.v1 + L.v2 * L.v2 + L.v3 * L.v3)};
-        const double zr[6] = {Rr.rho, 0.5 * Rr.v1, 0.5 * Rr.v2, 0.5 * Rr.v3, 2.0 * Rr.beta,
-                              0.25 * (Rr.v1 * Rr.v1 + Rr.v2 * Rr.v2 + Rr.v3 * Rr.v3)};
+        const double zl[5] = {L.rho, 0.5 * L.v1, 0.5 * L.v2, 0.5 * L.v3, 2.0 * L.beta};
+        const double zr[5] = {Rr.rho, 0.5 * Rr.v1, 0.5 * Rr.v2, 0.5 * Rr.v3, 2.0 * Rr.beta};
         ec_pair64(zl, zr, hg, a1, a2, a3, f);
         return;
     }
@@ -709,7 +782,7 @@ __device__ __forceinline__ void split_pair(const R *L, const R *Rr, R gamma, R h
 //
 // Per-node inputs scaled by powers of two (exact), so that the arithmetic
 // means of a pair are plain sums:
-//   EC         rho, v/2, rho/p, |v|^2/4                 (ec_pair64)
+//   EC         rho, v/2, rho/p                          (ec_pair64)
 //   KG         rho/2, v/2, p/2, e/2
 //   PIROZZOLI  rho/2, v/2, p/2, h/2
 //   DUCROS     rho/2, v/2, p/2, (rho e + p)/2
@@ -718,7 +791,7 @@ __device__ __forceinline__ void split_pair(const R *L, const R *Rr, R gamma, R h
 template <int FORM>
 constexpr int split_slots64()
 {
-    return FORM == HS3D_VOL_IR ? 7 : 6;
+    return FORM == HS3D_VOL_IR ? 7 : FORM == HS3D_VOL_EC ? 5 : 6;
 }
 
 template <int FORM>
@@ -733,7 +806,6 @@ __device__ __forceinline__ void split_node64(const Prim<double> &q, double *z)
         if constexpr (FORM == HS3D_VOL_EC) {
             z[0] = q.rho;
             z[4] = div_(q.rho, q.p);
-            z[5] = z[1] * z[1] + z[2] * z[2] + z[3] * z[3];
         } else {
             z[0] = 0.5 * q.rho;
             z[4] = 0.5 * q.p;

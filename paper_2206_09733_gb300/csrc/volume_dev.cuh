@@ -133,6 +133,16 @@ constexpr int dev_min_blocks()
     return (FORM == HS3D_VOL_STANDARD && n3 <= 64) ? 5 : 4;
 }
 
+// Viscous flux from the gradient kernel's values: stress and heat flux, or the
+// twelve gradients on the mortar path.
+template <bool MORT>
+__device__ __forceinline__ void dev_visc(const Prim<float> &q, const float *G, const Item &it, float a1, float a2,
+                                         float a3, float f[5])
+{
+    if constexpr (MORT) visc_flux_grad(q, G, it.muf, it.kappaf, a1, a2, a3, f);
+    else visc_flux(q, G, a1, a2, a3, f);
+}
+
 // One tile (epb elements) of the element kernel; returns true on the
 // thread that initialised its element's bulk-copy barrier.  MORT: the items
 // take their face fluxes from the mortar kernels (Item::face6).
@@ -148,6 +158,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
     constexpr int PER = dev_per_node<FORM, NS>();
     constexpr int VOFF = dev_visc_off<FORM, NS>();
     constexpr int KP = n / 2;
+    constexpr int NG = MORT ? 12 : kVisc;
     constexpr bool BULK = (n % 2 == 0);
     constexpr int D2 = (n2 + 3) & ~3;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -190,7 +201,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
             // their per-thread loads (-3% at 24^3; at N = 3 it measured +1-2%)
             prefetch_l2_block(itp->Jaf + (size_t)e * 9 * n3, sizeof(float) * 9 * n3, p, n3);
             if (LM) prefetch_l2_block(itp->Jalo + (size_t)e * 9 * n3, sizeof(float) * 9 * n3, p, n3);
-            if (NS) prefetch_l2_block((const float *)itp->grad + (size_t)e * 12 * n3, sizeof(float) * 12 * n3, p, n3);
+            if (NS) prefetch_l2_block((const float *)itp->grad + (size_t)e * NG * n3, sizeof(float) * NG * n3, p, n3);
         }
         const double *U = itp->u + (size_t)e * 5 * n3;
 #pragma unroll
@@ -262,11 +273,11 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
         const float *JA = it.Jaf + (size_t)e * 9 * n3;
 #pragma unroll
         for (int k = 0; k < 9; ++k) ja[k] = JA[k * n3 + p];
-        float G[12];
+        float G[NG];
         if (NS) {
-            const float *Gp = (const float *)it.grad + (size_t)e * 12 * n3 + p;
+            const float *Gp = (const float *)it.grad + (size_t)e * NG * n3 + p;
 #pragma unroll
-            for (int k = 0; k < 12; ++k) G[k] = Gp[k * n3];
+            for (int k = 0; k < NG; ++k) G[k] = Gp[k * n3];
         }
         if constexpr (LM) {
             // Ja^d.m' in float-float: m' = (mh, ml) from the FP64 deviation,
@@ -293,7 +304,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                 dflux_euler_rest(dv, A, dH, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], f);
                 if (NS) {
                     float fv[5];
-                    visc_flux(q, G, it.muf, it.kappaf, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fv);
+                    dev_visc<MORT>(q, G, it, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fv);
 #pragma unroll
                     for (int v = 0; v < 4; ++v) f[v] -= fv[v + 1];
                 }
@@ -338,7 +349,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                 }
                 if (NS) {
                     float fv[5];
-                    visc_flux(q, G, it.muf, it.kappaf, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fv);
+                    dev_visc<MORT>(q, G, it, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fv);
 #pragma unroll
                     for (int v = 0; v < 4; ++v) S[(VOFF + d * 4 + v) * n3 + p] = fv[v + 1];
                 }
@@ -360,7 +371,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                 for (int v = 0; v < 5; ++v) V[v] += dd * fe[v];
                 if (NS) {
                     float fv[5];
-                    visc_flux(q, G, it.muf, it.kappaf, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fv);
+                    dev_visc<MORT>(q, G, it, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fv);
 #pragma unroll
                     for (int v = 0; v < 4; ++v) S[(VOFF + d * 4 + v) * n3 + p] = fv[v + 1];
                 }
@@ -641,11 +652,11 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
 #pragma unroll
             for (int v = 0; v < 5; ++v) ad[v] = AD[v];
             const Prim<float> q = dev_prim(make_dev(u, ad, A, it.gm1f), A);
-            float G[12];
+            float G[NG];
             if (NS) {
-                const float *Gp = (const float *)it.grad + (size_t)e * 12 * n3 + p;
+                const float *Gp = (const float *)it.grad + (size_t)e * NG * n3 + p;
 #pragma unroll
-                for (int k = 0; k < 12; ++k) G[k] = Gp[k * n3];
+                for (int k = 0; k < NG; ++k) G[k] = Gp[k * n3];
             }
             const float *JA = it.Jaf + (size_t)e * 9 * n3 + p;
 #pragma unroll
@@ -655,7 +666,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                 euler_flux(q, q.E, a1, a2, a3, own[d]);
                 if (NS) {
                     float fv[5];
-                    visc_flux(q, G, it.muf, it.kappaf, a1, a2, a3, fv);
+                    dev_visc<MORT>(q, G, it, a1, a2, a3, fv);
 #pragma unroll
                     for (int v = 1; v < 5; ++v) own[d][v] -= fv[v];
                 }

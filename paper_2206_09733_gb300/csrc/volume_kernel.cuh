@@ -26,11 +26,12 @@
 //   - split forms leave out the diagonal pair: D_ii is zero inside and
 //     2 D_ii = +-1/w at the two ends, where F#(u_i, u_i).(2 Ja_i) D_ii is
 //     exactly the own Euler flux that the surface term (1/w)(F* - F~_in)
-//     takes off again, so neither is formed and the surface term is
-//     +-(1/w)(F* + F~_v);
+//     takes off again, so neither is formed; of the viscous part the
+//     diagonal takes half of the surface term's, and +-(1/w)(F* + F~_v/2)
+//     remains;
 //   - the two faces of a direction share one instruction sequence (a lane is
 //     on at most one of them).
-// 16^3 elements of N = 3, NS, Chandrashekar form, one launch: 365 -> 261 us (441 FP64 instructions per warp, pipe 85% busy).
+// 16^3 elements of N = 3, NS, Chandrashekar form, one launch: 365 -> 235 us.
 //
 // One thread per node, `epb` elements per CTA (a kernel argument).  The
 // element's contravariant fluxes (standard form) or its per-node two-point-flux
@@ -270,17 +271,17 @@ k_volume(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int stage
 #pragma unroll
         for (int v = 0; v < 5; ++v) u[v] = it.u[node + v * n3];
         const Prim<double> q = prim_from_u<double>(u, P.gm1);
-        double G[12];
+        double G[kVisc];
         if (NS) {
-            const double *Gp = (const double *)it.grad + (size_t)e * 12 * n3 + p;
+            const double *Gp = (const double *)it.grad + (size_t)e * kVisc * n3 + p;
 #pragma unroll
-            for (int k = 0; k < 12; ++k) G[k] = Gp[k * n3];
+            for (int k = 0; k < kVisc; ++k) G[k] = Gp[k * n3];
         }
         if constexpr (STD || NS) {
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 double fe[5], fv[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-                if (NS) visc_flux(q, G, P.mu, P.kappa, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fv);
+                if (NS) visc_flux(q, G, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fv);
                 if constexpr (STD) {
                     euler_flux(q, q.E, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fe);
 #pragma unroll
@@ -365,7 +366,7 @@ k_volume(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int stage
                 const int ta = (d == 0) ? ijk[1] : ijk[0];
                 const int tb = (d == 2) ? ijk[1] : ijk[2];
                 const int l = ta + n * tb;
-                const int base = p - i * sd;
+                const int base = p - i * sd;   // (viscous fluxes)
                 const double *Drow = sD + i * n;
                 // the other n - 1 nodes of the line, the pair (i, i + k mod n) with
                 // pair thread x n^2 + l in slot k - 1 (x = i) or n - k - 1 (x = m)
@@ -387,11 +388,7 @@ k_volume(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int stage
                     const double *F = PB + (slot - 1) * n3 + x * n2 + l;
 #pragma unroll
                     for (int v = 0; v < 5; ++v) V[v] += Dm * F[v * KP * n3];
-                }
-                if (NS) {
-#pragma unroll
-                    for (int m = 0; m < n; ++m) {
-                        const double Dm = Drow[m];
+                    if (NS) {
 #pragma unroll
                         for (int v = 1; v < 5; ++v) V[v] -= Dm * S[(ZS + 9 + d * 4 + v - 1) * n3 + base + m * sd];
                     }
@@ -404,7 +401,7 @@ k_volume(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int stage
         const Item &it = *itp;
         // surface term: +-(1/w)(F* - F~) on the +-d face (standard form: the
         // difference is formed first, it is small where the large fluxes nearly
-        // cancel; split forms: +-(1/w)(F* + F~_v), see the top)
+        // cancel; split forms: +-(1/w)(F* + F~_v/2), see the top)
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             if (ijk[d] != N && ijk[d] != 0) continue;
@@ -415,10 +412,12 @@ k_volume(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int stage
             const double *F = F6 + (2 * d + (plus ? 1 : 0)) * 5 * n2 + ta + n * tb;
 #pragma unroll
             for (int v = 0; v < 5; ++v) {
-                double f = F[v * n2];
-                if constexpr (STD) f -= S[(d * 5 + v) * n3 + p];
-                else if (NS && v > 0) f += S[(ZS + 9 + d * 4 + v - 1) * n3 + p];
-                V[v] = fma(sw, f, V[v]);
+                if constexpr (STD) {
+                    V[v] = fma(sw, F[v * n2] - S[(d * 5 + v) * n3 + p], V[v]);
+                } else {
+                    V[v] = fma(sw, F[v * n2], V[v]);
+                    if (NS && v > 0) V[v] = fma(0.5 * sw, S[(ZS + 9 + d * 4 + v - 1) * n3 + p], V[v]);
+                }
             }
         }
         node_update<double, NS>(it, e, p, n3, V, u, stage, rkA, rkB, lam_slot, lc, lv, lam_active);
