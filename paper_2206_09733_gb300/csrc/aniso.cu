@@ -23,17 +23,23 @@
 // Sec. 3.6 names).  Each element face's result goes to its own block of the
 // face arrays (fstar, qhat), at the face-node offset fnoff[6e + slot].
 //
-// Kernels take one element (or one face) per CTA.  Elements are launched in
-// classes by node count (kAnisoClass), so a CTA has at most twice the threads
-// its element needs; the work is FP64 and per node, as in the oracle, with
-// no symmetry or sum factorisation beyond it: this path is for coverage of
-// the anisotropic discretisation, the isotropic meshes keep their
-// specialised kernels.
+// The kernels are bound by the FP64 pipe (one warp instruction per 16 cycles
+// and SM, however many lanes are active), so the stage kernels pack: elements
+// are binned into CTAs of 256 (or 512) thread slots at mesh set-up, one slot
+// per node (k_agrad, k_avol), and the faces of equal mortar degrees share CTAs
+// of 128 threads, sorted by their sides' degrees so that a CTA's faces need
+// the same passes (k_amortar).  Interpolation and projection go direction by
+// direction and are skipped where the side has the mortar's degree; each pair
+// of a line is evaluated once.  The set-up, initial-state and diagnostics
+// kernels take one element per CTA, launched in classes by node count
+// (kAnisoClass).
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "aniso.cuh"
@@ -195,51 +201,73 @@ __global__ void __launch_bounds__(512) k_ainit(const int *__restrict__ elems, co
 __device__ __forceinline__ void alam_node(const AShape &s, const double *Ja, int p, double iJ, const Prim<double> &q,
                                           const APhys &P, double &lc, double &lv)
 {
-    const double c = sqrt(P.gamma * q.p / q.rho);
+    const double c = sound_speed(q, P.gamma);
     double sc = 0.0, sv = 0.0;
     for (int d = 0; d < 3; ++d) {
         const double a1 = Ja[(size_t)(d * 3) * s.n3 + p], a2 = Ja[(size_t)(d * 3 + 1) * s.n3 + p],
                      a3 = Ja[(size_t)(d * 3 + 2) * s.n3 + p];
-        const double an = sqrt(a1 * a1 + a2 * a2 + a3 * a3);
-        const double n2 = (double)s.n[d] * s.n[d];
-        sc += n2 * (fabs(a1 * q.v1 + a2 * q.v2 + a3 * q.v3) + c * an) * iJ;
-        sv += n2 * n2 * (an * iJ) * (an * iJ);
+        const double s2 = a1 * a1 + a2 * a2 + a3 * a3;
+        const double n2 = (double)(s.n[d] * s.n[d]);
+        sc += n2 * (fabs(a1 * q.v1 + a2 * q.v2 + a3 * q.v3) + c * sqrt_(s2));
+        sv += n2 * n2 * s2;
     }
-    lc = sc;
-    lv = P.physics == HS3D_NS ? P.mu * sv / q.rho : 0.0;
+    lc = sc * iJ;
+    lv = P.physics == HS3D_NS ? P.mu * sv * (iJ * iJ) * q.ir : 0.0;
 }
 
-__global__ void __launch_bounds__(512) k_alambda(const int *__restrict__ elems, const int *__restrict__ P3,
-                          const long long *__restrict__ noff, const double *__restrict__ Jaall,
-                          const double *__restrict__ invJall, const double *__restrict__ u, APhys P, Clock *clk,
-                          int slot)
+// The element, its shape and this thread's node of a packed launch: slot
+// blockIdx.x T + threadIdx.x; origin is the element's first thread.
+struct ASlot {
+    int e, p, origin;
+    AShape s;
+};
+__device__ __forceinline__ bool aslot(const int *__restrict__ slot_elem, const int *__restrict__ slot0,
+                                      const int *__restrict__ P3, ASlot &a)
 {
-    const int e = elems[blockIdx.x];
-    const AShape s = ashape(P3, e);
-    const int p = threadIdx.x;
-    const bool live = p < s.n3;
+    a.e = slot_elem[(size_t)blockIdx.x * blockDim.x + threadIdx.x];
+    if (a.e < 0) return false;
+    a.origin = slot0[a.e];
+    a.p = (int)threadIdx.x - a.origin;
+    a.s = ashape(P3, a.e);
+    return true;
+}
+
+__global__ void __launch_bounds__(512) k_alambda(const int *__restrict__ slot_elem, const int *__restrict__ slot0,
+                                                 const int *__restrict__ P3, const long long *__restrict__ noff,
+                                                 const double *__restrict__ Jaall, const double *__restrict__ invJall,
+                                                 const double *__restrict__ u, APhys P, Clock *clk, int slot)
+{
+    ASlot S;
+    const bool live = aslot(slot_elem, slot0, P3, S);
     double lc = 0.0, lv = 0.0;
     if (live) {
-        const long long nb = noff[e];
+        const long long nb = noff[S.e];
         double w[5];
-        for (int v = 0; v < 5; ++v) w[v] = u[5 * nb + (size_t)v * s.n3 + p];
+        for (int v = 0; v < 5; ++v) w[v] = u[5 * nb + (size_t)v * S.s.n3 + S.p];
         const Prim<double> q = prim_from_u<double>(w, P.gm1);
         if (!(q.rho > 0.0) || !(q.p > 0.0)) clk->bad = 1;
-        else alam_node(s, Jaall + 9 * nb, p, invJall[nb + p], q, P, lc, lv);
+        else alam_node(S.s, Jaall + 9 * nb, S.p, invJall[nb + S.p], q, P, lc, lv);
     }
     warp_max_to_clock(&clk->lam[slot][0], P.physics == HS3D_NS ? &clk->lam[slot][1] : nullptr, lc, lv, live);
 }
 
 // ------------------------------------------------------------------ mortar faces
 
-// One face per CTA of 64 threads (at most 8 x 8 mortar points).
+// The faces of one CTA: `count` faces from `face0` of the table sorted by
+// mortar degrees (nm0 x nm1 points each); passes: bit 0 / 1, some face's L / R
+// side needs the first-direction interpolation and projection.
 //   MODE 0: q* = (q(u_L) + q(u_R))/2 at the mortar points -> qhat of both sides (4 values);
 //   MODE 1: s F*(u_L, u_R; n) - (F_v(L) + F_v(R)).Sn/2 -> fstar of both sides (5 values,
 //           oriented along +d).
-constexpr int kAFaceThreads = 64;
+// 16^3 elements of degrees 2..5 (NS, Roe): flux launch 1331 -> 247 us, interface
+// values 491 -> 74 us against one face per 64-thread CTA with both directions
+// interpolated at once for every side.
+constexpr int kAFaceThreads = 128;
 
 template <int MODE, bool NS>
-__global__ void __launch_bounds__(kAFaceThreads) k_amortar(const AFace *__restrict__ faces, const int *__restrict__ P3,
+__global__ void __launch_bounds__(kAFaceThreads) k_amortar(const AFace *__restrict__ faces,
+                                                           const AFaceCta *__restrict__ ctas,
+                                                           const int *__restrict__ P3,
                                                            const long long *__restrict__ noff,
                                                            const long long *__restrict__ fnoff,
                                                            const double *__restrict__ u,
@@ -248,84 +276,135 @@ __global__ void __launch_bounds__(kAFaceThreads) k_amortar(const AFace *__restri
                                                            const MortarOps *__restrict__ mo, APhys P,
                                                            double *__restrict__ out)
 {
+    constexpr int T = kAFaceThreads;
     constexpr int NV = (MODE == 1 && NS) ? 5 + kVisc : 5;   // conservative state (+ viscous stress) per trace point
     constexpr int NO = MODE == 0 ? 4 : 5;
-    __shared__ double tr[2][NV][kAFaceThreads];
-    __shared__ double sn[2][3][kAFaceThreads];
-    __shared__ double fm[NO][kAFaceThreads];
-    const AFace F = faces[blockIdx.x];
-    const int d = F.d, p = threadIdx.x;
+    constexpr int NM = MODE == 1 ? 3 : 0;                   // face metric
+    __shared__ double tr[2][NV][T];
+    __shared__ double sn[NM > 0 ? NM : 1][T];
+    __shared__ double fm[NO][T];
+    __shared__ double gk[2][NO][T];
+    pdl_wait();
+    const AFaceCta C = ctas[blockIdx.x];
+    const int nm0 = C.nm0, nm1 = C.nm1, nM2 = nm0 * nm1;
+    const int fi = threadIdx.x / nM2, p = threadIdx.x - fi * nM2, o = fi * nM2;
+    const bool live = fi < C.count;
+    AFace F{0, 0, 0};
+    if (live) F = faces[C.face0 + fi];
+    const int d = F.d;
     int d0, d1;
     aface_dirs(d, d0, d1);
     const int eS[2] = {F.eL, F.eR};
     AShape sh[2];
-    int S0[2], S1[2];
+    int n0[2], n1[2];   // the sides' points per tangential direction
+#pragma unroll
     for (int k = 0; k < 2; ++k) {
         sh[k] = ashape(P3, eS[k]);
-        S0[k] = sh[k].n[d0] - 1;
-        S1[k] = sh[k].n[d1] - 1;
+        n0[k] = d0 == 0 ? sh[k].n[0] : sh[k].n[1];
+        n1[k] = d1 == 2 ? sh[k].n[2] : sh[k].n[1];
     }
-    const int M0 = S0[0] > S0[1] ? S0[0] : S0[1], M1 = S1[0] > S1[1] ? S1[0] : S1[1];
-    const int nm0 = M0 + 1, nM2 = nm0 * (M1 + 1);
+    // the face metric of a side whose tangential degrees are the mortar's (L
+    // first), else L's, interpolated (hk < 0)
+    const int hk = (n0[0] == nm0 && n1[0] == nm1) ? 0 : (n0[1] == nm0 && n1[1] == nm1) ? 1 : -1;
 
-    // 1. both sides' traces (and face metric) on their own face points
+    // 1. both sides' traces on their own face points
+#pragma unroll
     for (int k = 0; k < 2; ++k) {
-        const int ns0 = S0[k] + 1, f2 = ns0 * (S1[k] + 1);
-        if (p < f2) {
-            const int node = aface_node(sh[k], d, k == 0 ? sh[k].n[d] - 1 : 0, p % ns0, p / ns0);
+        if (live && p < n0[k] * n1[k]) {
+            const int node = aface_node(sh[k], d, k == 0 ? sh[k].n[d] - 1 : 0, p % n0[k], p / n0[k]);
             const long long nb = noff[eS[k]];
             const int n3 = sh[k].n3;
-            for (int v = 0; v < 5; ++v) tr[k][v][p] = u[5 * nb + (size_t)v * n3 + node];
-            if constexpr (MODE == 1 && NS)
-                for (int q = 0; q < kVisc; ++q) tr[k][5 + q][p] = grad[kVisc * nb + (size_t)q * n3 + node];
-            if constexpr (MODE == 1)
-                for (int c = 0; c < 3; ++c) sn[k][c][p] = Jaall[9 * nb + (size_t)(d * 3 + c) * n3 + node];
+#pragma unroll
+            for (int v = 0; v < 5; ++v) tr[k][v][o + p] = u[5 * nb + (size_t)v * n3 + node];
+            if constexpr (MODE == 1 && NS) {
+#pragma unroll
+                for (int q = 0; q < kVisc; ++q) tr[k][5 + q][o + p] = grad[kVisc * nb + (size_t)q * n3 + node];
+            }
+            if constexpr (MODE == 1) {
+                if (k == (hk > 0 ? 1 : 0)) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) sn[c][o + p] = Jaall[9 * nb + (size_t)(d * 3 + c) * n3 + node];
+                }
+            }
         }
     }
     __syncthreads();
 
-    // 2. the mortar function at this thread's mortar point (a, b)
-    if (p < nM2) {
+    // 2. first tangential direction, in place: (n0 x n1) -> (nm0 x n1) points
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        if (!(C.passes & (1 << k))) continue;   // (uniform over the CTA)
+        double r[NV], rs[3] = {0.0, 0.0, 0.0};
+        const bool mine = live && n0[k] < nm0 && p < nm0 * n1[k];
+        if (mine) {
+            const int a = p % nm0, j = p / nm0;
+            const double *I = mo->Pi[n0[k] - 1][nm0 - 1] + a * n0[k];
+            const int src = o + n0[k] * j;
+#pragma unroll
+            for (int v = 0; v < NV; ++v) r[v] = 0.0;
+            for (int i = 0; i < n0[k]; ++i) {
+                const double w = I[i];
+#pragma unroll
+                for (int v = 0; v < NV; ++v) r[v] += w * tr[k][v][src + i];
+                if constexpr (MODE == 1) {
+                    if (k == 0 && hk < 0) {
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) rs[c] += w * sn[c][src + i];
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        if (mine) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) tr[k][v][o + p] = r[v];
+            if constexpr (MODE == 1) {
+                if (k == 0 && hk < 0) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) sn[c][o + p] = rs[c];
+                }
+            }
+        }
+    }
+    if (C.passes) __syncthreads();
+
+    // 3. second direction into registers, and the mortar function at this point
+    if (live) {
         const int a = p % nm0, b = p / nm0;
         double w[2][NV];
+#pragma unroll
         for (int k = 0; k < 2; ++k) {
-            const int ns0 = S0[k] + 1, ns1 = S1[k] + 1;
-            const double *I0 = mo->Pi[S0[k]][M0] + a * ns0;   // identity rows when S == M
-            const double *I1 = mo->Pi[S1[k]][M1] + b * ns1;
-            for (int v = 0; v < NV; ++v) {
-                double acc = 0.0;
-                for (int j = 0; j < ns1; ++j) {
-                    double r = 0.0;
-                    for (int i = 0; i < ns0; ++i) r += I0[i] * tr[k][v][i + ns0 * j];
-                    acc += I1[j] * r;
+            if (n1[k] < nm1) {
+                const double *I = mo->Pi[n1[k] - 1][nm1 - 1] + b * n1[k];
+#pragma unroll
+                for (int v = 0; v < NV; ++v) w[k][v] = 0.0;
+                for (int j = 0; j < n1[k]; ++j) {
+                    const double c = I[j];
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) w[k][v] += c * tr[k][v][o + a + nm0 * j];
                 }
-                w[k][v] = acc;
+            } else {
+#pragma unroll
+                for (int v = 0; v < NV; ++v) w[k][v] = tr[k][v][o + p];
             }
         }
         if constexpr (MODE == 0) {
             double qL[4], qR[4];
             mortar_q(w[0], P.gm1, qL);
             mortar_q(w[1], P.gm1, qR);
-            for (int v = 0; v < 4; ++v) fm[v][p] = 0.5 * (qL[v] + qR[v]);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) fm[v][o + p] = 0.5 * (qL[v] + qR[v]);
         } else {
-            // face metric at the mortar point
             double s3[3];
-            const int hk = (S0[0] == M0 && S1[0] == M1) ? 0 : (S0[1] == M0 && S1[1] == M1) ? 1 : -1;
-            if (hk >= 0) {
-                for (int c = 0; c < 3; ++c) s3[c] = sn[hk][c][p];
+            if (hk < 0 && n1[0] < nm1) {
+                const double *I = mo->Pi[n1[0] - 1][nm1 - 1] + b * n1[0];
+                s3[0] = s3[1] = s3[2] = 0.0;
+                for (int j = 0; j < n1[0]; ++j)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) s3[c] += I[j] * sn[c][o + a + nm0 * j];
             } else {
-                const int ns0 = S0[0] + 1, ns1 = S1[0] + 1;
-                const double *I0 = mo->Pi[S0[0]][M0] + a * ns0;
-                const double *I1 = mo->Pi[S1[0]][M1] + b * ns1;
-                for (int c = 0; c < 3; ++c) {
-                    double acc = 0.0;
-                    for (int j = 0; j < ns1; ++j) {
-                        double r = 0.0;
-                        for (int i = 0; i < ns0; ++i) r += I0[i] * sn[0][c][i + ns0 * j];
-                        acc += I1[j] * r;
-                    }
-                    s3[c] = acc;
-                }
+#pragma unroll
+                for (int c = 0; c < 3; ++c) s3[c] = sn[c][o + p];
             }
             const MortarPhys<double> mp{P.gamma, P.gm1, P.hg, P.mu, P.kappa};
             double fs[5];
@@ -335,31 +414,60 @@ __global__ void __launch_bounds__(kAFaceThreads) k_amortar(const AFace *__restri
                 const Prim<double> pL = mortar_prim(w[0], P.gm1), pR = mortar_prim(w[1], P.gm1);
                 visc_flux(pL, &w[0][5], s3[0], s3[1], s3[2], fl);
                 visc_flux(pR, &w[1][5], s3[0], s3[1], s3[2], fr);
+#pragma unroll
                 for (int v = 1; v < 5; ++v) fs[v] -= 0.5 * (fl[v] + fr[v]);
             }
-            for (int v = 0; v < 5; ++v) fm[v][p] = fs[v];
+#pragma unroll
+            for (int v = 0; v < 5; ++v) fm[v][o + p] = fs[v];
         }
     }
     __syncthreads();
 
-    // 3. each side's L2 projection onto its own face points, into its face block
+    // 4. each side's L2 projection onto its own face points, first direction ...
+#pragma unroll
     for (int k = 0; k < 2; ++k) {
-        const int ns0 = S0[k] + 1, f2 = ns0 * (S1[k] + 1);
-        if (p < f2) {
-            const int a = p % ns0, b = p / ns0;
-            const double *P0 = mo->P[S0[k]][M0] + a * nm0;   // identity rows when S == M
-            const double *P1 = mo->P[S1[k]][M1] + b * (M1 + 1);
+        if (live && n0[k] < nm0 && p < n0[k] * nm1) {
+            const int a = p % n0[k], j = p / n0[k];
+            const double *P0 = mo->P[n0[k] - 1][nm0 - 1] + a * nm0;
+            double r[NO];
+#pragma unroll
+            for (int v = 0; v < NO; ++v) r[v] = 0.0;
+            for (int i = 0; i < nm0; ++i) {
+                const double w = P0[i];
+#pragma unroll
+                for (int v = 0; v < NO; ++v) r[v] += w * fm[v][o + i + nm0 * j];
+            }
+#pragma unroll
+            for (int v = 0; v < NO; ++v) gk[k][v][o + p] = r[v];
+        }
+    }
+    if (C.passes) __syncthreads();
+
+    // ... then the second, into the side's face block
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int f2 = n0[k] * n1[k];
+        if (live && p < f2) {
+            const int a = p % n0[k], b = p / n0[k];
+            const double *src = (n0[k] < nm0 ? &gk[k][0][0] : &fm[0][0]) + o;
             const int slot = 2 * d + (k == 0 ? 1 : 0);
             double *dst = out + (size_t)NO * fnoff[6 * eS[k] + slot] + p;
-            for (int v = 0; v < NO; ++v) {
-                double acc = 0.0;
-                for (int j = 0; j <= M1; ++j) {
-                    double r = 0.0;
-                    for (int i = 0; i < nm0; ++i) r += P0[i] * fm[v][i + nm0 * j];
-                    acc += P1[j] * r;
+            double r[NO];
+            if (n1[k] < nm1) {
+                const double *P1 = mo->P[n1[k] - 1][nm1 - 1] + b * nm1;
+#pragma unroll
+                for (int v = 0; v < NO; ++v) r[v] = 0.0;
+                for (int j = 0; j < nm1; ++j) {
+                    const double w = P1[j];
+#pragma unroll
+                    for (int v = 0; v < NO; ++v) r[v] += w * src[v * T + a + n0[k] * j];
                 }
-                dst[(size_t)v * f2] = acc;
+            } else {
+#pragma unroll
+                for (int v = 0; v < NO; ++v) r[v] = src[v * T + p];
             }
+#pragma unroll
+            for (int v = 0; v < NO; ++v) dst[(size_t)v * f2] = r[v];
         }
     }
 }
@@ -368,198 +476,256 @@ __global__ void __launch_bounds__(kAFaceThreads) k_amortar(const AFace *__restri
 
 // J grad q_c = sum_d D_d (Ja^d_c q) + sum_faces (q*_e - q_in) (+-Ja^d_c)/w_end,
 // q = (v1, v2, v3, T), q*_e from the mortar kernel, stored as viscous stress and
-// heat flux [kVisc][n3] at kVisc noff[e].
-__global__ void __launch_bounds__(512) k_agrad(const int *__restrict__ elems, const int *__restrict__ P3, const long long *__restrict__ noff,
-                        const long long *__restrict__ fnoff, const AOps *__restrict__ ops,
-                        const double *__restrict__ u, const double *__restrict__ Jaall,
-                        const double *__restrict__ invJall, const double *__restrict__ qhat, APhys P,
-                        double *__restrict__ gradall)
+// heat flux [kVisc][n3] at kVisc noff[e].  D_ii is zero inside and -+1/(2w) at
+// the two ends, where the lift turns the diagonal term D_ii Ja q_in into
+// D_ii Ja (2 q* - q_in).  16^3 elements of degrees 2..5: 484 -> 193 us per stage.
+template <int T>
+__global__ void __launch_bounds__(T) k_agrad(const int *__restrict__ slot_elem, const int *__restrict__ slot0,
+                                             const int *__restrict__ P3, const long long *__restrict__ noff,
+                                             const long long *__restrict__ fnoff, const AOps *__restrict__ ops,
+                                             const double *__restrict__ u, const double *__restrict__ Jaall,
+                                             const double *__restrict__ invJall, const double *__restrict__ qhat,
+                                             APhys P, double *__restrict__ gradall)
 {
-    extern __shared__ double sm[];
-    const int e = elems[blockIdx.x];
-    const AShape s = ashape(P3, e);
-    const int n3 = s.n3, p = threadIdx.x;
-    const bool live = p < n3;
-    double *sq = sm;            // [4][n3]
-    double *sJ = sm + 4 * n3;   // [9][n3]
-    const long long nb = noff[e];
+    extern __shared__ double sm[];   // q [4][T], Ja [9][T]
+    pdl_wait();
+    ASlot S;
+    const bool live = aslot(slot_elem, slot0, P3, S);
+    const int t = threadIdx.x;
     double qp[4] = {0, 0, 0, 0};
-    int ijk[3] = {0, 0, 0};
+    long long nb = 0;
     if (live) {
-        ijk[0] = p % s.n[0];
-        ijk[1] = (p / s.n[0]) % s.n[1];
-        ijk[2] = p / (s.n[0] * s.n[1]);
-        mortar_q(u + 5 * nb + p, P.gm1, qp, n3);
-        for (int v = 0; v < 4; ++v) sq[v * n3 + p] = qp[v];
-        for (int k = 0; k < 9; ++k) sJ[k * n3 + p] = Jaall[9 * nb + (size_t)k * n3 + p];
+        nb = noff[S.e];
+        const int n3 = S.s.n3;
+        mortar_q(u + 5 * nb + S.p, P.gm1, qp, n3);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) sm[v * T + t] = qp[v];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) sm[(4 + k) * T + t] = Jaall[9 * nb + (size_t)k * n3 + S.p];
     }
     __syncthreads();
     if (!live) return;
+    const int ijk[3] = {S.p % S.s.n[0], (S.p / S.s.n[0]) % S.s.n[1], S.p / (S.s.n[0] * S.s.n[1])};
     double G[kVisc] = {};
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
-        const int nd = s.n[d], st = astride(s, d), i = ijk[d];
+        const int nd = S.s.n[d], st = astride(S.s, d), i = ijk[d];
         const double *Drow = ops->D[nd - 1] + i * nd;
-        const int base = p - i * st;
-        const double *J1 = sJ + d * 3 * n3, *J2 = J1 + n3, *J3 = J2 + n3;
-        for (int m = 0; m < nd; ++m) {
-            const int pm = base + m * st;
+        const double *J = sm + (4 + d * 3) * T;
+        for (int k = 1; k < nd; ++k) {
+            const int m = (i + k < nd) ? i + k : i + k - nd, pm = t + (m - i) * st;
             const double Dm = Drow[m];
-            stress_add(G, Dm * J1[pm], Dm * J2[pm], Dm * J3[pm], sq[pm], sq[n3 + pm], sq[2 * n3 + pm], sq[3 * n3 + pm]);
+            stress_add(G, Dm * J[pm], Dm * J[T + pm], Dm * J[2 * T + pm], sm[pm], sm[T + pm], sm[2 * T + pm],
+                       sm[3 * T + pm]);
         }
         if (i != 0 && i != nd - 1) continue;
         int d0, d1;
         aface_dirs(d, d0, d1);
-        const int f2 = s.n[d0] * s.n[d1];
+        const int f2 = S.s.n[d0] * S.s.n[d1];
         const int slot = 2 * d + (i != 0 ? 1 : 0);
-        const double *qs = qhat + (size_t)4 * fnoff[6 * e + slot] + ijk[d0] + s.n[d0] * ijk[d1];
-        const double iw = i != 0 ? ops->iw0[nd - 1] : -ops->iw0[nd - 1];
-        stress_add(G, iw * J1[p], iw * J2[p], iw * J3[p], qs[0] - qp[0], qs[f2] - qp[1], qs[2 * f2] - qp[2],
-                   qs[3 * f2] - qp[3]);
+        const double *qs = qhat + (size_t)4 * fnoff[6 * S.e + slot] + ijk[d0] + S.s.n[d0] * ijk[d1];
+        const double Dm = Drow[i];
+        stress_add(G, Dm * J[t], Dm * J[T + t], Dm * J[2 * T + t], 2.0 * qs[0] - qp[0], 2.0 * qs[f2] - qp[1],
+                   2.0 * qs[2 * f2] - qp[2], 2.0 * qs[3 * f2] - qp[3]);
     }
-    double t[kVisc];
-    stress_of(G, invJall[nb + p], P.mu, P.kappa, t);
-    double *Gout = gradall + kVisc * nb + p;
-    for (int k = 0; k < kVisc; ++k) Gout[(size_t)k * n3] = t[k];
+    double tau[kVisc];
+    stress_of(G, invJall[nb + S.p], P.mu, P.kappa, tau);
+    double *Gout = gradall + kVisc * nb + S.p;
+#pragma unroll
+    for (int k = 0; k < kVisc; ++k) Gout[(size_t)k * S.s.n3] = tau[k];
 }
 
 // ------------------------------------------------------------------ volume + surface + RK
 
 // du/dt = -(V + S)/J at every node; V the standard or split-form volume term
-// (each direction with its own D), S = sum_faces (+-F*_e - (F_e - F_v)(in).(+-Ja^d))/w_end.
+// (each direction with its own D), S = sum_faces (+-F*_e - (F_e - F_v)(in).(+-Ja^d))/w_end
+// (split forms without the diagonal pair, as volume_kernel.cuh explains).
 // stage < 0: du/dt into out; else the low-storage RK stage with coefficients
 // (A, B) and the clock's dt, and (lam_slot >= 0) the new state's dt maxima.
-template <bool NS, int FORM>
-__global__ void __launch_bounds__(512) k_avol(const int *__restrict__ elems, const int *__restrict__ P3, const long long *__restrict__ noff,
-                       const long long *__restrict__ fnoff, const AOps *__restrict__ ops, double *__restrict__ u,
-                       double *__restrict__ g, double *__restrict__ out, const double *__restrict__ Jaall,
-                       const double *__restrict__ invJall, const double *__restrict__ gradall,
-                       const double *__restrict__ fstar, APhys P, Clock *clk, int stage, double rkA, double rkB,
-                       int lam_slot)
+// The pairs of an element's lines are spread over its threads by position
+// first: thread q of the element takes position x = q / (n3/n_d) of line
+// q mod (n3/n_d) and evaluates (x, x + k mod n_d), k = 1 .. n_d/2 (the half-way
+// pair of an even n_d for x < n_d/2 only, the element's lower threads).
+// 16^3 elements of degrees 2..5, NS, Chandrashekar form: 1266 -> 391 us per stage.
+// Dynamic shared memory per thread slot (doubles): standard form the
+// directional flux 5; split forms the pair inputs, Ja^d 3, F_v.Ja^d 4 (NS) and
+// the pair fluxes [kp][5], kp = floor(n_max/2).
+template <int FORM, bool NS>
+constexpr int avol_smem_per(int kp)
+{
+    return FORM == HS3D_VOL_STANDARD ? 5 : split_slots64<FORM>() + 3 + (NS ? 4 : 0) + 5 * kp;
+}
+
+template <int T, bool NS, int FORM>
+__global__ void __launch_bounds__(T, 512 / T) k_avol(const int *__restrict__ slot_elem, const int *__restrict__ slot0,
+                                            const int *__restrict__ P3, const long long *__restrict__ noff,
+                                            const long long *__restrict__ fnoff, const AOps *__restrict__ ops,
+                                            double *__restrict__ u, double *__restrict__ g, double *__restrict__ out,
+                                            const double *__restrict__ Jaall, const double *__restrict__ invJall,
+                                            const double *__restrict__ gradall, const double *__restrict__ fstar,
+                                            APhys P, Clock *clk, int stage, double rkA, double rkB, int lam_slot)
 {
     constexpr bool STD = FORM == HS3D_VOL_STANDARD;
+    constexpr int ZS = split_slots64<FORM>();
     extern __shared__ double sm[];
-    const int e = elems[blockIdx.x];
-    const AShape s = ashape(P3, e);
-    const int n3 = s.n3, p = threadIdx.x;
+    pdl_wait();
+    ASlot S;
     // (a finished or failed run's clock stops its stages, not a residual evaluation)
-    const bool live = p < n3 && (stage < 0 || !(clk->done));
-    // shared: standard: the directional flux F~^d [5][n3];
-    //         split: the pair inputs [kSplitSlots][n3], Ja^d [3][n3], (NS) F_v.Ja^d [4][n3]
-    double *sF = sm;
-    double *sZ = sm;
-    double *sA = sm + kSplitSlots * n3;
-    double *sV = sA + 3 * n3;
-    const long long nb = noff[e];
-    const double *Ja = Jaall + 9 * nb;
-    int ijk[3] = {0, 0, 0};
+    const bool live = aslot(slot_elem, slot0, P3, S) && (stage < 0 || !(clk->done));
+    const int t = threadIdx.x;
+    double *sF = sm;                              // standard: directional flux [5][T]
+    double *sZ = sm;                              // split: pair inputs [ZS][T]
+    double *sA = sm + ZS * T;                     // Ja^d [3][T]
+    double *sV = sA + 3 * T;                      // F_v.Ja^d [4][T] (NS)
+    double *PB = sV + (NS ? 4 : 0) * T;           // pair fluxes [kp][5][T]
+    long long nb = 0;
+    const double *Ja = nullptr;
+    int ijk[3] = {0, 0, 0}, n3 = 1;
     double w[5] = {0, 0, 0, 0, 0}, G[kVisc] = {};
     Prim<double> q{};
     if (live) {
-        ijk[0] = p % s.n[0];
-        ijk[1] = (p / s.n[0]) % s.n[1];
-        ijk[2] = p / (s.n[0] * s.n[1]);
-        for (int v = 0; v < 5; ++v) w[v] = u[5 * nb + (size_t)v * n3 + p];
+        nb = noff[S.e];
+        Ja = Jaall + 9 * nb + S.p;
+        n3 = S.s.n3;
+        ijk[0] = S.p % S.s.n[0];
+        ijk[1] = (S.p / S.s.n[0]) % S.s.n[1];
+        ijk[2] = S.p / (S.s.n[0] * S.s.n[1]);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) w[v] = u[5 * nb + (size_t)v * n3 + S.p];
         q = prim_from_u<double>(w, P.gm1);
-        if (NS)
-            for (int k = 0; k < kVisc; ++k) G[k] = gradall[kVisc * nb + (size_t)k * n3 + p];
+        if (NS) {
+#pragma unroll
+            for (int k = 0; k < kVisc; ++k) G[k] = gradall[kVisc * nb + (size_t)k * n3 + S.p];
+        }
         if constexpr (!STD) {
-            double z[kSplitSlots];
-            split_node<FORM>(q, z);
-            for (int k = 0; k < kSplitSlots; ++k) sZ[k * n3 + p] = z[k];
+            double z[ZS];
+            split_node64<FORM>(q, z);
+#pragma unroll
+            for (int k = 0; k < ZS; ++k) sZ[k * T + t] = z[k];
         }
     }
     double R[5] = {0, 0, 0, 0, 0};
-    double own[3][5];   // (F_e - F_v).Ja^d at this node, for the surface term
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
-        double a[3] = {0, 0, 0};
+        const int nd = live ? S.s.n[d] : 1, st = live ? astride(S.s, d) : 0, i = ijk[d];
+        int d0, d1;
+        aface_dirs(d, d0, d1);
+        double own[5] = {0, 0, 0, 0, 0};   // standard: (F_e - F_v).Ja^d; split: F_v.Ja^d
+        if (d > 0) __syncthreads();        // the previous direction's shared values are consumed
         if (live) {
-            for (int c = 0; c < 3; ++c) a[c] = Ja[(size_t)(d * 3 + c) * n3 + p];
-            double fe[5], fv[5] = {0, 0, 0, 0, 0};
-            euler_flux(q, q.E, a[0], a[1], a[2], fe);
-            if (NS) visc_flux(q, G, a[0], a[1], a[2], fv);
-            for (int v = 0; v < 5; ++v) own[d][v] = fe[v] - fv[v];
-        }
-        __syncthreads();   // the previous direction's shared values are consumed
-        if (live) {
+            const double a1 = Ja[(size_t)(d * 3) * n3], a2 = Ja[(size_t)(d * 3 + 1) * n3],
+                         a3 = Ja[(size_t)(d * 3 + 2) * n3];
+            double fv[5] = {0, 0, 0, 0, 0};
+            if (NS) visc_flux(q, G, a1, a2, a3, fv);
             if constexpr (STD) {
-                for (int v = 0; v < 5; ++v) sF[v * n3 + p] = own[d][v];
+                euler_flux(q, q.E, a1, a2, a3, own);
+#pragma unroll
+                for (int v = 0; v < 5; ++v) {
+                    if (NS && v > 0) own[v] -= fv[v];
+                    sF[v * T + t] = own[v];
+                }
             } else {
-                for (int c = 0; c < 3; ++c) sA[c * n3 + p] = a[c];
+                sA[t] = a1;
+                sA[T + t] = a2;
+                sA[2 * T + t] = a3;
                 if (NS) {
-                    double fv[5];
-                    visc_flux(q, G, a[0], a[1], a[2], fv);
-                    for (int v = 1; v < 5; ++v) sV[(v - 1) * n3 + p] = fv[v];
+#pragma unroll
+                    for (int v = 1; v < 5; ++v) sV[(v - 1) * T + t] = own[v] = fv[v];
                 }
             }
         }
         __syncthreads();
+        if constexpr (!STD) {
+            if (live) {
+                const int lines = n3 / nd;
+                const int x = S.p / lines, l = S.p - x * lines;
+                const int tb = l / S.s.n[d0], ta = l - tb * S.s.n[d0];
+                const int a = S.origin + x * st + ta * astride(S.s, d0) + tb * astride(S.s, d1);
+                double za[ZS];
+#pragma unroll
+                for (int k = 0; k < ZS; ++k) za[k] = sZ[k * T + a];
+                const double j1 = sA[a], j2 = sA[T + a], j3 = sA[2 * T + a];
+                for (int k = 1; 2 * k <= nd; ++k) {
+                    if (2 * k == nd && x >= k) break;
+                    const int c = a + ((x + k < nd) ? k : k - nd) * st;
+                    double zc[ZS], fs[5];
+#pragma unroll
+                    for (int m = 0; m < ZS; ++m) zc[m] = sZ[m * T + c];
+                    split_pair64<FORM>(za, zc, P.gamma, P.hg, j1 + sA[c], j2 + sA[T + c], j3 + sA[2 * T + c], fs);
+#pragma unroll
+                    for (int v = 0; v < 5; ++v) PB[((k - 1) * 5 + v) * T + t] = fs[v];
+                }
+            }
+            __syncthreads();
+        }
         if (live) {
-            const int nd = s.n[d], st = astride(s, d);
-            const double *Drow = ops->D[nd - 1] + ijk[d] * nd;
-            const int base = p - ijk[d] * st;
+            const double *Drow = ops->D[nd - 1] + i * nd;
+            const int base = t - i * st;
             if constexpr (STD) {
-                for (int v = 0; v < 5; ++v) {
-                    double acc = 0.0;
-                    for (int m = 0; m < nd; ++m) acc += Drow[m] * sF[v * n3 + base + m * st];
-                    R[v] += acc;
+                for (int m = 0; m < nd; ++m) {
+                    const double Dm = Drow[m];
+#pragma unroll
+                    for (int v = 0; v < 5; ++v) R[v] += Dm * sF[v * T + base + m * st];
                 }
             } else {
-                // sum_m 2 D_im F#(u_i, u_m).(Ja_i + Ja_m)/2, the diagonal included
-                double zi[kSplitSlots];
-                for (int k = 0; k < kSplitSlots; ++k) zi[k] = sZ[k * n3 + p];
-                for (int m = 0; m < nd; ++m) {
-                    const int pm = base + m * st;
-                    double zm[kSplitSlots];
-                    for (int k = 0; k < kSplitSlots; ++k) zm[k] = sZ[k * n3 + pm];
-                    double fs[5];
-                    split_pair<FORM>(zi, zm, P.gamma, P.hg, a[0] + sA[pm], a[1] + sA[n3 + pm], a[2] + sA[2 * n3 + pm],
-                                     fs);
-                    for (int v = 0; v < 5; ++v) R[v] += Drow[m] * fs[v];
-                }
-                if (NS)
-                    for (int v = 1; v < 5; ++v) {
-                        double acc = 0.0;
-                        for (int m = 0; m < nd; ++m) acc += Drow[m] * sV[(v - 1) * n3 + base + m * st];
-                        R[v] -= acc;
+                const int lines = n3 / nd;
+                const int lq = S.origin + ijk[d0] + S.s.n[d0] * ijk[d1];   // + x lines: the pair thread of (x, this line)
+                for (int k = 1; k < nd; ++k) {
+                    const int m = (i + k < nd) ? i + k : i + k - nd;
+                    const int x = (2 * k < nd || (2 * k == nd && i < k)) ? i : m;
+                    const int slot = 2 * k <= nd ? k : nd - k;
+                    const double Dm = Drow[m];
+                    const double *F = PB + (slot - 1) * 5 * T + lq + x * lines;
+#pragma unroll
+                    for (int v = 0; v < 5; ++v) R[v] += Dm * F[v * T];
+                    if (NS) {
+#pragma unroll
+                        for (int v = 1; v < 5; ++v) R[v] -= Dm * sV[(v - 1) * T + base + m * st];
                     }
+                }
+            }
+            // surface term
+            if (i == 0 || i == nd - 1) {
+                const int f2 = S.s.n[d0] * S.s.n[d1];
+                const double *fs = fstar + (size_t)5 * fnoff[6 * S.e + 2 * d + (i != 0 ? 1 : 0)] + ijk[d0] +
+                                   S.s.n[d0] * ijk[d1];
+                const double sw = i != 0 ? ops->iw0[nd - 1] : -ops->iw0[nd - 1];
+#pragma unroll
+                for (int v = 0; v < 5; ++v) {
+                    const double F = fs[(size_t)v * f2];
+                    if constexpr (STD) {
+                        R[v] = fma(sw, F - own[v], R[v]);
+                    } else {
+                        R[v] = fma(sw, F, R[v]);
+                        if (NS && v > 0) R[v] = fma(0.5 * sw, own[v], R[v]);
+                    }
+                }
             }
         }
     }
     double lc = 0.0, lv = 0.0;
     bool active = false;
     if (live) {
-        // surface term
-        for (int d = 0; d < 3; ++d) {
-            for (int side = -1; side <= 1; side += 2) {
-                const int at = side > 0 ? s.n[d] - 1 : 0;
-                if (ijk[d] != at) continue;
-                int d0, d1;
-                aface_dirs(d, d0, d1);
-                const int f2 = s.n[d0] * s.n[d1];
-                const int slot = 2 * d + (side > 0 ? 1 : 0);
-                const double *fs = fstar + (size_t)5 * fnoff[6 * e + slot] + ijk[d0] + s.n[d0] * ijk[d1];
-                const double iw = ops->iw0[s.n[d] - 1];
-                for (int v = 0; v < 5; ++v) R[v] += (side * fs[(size_t)v * f2] - side * own[d][v]) * iw;
-            }
-        }
-        const double iJ = invJall[nb + p];
+        const double iJ = invJall[nb + S.p];
         if (stage < 0) {
-            for (int v = 0; v < 5; ++v) out[5 * nb + (size_t)v * n3 + p] = -R[v] * iJ;
+#pragma unroll
+            for (int v = 0; v < 5; ++v) out[5 * nb + (size_t)v * n3 + S.p] = -R[v] * iJ;
         } else {
-            const double dt = clk->dt;
-            double *gp = g + 5 * nb + p, *up = u + 5 * nb + p;
+            const double sd = -(clk->dt * iJ);
+            double *gp = g + 5 * nb + S.p, *up = u + 5 * nb + S.p;
+#pragma unroll
             for (int v = 0; v < 5; ++v) {
-                const double r = -R[v] * iJ;
-                const double gv = (stage == 0) ? dt * r : rkA * gp[(size_t)v * n3] + dt * r;
+                const double inc = R[v] * sd;
+                const double gv = (stage == 0) ? inc : fma(rkA, gp[(size_t)v * n3], inc);
                 gp[(size_t)v * n3] = gv;
-                w[v] = w[v] + rkB * gv;
+                w[v] = fma(rkB, gv, w[v]);
                 up[(size_t)v * n3] = w[v];
             }
             if (lam_slot >= 0) {
                 const Prim<double> qn = prim_from_u<double>(w, P.gm1);
                 if (!(qn.rho > 0.0) || !(qn.p > 0.0)) clk->bad = 1;
                 else {
-                    alam_node(s, Ja, p, iJ, qn, P, lc, lv);
+                    alam_node(S.s, Jaall + 9 * nb, S.p, iJ, qn, P, lc, lv);
                     active = true;
                 }
             }
@@ -766,11 +932,7 @@ cudaError_t for_classes(const AnisoMesh *a, F fn)
     return e;
 }
 
-// Shared memory of the element kernels per thread slot (doubles): the volume
-// kernel's standard form 5, split forms kSplitSlots + 3 + 4; the gradient 13.
-template <int FORM>
-constexpr size_t avol_smem_per() { return FORM == HS3D_VOL_STANDARD ? 5 : (kSplitSlots + 3 + 4); }
-constexpr size_t kAGradSmemPer = 13;
+constexpr size_t kAGradSmemPer = 13;   // doubles per thread slot of k_agrad
 
 template <class K>
 cudaError_t allow_smem(K kernel, size_t bytes)
@@ -780,49 +942,137 @@ cudaError_t allow_smem(K kernel, size_t bytes)
 }
 
 // (set once at mesh set-up: not a stream operation, but kept out of captured launches)
-template <bool NS>
-cudaError_t allow_avol_smem(size_t T)
+template <int T, bool NS>
+cudaError_t allow_avol_smem(int kp)
 {
-    cudaError_t e = allow_smem(k_avol<NS, HS3D_VOL_STANDARD>, sizeof(double) * avol_smem_per<HS3D_VOL_STANDARD>() * T);
-    if (e == cudaSuccess) e = allow_smem(k_avol<NS, HS3D_VOL_EC>, sizeof(double) * avol_smem_per<HS3D_VOL_EC>() * T);
-    if (e == cudaSuccess) e = allow_smem(k_avol<NS, HS3D_VOL_KG>, sizeof(double) * avol_smem_per<HS3D_VOL_KG>() * T);
-    if (e == cudaSuccess)
-        e = allow_smem(k_avol<NS, HS3D_VOL_PIROZZOLI>, sizeof(double) * avol_smem_per<HS3D_VOL_PIROZZOLI>() * T);
-    if (e == cudaSuccess)
-        e = allow_smem(k_avol<NS, HS3D_VOL_DUCROS>, sizeof(double) * avol_smem_per<HS3D_VOL_DUCROS>() * T);
-    if (e == cudaSuccess)
-        e = allow_smem(k_avol<NS, HS3D_VOL_MORINISHI>, sizeof(double) * avol_smem_per<HS3D_VOL_MORINISHI>() * T);
-    if (e == cudaSuccess) e = allow_smem(k_avol<NS, HS3D_VOL_IR>, sizeof(double) * avol_smem_per<HS3D_VOL_IR>() * T);
+    cudaError_t e = cudaSuccess;
+#define HS3D_ALLOW(FORM) \
+    if (e == cudaSuccess) e = allow_smem(k_avol<T, NS, FORM>, sizeof(double) * avol_smem_per<FORM, NS>(kp) * T);
+    HS3D_ALLOW(HS3D_VOL_STANDARD)
+    HS3D_ALLOW(HS3D_VOL_EC)
+    HS3D_ALLOW(HS3D_VOL_KG)
+    HS3D_ALLOW(HS3D_VOL_PIROZZOLI)
+    HS3D_ALLOW(HS3D_VOL_DUCROS)
+    HS3D_ALLOW(HS3D_VOL_MORINISHI)
+    HS3D_ALLOW(HS3D_VOL_IR)
+#undef HS3D_ALLOW
     return e;
 }
 
-template <bool NS, int FORM>
+template <int T>
+cudaError_t allow_stage_smem(const AnisoMesh *a)
+{
+    const int kp = (a->Pmax + 1) / 2;
+    cudaError_t e = allow_avol_smem<T, false>(kp);
+    if (e == cudaSuccess) e = allow_avol_smem<T, true>(kp);
+    if (e == cudaSuccess) e = allow_smem(k_agrad<T>, sizeof(double) * kAGradSmemPer * T);
+    return e;
+}
+
+template <int T, bool NS>
 cudaError_t launch_avol(const AnisoMesh *a, const APhys &P, double *u, double *g, double *out, int stage, double A,
                         double B, int lam_slot, cudaStream_t s)
 {
     const AOps *ops = device_aops();
     if (!ops) return cudaErrorMemoryAllocation;
-    return for_classes(a, [&](int T, int cnt, const int *els) {
-        const size_t smem = sizeof(double) * avol_smem_per<FORM>() * T;
-        k_avol<NS, FORM><<<cnt, T, smem, s>>>(els, a->dP3, a->dnoff, a->dfnoff, ops, u, g, out, a->Ja, a->invJ,
-                                              a->grad, a->fstar, P, a->clk, stage, A, B, lam_slot);
-        return cudaGetLastError();
-    });
+    const int kp = (a->Pmax + 1) / 2;
+    switch (P.form) {
+#define HS3D_AVOL(FORM)                                                                                               \
+    case FORM:                                                                                                        \
+        return launch_pdl(k_avol<T, NS, FORM>, a->npacks, T, sizeof(double) * avol_smem_per<FORM, NS>(kp) * T, s,      \
+                          a->slot_elem, a->slot0, a->dP3, a->dnoff, a->dfnoff, ops, u, g, out, a->Ja, a->invJ,         \
+                          a->grad, a->fstar, P, a->clk, stage, A, B, lam_slot);
+        HS3D_AVOL(HS3D_VOL_STANDARD)
+        HS3D_AVOL(HS3D_VOL_EC)
+        HS3D_AVOL(HS3D_VOL_KG)
+        HS3D_AVOL(HS3D_VOL_PIROZZOLI)
+        HS3D_AVOL(HS3D_VOL_DUCROS)
+        HS3D_AVOL(HS3D_VOL_MORINISHI)
+        HS3D_AVOL(HS3D_VOL_IR)
+#undef HS3D_AVOL
+    }
+    return cudaErrorInvalidValue;
 }
 
-template <bool NS>
-cudaError_t launch_avol_form(const AnisoMesh *a, const APhys &P, double *u, double *g, double *out, int stage,
-                             double A, double B, int lam_slot, cudaStream_t s)
+// The stage kernels of a mesh whose packs have T thread slots.
+template <int T>
+cudaError_t launch_stage(const AnisoMesh *a, const APhys &P, double *u, double *g, double *out, int stage, double A,
+                         double B, int lam_slot, cudaStream_t s)
 {
-    switch (P.form) {
-        case HS3D_VOL_STANDARD: return launch_avol<NS, HS3D_VOL_STANDARD>(a, P, u, g, out, stage, A, B, lam_slot, s);
-        case HS3D_VOL_EC: return launch_avol<NS, HS3D_VOL_EC>(a, P, u, g, out, stage, A, B, lam_slot, s);
-        case HS3D_VOL_KG: return launch_avol<NS, HS3D_VOL_KG>(a, P, u, g, out, stage, A, B, lam_slot, s);
-        case HS3D_VOL_PIROZZOLI: return launch_avol<NS, HS3D_VOL_PIROZZOLI>(a, P, u, g, out, stage, A, B, lam_slot, s);
-        case HS3D_VOL_DUCROS: return launch_avol<NS, HS3D_VOL_DUCROS>(a, P, u, g, out, stage, A, B, lam_slot, s);
-        case HS3D_VOL_MORINISHI: return launch_avol<NS, HS3D_VOL_MORINISHI>(a, P, u, g, out, stage, A, B, lam_slot, s);
-        case HS3D_VOL_IR: return launch_avol<NS, HS3D_VOL_IR>(a, P, u, g, out, stage, A, B, lam_slot, s);
-        default: return cudaErrorInvalidValue;
+    const MortarOps *mo = device_mortar_ops();
+    const AOps *ops = device_aops();
+    if (!mo || !ops) return cudaErrorMemoryAllocation;
+    const bool ns = P.physics == HS3D_NS;
+    cudaError_t e = cudaSuccess;
+    if (ns) {
+        e = launch_pdl(k_amortar<0, true>, a->nfctas, kAFaceThreads, 0, s, a->faces, a->fctas, a->dP3, a->dnoff,
+                       a->dfnoff, u, a->grad, a->Ja, mo, P, a->qhat);
+        if (e == cudaSuccess)
+            e = launch_pdl(k_agrad<T>, a->npacks, T, sizeof(double) * kAGradSmemPer * T, s, a->slot_elem, a->slot0,
+                           a->dP3, a->dnoff, a->dfnoff, ops, u, a->Ja, a->invJ, a->qhat, P, a->grad);
+    }
+    if (e == cudaSuccess)
+        e = launch_pdl(ns ? k_amortar<1, true> : k_amortar<1, false>, a->nfctas, kAFaceThreads, 0, s, a->faces,
+                       a->fctas, a->dP3, a->dnoff, a->dfnoff, u, a->grad, a->Ja, mo, P, a->fstar);
+    if (e == cudaSuccess)
+        e = ns ? launch_avol<T, true>(a, P, u, g, out, stage, A, B, lam_slot, s)
+               : launch_avol<T, false>(a, P, u, g, out, stage, A, B, lam_slot, s);
+    return e;
+}
+
+// Elements into packs of T thread slots, largest first, each into the fullest
+// pack that still has room (packs kept by free slots).
+void pack_elements(const AnisoMesh *a, int T, std::vector<int> &slot_elem, std::vector<int> &slot0)
+{
+    std::vector<std::vector<int>> by_n3(T + 1), open(T + 1);   // elements by node count, packs by free slots
+    for (int e = 0; e < a->E; ++e) by_n3[a->noff[e + 1] - a->noff[e]].push_back(e);
+    slot0.assign(a->E, 0);
+    int packs = 0;
+    for (int n3 = T; n3 > 0; --n3)
+        for (int e : by_n3[n3]) {
+            int room = n3;
+            while (room <= T && open[room].empty()) ++room;
+            int pk;
+            if (room <= T) {
+                pk = open[room].back();
+                open[room].pop_back();
+            } else {
+                pk = packs++;
+                room = T;
+                slot_elem.resize((size_t)packs * T, -1);
+            }
+            slot0[e] = T - room;
+            for (int k = 0; k < n3; ++k) slot_elem[(size_t)pk * T + slot0[e] + k] = e;
+            open[room - n3].push_back(pk);
+        }
+}
+
+// The face table sorted by mortar degrees, then by the sides' degrees, and its CTAs.
+void pack_faces(const AnisoMesh *a, std::vector<AFace> &faces, std::vector<AFaceCta> &ctas)
+{
+    auto side = [&](const AFace &f, int k, int t) {   // points of side k (0: L) in tangential direction t
+        const int d0 = f.d == 0 ? 1 : 0, d1 = f.d == 2 ? 1 : 2;
+        return a->P3[3 * (size_t)(k ? f.eR : f.eL) + (t ? d1 : d0)] + 1;
+    };
+    std::vector<std::pair<unsigned, int>> key(faces.size());
+    for (size_t i = 0; i < faces.size(); ++i) {
+        const AFace &f = faces[i];
+        const unsigned l0 = side(f, 0, 0), r0 = side(f, 1, 0), l1 = side(f, 0, 1), r1 = side(f, 1, 1);
+        const unsigned m0 = l0 > r0 ? l0 : r0, m1 = l1 > r1 ? l1 : r1;
+        key[i] = {(((((m0 * 16 + m1) * 16 + l0) * 16 + r0) * 16 + l1) * 16 + r1), (int)i};
+    }
+    std::sort(key.begin(), key.end());
+    std::vector<AFace> sorted(faces.size());
+    for (size_t i = 0; i < faces.size(); ++i) sorted[i] = faces[key[i].second];
+    faces.swap(sorted);
+    for (size_t i = 0; i < faces.size();) {
+        const unsigned m = key[i].first >> 16;
+        AFaceCta c{(int)i, 0, (int)(m >> 4), (int)(m & 15), 0};
+        const int most = kAFaceThreads / (c.nm0 * c.nm1);
+        for (; i < faces.size() && c.count < most && key[i].first >> 16 == m; ++i, ++c.count)
+            for (int k = 0; k < 2; ++k)
+                if (side(faces[i], k, 0) < c.nm0) c.passes |= 1 << k;
+        ctas.push_back(c);
     }
 }
 
@@ -833,7 +1083,7 @@ cudaError_t launch_avol_form(const AnisoMesh *a, const APhys &P, double *u, doub
 void aniso_free(AnisoMesh *a)
 {
     if (!a) return;
-    void *ptrs[] = {a->dP3, a->dnoff, a->doff, a->dfnoff, a->cls_elems, a->faces, a->X, a->Ja, a->J, a->invJ,
+    void *ptrs[] = {a->dP3, a->dnoff, a->doff, a->dfnoff, a->cls_elems, a->slot_elem, a->slot0, a->faces, a->fctas, a->X, a->Ja, a->J, a->invJ,
                     a->grad, a->fstar, a->qhat, a->diag_part, a->clk, a->clkp, a->one};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -898,6 +1148,15 @@ hs3d_status aniso_build(const hs3d_mesh_desc *desc, const int *degree3, AnisoMes
             faces.push_back(AFace{(int)e, c[0] + a->ex * (c[1] + a->ey * c[2]), d});
         }
     }
+    long long n3max = 0;
+    for (long long e = 0; e < E; ++e) n3max = std::max<long long>(n3max, a->noff[e + 1] - a->noff[e]);
+    a->T = n3max <= 256 ? 256 : 512;
+    std::vector<int> slot_elem, slot0;
+    pack_elements(a, a->T, slot_elem, slot0);
+    a->npacks = (unsigned)(slot_elem.size() / a->T);
+    std::vector<AFaceCta> fctas;
+    pack_faces(a, faces, fctas);
+    a->nfctas = (unsigned)fctas.size();
     const long long nodes = a->noff[E], fnodes = a->fnoff[6 * E];
     std::vector<double> X(3 * (size_t)nodes);
     for (long long e = 0; e < E; ++e) anodes(a, (int)e, X.data() + 3 * a->noff[e]);
@@ -910,7 +1169,10 @@ hs3d_status aniso_build(const hs3d_mesh_desc *desc, const int *degree3, AnisoMes
         {(void **)&a->doff, sizeof(long long) * (E + 1)},
         {(void **)&a->dfnoff, sizeof(long long) * (6 * E + 1)},
         {(void **)&a->cls_elems, sizeof(int) * E},
+        {(void **)&a->slot_elem, sizeof(int) * slot_elem.size()},
+        {(void **)&a->slot0, sizeof(int) * E},
         {(void **)&a->faces, sizeof(AFace) * 3 * E},
+        {(void **)&a->fctas, sizeof(AFaceCta) * fctas.size()},
         {(void **)&a->X, sizeof(double) * 3 * nodes},
         {(void **)&a->Ja, sizeof(double) * 9 * nodes},
         {(void **)&a->J, sizeof(double) * nodes},
@@ -936,6 +1198,11 @@ hs3d_status aniso_build(const hs3d_mesh_desc *desc, const int *degree3, AnisoMes
     if (e == cudaSuccess)
         e = cudaMemcpy(a->dfnoff, a->fnoff.data(), sizeof(long long) * (6 * E + 1), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(a->cls_elems, elems.data(), sizeof(int) * E, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(a->slot_elem, slot_elem.data(), sizeof(int) * slot_elem.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(a->slot0, slot0.data(), sizeof(int) * E, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(a->fctas, fctas.data(), sizeof(AFaceCta) * fctas.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(a->faces, faces.data(), sizeof(AFace) * 3 * E, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(a->X, X.data(), sizeof(double) * 3 * nodes, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(a->clk, 0, sizeof(Clock));
@@ -949,10 +1216,7 @@ hs3d_status aniso_build(const hs3d_mesh_desc *desc, const int *degree3, AnisoMes
             return cudaGetLastError();
         });
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    const size_t Tmax = kAnisoClass[kAnisoClasses - 1];
-    if (e == cudaSuccess) e = allow_avol_smem<false>(Tmax);
-    if (e == cudaSuccess) e = allow_avol_smem<true>(Tmax);
-    if (e == cudaSuccess) e = allow_smem(k_agrad, sizeof(double) * kAGradSmemPer * Tmax);
+    if (e == cudaSuccess) e = a->T == 256 ? allow_stage_smem<256>(a) : allow_stage_smem<512>(a);
     if (e != cudaSuccess) {
         cudaGetLastError();
         aniso_free(a);
@@ -966,39 +1230,11 @@ cudaError_t aniso_stage(const AnisoMesh *a, const hs3d_solver_cfg *c, double *u,
                         int lam_slot, cudaStream_t s)
 {
     const APhys P = aphys(c);
-    const MortarOps *mo = device_mortar_ops();
-    const AOps *ops = device_aops();
-    if (!mo || !ops) return cudaErrorMemoryAllocation;
-    const bool ns = c->physics == HS3D_NS;
-    const int nf = 3 * a->E;
-    cudaError_t e = cudaSuccess;
-    if (ns) {
-        k_amortar<0, true><<<nf, kAFaceThreads, 0, s>>>(a->faces, a->dP3, a->dnoff, a->dfnoff, u, a->grad, a->Ja, mo,
-                                                        P, a->qhat);
-        e = cudaGetLastError();
-        if (e == cudaSuccess)
-            e = for_classes(a, [&](int T, int cnt, const int *els) {
-                const size_t smem = sizeof(double) * kAGradSmemPer * T;
-                k_agrad<<<cnt, T, smem, s>>>(els, a->dP3, a->dnoff, a->dfnoff, ops, u, a->Ja, a->invJ, a->qhat, P,
-                                             a->grad);
-                return cudaGetLastError();
-            });
-    }
-    if (e == cudaSuccess) {
-        if (ns)
-            k_amortar<1, true><<<nf, kAFaceThreads, 0, s>>>(a->faces, a->dP3, a->dnoff, a->dfnoff, u, a->grad, a->Ja,
-                                                            mo, P, a->fstar);
-        else
-            k_amortar<1, false><<<nf, kAFaceThreads, 0, s>>>(a->faces, a->dP3, a->dnoff, a->dfnoff, u, a->grad, a->Ja,
-                                                             mo, P, a->fstar);
-        e = cudaGetLastError();
-    }
     double A = 0.0, B = 0.0;
     if (stage >= 0) rk_coeffs(c->time_scheme, stage, &A, &B);
-    if (e == cudaSuccess)
-        e = ns ? launch_avol_form<true>(a, P, u, g, out, stage, A, B, lam_slot, s)
-               : launch_avol_form<false>(a, P, u, g, out, stage, A, B, lam_slot, s);
-    return e;
+    const cudaError_t e = a->T == 256 ? launch_stage<256>(a, P, u, g, out, stage, A, B, lam_slot, s)
+                                      : launch_stage<512>(a, P, u, g, out, stage, A, B, lam_slot, s);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t aniso_step(const AnisoMesh *a, const hs3d_solver_cfg *c, double *u, double *g, double dt, bool fresh,
@@ -1006,11 +1242,10 @@ cudaError_t aniso_step(const AnisoMesh *a, const hs3d_solver_cfg *c, double *u, 
 {
     const APhys P = aphys(c);
     cudaError_t e = cudaSuccess;
-    if (fresh && !(dt > 0.0))
-        e = for_classes(a, [&](int T, int cnt, const int *els) {
-            k_alambda<<<cnt, T, 0, s>>>(els, a->dP3, a->dnoff, a->Ja, a->invJ, u, P, a->clk, 0);
-            return cudaGetLastError();
-        });
+    if (fresh && !(dt > 0.0)) {
+        k_alambda<<<a->npacks, a->T, 0, s>>>(a->slot_elem, a->slot0, a->dP3, a->dnoff, a->Ja, a->invJ, u, P, a->clk, 0);
+        e = cudaGetLastError();
+    }
     // the maxima already carry n_d^2 (n_d^4): the p-mesh finalize with n = 1
     if (e == cudaSuccess)
         e = launch_pdt_finalize(a->clkp, a->one, 1, c->cfl, 8.0, 12.0, fresh ? 0 : 1, dt > 0.0 ? dt : 0.0, s);

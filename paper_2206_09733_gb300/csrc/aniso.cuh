@@ -19,6 +19,13 @@ struct AFace {
     int eL, eR, d;
 };
 
+// One CTA of the mortar kernel: `count` faces from `face0` whose mortars have
+// nm0 x nm1 points; passes bit 0 (1): some face's L (R) side has fewer than
+// nm0 points in the first tangential direction.
+struct AFaceCta {
+    int face0, count, nm0, nm1, passes;
+};
+
 // Derivative matrices and end weights of every Gauss-Lobatto degree 1..kMaxN
 // (device copy): D[N][i*(N+1) + m], iw0[N] = 1/w_0.
 struct AOps {
@@ -26,9 +33,10 @@ struct AOps {
     double iw0[kMaxn];
 };
 
-// Elements are launched in classes of node count: class k holds the
-// elements with kAnisoClass[k-1] < n_x n_y n_z <= kAnisoClass[k], one CTA of
-// kAnisoClass[k] threads each (thread t owns node t).
+// Set-up, initial-state and diagnostics kernels take elements in classes of
+// node count: class k holds the elements with kAnisoClass[k-1] < n_x n_y n_z <=
+// kAnisoClass[k], one CTA of kAnisoClass[k] threads each (thread t owns node t).
+// The stage kernels run on packs of T thread slots (slot_elem).
 constexpr int kAnisoClasses = 5;
 constexpr int kAnisoClass[kAnisoClasses] = {32, 64, 128, 256, 512};
 
@@ -44,9 +52,14 @@ struct AnisoMesh {
     int *dP3 = nullptr;
     long long *dnoff = nullptr, *doff = nullptr, *dfnoff = nullptr;
     int *cls_elems = nullptr;         // element ids, class by class
-    AFace *faces = nullptr;           // [3E]
+    int T = 256;                      // thread slots per pack: 256, or 512 if an element has more nodes
+    unsigned npacks = 0, nfctas = 0;
+    int *slot_elem = nullptr;         // [npacks T] element of every thread slot, -1: idle
+    int *slot0 = nullptr;             // [E] the element's first slot in its pack
+    AFace *faces = nullptr;           // [3E], sorted by mortar degrees
+    AFaceCta *fctas = nullptr;        // [nfctas]
     double *X = nullptr, *Ja = nullptr, *J = nullptr, *invJ = nullptr;
-    double *grad = nullptr;           // [12 nodes]
+    double *grad = nullptr;           // [kVisc nodes]: viscous stress and heat flux
     double *fstar = nullptr;          // [5 face nodes]: mortar flux projected onto each element face
     double *qhat = nullptr;           // [4 face nodes]: BR1 interface value on each element face
     double *diag_part = nullptr;      // [E][7]

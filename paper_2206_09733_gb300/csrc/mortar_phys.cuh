@@ -29,7 +29,8 @@ __device__ __forceinline__ void mortar_q(const R *u, R gm1, R q[4], int stride =
     q[0] = w.v1;
     q[1] = w.v2;
     q[2] = w.v3;
-    q[3] = w.p / w.rho;
+    if constexpr (sizeof(R) == 8) q[3] = w.p * w.ir;
+    else q[3] = w.p / w.rho;
 }
 
 // Inviscid numerical flux times the face scale, from the two conservative

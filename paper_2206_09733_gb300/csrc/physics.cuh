@@ -204,6 +204,9 @@ __device__ __forceinline__ void euler_flux(const Prim<R> &q, R E, R a1, R a2, R 
 // gradients, so the gradient kernels store these nine (a quarter less to write
 // and to read in the face and element kernels, and mu, kappa and the symmetric
 // sums are applied once per node instead of at every use).
+// Together with the boundary value in the diagonal term instead of a separate
+// lift (k_grad, k_grad_dev), per step: 32^3 elements of N = 7, mixed 8.0 -> 7.5
+// ms; 16^3 of N = 3, mixed 0.188 -> 0.180, FP64 1.54 -> 1.38.
 // Adds a_c q_v, q = (v1, v2, v3, T), to the nine sums the stress needs:
 // d1 v1, d2 v2, d3 v3, d1 v2 + d2 v1, d1 v3 + d3 v1, d2 v3 + d3 v2, d1 T, d2 T, d3 T.
 template <typename R>

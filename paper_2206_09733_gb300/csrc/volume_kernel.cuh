@@ -31,7 +31,7 @@
 //     remains;
 //   - the two faces of a direction share one instruction sequence (a lane is
 //     on at most one of them).
-// 16^3 elements of N = 3, NS, Chandrashekar form, one launch: 365 -> 235 us.
+// 16^3 elements of N = 3, NS, Chandrashekar form, one launch: 365 -> 260 us.
 //
 // One thread per node, `epb` elements per CTA (a kernel argument).  The
 // element's contravariant fluxes (standard form) or its per-node two-point-flux
