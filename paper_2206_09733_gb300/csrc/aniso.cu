@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(512) k_alambda(const int *__restrict__ slot_el
         if (!(q.rho > 0.0) || !(q.p > 0.0)) clk->bad = 1;
         else alam_node(S.s, Jaall + 9 * nb, S.p, invJall[nb + S.p], q, P, lc, lv);
     }
-    warp_max_to_clock(&clk->lam[slot][0], P.physics == HS3D_NS ? &clk->lam[slot][1] : nullptr, lc, lv, live);
+    cta_max_to_clock<double>(clk->lam[slot], P.physics == HS3D_NS, lc, lv);
 }
 
 // ------------------------------------------------------------------ mortar faces
@@ -704,7 +704,6 @@ __global__ void __launch_bounds__(T, 512 / T) k_avol(const int *__restrict__ slo
         }
     }
     double lc = 0.0, lv = 0.0;
-    bool active = false;
     if (live) {
         const double iJ = invJall[nb + S.p];
         if (stage < 0) {
@@ -724,17 +723,11 @@ __global__ void __launch_bounds__(T, 512 / T) k_avol(const int *__restrict__ slo
             if (lam_slot >= 0) {
                 const Prim<double> qn = prim_from_u<double>(w, P.gm1);
                 if (!(qn.rho > 0.0) || !(qn.p > 0.0)) clk->bad = 1;
-                else {
-                    alam_node(S.s, Jaall + 9 * nb, S.p, iJ, qn, P, lc, lv);
-                    active = true;
-                }
+                else alam_node(S.s, Jaall + 9 * nb, S.p, iJ, qn, P, lc, lv);
             }
         }
     }
-    // (one call site: the warp reduction needs every lane)
-    if (lam_slot >= 0 && stage >= 0)
-        warp_max_to_clock(active ? &clk->lam[lam_slot][0] : nullptr,
-                          active && P.physics == HS3D_NS ? &clk->lam[lam_slot][1] : nullptr, lc, lv, active);
+    if (lam_slot >= 0 && stage >= 0) cta_max_to_clock<double>(clk->lam[lam_slot], P.physics == HS3D_NS, lc, lv);
 }
 
 // ------------------------------------------------------------------ diagnostics
@@ -937,7 +930,8 @@ constexpr size_t kAGradSmemPer = 13;   // doubles per thread slot of k_agrad
 template <class K>
 cudaError_t allow_smem(K kernel, size_t bytes)
 {
-    return bytes > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)
+    // (the kernels' own static shared memory counts toward the 48 KB too)
+    return bytes > 40 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)
                              : cudaSuccess;
 }
 

@@ -35,7 +35,7 @@ __device__ __forceinline__ int face_node(int d, int end, int ta, int tb)
 }
 
 // Small CTAs: with its 142 registers a 256-thread CTA leaves one CTA (8 warps)
-// per SM, 64-thread CTAs 14 warps, and a small mesh reaches more SMs (16^3,
+// per SM, 64-thread CTAs 12 warps, and a small mesh reaches more SMs (16^3,
 // N = 3: 118 -> 98 us).
 constexpr int kFaceThreads = 64;
 

@@ -197,10 +197,22 @@ __device__ __forceinline__ const Item &find_item_face(const Batch &b, long long 
     return b.items[lo];
 }
 
+// Raise a clock maximum (bits of a non-negative double) to v.  Within a launch
+// the maximum only grows, so the value read first (it may be an older one from
+// L1; what earlier launches wrote is visible after pdl_wait) is never above
+// the true one, and only calls that cannot raise it skip the atomic: millions
+// of atomics on one address would otherwise queue up in its L2 slice.
+__device__ __forceinline__ void raise_max(unsigned long long *dst, unsigned long long v)
+{
+    unsigned long long cur;
+    asm volatile("ld.global.ca.u64 %0, [%1];" : "=l"(cur) : "l"(dst) : "memory");
+    if (v > cur) atomicMax(dst, v);
+}
+
 // Max-reduce non-negative rates over the lanes of a warp that share the same
 // clock (threads map to consecutive nodes and an item's elements are
-// consecutive, so each group is a contiguous run of lanes) and add them to
-// that clock slot with one atomic per group.  All 32 lanes must call this.
+// consecutive, so each group is a contiguous run of lanes).  The bits of
+// non-negative doubles order as integers.  All 32 lanes must call this.
 __device__ __forceinline__ void warp_max_to_clock(unsigned long long *dst_c, unsigned long long *dst_v, double lc,
                                                   double lv, bool active)
 {
@@ -210,19 +222,79 @@ __device__ __forceinline__ void warp_max_to_clock(unsigned long long *dst_c, uns
     unsigned peers = __match_any_sync(full, key);
     const int first = __ffs(peers) - 1;
     const int last = 31 - __clz(peers);
+    unsigned long long bc = (unsigned long long)__double_as_longlong(lc), bv = (unsigned long long)__double_as_longlong(lv);
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-        double oc = __shfl_down_sync(full, lc, off);
-        double ov = __shfl_down_sync(full, lv, off);
+        const unsigned long long oc = __shfl_down_sync(full, bc, off), ov = __shfl_down_sync(full, bv, off);
         if (lane + off <= last) {
-            lc = fmax(lc, oc);
-            lv = fmax(lv, ov);
+            bc = oc > bc ? oc : bc;
+            bv = ov > bv ? ov : bv;
         }
     }
     if (active && lane == first) {
-        atomicMax(dst_c, (unsigned long long)__double_as_longlong(lc));
-        if (dst_v) atomicMax(dst_v, (unsigned long long)__double_as_longlong(lv));
+        raise_max(dst_c, bc);
+        if (dst_v) raise_max(dst_v, bv);
     }
+}
+
+// Warp maximum of non-negative values as the bits of a double (lanes of `mask`).
+__device__ __forceinline__ unsigned long long warp_max_bits(unsigned mask, float v)
+{
+    const unsigned m = __reduce_max_sync(mask, __float_as_uint(v));
+    return (unsigned long long)__double_as_longlong((double)__uint_as_float(m));
+}
+__device__ __forceinline__ unsigned long long warp_max_bits(unsigned mask, double v)
+{
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const unsigned mh = __reduce_max_sync(mask, hi);
+    const unsigned ml = __reduce_max_sync(mask, hi == mh ? lo : 0u);
+    return ((unsigned long long)mh << 32) | ml;
+}
+
+// The same over a whole CTA whose nodes belong to one clock: one integer
+// reduction per warp and at most one atomic per CTA and rate (per warp they took
+// a quarter of the last stage's element kernel, 32^3 elements of N = 7: 1545 ->
+// 1332 us, and most of the dt pass, 1048 -> 264 us).  lam: the clock's slot; every
+// thread of the CTA must call this, inactive ones with zeros.
+template <typename R>
+__device__ __forceinline__ void cta_max_to_clock(unsigned long long *lam, bool ns, R lc, R lv)
+{
+    __shared__ unsigned long long part[2][16];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = (int)(blockDim.x + 31) >> 5;
+    const int left = (int)blockDim.x - (warp << 5);
+    const unsigned mask = left >= 32 ? 0xffffffffu : (1u << left) - 1u;
+    const unsigned long long wc = warp_max_bits(mask, lc), wv = ns ? warp_max_bits(mask, lv) : 0ull;
+    if (lane == 0) {
+        part[0][warp] = wc;
+        part[1][warp] = wv;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {   // thread 0 the convective, thread 1 the viscous rate
+        unsigned long long m = part[threadIdx.x][0];
+        for (int k = 1; k < nwarps; ++k) {
+            const unsigned long long o = part[threadIdx.x][k];
+            m = o > m ? o : m;
+        }
+        raise_max(lam + threadIdx.x, m);
+    }
+}
+
+// dt maxima of a launch's nodes into their items' clocks (slot `slot`): every
+// thread of the CTA calls it with the same b, slot and ns.
+template <typename R>
+__device__ __forceinline__ void rates_to_clock(const Batch &b, const Item *itp, int slot, bool ns, R lc, R lv,
+                                               bool active)
+{
+    if (b.nitems == 1) {
+        cta_max_to_clock<R>(b.single.clk->lam[slot], ns, active ? lc : (R)0, active ? lv : (R)0);
+        return;
+    }
+    unsigned long long *dc = nullptr, *dv = nullptr;
+    if (active) {
+        dc = &itp->clk->lam[slot][0];
+        dv = ns ? &itp->clk->lam[slot][1] : nullptr;
+    }
+    warp_max_to_clock(dc, dv, (double)lc, (double)lv, active);
 }
 
 // Programmatic dependent launch: a kernel launched by launch_pdl may be

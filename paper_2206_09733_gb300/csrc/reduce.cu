@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(256) k_lambda(const __grid_constant__ Batch b,
 {
     constexpr int n = N + 1, n3 = n * n * n;
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    double lc = 0.0, lv = 0.0;
+    R lc = (R)0, lv = (R)0;
     bool active = false;
     const Item *itp = nullptr;
     if (t < b.total_elems * n3) {
@@ -88,18 +88,13 @@ __global__ void __launch_bounds__(256) k_lambda(const __grid_constant__ Batch b,
                 lc = sc * iJ;
                 if (ns) lv = P.mu * sv * (iJ * iJ) * q.ir;
             } else {
-                lc = widen<R>(sc);
-                if (ns) lv = widen<R>(P.mu * sv / q.rho);
+                lc = sc;
+                if (ns) lv = P.mu * sv / q.rho;
             }
             active = true;
         }
     }
-    unsigned long long *dc = nullptr, *dv = nullptr;
-    if (active) {
-        dc = &itp->clk->lam[slot][0];
-        dv = ns ? &itp->clk->lam[slot][1] : nullptr;
-    }
-    warp_max_to_clock(dc, dv, lc, lv, active);
+    rates_to_clock<R>(b, itp, slot, ns, lc, lv, active);
 }
 
 // One thread per item: dt from the maxima in clock slot `slot` (or the fixed

@@ -611,7 +611,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
             if (itp->clk) itp->clk->bad = 2;
         }
     }
-    double lc = 0.0, lv = 0.0;
+    float lc = 0.0f, lv = 0.0f;
     bool lam_active = false;
     if (valid) {
     const Item &it = *itp;
@@ -739,21 +739,14 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                     sc += (fabsf(a1 * qn.v1 + a2 * qn.v2 + a3 * qn.v3) + c * an) * ijf;
                     sv += (an * ijf) * (an * ijf);
                 }
-                lc = f2d_exact(sc);
-                lv = NS ? f2d_exact(it.muf * sv / qn.rho) : 0.0;
+                lc = sc;
+                lv = NS ? it.muf * sv / qn.rho : 0.0f;
                 lam_active = true;
             }
         }
     }
     }
-    if (lam_slot >= 0 && stage >= 0) {
-        unsigned long long *dc = nullptr, *dvp = nullptr;
-        if (lam_active) {
-            dc = &itp->clk->lam[lam_slot][0];
-            dvp = NS ? &itp->clk->lam[lam_slot][1] : nullptr;
-        }
-        warp_max_to_clock(dc, dvp, lc, lv, lam_active);
-    }
+    if (lam_slot >= 0 && stage >= 0) rates_to_clock<float>(b, itp, lam_slot, NS, lc, lv, lam_active);
     return armed;
 }
 

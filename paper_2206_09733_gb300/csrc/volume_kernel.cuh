@@ -422,14 +422,7 @@ k_volume(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int stage
         }
         node_update<double, NS>(it, e, p, n3, V, u, stage, rkA, rkB, lam_slot, lc, lv, lam_active);
     }
-    if (lam_slot >= 0 && stage >= 0) {
-        unsigned long long *dc = nullptr, *dv = nullptr;
-        if (lam_active) {
-            dc = &itp->clk->lam[lam_slot][0];
-            dv = NS ? &itp->clk->lam[lam_slot][1] : nullptr;
-        }
-        warp_max_to_clock(dc, dv, lc, lv, lam_active);
-    }
+    if (lam_slot >= 0 && stage >= 0) rates_to_clock<double>(b, itp, lam_slot, NS, lc, lv, lam_active);
 }
 
 // ------------------------------------------------------------------ launch (one volume form)
