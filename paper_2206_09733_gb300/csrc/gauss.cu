@@ -476,7 +476,7 @@ template <int N>
 static int gauss_epb(int prec, int which, long long elems)
 {
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
-    int epb = spread_elems(elems_per_block_p(N, prec, which), elems);
+    int epb = spread_elems(elems_per_block_p(N, prec, which, kSmallCta), elems);
     if (epb * n3 > gauss_threads<N>()) epb = gauss_threads<N>() / n3;
     return epb < 1 ? 1 : epb;
 }

@@ -45,16 +45,12 @@ static int prec_slot(int prec) { return prec == HS3D_FP64 ? 0 : 1; }
 
 int tuned_elems_per_block(int N, int prec, int which) { return g_epb[N][prec_slot(prec)][which]; }
 
-int elems_per_block_p(int N, int prec, int which)
+int elems_per_block_p(int N, int prec, int which, int threads)
 {
-    int v = g_epb[N][prec_slot(prec)][which];
+    const int v = g_epb[N][prec_slot(prec)][which];
     if (v > 0) return v;
-    // FP64 element kernel: 128 threads' worth (its ~110 registers and 22 KB of
-    // shared memory per 64-node element leave two 256-thread CTAs per SM, whose
-    // barriers stall half the warps at once; four of 128: 16^3 elements of N = 3,
-    // Chandrashekar form -8% per step), else 256
-    int n3 = (N + 1) * (N + 1) * (N + 1);
-    int e = (prec == HS3D_FP64 && which == 1 ? 128 : 256) / n3;
+    const int n3 = (N + 1) * (N + 1) * (N + 1);
+    const int e = threads / n3;
     return e < 1 ? 1 : e;
 }
 

@@ -118,19 +118,20 @@ __device__ __forceinline__ int dev_line_node(int d, int idx, int ta, int tb)
     return ta + n * (tb + n * idx);
 }
 
-// Minimum resident CTAs asked of the compiler (its register budget), for
-// CTAs of up to 256 threads: the split forms 4 (64 registers; with about
-// 55 KB of shared memory per CTA, 4 are resident; ~56 bytes of spills per
+// Minimum resident CTAs asked of the compiler (its register budget), in CTAs
+// of 256 threads: the split forms 4 (64 registers; ~56 bytes of spills per
 // thread, and still 8-12% faster than 3 CTAs at 80 registers, 16^3 and 32^3
-// N = 3, EC and KG); the standard form 5 up to N = 3 (48 registers, ~50
-// bytes of spills: -4% at 64^3 N = 3) and 4 above (no spills; 5 measured
-// +3% at N = 4).
-template <int N, int FORM>
+// N = 3, EC and KG; 5: +30%); the standard form 5 (48 registers) for Euler and
+// 4 for Navier-Stokes below N = 5 (with the viscous values 48 registers
+// spill).  Measured with 128-thread CTAs, 5 against 4: Euler 64^3 N = 3 -7%,
+// 52^3 N = 4 -3%, 24^3 N = 5 -5%; NS 48^3 N = 2 +3%, 40^3 N = 3 +3%, 30^3 N = 4
+// +2%, 24^3 N = 5 -1%.
+template <int N, bool NS, int FORM>
 constexpr int dev_min_blocks()
 {
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
     if (n3 > 256) return 2;
-    return (FORM == HS3D_VOL_STANDARD && n3 <= 64) ? 5 : 4;
+    return (FORM == HS3D_VOL_STANDARD && (!NS || n3 > 125)) ? 5 : 4;
 }
 
 // Viscous flux from the gradient kernel's values: stress and heat flux, or the
@@ -765,7 +766,7 @@ __device__ __noinline__ bool volume_dev_tile_call(const Batch &b, const Ops *__r
 // reusing their shared memory; a tile's element barriers are invalidated
 // before the next tile initialises them again.
 template <int N, bool NS, int FORM, bool PERSIST, bool MORT = false>
-__global__ void __launch_bounds__(dev_threads<N>(), dev_min_blocks<N, FORM>())
+__global__ void __launch_bounds__(dev_threads<N>(), dev_min_blocks<N, NS, FORM>())
 k_volume_dev(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int stage, double rkA, double rkB,
              int lam_slot, int epb, long long ntiles)
 {
@@ -792,7 +793,7 @@ template <int N, bool NS, int FORM>
 static cudaError_t vol_dev_launch2(const Batch &b, int stage, double rkA, double rkB, int lam_slot, cudaStream_t s)
 {
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
-    int epb = spread_elems(elems_per_block_p(N, HS3D_MIXED32, 1), b.total_elems);
+    int epb = spread_elems(elems_per_block_p(N, HS3D_MIXED32, 1, is_standard(FORM) ? kSmallCta : 256), b.total_elems);
     if (epb * n3 > dev_threads<N>()) epb = dev_threads<N>() / n3;
     if (epb < 1) epb = 1;
     const int threads = ((epb * n3) + 31) & ~31;

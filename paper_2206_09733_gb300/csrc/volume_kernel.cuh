@@ -431,7 +431,7 @@ template <int N, bool NS, int FORM>
 static cudaError_t vol_launch2(const Batch &b, int stage, double rkA, double rkB, int lam_slot, cudaStream_t s)
 {
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
-    int epb = spread_elems(elems_per_block_p(N, HS3D_FP64, 1), b.total_elems);
+    int epb = spread_elems(elems_per_block_p(N, HS3D_FP64, 1, kSmallCta), b.total_elems);
     int threads = epb * n3;
     if (threads > vol_threads<N>()) {
         epb = vol_threads<N>() / n3;
