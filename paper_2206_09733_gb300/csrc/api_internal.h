@@ -24,6 +24,8 @@ struct hs3d_mesh {
     void *grad = nullptr;           // scratch, sized for FP64
     hs3d::Clock *clk = nullptr;
     double *diag_partials = nullptr;
+    void *slab = nullptr;           // the one allocation behind the arrays above
+    float *uf_own = nullptr;        // uf where a p-mesh allocated it for its bucket
     size_t bytes = 0;
     cudaStream_t stream = nullptr;  // private stream for set-up and graph capture
     // graph cache of hs3d_rk3_run: the two most recently used (cfg, u, g, dt)

@@ -122,8 +122,7 @@ namespace hs3d {
 
 static void release(hs3d_server *S, ServerReq *r)
 {
-    if (r->u) cudaFree(r->u);
-    if (r->g) cudaFree(r->g);
+    if (r->u) cudaFree(r->u);   // (g is the second half of u's allocation)
     if (r->mesh) mesh_free(r->mesh);
     r->u = r->g = nullptr;
     r->mesh = nullptr;
@@ -141,11 +140,11 @@ static hs3d_status admit(hs3d_server *S, ServerReq *r)
     hs3d_status st = mesh_build(&d, &r->mesh);
     if (st != HS3D_OK) return st;
     size_t sz = sizeof(double) * (size_t)r->mesh->E * 5 * r->mesh->n3;
-    cudaError_t e = cudaMalloc(&r->u, sz);
-    if (e == cudaSuccess) e = cudaMalloc(&r->g, sz);
+    const size_t half = (sz + 255) & ~(size_t)255;   // state, then RK register
+    cudaError_t e = cudaMalloc(&r->u, half + sz);
+    if (e == cudaSuccess) r->g = (double *)((char *)r->u + half);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        if (r->u) cudaFree(r->u);
         r->u = nullptr;
         mesh_free(r->mesh);
         r->mesh = nullptr;
@@ -164,7 +163,6 @@ static hs3d_status admit(hs3d_server *S, ServerReq *r)
     if (e == cudaSuccess) e = cudaStreamSynchronize(S->stream);
     if (e != cudaSuccess) {
         cudaFree(r->u);
-        cudaFree(r->g);
         r->u = r->g = nullptr;
         mesh_free(r->mesh);
         r->mesh = nullptr;
