@@ -789,9 +789,23 @@ k_volume_dev(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int s
 
 // ------------------------------------------------------------------ launch (one volume form)
 
+// The standard form at N = 7 without mortars has its own kernel (volume_row.cuh).
+template <int N, int FORM>
+constexpr bool has_row_kernel()
+{
+    return is_standard(FORM) && N == 7;
+}
+template <int N, bool NS>
+static cudaError_t vol_row_launch(const Batch &b, int stage, double rkA, double rkB, int lam_slot, cudaStream_t s);
+template <int N>
+static cudaError_t vol_row_prep();
+
 template <int N, bool NS, int FORM>
 static cudaError_t vol_dev_launch2(const Batch &b, int stage, double rkA, double rkB, int lam_slot, cudaStream_t s)
 {
+    if constexpr (has_row_kernel<N, FORM>()) {
+        if (!b.mortar) return vol_row_launch<N, NS>(b, stage, rkA, rkB, lam_slot, s);
+    }
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
     int epb = spread_elems(elems_per_block_p(N, HS3D_MIXED32, 1, is_standard(FORM) ? kSmallCta : 256), b.total_elems);
     if (epb * n3 > dev_threads<N>()) epb = dev_threads<N>() / n3;
@@ -801,16 +815,20 @@ static cudaError_t vol_dev_launch2(const Batch &b, int stage, double rkA, double
     const unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);
     const Ops *ops = device_ops(N);
     if (!ops) return cudaErrorMemoryAllocation;
-    if (b.persistent && !b.mortar) {
-        const unsigned grid = persistent_grid(k_volume_dev<N, NS, FORM, true>, threads, smem, blocks);
-        return launch_pdl(k_volume_dev<N, NS, FORM, true>, grid, threads, smem, s, b, ops, stage, rkA, rkB,
-                          stage >= 0 ? lam_slot : -1, epb, (long long)blocks);
-    }
     if (b.mortar)
         return launch_pdl(k_volume_dev<N, NS, FORM, false, true>, blocks, threads, smem, s, b, ops, stage, rkA, rkB,
                           stage >= 0 ? lam_slot : -1, epb, (long long)blocks);
-    return launch_pdl(k_volume_dev<N, NS, FORM, false>, blocks, threads, smem, s, b, ops, stage, rkA, rkB,
-                      stage >= 0 ? lam_slot : -1, epb, (long long)blocks);
+    if constexpr (has_row_kernel<N, FORM>()) {
+        return cudaErrorInvalidValue;   // (taken above)
+    } else {
+        if (b.persistent) {
+            const unsigned grid = persistent_grid(k_volume_dev<N, NS, FORM, true>, threads, smem, blocks);
+            return launch_pdl(k_volume_dev<N, NS, FORM, true>, grid, threads, smem, s, b, ops, stage, rkA, rkB,
+                              stage >= 0 ? lam_slot : -1, epb, (long long)blocks);
+        }
+        return launch_pdl(k_volume_dev<N, NS, FORM, false>, blocks, threads, smem, s, b, ops, stage, rkA, rkB,
+                          stage >= 0 ? lam_slot : -1, epb, (long long)blocks);
+    }
 }
 
 template <int FORM>
@@ -841,10 +859,15 @@ static cudaError_t prep_vol_dev_kernel(K kernel)
 template <int N, int FORM>
 static cudaError_t prep_vol_dev_n()
 {
-    cudaError_t e = prep_vol_dev_kernel(k_volume_dev<N, false, FORM, false>);
-    if (e == cudaSuccess) e = prep_vol_dev_kernel(k_volume_dev<N, true, FORM, false>);
-    if (e == cudaSuccess) e = prep_vol_dev_kernel(k_volume_dev<N, false, FORM, true>);
-    if (e == cudaSuccess) e = prep_vol_dev_kernel(k_volume_dev<N, true, FORM, true>);
+    cudaError_t e = cudaSuccess;
+    if constexpr (has_row_kernel<N, FORM>()) {
+        e = vol_row_prep<N>();
+    } else {
+        e = prep_vol_dev_kernel(k_volume_dev<N, false, FORM, false>);
+        if (e == cudaSuccess) e = prep_vol_dev_kernel(k_volume_dev<N, true, FORM, false>);
+        if (e == cudaSuccess) e = prep_vol_dev_kernel(k_volume_dev<N, false, FORM, true>);
+        if (e == cudaSuccess) e = prep_vol_dev_kernel(k_volume_dev<N, true, FORM, true>);
+    }
     if (e == cudaSuccess) e = prep_vol_dev_kernel(k_volume_dev<N, false, FORM, false, true>);
     if (e == cudaSuccess) e = prep_vol_dev_kernel(k_volume_dev<N, true, FORM, false, true>);
     return e;

@@ -2,6 +2,7 @@
 // precisions, Euler and Navier-Stokes.
 #include "volume_dev.cuh"
 #include "volume_kernel.cuh"
+#include "volume_row.cuh"
 
 namespace hs3d {
 HS3D_VOLUME_FORM_TU(HS3D_VOL_STANDARD)
