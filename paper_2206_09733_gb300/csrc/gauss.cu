@@ -206,6 +206,31 @@ k_grad_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops)
     R *sq = su + 5 * n3;
     R *sja = sq + 4 * n3;
     R *slift = sja + 9 * n3;
+    // this thread's face points: the neighbours' interpolated traces and the face
+    // metric come before the barrier, so that their loads (5 n values from another
+    // element) overlap the element's own instead of following them (32^3, N = 3:
+    // the run 4.48 -> 4.19 ms)
+    constexpr int IT = (6 * n2 + n3 - 1) / n3;
+    R un[IT][5], sf[IT][3];
+    if (valid) {
+        const Item &it = *itp;
+        const Nbrs nbs = elem_nbrs(e, it.ex, it.ey, it.ez);
+#pragma unroll
+        for (int c = 0; c < IT; ++c) {
+            const int t = p + c * n3;
+            if (t < 6 * n2) {
+                const int slot = t / n2, ab = t - slot * n2;
+                const int d = slot >> 1, plus = slot & 1;
+                const int nb = nbr_of_slot(nbs, slot);
+                trace_u<n, R>(it, ops, nb, d, plus ? 0 : 1, ab % n, ab / n, un[c]);
+                // own face metric: this face's normal, held by its minus-side element
+                const R *Sf = gnormal<R>(it) + ((size_t)d * it.E + (plus ? e : nb)) * 3 * n2 + ab;
+                sf[c][0] = Sf[0];
+                sf[c][1] = Sf[n2];
+                sf[c][2] = Sf[2 * n2];
+            }
+        }
+    }
     if (valid) {
         const Item &it = *itp;
         const R gm1 = phys_of<R>(it).gm1;
@@ -220,7 +245,7 @@ k_grad_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops)
         sq[0 * n3 + p] = qp.v1;
         sq[1 * n3 + p] = qp.v2;
         sq[2 * n3 + p] = qp.v3;
-        sq[3 * n3 + p] = qp.p / qp.rho;
+        sq[3 * n3 + p] = temperature(qp);
         const R *JA = gmetric<R>(it) + (size_t)e * 9 * n3 + p;
 #pragma unroll
         for (int k = 0; k < 9; ++k) sja[k * n3 + p] = JA[k * n3];
@@ -231,13 +256,14 @@ k_grad_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops)
         // interpolated products Ja^d_c q, times the face metric
         const Item &it = *itp;
         const R gm1 = phys_of<R>(it).gm1;
-        const Nbrs nbs = elem_nbrs(e, it.ex, it.ey, it.ez);
-        for (int t = p; t < 6 * n2; t += n3) {
+#pragma unroll
+        for (int c = 0; c < IT; ++c) {
+            const int t = p + c * n3;
+            if (t >= 6 * n2) break;
             const int slot = t / n2, ab = t - slot * n2;
             const int d = slot >> 1, plus = slot & 1;
             const int ta = ab % n, tb = ab / n;
-            const int nb = nbr_of_slot(nbs, slot);
-            R uo[5], un[5];
+            R uo[5];
 #pragma unroll
             for (int v = 0; v < 5; ++v) uo[v] = (R)0;
 #pragma unroll
@@ -247,14 +273,9 @@ k_grad_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops)
 #pragma unroll
                 for (int v = 0; v < 5; ++v) uo[v] += l * su[v * n3 + pj];
             }
-            trace_u<n, R>(it, ops, nb, d, plus ? 0 : 1, ta, tb, un);
-            const Prim<R> po = prim_of<R>(uo, gm1), pn = prim_of<R>(un, gm1);
+            const Prim<R> po = prim_of<R>(uo, gm1), pn = prim_of<R>(un[c], gm1);
             const R qs[4] = {(R)0.5 * (po.v1 + pn.v1), (R)0.5 * (po.v2 + pn.v2), (R)0.5 * (po.v3 + pn.v3),
-                             (R)0.5 * (po.p / po.rho + pn.p / pn.rho)};
-            // own face metric: this face's normal, held by its minus-side element
-            const int owner = plus ? e : nb;
-            const R *Sf = gnormal<R>(it) + ((size_t)d * it.E + owner) * 3 * n2 + ab;
-            const R sf[3] = {Sf[0], Sf[n2], Sf[2 * n2]};
+                             (R)0.5 * (temperature(po) + temperature(pn))};
             const R sg = plus ? (R)1 : (R)-1;
             // interpolated products (Ja^d_c q_v)(+-1): line node by line node,
             // each node's 3 metric terms and 4 variables read once
@@ -267,19 +288,19 @@ k_grad_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops)
                 const int pj = gline<n>(d, j, ta, tb);
                 R jac[3], qv[4];
 #pragma unroll
-                for (int c = 0; c < 3; ++c) jac[c] = sja[(d * 3 + c) * n3 + pj];
+                for (int x = 0; x < 3; ++x) jac[x] = sja[(d * 3 + x) * n3 + pj];
 #pragma unroll
                 for (int v = 0; v < 4; ++v) qv[v] = sq[v * n3 + pj];
 #pragma unroll
                 for (int v = 0; v < 4; ++v)
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) jq[v * 3 + c] += l * (jac[c] * qv[v]);
+                    for (int x = 0; x < 3; ++x) jq[v * 3 + x] += l * (jac[x] * qv[v]);
             }
 #pragma unroll
             for (int v = 0; v < 4; ++v)
 #pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    slift[(slot * 12 + v * 3 + c) * n2 + ab] = sg * (qs[v] * sf[c] - jq[v * 3 + c]);
+                for (int x = 0; x < 3; ++x)
+                    slift[(slot * 12 + v * 3 + x) * n2 + ab] = sg * (qs[v] * sf[c][x] - jq[v * 3 + x]);
         }
     }
     __syncthreads();

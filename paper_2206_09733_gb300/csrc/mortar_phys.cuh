@@ -29,8 +29,7 @@ __device__ __forceinline__ void mortar_q(const R *u, R gm1, R q[4], int stride =
     q[0] = w.v1;
     q[1] = w.v2;
     q[2] = w.v3;
-    if constexpr (sizeof(R) == 8) q[3] = w.p * w.ir;
-    else q[3] = w.p / w.rho;
+    q[3] = temperature(w);
 }
 
 // Inviscid numerical flux times the face scale, from the two conservative

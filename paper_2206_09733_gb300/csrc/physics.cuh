@@ -279,12 +279,18 @@ __device__ __forceinline__ void visc_flux_grad(const Prim<R> &q, const R G[12], 
     f[4] = q.v1 * s1 + q.v2 * s2 + q.v3 * s3 + kappa * (G[9] * a1 + G[10] * a2 + G[11] * a3);
 }
 
-// Speed of sound and total enthalpy of a state.
+// Speed of sound, temperature p/rho and total enthalpy of a state.
 template <typename R>
 __device__ __forceinline__ R sound_speed(const Prim<R> &q, R gamma)
 {
     if constexpr (sizeof(R) == 8) return sqrt_(gamma * q.p * q.ir);
     else return sqrt(gamma * q.p / q.rho);
+}
+template <typename R>
+__device__ __forceinline__ R temperature(const Prim<R> &q)
+{
+    if constexpr (sizeof(R) == 8) return q.p * q.ir;
+    else return q.p / q.rho;
 }
 template <typename R>
 __device__ __forceinline__ R enthalpy(const Prim<R> &q, R E)
