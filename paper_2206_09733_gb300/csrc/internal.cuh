@@ -563,8 +563,8 @@ int elems_per_block_p(int N, int prec, int which, int threads = 256);
 // as many warps are resident as with 256 threads, but a barrier or a late load
 // stalls half as many at once.  Measured, 256 -> 128: FP64 element kernel (EC,
 // 16^3, N = 3) -8% per step; standard form, mixed: 64^3 N = 3 14.71 -> 13.74 ms,
-// 53x52x51 N = 4 17.95 -> 16.93; Gauss-Legendre 32^3 N = 3 4.76 -> 4.47.  The mixed
-// split-form kernel and the BR1 gradients of Lobatto meshes do not gain (+1%, 0).
+// 53x52x51 N = 4 17.95 -> 16.93; Gauss-Legendre 32^3 N = 3 4.76 -> 4.47; mixed
+// Chandrashekar form 24^3 N = 4 -1%.  The BR1 gradients of Lobatto meshes do not gain.
 constexpr int kSmallCta = 128;
 int tuned_elems_per_block(int N, int prec, int which);   // 0 if untuned
 void set_elems_per_block_p(int N, int prec, int which, int epb);

@@ -45,9 +45,12 @@ constexpr bool dev_lowmach()
     return FORM == HS3D_VOL_STANDARD || FORM == HS3D_VOL_EC;
 }
 
-template <int N>
+// Largest CTA: 128 threads for the Chandrashekar form at N = 3 (dev_min_blocks),
+// else 256 or one element.
+template <int N, int FORM>
 constexpr int dev_threads()
 {
+    if (FORM == HS3D_VOL_EC && N == 3) return 128;
     constexpr int t = ((N + 1) * (N + 1) * (N + 1) > 256) ? (N + 1) * (N + 1) * (N + 1) : 256;
     return (t + 31) & ~31;
 }
@@ -126,10 +129,14 @@ __device__ __forceinline__ int dev_line_node(int d, int idx, int ta, int tb)
 // spill).  Measured with 128-thread CTAs, 5 against 4: Euler 64^3 N = 3 -7%,
 // 52^3 N = 4 -3%, 24^3 N = 5 -5%; NS 48^3 N = 2 +3%, 40^3 N = 3 +3%, 30^3 N = 4
 // +2%, 24^3 N = 5 -1%.
+// Chandrashekar form at N = 3: seven CTAs of 128 threads (72 registers, no
+// spills): 16^3 elements, NS 709 -> 698 us per 4 steps, Euler 512 -> 503, 32^3
+// unchanged (8: +0.6%, +4% at 32^3; 6: +1.4%; 5: +0.5%).
 template <int N, bool NS, int FORM>
 constexpr int dev_min_blocks()
 {
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
+    if (FORM == HS3D_VOL_EC && N == 3) return 7;
     if (n3 > 256) return 2;
     return (FORM == HS3D_VOL_STANDARD && (!NS || n3 > 125)) ? 5 : 4;
 }
@@ -766,7 +773,7 @@ __device__ __noinline__ bool volume_dev_tile_call(const Batch &b, const Ops *__r
 // reusing their shared memory; a tile's element barriers are invalidated
 // before the next tile initialises them again.
 template <int N, bool NS, int FORM, bool PERSIST, bool MORT = false>
-__global__ void __launch_bounds__(dev_threads<N>(), dev_min_blocks<N, NS, FORM>())
+__global__ void __launch_bounds__(dev_threads<N, FORM>(), dev_min_blocks<N, NS, FORM>())
 k_volume_dev(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int stage, double rkA, double rkB,
              int lam_slot, int epb, long long ntiles)
 {
@@ -807,8 +814,8 @@ static cudaError_t vol_dev_launch2(const Batch &b, int stage, double rkA, double
         if (!b.mortar) return vol_row_launch<N, NS>(b, stage, rkA, rkB, lam_slot, s);
     }
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
-    int epb = spread_elems(elems_per_block_p(N, HS3D_MIXED32, 1, is_standard(FORM) ? kSmallCta : 256), b.total_elems);
-    if (epb * n3 > dev_threads<N>()) epb = dev_threads<N>() / n3;
+    int epb = spread_elems(elems_per_block_p(N, HS3D_MIXED32, 1, (is_standard(FORM) || FORM == HS3D_VOL_EC) ? kSmallCta : 256), b.total_elems);
+    if (epb * n3 > dev_threads<N, FORM>()) epb = dev_threads<N, FORM>() / n3;
     if (epb < 1) epb = 1;
     const int threads = ((epb * n3) + 31) & ~31;
     const size_t smem = dev_smem_bytes<N, NS, FORM>(epb);
