@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(512) k_alambda(const int *__restrict__ slot_el
                                                  const double *__restrict__ Jaall, const double *__restrict__ invJall,
                                                  const double *__restrict__ u, APhys P, Clock *clk, int slot)
 {
-    ASlot S;
+    ASlot S{};
     const bool live = aslot(slot_elem, slot0, P3, S);
     double lc = 0.0, lv = 0.0;
     if (live) {
@@ -478,7 +478,8 @@ __global__ void __launch_bounds__(kAFaceThreads) k_amortar(const AFace *__restri
 // q = (v1, v2, v3, T), q*_e from the mortar kernel, stored as viscous stress and
 // heat flux [kVisc][n3] at kVisc noff[e].  D_ii is zero inside and -+1/(2w) at
 // the two ends, where the lift turns the diagonal term D_ii Ja q_in into
-// D_ii Ja (2 q* - q_in).  16^3 elements of degrees 2..5: 484 -> 193 us per stage.
+// D_ii Ja (2 q* - q_in); the nine stress products are formed once per node and
+// direction.  16^3 elements of degrees 2..5: 484 -> 174 us per stage.
 template <int T>
 __global__ void __launch_bounds__(T) k_agrad(const int *__restrict__ slot_elem, const int *__restrict__ slot0,
                                              const int *__restrict__ P3, const long long *__restrict__ noff,
@@ -487,47 +488,60 @@ __global__ void __launch_bounds__(T) k_agrad(const int *__restrict__ slot_elem, 
                                              const double *__restrict__ invJall, const double *__restrict__ qhat,
                                              APhys P, double *__restrict__ gradall)
 {
-    extern __shared__ double sm[];   // q [4][T], Ja [9][T]
+    extern __shared__ double sm[];   // the stress products of one direction [kVisc][T]
     pdl_wait();
-    ASlot S;
+    ASlot S{};
     const bool live = aslot(slot_elem, slot0, P3, S);
     const int t = threadIdx.x;
     double qp[4] = {0, 0, 0, 0};
     long long nb = 0;
+    int ijk[3] = {0, 0, 0}, n3 = 1;
     if (live) {
         nb = noff[S.e];
-        const int n3 = S.s.n3;
+        n3 = S.s.n3;
         mortar_q(u + 5 * nb + S.p, P.gm1, qp, n3);
-#pragma unroll
-        for (int v = 0; v < 4; ++v) sm[v * T + t] = qp[v];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) sm[(4 + k) * T + t] = Jaall[9 * nb + (size_t)k * n3 + S.p];
+        ijk[0] = S.p % S.s.n[0];
+        ijk[1] = (S.p / S.s.n[0]) % S.s.n[1];
+        ijk[2] = S.p / (S.s.n[0] * S.s.n[1]);
     }
-    __syncthreads();
-    if (!live) return;
-    const int ijk[3] = {S.p % S.s.n[0], (S.p / S.s.n[0]) % S.s.n[1], S.p / (S.s.n[0] * S.s.n[1])};
+    const double *Ja = Jaall + 9 * nb + S.p;
     double G[kVisc] = {};
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        const int nd = S.s.n[d], st = astride(S.s, d), i = ijk[d];
-        const double *Drow = ops->D[nd - 1] + i * nd;
-        const double *J = sm + (4 + d * 3) * T;
-        for (int k = 1; k < nd; ++k) {
-            const int m = (i + k < nd) ? i + k : i + k - nd, pm = t + (m - i) * st;
-            const double Dm = Drow[m];
-            stress_add(G, Dm * J[pm], Dm * J[T + pm], Dm * J[2 * T + pm], sm[pm], sm[T + pm], sm[2 * T + pm],
-                       sm[3 * T + pm]);
+        const int nd = live ? S.s.n[d] : 1, st = live ? astride(S.s, d) : 0, i = ijk[d];
+        double a1 = 0.0, a2 = 0.0, a3 = 0.0;
+        if (d > 0) __syncthreads();   // the previous direction's products are consumed
+        if (live) {
+            a1 = Ja[(size_t)(d * 3) * n3];
+            a2 = Ja[(size_t)(d * 3 + 1) * n3];
+            a3 = Ja[(size_t)(d * 3 + 2) * n3];
+            double w[kVisc] = {};
+            stress_add(w, a1, a2, a3, qp[0], qp[1], qp[2], qp[3]);
+#pragma unroll
+            for (int c = 0; c < kVisc; ++c) sm[c * T + t] = w[c];
         }
-        if (i != 0 && i != nd - 1) continue;
-        int d0, d1;
-        aface_dirs(d, d0, d1);
-        const int f2 = S.s.n[d0] * S.s.n[d1];
-        const int slot = 2 * d + (i != 0 ? 1 : 0);
-        const double *qs = qhat + (size_t)4 * fnoff[6 * S.e + slot] + ijk[d0] + S.s.n[d0] * ijk[d1];
-        const double Dm = Drow[i];
-        stress_add(G, Dm * J[t], Dm * J[T + t], Dm * J[2 * T + t], 2.0 * qs[0] - qp[0], 2.0 * qs[f2] - qp[1],
-                   2.0 * qs[2 * f2] - qp[2], 2.0 * qs[3 * f2] - qp[3]);
+        __syncthreads();
+        if (live) {
+            const double *Drow = ops->D[nd - 1] + i * nd;
+            for (int k = 1; k < nd; ++k) {
+                const int m = (i + k < nd) ? i + k : i + k - nd, pm = t + (m - i) * st;
+                const double Dm = Drow[m];
+#pragma unroll
+                for (int c = 0; c < kVisc; ++c) G[c] += Dm * sm[c * T + pm];
+            }
+            if (i == 0 || i == nd - 1) {
+                int d0, d1;
+                aface_dirs(d, d0, d1);
+                const int f2 = S.s.n[d0] * S.s.n[d1];
+                const int slot = 2 * d + (i != 0 ? 1 : 0);
+                const double *qs = qhat + (size_t)4 * fnoff[6 * S.e + slot] + ijk[d0] + S.s.n[d0] * ijk[d1];
+                const double Dm = Drow[i];
+                stress_add(G, Dm * a1, Dm * a2, Dm * a3, 2.0 * qs[0] - qp[0], 2.0 * qs[f2] - qp[1],
+                           2.0 * qs[2 * f2] - qp[2], 2.0 * qs[3 * f2] - qp[3]);
+            }
+        }
     }
+    if (!live) return;
     double tau[kVisc];
     stress_of(G, invJall[nb + S.p], P.mu, P.kappa, tau);
     double *Gout = gradall + kVisc * nb + S.p;
@@ -569,7 +583,7 @@ __global__ void __launch_bounds__(T, 512 / T) k_avol(const int *__restrict__ slo
     constexpr int ZS = split_slots64<FORM>();
     extern __shared__ double sm[];
     pdl_wait();
-    ASlot S;
+    ASlot S{};
     // (a finished or failed run's clock stops its stages, not a residual evaluation)
     const bool live = aslot(slot_elem, slot0, P3, S) && (stage < 0 || !(clk->done));
     const int t = threadIdx.x;
@@ -925,7 +939,7 @@ cudaError_t for_classes(const AnisoMesh *a, F fn)
     return e;
 }
 
-constexpr size_t kAGradSmemPer = 13;   // doubles per thread slot of k_agrad
+constexpr size_t kAGradSmemPer = kVisc;   // doubles per thread slot of k_agrad
 
 template <class K>
 cudaError_t allow_smem(K kernel, size_t bytes)

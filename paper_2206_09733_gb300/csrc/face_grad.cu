@@ -121,14 +121,23 @@ __device__ __forceinline__ void grad_vars(const double u[5], double gm1, double 
     out[3] = q.p * q.ir;
 }
 
-// Shared memory per element (doubles): q [4][n3], Ja [9][n3], neighbour
-// traces of q [6 faces][4][n2] (slot 2d: the -d face, slot 2d+1: the +d
-// face).  The neighbour traces are gathered by all threads of the element
-// before the barrier, so the lifting reads no global memory.
+// Shared memory per element (doubles): the nine stress products of one
+// direction, or of all three where they fit beside enough CTAs (n^3 <= 125: one
+// barrier per direction less), [1 or 3][9][n3], and the neighbour traces of q
+// [6 faces][4][n2] (slot 2d: the -d face, slot 2d+1: the +d face).  The products
+// Ja^d_c q_v are combined once per node and direction (12 FP64 instructions),
+// so that the contraction takes 9 multiply-adds per pair of nodes instead of 15
+// instructions (with the Roe flux's summed Euler part: 16^3, N = 3, two steps
+// 2.53 -> 2.45 ms; 11x12x13, N = 4, KG, RK4 1.65 -> 1.56).
+template <int N>
+constexpr int grad_buffers()
+{
+    return (N + 1) * (N + 1) * (N + 1) <= 125 ? 3 : 1;
+}
 template <int N>
 constexpr int grad_per_elem()
 {
-    return 13 * (N + 1) * (N + 1) * (N + 1) + 24 * (N + 1) * (N + 1);
+    return grad_buffers<N>() * kVisc * (N + 1) * (N + 1) * (N + 1) + 24 * (N + 1) * (N + 1);
 }
 
 template <int N>
@@ -152,9 +161,10 @@ __global__ void __launch_bounds__(grad_threads<N>()) k_grad(const __grid_constan
         e = (int)(ge - itp->elem_begin);
         if (itp->clk && itp->clk->done) valid = false;
     }
-    double *q = sE + (size_t)le * PER_ELEM;
-    double *ja = q + 4 * n3;
-    double *qn = ja + 9 * n3;
+    constexpr int NB = grad_buffers<N>();
+    double *W = sE + (size_t)le * PER_ELEM;
+    double *qn = W + NB * kVisc * n3;
+    double ja[9] = {}, qin[4] = {};
     if (valid) {
         const Item &it = *itp;
         const double gm1 = it.gm1;
@@ -188,7 +198,7 @@ __global__ void __launch_bounds__(grad_threads<N>()) k_grad(const __grid_constan
 #pragma unroll
         for (int v = 0; v < 5; ++v) uo[v] = U[v * n3];
 #pragma unroll
-        for (int k = 0; k < 9; ++k) ja[k * n3 + p] = JA[k * n3];
+        for (int k = 0; k < 9; ++k) ja[k] = JA[k * n3];
 #pragma unroll
         for (int k = 0; k < IT; ++k) {
             const int t = p + k * n3;
@@ -205,17 +215,22 @@ __global__ void __launch_bounds__(grad_threads<N>()) k_grad(const __grid_constan
                 for (int v = 0; v < 4; ++v) qn[(slot * 4 + v) * n2 + ab] = g4[v];
             }
         }
-        double qin[4];
         grad_vars(uo, gm1, qin);
-#pragma unroll
-        for (int v = 0; v < 4; ++v) q[v * n3 + p] = qin[v];
     }
-    __syncthreads();
-    if (!valid) return;
     const int ijk[3] = {p % n, (p / n) % n, p / n2};
     double acc[kVisc];
 #pragma unroll
     for (int k = 0; k < kVisc; ++k) acc[k] = 0.0;
+    // the other nodes of the line through this one
+    auto contract = [&](const double *Wd, const double *Drow, int base, int stride, int i) {
+#pragma unroll
+        for (int k = 1; k < n; ++k) {
+            const int m = (i + k < n) ? i + k : i + k - n;
+            const double Dm = Drow[m];
+#pragma unroll
+            for (int c = 0; c < kVisc; ++c) acc[c] += Dm * Wd[c * n3 + base + m * stride];
+        }
+    };
     // D_ii is zero inside and -+1/(2w) at the two ends, where the BR1 lift
     // +-(1/w)(q_out - q_in)/2 Ja turns the diagonal term D_ii Ja q_in into
     // D_ii Ja q_out: no separate lift
@@ -225,21 +240,34 @@ __global__ void __launch_bounds__(grad_threads<N>()) k_grad(const __grid_constan
         const int stride = (d == 0) ? 1 : (d == 1) ? n : n2;
         const int base = p - i * stride;
         const double *Drow = sD + i * n;
-        const double *J1 = ja + d * 3 * n3, *J2 = J1 + n3, *J3 = J2 + n3;
+        double *Wd = W + (NB == 3 ? d * kVisc * n3 : 0);
+        if (NB == 1 && d > 0) __syncthreads();   // the previous direction's products are consumed
+        if (valid) {
+            double w[kVisc] = {};
+            stress_add(w, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], qin[0], qin[1], qin[2], qin[3]);
 #pragma unroll
-        for (int k = 1; k < n; ++k) {
-            const int m = (i + k < n) ? i + k : i + k - n;
-            const int pm = base + m * stride;
-            const double Dm = Drow[m];
-            stress_add(acc, Dm * J1[pm], Dm * J2[pm], Dm * J3[pm], q[pm], q[n3 + pm], q[2 * n3 + pm], q[3 * n3 + pm]);
+            for (int c = 0; c < kVisc; ++c) Wd[c * n3 + p] = w[c];
         }
-        if (i == 0 || i == N) {
-            const int ta = (d == 0) ? ijk[1] : ijk[0];
-            const int tb = (d == 2) ? ijk[1] : ijk[2];
-            const double *Q = qn + (2 * d + (i == N ? 1 : 0)) * 4 * n2 + ta + n * tb;
-            const double Dm = Drow[i];
-            stress_add(acc, Dm * J1[p], Dm * J2[p], Dm * J3[p], Q[0], Q[n2], Q[2 * n2], Q[3 * n2]);
+        if (NB == 1 || d == 2) __syncthreads();
+        if (NB == 1 && valid) contract(Wd, Drow, base, stride, i);
+    }
+    if (!valid) return;
+    if constexpr (NB == 3) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int stride = (d == 0) ? 1 : (d == 1) ? n : n2;
+            contract(W + d * kVisc * n3, sD + ijk[d] * n, p - ijk[d] * stride, stride, ijk[d]);
         }
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const int i = ijk[d];
+        if (i != 0 && i != N) continue;
+        const int ta = (d == 0) ? ijk[1] : ijk[0];
+        const int tb = (d == 2) ? ijk[1] : ijk[2];
+        const double *Q = qn + (2 * d + (i == N ? 1 : 0)) * 4 * n2 + ta + n * tb;
+        const double Dm = sD[i * n + i];
+        stress_add(acc, Dm * ja[d * 3], Dm * ja[d * 3 + 1], Dm * ja[d * 3 + 2], Q[0], Q[n2], Q[2 * n2], Q[3 * n2]);
     }
     const Item &it = *itp;
     double t[kVisc];

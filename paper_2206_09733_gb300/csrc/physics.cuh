@@ -198,6 +198,20 @@ __device__ __forceinline__ void euler_flux(const Prim<R> &q, R E, R a1, R a2, R 
     f[4] = (E + q.p) * va;
 }
 
+// The sum of two states' Euler fluxes dotted with a (FP64: 22 instructions; two
+// fluxes and their sum take 31).
+__device__ __forceinline__ void euler_flux_sum(const Prim<double> &L, double EL, const Prim<double> &Rr, double ER,
+                                               double a1, double a2, double a3, double f[5])
+{
+    const double vaL = L.v1 * a1 + L.v2 * a2 + L.v3 * a3, vaR = Rr.v1 * a1 + Rr.v2 * a2 + Rr.v3 * a3;
+    const double mL = L.rho * vaL, mR = Rr.rho * vaR, p = L.p + Rr.p;
+    f[0] = mL + mR;
+    f[1] = mL * L.v1 + mR * Rr.v1 + p * a1;
+    f[2] = mL * L.v2 + mR * Rr.v2 + p * a2;
+    f[3] = mL * L.v3 + mR * Rr.v3 + p * a3;
+    f[4] = (EL + L.p) * vaL + (ER + Rr.p) * vaR;
+}
+
 // Viscous stress and heat flux, kVisc values per node: t11, t22, t33, t12,
 // t13, t23 of tau = mu (grad v + grad v^T) - 2/3 mu I div v, then
 // kappa grad T.  The viscous fluxes read nothing else of the twelve BR1
@@ -358,8 +372,12 @@ __device__ __forceinline__ void flux_roe(const Prim<R> &L, const R uL[5], const 
     norm_and_inverse(s1 * s1 + s2 * s2 + s3 * s3, s, is);
     R n1 = s1 * is, n2 = s2 * is, n3 = s3 * is;
     R fl[5], fr[5];
-    euler_flux(L, uL[4], s1, s2, s3, fl);
-    euler_flux(Rr, uR[4], s1, s2, s3, fr);
+    if constexpr (sizeof(R) == 8) {
+        euler_flux_sum(L, uL[4], Rr, uR[4], s1, s2, s3, fl);   // F_L + F_R
+    } else {
+        euler_flux(L, uL[4], s1, s2, s3, fl);
+        euler_flux(Rr, uR[4], s1, s2, s3, fr);
+    }
     R sl = sqrt_(L.rho), sr = sqrt_(Rr.rho);
     R iw;
     if constexpr (sizeof(R) == 8) iw = rcp_fast(sl + sr);
@@ -400,6 +418,14 @@ __device__ __forceinline__ void flux_roe(const Prim<R> &L, const R uL[5], const 
     R W2 = l1 * (vt2 - ct * n2) + l2 * (a2 * vt2 + sh2) + l5 * (vt2 + ct * n2);
     R W3 = l1 * (vt3 - ct * n3) + l2 * (a2 * vt3 + sh3) + l5 * (vt3 + ct * n3);
     R W4 = l1 * (Ht - ct * vnt) + l2 * (a2 * (R)0.5 * q2 + vt1 * sh1 + vt2 * sh2 + vt3 * sh3) + l5 * (Ht + ct * vnt);
+    if constexpr (sizeof(R) == 8) {
+        f[0] = 0.5 * (fl[0] - s * W0);
+        f[1] = 0.5 * (fl[1] - s * W1);
+        f[2] = 0.5 * (fl[2] - s * W2);
+        f[3] = 0.5 * (fl[3] - s * W3);
+        f[4] = 0.5 * (fl[4] - s * W4);
+        return;
+    }
     R hs = (R)0.5 * s;
     f[0] = (R)0.5 * (fl[0] + fr[0]) - hs * W0;
     f[1] = (R)0.5 * (fl[1] + fr[1]) - hs * W1;
