@@ -45,12 +45,14 @@ constexpr bool dev_lowmach()
     return FORM == HS3D_VOL_STANDARD || FORM == HS3D_VOL_EC;
 }
 
-// Largest CTA: 128 threads for the Chandrashekar form at N = 3 (dev_min_blocks),
-// else 256 or one element.
+// Largest CTA: 128 threads for the Chandrashekar form at N = 3 and 4
+// (dev_min_blocks), one element (216 threads, seven warps) at N = 5 and where an
+// element has more than 256 nodes, else 256.
 template <int N, int FORM>
 constexpr int dev_threads()
 {
-    if (FORM == HS3D_VOL_EC && N == 3) return 128;
+    if (FORM == HS3D_VOL_EC && (N == 3 || N == 4)) return 128;
+    if (N == 5) return 224;
     constexpr int t = ((N + 1) * (N + 1) * (N + 1) > 256) ? (N + 1) * (N + 1) * (N + 1) : 256;
     return (t + 31) & ~31;
 }
@@ -129,14 +131,17 @@ __device__ __forceinline__ int dev_line_node(int d, int idx, int ta, int tb)
 // spill).  Measured with 128-thread CTAs, 5 against 4: Euler 64^3 N = 3 -7%,
 // 52^3 N = 4 -3%, 24^3 N = 5 -5%; NS 48^3 N = 2 +3%, 40^3 N = 3 +3%, 30^3 N = 4
 // +2%, 24^3 N = 5 -1%.
-// Chandrashekar form at N = 3: seven CTAs of 128 threads (72 registers, no
-// spills): 16^3 elements, NS 709 -> 698 us per 4 steps, Euler 512 -> 503, 32^3
-// unchanged (8: +0.6%, +4% at 32^3; 6: +1.4%; 5: +0.5%).
+// Chandrashekar form at N = 3 and 4: seven CTAs of 128 threads (72 registers, no
+// spills): 16^3 elements of N = 3, NS 709 -> 698 us per 4 steps, Euler 512 -> 503,
+// 32^3 unchanged (8: +0.6%, +4% at 32^3; 6: +1.4%; 5: +0.5%), 24^3 of N = 4 -2%.
+// At N = 5 the bound of 224 threads lets four CTAs have 72 registers as well:
+// 24^3 elements, Chandrashekar form NS 8.98 -> 8.34 ms, Euler 6.70 -> 5.98,
+// standard form NS 5.00 -> 4.75.
 template <int N, bool NS, int FORM>
 constexpr int dev_min_blocks()
 {
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
-    if (FORM == HS3D_VOL_EC && N == 3) return 7;
+    if (FORM == HS3D_VOL_EC && (N == 3 || N == 4)) return 7;
     if (n3 > 256) return 2;
     return (FORM == HS3D_VOL_STANDARD && (!NS || n3 > 125)) ? 5 : 4;
 }
