@@ -227,9 +227,8 @@ hs3d_status mesh_build(const hs3d_mesh_desc *desc, hs3d_mesh **out)
         mesh_free(m);
         return fail(HS3D_ERR_NOMEM, "operator tables");
     }
-    e = launch_geometry(m->N, m->nodes, xyz_dev, m->ex, m->ey, m->ez, m->lo, m->hi, m->amp, m->X, m->Ja, m->Jaf, m->J, m->invJ,
+    e = launch_geometry(m->N, m->nodes, xyz_dev, m->ex, m->ey, m->ez, m->lo, m->hi, m->amp, m->X, m->Ja, m->Jaf, m->Jalo, m->J, m->invJ,
                         m->invJf, m->fn, m->fnf, m->stream);
-    if (e == cudaSuccess) e = launch_metric_lo(m->Ja, m->Jaf, m->Jalo, (long long)m->E * 9 * m->n3, m->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->clk, 0, sizeof(Clock), m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (xyz_dev) cudaFree(xyz_dev);

@@ -231,13 +231,15 @@ template <int N>
 __global__ void __launch_bounds__((N + 1) * (N + 1) * (N + 1))
 k_geometry(const double *__restrict__ xyz, int ex, int ey, int ez, double lo0, double lo1, double lo2, double hi0,
            double hi1, double hi2, double amp, const Ops *__restrict__ ops, double *__restrict__ X,
-           double *__restrict__ Ja, float *__restrict__ Jaf, double *__restrict__ J, double *__restrict__ invJ,
-           float *__restrict__ invJf, double *__restrict__ fn, float *__restrict__ fnf, double *__restrict__ dXout)
+           double *__restrict__ Ja, float *__restrict__ Jaf, float *__restrict__ Jalo, double *__restrict__ J,
+           double *__restrict__ invJ, float *__restrict__ invJf, double *__restrict__ fn, float *__restrict__ fnf,
+           double *__restrict__ dXout)
 {
     constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
     __shared__ double sD[n * n];
     __shared__ double sX[3][n3];
     __shared__ double sT[2][n3];
+    __shared__ double sx[3][n], ss[3][n];
     const int e = blockIdx.x;
     const int E = ex * ey * ez;
     const int p = threadIdx.x;
@@ -245,20 +247,24 @@ k_geometry(const double *__restrict__ xyz, int ex, int ey, int ez, double lo0, d
     for (int t = p; t < n * n; t += n3) sD[t] = ops->D[t];
     const double lo[3] = {lo0, lo1, lo2}, hi[3] = {hi0, hi1, hi2};
     const int ab[3] = {e % ex, (e / ex) % ey, e / (ex * ey)};
-    const int Ed[3] = {ex, ey, ez};
     double x[3];
     if (xyz) {
         for (int c = 0; c < 3; ++c) x[c] = xyz[((size_t)e * 3 + c) * n3 + p];
     } else {
-        double th[3];
-        for (int c = 0; c < 3; ++c) {
-            double L = hi[c] - lo[c];
-            double h = L / Ed[c];
-            x[c] = lo[c] + h * (ab[c] + 0.5 * (ops->xi[ijk[c]] + 1.0));
-            th[c] = -M_PI + 2.0 * M_PI * (x[c] - lo[c]) / L;
+        // position and sine per direction: 3 n of each an element, not 3 n^3 (the
+        // FP64 pipe bounds this kernel: 32^3 elements of N = 7 13.4 -> 9.6 ms
+        // together with the low part written here)
+        if (p < 3 * n) {
+            const int c = p / n, i = p - c * n;
+            const double l = c == 0 ? lo0 : c == 1 ? lo1 : lo2, L = (c == 0 ? hi0 : c == 1 ? hi1 : hi2) - l;
+            const double h = L / (c == 0 ? ex : c == 1 ? ey : ez);
+            const double x1 = l + h * ((c == 0 ? ab[0] : c == 1 ? ab[1] : ab[2]) + 0.5 * (ops->xi[i] + 1.0));
+            sx[c][i] = x1;
+            ss[c][i] = sin(-M_PI + 2.0 * M_PI * (x1 - l) / L);
         }
-        double s = sin(th[0]) * sin(th[1]) * sin(th[2]);
-        for (int c = 0; c < 3; ++c) x[c] += amp * ((hi[c] - lo[c]) / (2.0 * M_PI)) * s;
+        __syncthreads();
+        const double s = ss[0][ijk[0]] * ss[1][ijk[1]] * ss[2][ijk[2]];
+        for (int c = 0; c < 3; ++c) x[c] = sx[c][ijk[c]] + amp * ((hi[c] - lo[c]) / (2.0 * M_PI)) * s;
     }
     for (int c = 0; c < 3; ++c) sX[c][p] = x[c];
     __syncthreads();
@@ -279,8 +285,9 @@ k_geometry(const double *__restrict__ xyz, int ex, int ey, int ez, double lo0, d
     double Jp = a[0][0] * (a[1][1] * a[2][2] - a[1][2] * a[2][1]) + a[0][1] * (a[1][2] * a[2][0] - a[1][0] * a[2][2]) +
                 a[0][2] * (a[1][0] * a[2][1] - a[1][1] * a[2][0]);
     J[(size_t)e * n3 + p] = Jp;
-    invJ[(size_t)e * n3 + p] = 1.0 / Jp;
-    invJf[(size_t)e * n3 + p] = (float)(1.0 / Jp);
+    const double iJ = 1.0 / Jp;
+    invJ[(size_t)e * n3 + p] = iJ;
+    invJf[(size_t)e * n3 + p] = (float)iJ;
     for (int c = 0; c < 3; ++c) X[((size_t)e * 3 + c) * n3 + p] = x[c];
     if (dXout)   // dX_c/dxi_d, [E][c*3 + d][n3] (Gauss-Legendre meshes evaluate it at their nodes)
         for (int c = 0; c < 3; ++c)
@@ -296,7 +303,10 @@ k_geometry(const double *__restrict__ xyz, int ex, int ey, int ez, double lo0, d
             __syncthreads();
             double v = deriv(sT[0], i2) - deriv(sT[1], i1);
             Ja[(((size_t)e * 3 + i) * 3 + c) * n3 + p] = v;
-            Jaf[(((size_t)e * 3 + i) * 3 + c) * n3 + p] = (float)v;
+            const float vf = (float)v;
+            Jaf[(((size_t)e * 3 + i) * 3 + c) * n3 + p] = vf;
+            // low part of the FP32 metric terms (mixed path's float-float mass divergence)
+            if (Jalo) Jalo[(((size_t)e * 3 + i) * 3 + c) * n3 + p] = (float)(v - (double)vf);
             if (ijk[i] == N) {
                 // tangential (a,b) index of this node on the +i face
                 int ta = (i == 0) ? ijk[1] : ijk[0];
@@ -385,7 +395,7 @@ __global__ void k_facemetric_gauss(int n, long long total, const double *__restr
 }
 
 cudaError_t launch_geometry(int N, int nodes, const double *node_xyz_dev, int ex, int ey, int ez, const double *lo,
-                            const double *hi, double amp, double *X, double *Ja, float *Jaf, double *J, double *invJ,
+                            const double *hi, double amp, double *X, double *Ja, float *Jaf, float *Jalo, double *J, double *invJ,
                             float *invJf, double *fn, float *fnf, cudaStream_t s)
 {
     const Ops *ops = device_ops(N, HS3D_NODES_LOBATTO);
@@ -413,7 +423,7 @@ cudaError_t launch_geometry(int N, int nodes, const double *node_xyz_dev, int ex
 #define HS3D_GEO(NN)                                                                                            \
     case NN:                                                                                                    \
         k_geometry<NN><<<E, n3, 0, s>>>(node_xyz_dev, ex, ey, ez, lo[0], lo[1], lo[2], hi[0], hi[1], hi[2], amp, \
-                                        ops, XL, JaL, Jaf, J, invJ, invJf, fnL, fnf, dXL);                      \
+                                        ops, XL, JaL, Jaf, gauss ? nullptr : Jalo, J, invJ, invJf, fnL, fnf, dXL); \
         if (gauss)                                                                                              \
             k_geometry_gauss<NN><<<E, n3, 0, s>>>(XL, JaL, dXL, device_ops(N, HS3D_NODES_GAUSS), X, Ja, Jaf, J,  \
                                                   invJ, invJf);                                                 \
@@ -467,21 +477,6 @@ cudaError_t launch_init_state(int N, int E, const double *X, const hs3d_ic &ic, 
     int threads = 256;
     long long blocks = (total + threads - 1) / threads;
     k_init_state<<<(unsigned)blocks, threads, 0, s>>>(n3, total, X, ic, hi[0] - lo[0], hi[1] - lo[1], u);
-    return cudaGetLastError();
-}
-
-// Low part of the FP32 metric terms: Jalo = Ja - Jaf rounded to FP32.
-__global__ void k_metric_lo(const double *__restrict__ Ja, const float *__restrict__ Jaf, float *__restrict__ Jalo,
-                            long long count)
-{
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i < count) Jalo[i] = (float)(Ja[i] - (double)Jaf[i]);
-}
-
-cudaError_t launch_metric_lo(const double *Ja, const float *Jaf, float *Jalo, long long count, cudaStream_t s)
-{
-    if (count == 0) return cudaSuccess;
-    k_metric_lo<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(Ja, Jaf, Jalo, count);
     return cudaGetLastError();
 }
 

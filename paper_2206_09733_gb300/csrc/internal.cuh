@@ -508,7 +508,7 @@ __device__ __forceinline__ int nbr_of_slot(const Nbrs &r, int s)
 
 // Launch helpers implemented in the .cu files (return cudaError_t of the launch).
 cudaError_t launch_geometry(int N, int nodes, const double *node_xyz_dev, int ex, int ey, int ez, const double *lo,
-                            const double *hi, double amp, double *X, double *Ja, float *Jaf, double *J, double *invJ,
+                            const double *hi, double amp, double *X, double *Ja, float *Jaf, float *Jalo, double *J, double *invJ,
                             float *invJf, double *fn, float *fnf, cudaStream_t s);
 cudaError_t launch_init_state(int N, int E, const double *X, const hs3d_ic &ic, const double *lo, const double *hi,
                               double *u, cudaStream_t s);
@@ -534,8 +534,6 @@ cudaError_t prepare_gauss(int N);
 cudaError_t launch_face_dev(int N, int physics, int flux, const Batch &b, cudaStream_t s);
 cudaError_t launch_grad_dev(int N, const Batch &b, cudaStream_t s);
 cudaError_t prepare_grad_dev(int N);
-// Ja - Jaf rounded to FP32, one thread per value.
-cudaError_t launch_metric_lo(const double *Ja, const float *Jaf, float *Jalo, long long count, cudaStream_t s);
 // Low-storage RK schemes (HS3D_TIME_*): stage count and the stage's (A_k, B_k).
 int rk_stages(int scheme);
 void rk_coeffs(int scheme, int k, double *A, double *B);
