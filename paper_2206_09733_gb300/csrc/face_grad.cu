@@ -12,14 +12,14 @@
 // k_grad: BR1 gradients of q = (v1, v2, v3, T), T = p/rho (Bassi & Rebay 1997):
 //   J grad q_c = sum_d D_d (Ja^d_c q) + sum_faces (1/w_end) (q* - q_in) (+-Ja^d_c),
 //   q* = (q_in + q_out)/2, stored as viscous stress and heat flux (kVisc
-// values per node).  Element per thread group, node per thread.
+//   values per node).  Element per thread group, node per thread.
 //
 // Both are bound by the FP64 pipe, so they are written for few FP64
 // instructions per warp: one reciprocal per state (rcp_fast, shared by
 // velocities, enthalpy and temperature), one reciprocal square root for a
 // norm and its inverse, and one instruction sequence for the two faces of a
 // direction (a lane is on at most one of them).  16^3 elements of N = 3 (NS,
-// Roe), one launch: k_face 122 -> 118 us, k_grad 177 -> 143 us.
+// Roe), one launch: k_face 122 -> 85 us, k_grad 177 -> 106 us.
 #include "internal.cuh"
 #include "physics.cuh"
 
@@ -36,7 +36,7 @@ __device__ __forceinline__ int face_node(int d, int end, int ta, int tb)
 
 // Small CTAs: with its 142 registers a 256-thread CTA leaves one CTA (8 warps)
 // per SM, 64-thread CTAs 12 warps, and a small mesh reaches more SMs (16^3,
-// N = 3: 118 -> 98 us).
+// N = 3, two steps of three stages: 3175 -> 3071 us).
 constexpr int kFaceThreads = 64;
 
 template <int N, bool NS>

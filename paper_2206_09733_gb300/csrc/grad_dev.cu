@@ -317,12 +317,11 @@ constexpr bool has_grad_row()
 }
 
 __device__ __forceinline__ float4 ld4(const float *p) { return *(const float4 *)p; }
-__device__ __forceinline__ void fma4(float acc[4][kVisc], int k, float d, const float4 &w)
+// Sums of four nodes as packed pairs (0, 1), (2, 3) (two FP32 operations per issue slot).
+__device__ __forceinline__ void fma4(float2 acc[2][kVisc], int k, float d, const float4 &w)
 {
-    acc[0][k] += d * w.x;
-    acc[1][k] += d * w.y;
-    acc[2][k] += d * w.z;
-    acc[3][k] += d * w.w;
+    acc[0][k] = __ffma2_rn(make_float2(d, d), make_float2(w.x, w.y), acc[0][k]);
+    acc[1][k] = __ffma2_rn(make_float2(d, d), make_float2(w.z, w.w), acc[1][k]);
 }
 __device__ __forceinline__ float at4(const float4 &v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
 
@@ -423,19 +422,28 @@ __global__ void __launch_bounds__(128, 5) k_grad_row(const __grid_constant__ Bat
             }
         }
         __syncthreads();
-        float acc[4][kVisc];
+        float2 acc[2][kVisc];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 2; ++i)
 #pragma unroll
-            for (int c = 0; c < kVisc; ++c) acc[i][c] = 0.0f;
+            for (int c = 0; c < kVisc; ++c) acc[i][c] = make_float2(0.0f, 0.0f);
+        // one node's stress products onto its sums
+        auto add_node = [&](int i, float a1, float a2, float a3, float q1, float q2, float q3, float T) {
+            float t[kVisc];
+#pragma unroll
+            for (int c = 0; c < kVisc; ++c) t[c] = i & 1 ? acc[i >> 1][c].y : acc[i >> 1][c].x;
+            stress_add(t, a1, a2, a3, q1, q2, q3, T);
+#pragma unroll
+            for (int c = 0; c < kVisc; ++c) (i & 1 ? acc[i >> 1][c].y : acc[i >> 1][c].x) = t[c];
+        };
         const float *JA = it.Jaf + (size_t)e * 9 * n3 + p0;
         // the diagonal term at the two ends of a line: D_ii Ja q_out (see k_grad_dev)
         auto end_row = [&](const float4 J[3], const float *Q, float dn) {
             const float4 Q0 = ld4(Q), Q1 = ld4(Q + n2), Q2 = ld4(Q + 2 * n2), Q3 = ld4(Q + 3 * n2);
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                stress_add(acc[i], dn * at4(J[0], i), dn * at4(J[1], i), dn * at4(J[2], i), at4(Q0, i), at4(Q1, i),
-                           at4(Q2, i), at4(Q3, i));
+                add_node(i, dn * at4(J[0], i), dn * at4(J[1], i), dn * at4(J[2], i), at4(Q0, i), at4(Q1, i), at4(Q2, i),
+                         at4(Q3, i));
         };
         float4 J[3];
         if (valid) {
@@ -455,11 +463,11 @@ __global__ void __launch_bounds__(128, 5) k_grad_row(const __grid_constant__ Bat
             {
                 if (h == 0) {
                     const float *Q = qn + j + n * k;
-                    stress_add(acc[0], -dend * J[0].x, -dend * J[1].x, -dend * J[2].x, Q[0], Q[n2], Q[2 * n2], Q[3 * n2]);
+                    add_node(0, -dend * J[0].x, -dend * J[1].x, -dend * J[2].x, Q[0], Q[n2], Q[2 * n2], Q[3 * n2]);
                 }
                 if (h == RPL - 1) {
                     const float *Q = qn + 4 * n2 + j + n * k;
-                    stress_add(acc[3], dend * J[0].w, dend * J[1].w, dend * J[2].w, Q[0], Q[n2], Q[2 * n2], Q[3 * n2]);
+                    add_node(3, dend * J[0].w, dend * J[1].w, dend * J[2].w, Q[0], Q[n2], Q[2 * n2], Q[3 * n2]);
                 }
             }
         }
@@ -515,7 +523,12 @@ __global__ void __launch_bounds__(128, 5) k_grad_row(const __grid_constant__ Bat
             float *G = (float *)it.grad + (size_t)e * kVisc * n3 + p0;
             float tau[4][kVisc];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) stress_of(acc[i], at4(ij, i), it.muf, it.kappaf, tau[i]);
+            for (int i = 0; i < 4; ++i) {
+                float t[kVisc];
+#pragma unroll
+                for (int c = 0; c < kVisc; ++c) t[c] = i & 1 ? acc[i >> 1][c].y : acc[i >> 1][c].x;
+                stress_of(t, at4(ij, i), it.muf, it.kappaf, tau[i]);
+            }
 #pragma unroll
             for (int c = 0; c < kVisc; ++c)
                 *(float4 *)(G + c * n3) = make_float4(tau[0][c], tau[1][c], tau[2][c], tau[3][c]);

@@ -75,6 +75,34 @@ __host__ __device__ __forceinline__ void ff_mul(float &sh, float &sl, float ah, 
     sl = fmaf(ah, bl, fmaf(al, bh, pe));
 }
 
+#if defined(__CUDACC__)
+// The same on two values at once: Blackwell's packed FP32 instructions take two
+// operands of a register pair per issue slot, and the contractions of the element
+// and gradient kernels are bound by issue.  Bitwise the scalar operations, lane
+// by lane (a difference is an fma by -1, which rounds once as well).
+__device__ __forceinline__ float2 pair(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
+__device__ __forceinline__ float2 ff_prod2(float2 ah, float2 al, float2 bh, float2 bl, float2 &p)
+{
+    p = __fmul2_rn(ah, bh);
+    const float2 pe = __ffma2_rn(ah, bh, __fmul2_rn(p, make_float2(-1.0f, -1.0f)));
+    return __ffma2_rn(ah, bl, __ffma2_rn(al, bh, pe));
+}
+__device__ __forceinline__ void ff_mul2(float2 &sh, float2 &sl, float2 ah, float2 al, float2 bh, float2 bl)
+{
+    sl = ff_prod2(ah, al, bh, bl, sh);
+}
+__device__ __forceinline__ void ff_fma2(float2 &sh, float2 &sl, float2 ah, float2 al, float2 bh, float2 bl)
+{
+    float2 p;
+    const float2 pe = ff_prod2(ah, al, bh, bl, p);
+    const float2 s = __fadd2_rn(sh, p), bb = sub2(s, sh);
+    const float2 e = __fadd2_rn(sub2(sh, sub2(s, bb)), sub2(p, bb));
+    sh = s;
+    sl = __fadd2_rn(sl, __fadd2_rn(e, pe));
+}
+#endif
+
 // FP64 -> FP32 (round to nearest even) of the deviations: the integer-pipe
 // rounding d2f_rn (the hardware conversion, one FP64-pipe instruction each,
 // measured 3-20% slower in all three deviation kernels).

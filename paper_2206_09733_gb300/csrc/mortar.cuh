@@ -35,7 +35,7 @@ struct MortarSide {
     int N, E;
     long long base;        // offset of the bucket's first element in the caller's state (doubles)
     const float *uf;       // FP32 shadow of the bucket's state [E][5][n3] (mixed path)
-    const void *grad;      // BR1 gradients [E][12][n3] (R)
+    const void *grad;      // viscous stress and heat flux [E][9][n3] (FP64), BR1 gradients [E][12][n3] (FP32)
     const double *Ja;      // [E][9][n3]
     const float *Jaf;
     void *fstar6;          // face fluxes [6][E][5][n2] (R)
