@@ -57,21 +57,47 @@ constexpr int dev_threads()
     return (t + 31) & ~31;
 }
 
-// Staged floats per node:
-//   standard   [d][4] FP32 fluxes (momentum, energy rest), [d][hi, lo] of Ja^d.m'      18
-//   EC         rho', v'(3), beta', |v|^2 - |vbar|^2, m'(3), Ja - Ja_centre [d][3],
-//              [d][hi, lo] of Ja^d.m', NS: [d][4] viscous contravariant fluxes      24 (+12)
-//   other      7 two-point inputs, Jaf [d][3], NS: [d][4] viscous fluxes             16 (+12)
+// Staged floats per node, in groups of four that one 16-byte load brings (the
+// kernel is bound by issue: a line's contraction takes a load and two packed
+// multiply-adds a node in place of four of each, a Chandrashekar pair three loads in
+// place of twelve); viscous contravariant fluxes with the sign of a right-hand side.
+// Against single values: Euler standard form 64^3 N = 3 13.73 -> 13.39 ms (4 steps), 52^3
+// N = 4 16.47 -> 15.96, 24^3 N = 5 2.86 -> 2.73; Chandrashekar NS 16^3 N = 3 698 -> 680 us,
+// 24^3 N = 6 15.4 -> 14.7 ms; Pirozzoli NS 24^3 N = 5 5.53 -> 5.34:
+//   standard   [d] 4 FP32 fluxes (momentum, energy rest); [d][hi, lo] of Ja^d.m'       18
+//   EC         (rho', v'), (beta', |v|^2 - |vbar|^2, m1', m2'), [d] (Ja - Ja_centre, m3'),
+//              NS: [d] 4 viscous fluxes; [d][hi, lo] of Ja^d.m'                      26 (+12)
+//   other      singly 7 two-point inputs, Jaf [d][3]; NS: [d] 4 viscous fluxes       16 (+12)
 template <int FORM, bool NS>
 constexpr int dev_per_node()
 {
-    return (FORM == HS3D_VOL_STANDARD) ? 18 : (FORM == HS3D_VOL_EC ? 24 : 16) + (NS ? 12 : 0);
+    return (FORM == HS3D_VOL_STANDARD) ? 18 : (FORM == HS3D_VOL_EC ? 26 : 16) + (NS ? 12 : 0);
 }
 
 template <int FORM, bool NS>
 constexpr int dev_visc_off()
 {
-    return FORM == HS3D_VOL_EC ? 24 : 16;
+    return FORM == HS3D_VOL_EC ? 20 : 16;
+}
+
+// First of the mass pairs Ja^d.m' (hi, lo).
+template <int FORM, bool NS>
+constexpr int dev_mass_off()
+{
+    return FORM == HS3D_VOL_STANDARD ? 12 : NS ? 32 : 20;
+}
+
+// Floats per element of the staging and of the pair buffer (per slot: four fluxes
+// a node, then the mass remainder), in whole 16 bytes.
+template <int N, bool NS, int FORM>
+constexpr int dev_stage_floats()
+{
+    return (dev_per_node<FORM, NS>() * (N + 1) * (N + 1) * (N + 1) + 3) & ~3;
+}
+template <int N, int FORM>
+constexpr int dev_pair_floats()
+{
+    return FORM == HS3D_VOL_STANDARD ? 0 : (5 * ((N + 1) / 2) * (N + 1) * (N + 1) * (N + 1) + 3) & ~3;
 }
 
 // Per-element block of shared memory, 36 floats: the element's reference
@@ -85,14 +111,13 @@ static_assert(sizeof(Anchor) == 16 * sizeof(float) && offsetof(AnchorRec, a) == 
               "reference-state record layout");
 
 // Byte offset of the RK staging block (16-byte aligned): D, Dlo, per-element
-// blocks, per-node staging, face blocks, pair buffers (split forms).
+// blocks, per-node staging, pair buffers (split forms), face blocks.
 template <int N, bool NS, int FORM>
 __host__ __device__ constexpr size_t dev_rk_offset(int epb)
 {
-    constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
-    constexpr size_t pairs = (FORM == HS3D_VOL_STANDARD) ? 0 : (size_t)5 * (n / 2) * n3;
-    const size_t fl = 2 * ((n2 + 3) & ~3) + (size_t)epb * kDevElemBlock + (size_t)epb * dev_per_node<FORM, NS>() * n3 +
-                      (size_t)epb * 30 * n2 + (size_t)epb * pairs;
+    constexpr int n = N + 1, n2 = n * n;
+    const size_t fl = 2 * ((n2 + 3) & ~3) + (size_t)epb * (kDevElemBlock + dev_stage_floats<N, NS, FORM>() +
+                                                           dev_pair_floats<N, FORM>() + 30 * n2);
     return (sizeof(float) * fl + 15) & ~(size_t)15;
 }
 
@@ -156,6 +181,53 @@ __device__ __forceinline__ void dev_visc(const Prim<float> &q, const float *G, c
     else visc_flux(q, G, a1, a2, a3, f);
 }
 
+// One line of the float-float mass divergence, two nodes at a time (even and odd
+// ones summed apart); `first`: nothing summed before.  SEQ: node by node in
+// Ch.x + Cl.x (the mortar path, where the order of the sum is kept).
+template <int n, bool SEQ>
+__device__ __forceinline__ void mass_line(bool first, const float *D, const float *Dl, const float *wh, const float *wl,
+                                          int stride, float2 &Ch, float2 &Cl)
+{
+    if constexpr (SEQ) {
+#pragma unroll
+        for (int m = 0; m < n; ++m) {
+            if (first && m == 0) ff_mul(Ch.x, Cl.x, D[m], Dl[m], wh[m * stride], wl[m * stride]);
+            else ff_fma(Ch.x, Cl.x, D[m], Dl[m], wh[m * stride], wl[m * stride]);
+        }
+    } else {
+#pragma unroll
+        for (int m = 0; m + 1 < n; m += 2) {
+            float2 d2, l2;
+            if constexpr (n % 2 == 0) {
+                d2 = *(const float2 *)(D + m);
+                l2 = *(const float2 *)(Dl + m);
+            } else {
+                d2 = make_float2(D[m], D[m + 1]);
+                l2 = make_float2(Dl[m], Dl[m + 1]);
+            }
+            const float2 h2 = make_float2(wh[m * stride], wh[(m + 1) * stride]);
+            const float2 w2 = make_float2(wl[m * stride], wl[(m + 1) * stride]);
+            if (first && m == 0) ff_mul2(Ch, Cl, d2, l2, h2, w2);
+            else ff_fma2(Ch, Cl, d2, l2, h2, w2);
+        }
+        if constexpr (n % 2 == 1) ff_fma(Ch.x, Cl.x, D[n - 1], Dl[n - 1], wh[(n - 1) * stride], wl[(n - 1) * stride]);
+    }
+}
+
+// Chandrashekar pair inputs of node a: its state, momentum and metric deviations.
+__device__ __forceinline__ void ec_load(const float4 *S4, const float4 *DA, int n3, int a, ECDev &z, float dm[3],
+                                        float da[3])
+{
+    const float4 x = S4[a], y = S4[n3 + a], j = DA[a];
+    z = {x.x, x.y, x.z, x.w, y.x, y.y};
+    dm[0] = y.z;
+    dm[1] = y.w;
+    dm[2] = j.w;
+    da[0] = j.x;
+    da[1] = j.y;
+    da[2] = j.z;
+}
+
 // One tile (epb elements) of the element kernel; returns true on the
 // thread that initialised its element's bulk-copy barrier.  MORT: the items
 // take their face fluxes from the mortar kernels (Item::face6).
@@ -168,8 +240,8 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
     constexpr bool STD = (FORM == HS3D_VOL_STANDARD);
     constexpr bool EC = (FORM == HS3D_VOL_EC);
     constexpr bool LM = dev_lowmach<FORM>();
-    constexpr int PER = dev_per_node<FORM, NS>();
-    constexpr int VOFF = dev_visc_off<FORM, NS>();
+    constexpr int PER = dev_stage_floats<N, NS, FORM>(), PAIRS = dev_pair_floats<N, FORM>();
+    constexpr int VOFF = dev_visc_off<FORM, NS>(), WOFF = dev_mass_off<FORM, NS>();
     constexpr int KP = n / 2;
     constexpr int NG = MORT ? 12 : kVisc;
     constexpr bool BULK = (n % 2 == 0);
@@ -179,8 +251,8 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
     float *sDl = sD + D2;
     float *selem = sDl + D2;
     float *sbuf = selem + (size_t)epb * kDevElemBlock;
-    float *sface = sbuf + (size_t)epb * PER * n3;
-    float *spair = sface + (size_t)epb * 30 * n2;
+    float *spair = sbuf + (size_t)epb * PER;
+    float *sface = spair + (size_t)epb * PAIRS;
     float *sG = (float *)(smem_raw + dev_rk_offset<N, NS, FORM>(epb));
     float *sIJ = (float *)(sG + (STD ? (size_t)epb * 5 * n3 : 0));
     for (int t = threadIdx.x; t < n2; t += blockDim.x) {
@@ -198,9 +270,10 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
         if (itp->clk && itp->clk->done) valid = false;
     }
     const bool armed = BULK && valid && p == 0;
-    float *S = sbuf + (size_t)le * PER * n3;
+    float *S = sbuf + (size_t)le * PER;
+    float4 *S4 = (float4 *)S;   // groups of four, [group][n3]
     float *F6 = sface + (size_t)le * 30 * n2;
-    float *PB = spair + (size_t)le * 5 * KP * n3;
+    float *PB = spair + (size_t)le * PAIRS;
     double *AD = (double *)(selem + (size_t)le * kDevElemBlock);     // reference state, FP64 conserved
     Anchor *ANC = (Anchor *)(selem + (size_t)le * kDevElemBlock + 10);
     float *CEN = selem + (size_t)le * kDevElemBlock + 26;            // centre metric terms (EC)
@@ -233,7 +306,17 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
     }
     __syncthreads();
     float V[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    float Ch = 0.0f, Cl = 0.0f;   // float-float C (low-Mach forms)
+    float2 Ch = pair(0.0f), Cl = pair(0.0f);   // float-float C (low-Mach forms), even and odd nodes of a line
+    // four rest rows: V[1..4] += D f
+    auto add4 = [&](float D, const float4 &f) {
+        const float2 D2 = pair(D);
+        const float2 a = __ffma2_rn(D2, make_float2(f.x, f.y), make_float2(V[1], V[2]));
+        const float2 b = __ffma2_rn(D2, make_float2(f.z, f.w), make_float2(V[3], V[4]));
+        V[1] = a.x;
+        V[2] = a.y;
+        V[3] = b.x;
+        V[4] = b.y;
+    };
     float Hb = 0.0f;
     if (valid) {
         const Item &it = *itp;
@@ -296,7 +379,6 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
             // Ja^d.m' in float-float: m' = (mh, ml) from the FP64 deviation,
             // Ja = Jaf + Jalo
             const float *JL = it.Jalo + (size_t)e * 9 * n3;
-            constexpr int WOFF = STD ? 12 : 18;
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 float wh = 0.0f, wl = 0.0f;
@@ -321,28 +403,26 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
 #pragma unroll
                     for (int v = 0; v < 4; ++v) f[v] -= fv[v + 1];
                 }
-#pragma unroll
-                for (int v = 0; v < 4; ++v) S[(d * 4 + v) * n3 + p] = f[v];
+                S4[d * n3 + p] = make_float4(f[0], f[1], f[2], f[3]);
             }
         } else if constexpr (EC) {
             const ECDev z = ec_dev(dv, A);
-            S[0 * n3 + p] = z.dr;
-            S[1 * n3 + p] = z.dv1;
-            S[2 * n3 + p] = z.dv2;
-            S[3 * n3 + p] = z.dv3;
-            S[4 * n3 + p] = z.db;
-            S[5 * n3 + p] = z.q;
-            S[6 * n3 + p] = dv.dm1;
-            S[7 * n3 + p] = dv.dm2;
-            S[8 * n3 + p] = dv.dm3;
+            S4[p] = make_float4(z.dr, z.dv1, z.dv2, z.dv3);
+            S4[n3 + p] = make_float4(z.db, z.q, dv.dm1, dv.dm2);
             // metric terms as deviations from the centre node's, accurate to FP32
             // relative to the deviation (their differences enter e_im)
             const float *JL = it.Jalo + (size_t)e * 9 * n3;
 #pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                const float jc = JA[k * n3 + pc], jlc = JL[k * n3 + pc];
-                S[(9 + k) * n3 + p] = (ja[k] - jc) + (JL[k * n3 + p] - jlc);
-                if (p == 0) CEN[k] = jc;
+            for (int d = 0; d < 3; ++d) {
+                float da[3];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const int k = d * 3 + c;
+                    const float jc = JA[k * n3 + pc], jlc = JL[k * n3 + pc];
+                    da[c] = (ja[k] - jc) + (JL[k * n3 + p] - jlc);
+                    if (p == 0) CEN[k] = jc;
+                }
+                S4[(2 + d) * n3 + p] = make_float4(da[0], da[1], da[2], dv.dm3);
             }
             // the diagonal pair (i, i), nonzero on the boundary nodes only
             // (D_ii = 0 inside): the same two-point function as every other pair,
@@ -363,8 +443,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                 if (NS) {
                     float fv[5];
                     dev_visc<MORT>(q, G, it, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fv);
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) S[(VOFF + d * 4 + v) * n3 + p] = fv[v + 1];
+                    S4[(VOFF / 4 + d) * n3 + p] = make_float4(-fv[1], -fv[2], -fv[3], -fv[4]);
                 }
             }
         } else {
@@ -385,8 +464,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                 if (NS) {
                     float fv[5];
                     dev_visc<MORT>(q, G, it, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fv);
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) S[(VOFF + d * 4 + v) * n3 + p] = fv[v + 1];
+                    S4[(VOFF / 4 + d) * n3 + p] = make_float4(-fv[1], -fv[2], -fv[3], -fv[4]);
                 }
             }
         }
@@ -403,14 +481,9 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                 const float *Drow = sD + ijk[d] * n;
                 const float *Dlrow = sDl + ijk[d] * n;
 #pragma unroll
-                for (int m = 0; m < n; ++m) {
-                    const float Dm = Drow[m];
-                    const int pm = base + m * stride;
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) V[v + 1] += Dm * S[(d * 4 + v) * n3 + pm];
-                    if (d == 0 && m == 0) ff_mul(Ch, Cl, Dm, Dlrow[m], S[(12 + 2 * d) * n3 + pm], S[(13 + 2 * d) * n3 + pm]);
-                    else ff_fma(Ch, Cl, Dm, Dlrow[m], S[(12 + 2 * d) * n3 + pm], S[(13 + 2 * d) * n3 + pm]);
-                }
+                for (int m = 0; m < n; ++m) add4(Drow[m], S4[d * n3 + base + m * stride]);
+                const float *wh = S + (WOFF + 2 * d) * n3 + base;
+                mass_line<n, MORT>(d == 0, Drow, Dlrow, wh, wh + n3, stride, Ch, Cl);
             }
         }
     } else {
@@ -430,7 +503,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                 const int x = ijk[d];
                 const int lane = threadIdx.x & 31;
                 const float *Drow = sD + x * n;
-                const float *DA = S + (9 + d * 3) * n3;   // Chandrashekar form: metric deviations
+                const float4 *DA = S4 + (2 + d) * n3;     // Chandrashekar form: metric deviations, m3'
                 const float *SJ = S + (7 + d * 3) * n3;   // other split forms: metric terms
                 ECDev za{};
                 float dma[3] = {0.0f, 0.0f, 0.0f}, da[3] = {0.0f, 0.0f, 0.0f};
@@ -440,13 +513,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                 for (int q = 0; q < kSplitSlots; ++q) zo[q] = 0.0f;
                 if (valid) {
                     if constexpr (EC) {
-                        za = {S[p], S[n3 + p], S[2 * n3 + p], S[3 * n3 + p], S[4 * n3 + p], S[5 * n3 + p]};
-                        dma[0] = S[6 * n3 + p];
-                        dma[1] = S[7 * n3 + p];
-                        dma[2] = S[8 * n3 + p];
-                        da[0] = DA[p];
-                        da[1] = DA[n3 + p];
-                        da[2] = DA[2 * n3 + p];
+                        ec_load(S4, DA, n3, p, za, dma, da);
                         c1 = 2.0f * CEN[d * 3];
                         c2 = 2.0f * CEN[d * 3 + 1];
                         c3 = 2.0f * CEN[d * 3 + 2];
@@ -469,13 +536,13 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                         const int xm = (x + k < n) ? x + k : x + k - n;
                         const int c = p + (xm - x) * sd;
                         if constexpr (EC) {
-                            const ECDev zc = {S[c], S[n3 + c], S[2 * n3 + c], S[3 * n3 + c], S[4 * n3 + c], S[5 * n3 + c]};
-                            const float dc[3] = {DA[c], DA[n3 + c], DA[2 * n3 + c]};
+                            ECDev zc;
+                            float dmc[3], dc[3];
+                            ec_load(S4, DA, n3, c, zc, dmc, dc);
                             float frho, rmass, fm[3], rest;
                             dflux_ec(za, zc, A, hg, c1 + da[0] + dc[0], c2 + da[1] + dc[1], c3 + da[2] + dc[2], frho,
                                      rmass, fm, rest);
-                            const float dm1 = dma[0] - S[6 * n3 + c], dm2 = dma[1] - S[7 * n3 + c],
-                                        dm3 = dma[2] - S[8 * n3 + c];
+                            const float dm1 = dma[0] - dmc[0], dm2 = dma[1] - dmc[1], dm3 = dma[2] - dmc[2];
                             fp[0] = rmass - 0.5f * (dm1 * (da[0] - dc[0]) + dm2 * (da[1] - dc[1]) + dm3 * (da[2] - dc[2]));
                             fp[1] = fm[0];
                             fp[2] = fm[1];
@@ -506,17 +573,11 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                     const int base = p - x * sd;
                     const float *Dlrow = sDl + x * n;
 #pragma unroll
-                    for (int m = 0; m < n; ++m) {
-                        const float Dm = Drow[m];
-                        const int pm = base + m * sd;
-                        if (NS) {
-#pragma unroll
-                            for (int v = 0; v < 4; ++v) V[v + 1] -= Dm * S[(VOFF + d * 4 + v) * n3 + pm];
-                        }
-                        if constexpr (EC) {
-                            if (d == 0 && m == 0) ff_mul(Ch, Cl, Dm, Dlrow[m], S[(18 + 2 * d) * n3 + pm], S[(19 + 2 * d) * n3 + pm]);
-                            else ff_fma(Ch, Cl, Dm, Dlrow[m], S[(18 + 2 * d) * n3 + pm], S[(19 + 2 * d) * n3 + pm]);
-                        }
+                    for (int m = 0; m < n; ++m)
+                        if (NS) add4(Drow[m], S4[(VOFF / 4 + d) * n3 + base + m * sd]);
+                    if constexpr (EC) {
+                        const float *wh = S + (WOFF + 2 * d) * n3 + base;
+                        mass_line<n, MORT>(d == 0, Drow, Dlrow, wh, wh + n3, sd, Ch, Cl);
                     }
                 }
                 continue;
@@ -531,28 +592,26 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                 const int x = ijk[d];
                 const int a = p;
                 if constexpr (EC) {
-                    const ECDev za = {S[a], S[n3 + a], S[2 * n3 + a], S[3 * n3 + a], S[4 * n3 + a], S[5 * n3 + a]};
-                    const float dma[3] = {S[6 * n3 + a], S[7 * n3 + a], S[8 * n3 + a]};
-                    const float *DA = S + (9 + d * 3) * n3;
-                    const float da[3] = {DA[a], DA[n3 + a], DA[2 * n3 + a]};
+                    const float4 *DA = S4 + (2 + d) * n3;
+                    ECDev za;
+                    float dma[3], da[3];
+                    ec_load(S4, DA, n3, a, za, dma, da);
                     const float c1 = 2.0f * CEN[d * 3], c2 = 2.0f * CEN[d * 3 + 1], c3 = 2.0f * CEN[d * 3 + 2];
 #pragma unroll
                     for (int k = 1; k <= KP; ++k) {
                         if (2 * k == n && x >= KP) break;
                         const int xm = (x + k < n) ? x + k : x + k - n;
                         const int c = a + (xm - x) * sd;
-                        const ECDev zc = {S[c], S[n3 + c], S[2 * n3 + c], S[3 * n3 + c], S[4 * n3 + c], S[5 * n3 + c]};
-                        const float dc[3] = {DA[c], DA[n3 + c], DA[2 * n3 + c]};
+                        ECDev zc;
+                        float dmc[3], dc[3];
+                        ec_load(S4, DA, n3, c, zc, dmc, dc);
                         float frho, rmass, fm[3], rest;
                         dflux_ec(za, zc, A, hg, c1 + da[0] + dc[0], c2 + da[1] + dc[1], c3 + da[2] + dc[2], frho, rmass,
                                  fm, rest);
-                        const float dm1 = dma[0] - S[6 * n3 + c], dm2 = dma[1] - S[7 * n3 + c], dm3 = dma[2] - S[8 * n3 + c];
+                        const float dm1 = dma[0] - dmc[0], dm2 = dma[1] - dmc[1], dm3 = dma[2] - dmc[2];
                         const float em = rmass - 0.5f * (dm1 * (da[0] - dc[0]) + dm2 * (da[1] - dc[1]) + dm3 * (da[2] - dc[2]));
-                        PB[(0 * KP + k - 1) * n3 + p] = em;
-                        PB[(1 * KP + k - 1) * n3 + p] = fm[0];
-                        PB[(2 * KP + k - 1) * n3 + p] = fm[1];
-                        PB[(3 * KP + k - 1) * n3 + p] = fm[2];
-                        PB[(4 * KP + k - 1) * n3 + p] = rest;
+                        PB[(4 * KP + k - 1) * n3 + p] = em;
+                        ((float4 *)PB)[(k - 1) * n3 + p] = make_float4(fm[0], fm[1], fm[2], rest);
                     }
                 } else {
                     float za[kSplitSlots];
@@ -570,8 +629,8 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                         for (int qq = 0; qq < kSplitSlots; ++qq) zc[qq] = S[qq * n3 + c];
                         float fs[5];
                         split_pair<FORM>(za, zc, gam, hg, j1 + SJ[c], j2 + SJ[n3 + c], j3 + SJ[2 * n3 + c], fs);
-#pragma unroll
-                        for (int v = 0; v < 5; ++v) PB[(v * KP + k - 1) * n3 + p] = fs[v];
+                        PB[(4 * KP + k - 1) * n3 + p] = fs[0];
+                        ((float4 *)PB)[(k - 1) * n3 + p] = make_float4(fs[1], fs[2], fs[3], fs[4]);
                     }
                 }
             }
@@ -598,19 +657,15 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                             x = (i < KP) ? i : m;
                         }
                         // (the pair sits with the thread of its node x, in slot k - 1)
-                        const float *F = PB + (slot - 1) * n3 + base + x * sd;
-#pragma unroll
-                        for (int v = 0; v < 5; ++v) V[v] += Dm * F[v * KP * n3];
+                        const int at = (slot - 1) * n3 + base + x * sd;
+                        V[0] += Dm * PB[4 * KP * n3 + at];
+                        add4(Dm, ((const float4 *)PB)[at]);
                     }
-                    const int pm = base + m * sd;
-                    if (NS) {
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) V[v + 1] -= Dm * S[(VOFF + d * 4 + v) * n3 + pm];
-                    }
-                    if constexpr (EC) {
-                        if (d == 0 && m == 0) ff_mul(Ch, Cl, Dm, Dlrow[m], S[(18 + 2 * d) * n3 + pm], S[(19 + 2 * d) * n3 + pm]);
-                        else ff_fma(Ch, Cl, Dm, Dlrow[m], S[(18 + 2 * d) * n3 + pm], S[(19 + 2 * d) * n3 + pm]);
-                    }
+                    if (NS) add4(Dm, S4[(VOFF / 4 + d) * n3 + base + m * sd]);
+                }
+                if constexpr (EC) {
+                    const float *wh = S + (WOFF + 2 * d) * n3 + base;
+                    mass_line<n, MORT>(d == 0, Drow, Dlrow, wh, wh + n3, sd, Ch, Cl);
                 }
             }
             // (after the last direction the pair buffer is not written again)
@@ -648,7 +703,13 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
     // volume rows: mass = C (+ the split form's remainder), energy = Hbar mass + rest
     float Vr = V[0];
     if constexpr (LM) {
-        Vr = (Ch + Cl) + V[0];
+        if constexpr (MORT) {
+            Vr = (Ch.x + Cl.x) + V[0];
+        } else {
+            float c, ce;
+            two_sum(Ch.x, Ch.y, c, ce);
+            Vr = (c + (ce + (Cl.x + Cl.y))) + V[0];
+        }
         V[4] += Hb * Vr;
     }
     V[0] = Vr;
