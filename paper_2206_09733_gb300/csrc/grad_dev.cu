@@ -29,12 +29,12 @@ constexpr int grad_dev_threads()
     return ((N + 1) * (N + 1) * (N + 1) > 256) ? (N + 1) * (N + 1) * (N + 1) : 256;
 }
 
-// Shared-memory floats per element: metric terms [9][n3], q' [4][n3],
-// neighbour-trace deviations [6][4][n2].
+// Shared-memory floats per element: q' [n3] and neighbour-trace deviations [6][n2]
+// in groups of four (one 16-byte load each), metric terms [9][n3].
 template <int N>
 constexpr int grad_dev_per_elem()
 {
-    return 13 * (N + 1) * (N + 1) * (N + 1) + 24 * (N + 1) * (N + 1);
+    return (13 * (N + 1) * (N + 1) * (N + 1) + 24 * (N + 1) * (N + 1) + 3) & ~3;
 }
 
 template <int n>
@@ -80,9 +80,9 @@ __device__ __forceinline__ bool grad_dev_tile(const Batch &b, const Ops *__restr
         if (itp->clk && itp->clk->done) valid = false;
     }
     const bool armed = BULK && valid && p == 0;
-    float *ja = sE + (size_t)le * PER;
-    float *q = ja + 9 * n3;
-    float *qn = q + 4 * n3;
+    float4 *q = (float4 *)(sE + (size_t)le * PER);
+    float4 *qn = q + n3;
+    float *ja = (float *)(qn + 6 * n2);
     float qin[4];
     if (valid) {
         const Item &it = *itp;
@@ -115,10 +115,7 @@ __device__ __forceinline__ bool grad_dev_tile(const Batch &b, const Ops *__restr
                 if (t < 6 * n2) {
                     const int slot = t / n2, ab = t - slot * n2;
                     const float *src = (const float *)it.qhat6 + ((size_t)slot * it.E + e) * 4 * n2 + ab;
-                    qn[(slot * 4 + 0) * n2 + ab] = src[0] - A.v1;
-                    qn[(slot * 4 + 1) * n2 + ab] = src[n2] - A.v2;
-                    qn[(slot * 4 + 2) * n2 + ab] = src[2 * n2] - A.v3;
-                    qn[(slot * 4 + 3) * n2 + ab] = src[3 * n2] - Tb;
+                    qn[t] = make_float4(src[0] - A.v1, src[n2] - A.v2, src[2 * n2] - A.v3, src[3 * n2] - Tb);
                 }
             }
         } else {
@@ -141,17 +138,14 @@ __device__ __forceinline__ bool grad_dev_tile(const Batch &b, const Ops *__restr
             for (int k = 0; k < IT; ++k) {
                 const int t = p + k * n3;
                 if (t < 6 * n2) {
-                    const int slot = t / n2, ab = t - slot * n2;
                     float g4[4];
                     grad_dev_vars(make_dev_rec(raw[k], A, R.Elo, gm1), A, Tb, rT, g4);
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) qn[(slot * 4 + v) * n2 + ab] = g4[v];
+                    qn[t] = make_float4(g4[0], g4[1], g4[2], g4[3]);
                 }
             }
         }
         grad_dev_vars(make_dev_rec(uo, A, R.Elo, gm1), A, Tb, rT, qin);
-#pragma unroll
-        for (int v = 0; v < 4; ++v) q[v * n3 + p] = qin[v];
+        q[p] = make_float4(qin[0], qin[1], qin[2], qin[3]);
         if constexpr (!BULK) {
             const float *JA = it.Jaf + (size_t)e * 9 * n3 + p;
 #pragma unroll
@@ -170,65 +164,22 @@ __device__ __forceinline__ bool grad_dev_tile(const Batch &b, const Ops *__restr
     }
     const int ijk[3] = {p % n, (p / n) % n, p / n2};
     const Item &it = *itp;
-    if constexpr (MORT) {
-        // the twelve gradients, every rounding as the mortar path's FP32 fluxes
-        // expect it (visc_flux_grad)
-        if (!landed) qin[0] = qin[1] = qin[2] = qin[3] = NAN;
-        float acc[12];
+    if (MORT && !landed) qin[0] = qin[1] = qin[2] = qin[3] = NAN;
+    // the twelve sums d q_v / dx_c, as packed pairs of v: (v1, v2) and (v3, T) share
+    // the metric factor, one 16-byte load brings q (against single values, the run:
+    // NS standard form, 24^3 N = 5 4.63 -> 4.47 ms, 24^3 N = 6 10.10 -> 9.89, 30^3 N = 4
+    // 6.61 -> 6.53, 40^3 N = 3 6.04 -> 6.01)
+    float2 a01[3], a23[3];
 #pragma unroll
-        for (int k = 0; k < 12; ++k) acc[k] = 0.0f;
+    for (int c = 0; c < 3; ++c) a01[c] = a23[c] = pair(0.0f);
+    auto add = [&](float s1, float s2, float s3, const float4 &Q) {
+        const float s[3] = {s1, s2, s3};
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const int stride = (d == 0) ? 1 : (d == 1) ? n : n2;
-            const int base = p - ijk[d] * stride;
-            const float *Drow = sD + ijk[d] * n;
-#pragma unroll
-            for (int m = 0; m < n; ++m) {
-                const int pm = base + m * stride;
-                const float Dm = Drow[m];
-                const float a1 = Dm * ja[(d * 3 + 0) * n3 + pm], a2 = Dm * ja[(d * 3 + 1) * n3 + pm],
-                            a3 = Dm * ja[(d * 3 + 2) * n3 + pm];
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const float qv = q[v * n3 + pm];
-                    acc[v * 3 + 0] += a1 * qv;
-                    acc[v * 3 + 1] += a2 * qv;
-                    acc[v * 3 + 2] += a3 * qv;
-                }
-            }
+        for (int c = 0; c < 3; ++c) {
+            a01[c] = __ffma2_rn(pair(s[c]), make_float2(Q.x, Q.y), a01[c]);
+            a23[c] = __ffma2_rn(pair(s[c]), make_float2(Q.z, Q.w), a23[c]);
         }
-        // surface lifting of the BR1 jumps (q* - q_in) = (q_out - q_in)/2
-        const float iw = ops->iw0f;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const int ta = (d == 0) ? ijk[1] : ijk[0];
-            const int tb = (d == 2) ? ijk[1] : ijk[2];
-            const int ab = ta + n * tb;
-#pragma unroll
-            for (int plus = 0; plus < 2; ++plus) {
-                if (ijk[d] != (plus ? N : 0)) continue;
-                const float sg = plus ? 1.0f : -1.0f;
-                const float n1 = sg * ja[(d * 3 + 0) * n3 + p], n2_ = sg * ja[(d * 3 + 1) * n3 + p],
-                            n3_ = sg * ja[(d * 3 + 2) * n3 + p];
-                const int slot = 2 * d + plus;
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const float j = 0.5f * (qn[(slot * 4 + v) * n2 + ab] - qin[v]) * iw;
-                    acc[v * 3 + 0] += j * n1;
-                    acc[v * 3 + 1] += j * n2_;
-                    acc[v * 3 + 2] += j * n3_;
-                }
-            }
-        }
-        const float ij = it.invJf[(size_t)e * n3 + p];
-        float *G = (float *)it.grad + (size_t)e * 12 * n3 + p;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) G[k * n3] = acc[k] * ij;
-        return armed;
-    }
-    float acc[kVisc];
-#pragma unroll
-    for (int k = 0; k < kVisc; ++k) acc[k] = 0.0f;
+    };
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         const int i = ijk[d];
@@ -240,23 +191,57 @@ __device__ __forceinline__ bool grad_dev_tile(const Batch &b, const Ops *__restr
         for (int m = 0; m < n; ++m) {
             const int pm = base + m * stride;
             const float Dm = Drow[m];
-            stress_add(acc, Dm * J1[pm], Dm * J2[pm], Dm * J3[pm], q[pm], q[n3 + pm], q[2 * n3 + pm], q[3 * n3 + pm]);
+            add(Dm * J1[pm], Dm * J2[pm], Dm * J3[pm], q[pm]);
         }
-        // the two ends: D_ii Ja q_in + (+-1/w)(q_out - q_in)/2 Ja = D_ii Ja q_out,
-        // D_ii = +-1/(2w) (sD holds zero on the diagonal)
-        if (i == 0 || i == N) {
-            const int ta = (d == 0) ? ijk[1] : ijk[0];
-            const int tb = (d == 2) ? ijk[1] : ijk[2];
-            const float *Q = qn + (2 * d + (i == N ? 1 : 0)) * 4 * n2 + ta + n * tb;
-            const float Dm = i == N ? dend : -dend;
-            stress_add(acc, Dm * J1[p], Dm * J2[p], Dm * J3[p], Q[0], Q[n2], Q[2 * n2], Q[3 * n2]);
+        if constexpr (!MORT) {
+            // the two ends: D_ii Ja q_in + (+-1/w)(q_out - q_in)/2 Ja = D_ii Ja q_out,
+            // D_ii = +-1/(2w) (sD holds zero on the diagonal)
+            if (i == 0 || i == N) {
+                const int ta = (d == 0) ? ijk[1] : ijk[0];
+                const int tb = (d == 2) ? ijk[1] : ijk[2];
+                const float Dm = i == N ? dend : -dend;
+                add(Dm * J1[p], Dm * J2[p], Dm * J3[p], qn[(2 * d + (i == N ? 1 : 0)) * n2 + ta + n * tb]);
+            }
         }
     }
-    float tau[kVisc];
-    stress_of(acc, landed ? it.invJf[(size_t)e * n3 + p] : NAN, it.muf, it.kappaf, tau);
-    float *G = (float *)it.grad + (size_t)e * kVisc * n3 + p;
+    if constexpr (MORT) {
+        // surface lifting of the BR1 jumps (q* - q_in) = (q_out - q_in)/2; the twelve
+        // gradients stay, every rounding as the mortar path's FP32 fluxes expect it
+        // (visc_flux_grad)
+        const float iw = ops->iw0f;
 #pragma unroll
-    for (int k = 0; k < kVisc; ++k) G[k * n3] = tau[k];
+        for (int d = 0; d < 3; ++d) {
+            const int ta = (d == 0) ? ijk[1] : ijk[0];
+            const int tb = (d == 2) ? ijk[1] : ijk[2];
+            const int ab = ta + n * tb;
+#pragma unroll
+            for (int plus = 0; plus < 2; ++plus) {
+                if (ijk[d] != (plus ? N : 0)) continue;
+                const float sg = plus ? 1.0f : -1.0f;
+                const float4 Q = qn[(2 * d + plus) * n2 + ab];
+                add(sg * ja[(d * 3 + 0) * n3 + p], sg * ja[(d * 3 + 1) * n3 + p], sg * ja[(d * 3 + 2) * n3 + p],
+                    make_float4(0.5f * (Q.x - qin[0]) * iw, 0.5f * (Q.y - qin[1]) * iw, 0.5f * (Q.z - qin[2]) * iw,
+                                0.5f * (Q.w - qin[3]) * iw));
+            }
+        }
+        const float ij = it.invJf[(size_t)e * n3 + p];
+        float *G = (float *)it.grad + (size_t)e * 12 * n3 + p;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            G[c * n3] = a01[c].x * ij;
+            G[(3 + c) * n3] = a01[c].y * ij;
+            G[(6 + c) * n3] = a23[c].x * ij;
+            G[(9 + c) * n3] = a23[c].y * ij;
+        }
+    } else {
+        const float acc[kVisc] = {a01[0].x, a01[1].y, a23[2].x, a01[0].y + a01[1].x, a23[0].x + a01[2].x,
+                                  a23[1].x + a01[2].y, a23[0].y, a23[1].y, a23[2].y};
+        float tau[kVisc];
+        stress_of(acc, landed ? it.invJf[(size_t)e * n3 + p] : NAN, it.muf, it.kappaf, tau);
+        float *G = (float *)it.grad + (size_t)e * kVisc * n3 + p;
+#pragma unroll
+        for (int k = 0; k < kVisc; ++k) G[k * n3] = tau[k];
+    }
     return armed;
 }
 
