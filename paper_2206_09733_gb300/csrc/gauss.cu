@@ -153,6 +153,53 @@ __global__ void __launch_bounds__(256) k_face_gauss(const __grid_constant__ Batc
 
 // ------------------------------------------------------------------ BR1 gradients
 
+// Four values a point in shared memory.  FP32: side by side, one 16-byte access and
+// packed multiply-adds (these kernels issue more shared-memory and FP32
+// instructions than anything else); FP64: four arrays of `S` values, consecutive
+// threads on consecutive words.  Either way 4 S values, rounded the same.
+// Runs of 4 steps, NS, against single values: 32^3 N = 3 4.20 -> 4.02 ms, 24^3 N = 4 4.01 ->
+// 3.71, 20^3 N = 5 4.56 -> 4.11, 16^3 N = 7 6.60 -> 6.08; Euler 32^3 N = 3 1.95 -> 1.82.
+template <typename R>
+struct Four {
+    R x[4];
+};
+template <int S, typename R>
+__device__ __forceinline__ Four<R> ld_four(const R *base, int i)
+{
+    if constexpr (sizeof(R) == 4) {
+        const float4 v = ((const float4 *)base)[i];
+        return {v.x, v.y, v.z, v.w};
+    } else {
+        return {base[i], base[S + i], base[2 * S + i], base[3 * S + i]};
+    }
+}
+template <int S, typename R>
+__device__ __forceinline__ void st_four(R *base, int i, R a, R b, R c, R d)
+{
+    if constexpr (sizeof(R) == 4) {
+        ((float4 *)base)[i] = make_float4(a, b, c, d);
+    } else {
+        base[i] = a;
+        base[S + i] = b;
+        base[2 * S + i] = c;
+        base[3 * S + i] = d;
+    }
+}
+// a += s f
+template <typename R>
+__device__ __forceinline__ void add_four(Four<R> &a, R s, const Four<R> &f)
+{
+    if constexpr (sizeof(R) == 4) {
+        const float2 s2 = make_float2(s, s);
+        const float2 lo = __ffma2_rn(s2, make_float2(f.x[0], f.x[1]), make_float2(a.x[0], a.x[1]));
+        const float2 hi = __ffma2_rn(s2, make_float2(f.x[2], f.x[3]), make_float2(a.x[2], a.x[3]));
+        a = {lo.x, lo.y, hi.x, hi.y};
+    } else {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) a.x[v] += s * f.x[v];
+    }
+}
+
 template <int N>
 constexpr int gauss_threads()
 {
@@ -162,7 +209,7 @@ constexpr int gauss_threads()
 template <int N>
 constexpr int grad_gauss_per_elem()
 {
-    return 18 * (N + 1) * (N + 1) * (N + 1) + 72 * (N + 1) * (N + 1);
+    return (18 * (N + 1) * (N + 1) * (N + 1) + 72 * (N + 1) * (N + 1) + 3) & ~3;
 }
 
 template <typename R>
@@ -189,7 +236,7 @@ k_grad_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops)
     constexpr int PER = grad_gauss_per_elem<N>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R *sD = (R *)smem_raw;
-    R *sE = sD + ((n * n + 1) & ~1);
+    R *sE = sD + ((n * n + 3) & ~3);
     const int epb = blockDim.x / n3;
     for (int t = threadIdx.x; t < n * n; t += blockDim.x) sD[t] = ops_D<R>(ops, t);
     const int le = threadIdx.x / n3, p = threadIdx.x - le * n3;
@@ -202,10 +249,11 @@ k_grad_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops)
         e = (int)(ge - itp->elem_begin);
         if (itp->clk && itp->clk->done) valid = false;
     }
-    R *su = sE + (size_t)le * PER;
-    R *sq = su + 5 * n3;
-    R *sja = sq + 4 * n3;
-    R *slift = sja + 9 * n3;
+    R *su = sE + (size_t)le * PER;   // mass and momentum in fours, then energy
+    R *sq = su + 4 * n3;
+    R *slift = sq + 4 * n3;          // [6 slots][3 directions][n2] fours
+    R *su4 = slift + 72 * n2;
+    R *sja = su4 + n3;
     // this thread's face points: the neighbours' interpolated traces and the face
     // metric come before the barrier, so that their loads (5 n values from another
     // element) overlap the element's own instead of following them (32^3, N = 3:
@@ -239,13 +287,11 @@ k_grad_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops)
         for (int v = 0; v < 5; ++v) {
             if constexpr (sizeof(R) == 8) uu[v] = it.u[(size_t)e * 5 * n3 + p + (size_t)v * n3];
             else uu[v] = it.uf[(size_t)e * 5 * n3 + p + (size_t)v * n3];
-            su[v * n3 + p] = uu[v];
         }
+        st_four<n3>(su, p, uu[0], uu[1], uu[2], uu[3]);
+        su4[p] = uu[4];
         const Prim<R> qp = prim_of<R>(uu, gm1);
-        sq[0 * n3 + p] = qp.v1;
-        sq[1 * n3 + p] = qp.v2;
-        sq[2 * n3 + p] = qp.v3;
-        sq[3 * n3 + p] = temperature(qp);
+        st_four<n3>(sq, p, qp.v1, qp.v2, qp.v3, temperature(qp));
         const R *JA = gmetric<R>(it) + (size_t)e * 9 * n3 + p;
 #pragma unroll
         for (int k = 0; k < 9; ++k) sja[k * n3 + p] = JA[k * n3];
@@ -263,53 +309,49 @@ k_grad_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops)
             const int slot = t / n2, ab = t - slot * n2;
             const int d = slot >> 1, plus = slot & 1;
             const int ta = ab % n, tb = ab / n;
-            R uo[5];
-#pragma unroll
-            for (int v = 0; v < 5; ++v) uo[v] = (R)0;
+            Four<R> o{};
+            R o4 = (R)0;
 #pragma unroll
             for (int j = 0; j < n; ++j) {
                 const R l = plus ? ops_rb<R>(ops, j) : ops_lb<R>(ops, j);
                 const int pj = gline<n>(d, j, ta, tb);
-#pragma unroll
-                for (int v = 0; v < 5; ++v) uo[v] += l * su[v * n3 + pj];
+                add_four(o, l, ld_four<n3>(su, pj));
+                o4 += l * su4[pj];
             }
+            const R uo[5] = {o.x[0], o.x[1], o.x[2], o.x[3], o4};
             const Prim<R> po = prim_of<R>(uo, gm1), pn = prim_of<R>(un[c], gm1);
             const R qs[4] = {(R)0.5 * (po.v1 + pn.v1), (R)0.5 * (po.v2 + pn.v2), (R)0.5 * (po.v3 + pn.v3),
                              (R)0.5 * (temperature(po) + temperature(pn))};
             const R sg = plus ? (R)1 : (R)-1;
             // interpolated products (Ja^d_c q_v)(+-1): line node by line node,
             // each node's 3 metric terms and 4 variables read once
-            R jq[12];
-#pragma unroll
-            for (int k = 0; k < 12; ++k) jq[k] = (R)0;
+            Four<R> jq[3]{};
 #pragma unroll
             for (int j = 0; j < n; ++j) {
                 const R l = plus ? ops_rb<R>(ops, j) : ops_lb<R>(ops, j);
                 const int pj = gline<n>(d, j, ta, tb);
-                R jac[3], qv[4];
+                const Four<R> qv = ld_four<n3>(sq, pj);
 #pragma unroll
-                for (int x = 0; x < 3; ++x) jac[x] = sja[(d * 3 + x) * n3 + pj];
-#pragma unroll
-                for (int v = 0; v < 4; ++v) qv[v] = sq[v * n3 + pj];
-#pragma unroll
-                for (int v = 0; v < 4; ++v)
-#pragma unroll
-                    for (int x = 0; x < 3; ++x) jq[v * 3 + x] += l * (jac[x] * qv[v]);
+                for (int x = 0; x < 3; ++x) {
+                    const R jac = sja[(d * 3 + x) * n3 + pj];
+                    const Four<R> t = {jac * qv.x[0], jac * qv.x[1], jac * qv.x[2], jac * qv.x[3]};
+                    add_four(jq[x], l, t);
+                }
             }
 #pragma unroll
-            for (int v = 0; v < 4; ++v)
+            for (int x = 0; x < 3; ++x) {
+                R lift[4];
 #pragma unroll
-                for (int x = 0; x < 3; ++x)
-                    slift[(slot * 12 + v * 3 + x) * n2 + ab] = sg * (qs[v] * sf[c][x] - jq[v * 3 + x]);
+                for (int v = 0; v < 4; ++v) lift[v] = sg * (qs[v] * sf[c][x] - jq[x].x[v]);
+                st_four<n2>(slift + (slot * 3 + x) * 4 * n2, ab, lift[0], lift[1], lift[2], lift[3]);
+            }
         }
     }
     __syncthreads();
     if (!valid) return;
     const Item &it = *itp;
     const int ijk[3] = {p % n, (p / n) % n, p / n2};
-    R acc[12];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = (R)0;
+    Four<R> acc[3]{};   // d (v, T) / dx_c
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         const int stride = (d == 0) ? 1 : (d == 1) ? n : n2;
@@ -319,15 +361,9 @@ k_grad_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops)
         for (int m = 0; m < n; ++m) {
             const int pm = base + m * stride;
             const R Dm = Drow[m];
-            const R a1 = Dm * sja[(d * 3 + 0) * n3 + pm], a2 = Dm * sja[(d * 3 + 1) * n3 + pm],
-                    a3 = Dm * sja[(d * 3 + 2) * n3 + pm];
+            const Four<R> qv = ld_four<n3>(sq, pm);
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const R qv = sq[v * n3 + pm];
-                acc[v * 3 + 0] += a1 * qv;
-                acc[v * 3 + 1] += a2 * qv;
-                acc[v * 3 + 2] += a3 * qv;
-            }
+            for (int c = 0; c < 3; ++c) add_four(acc[c], Dm * sja[(d * 3 + c) * n3 + pm], qv);
         }
     }
 #pragma unroll
@@ -338,15 +374,19 @@ k_grad_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops)
         const int ab = ta + n * tb;
         const R wp = ops_rbw<R>(ops, i), wm = ops_lbw<R>(ops, i);
 #pragma unroll
-        for (int k = 0; k < 12; ++k)
-            acc[k] += wp * slift[((2 * d + 1) * 12 + k) * n2 + ab] + wm * slift[((2 * d) * 12 + k) * n2 + ab];
+        for (int c = 0; c < 3; ++c) {
+            const Four<R> lp = ld_four<n2>(slift + ((2 * d + 1) * 3 + c) * 4 * n2, ab);
+            const Four<R> lm = ld_four<n2>(slift + (2 * d * 3 + c) * 4 * n2, ab);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[c].x[v] += wp * lp.x[v] + wm * lm.x[v];
+        }
     }
     R ij;
     if constexpr (sizeof(R) == 8) ij = it.invJ[(size_t)e * n3 + p];
     else ij = it.invJf[(size_t)e * n3 + p];
     R *G = (R *)it.grad + (size_t)e * 12 * n3 + p;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) G[k * n3] = acc[k] * ij;
+    for (int k = 0; k < 12; ++k) G[k * n3] = acc[k % 3].x[k / 3] * ij;
 }
 
 // ------------------------------------------------------------------ element kernel (standard form)
@@ -360,11 +400,12 @@ k_volume_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int
 {
     constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
     constexpr int FACEVALS = 6 * 5 * n2;
+    constexpr int PER = (15 * n3 + 3) & ~3;   // contravariant fluxes: [3] fours, [3] energy
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R *sD = (R *)smem_raw;
     const int epb = blockDim.x / n3;
-    R *sbuf = sD + ((n * n + 1) & ~1);
-    R *sface = sbuf + (size_t)epb * 15 * n3;
+    R *sbuf = sD + ((n * n + 3) & ~3);
+    R *sface = sbuf + (size_t)epb * PER;
     for (int t = threadIdx.x; t < n * n; t += blockDim.x) sD[t] = ops_D<R>(ops, t);
     const int le = threadIdx.x / n3, p = threadIdx.x - le * n3;
     const long long ge = blockIdx.x * (long long)epb + le;
@@ -376,7 +417,7 @@ k_volume_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int
         e = (int)(ge - itp->elem_begin);
         if (itp->clk && itp->clk->done) valid = false;
     }
-    R *S = sbuf + (size_t)le * 15 * n3;
+    R *S = sbuf + (size_t)le * PER, *SE = S + 12 * n3;
     R *F6 = sface + (size_t)le * FACEVALS;
     const int ijk[3] = {p % n, (p / n) % n, p / n2};
     double u[5];
@@ -419,7 +460,9 @@ k_volume_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int
             euler_flux(q, q.E, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fe);
             if (NS) visc_flux_grad(q, G, P.mu, P.kappa, ja[d * 3], ja[d * 3 + 1], ja[d * 3 + 2], fv);
 #pragma unroll
-            for (int v = 0; v < 5; ++v) S[(d * 5 + v) * n3 + p] = NS ? fe[v] - fv[v] : fe[v];
+            for (int v = 0; v < 5; ++v) fe[v] = NS ? fe[v] - fv[v] : fe[v];
+            st_four<n3>(S + d * 4 * n3, p, fe[0], fe[1], fe[2], fe[3]);
+            SE[d * n3 + p] = fe[4];
         }
     }
     cp_async_wait_all();
@@ -430,14 +473,18 @@ k_volume_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int
             const int slot = t / n2, ab = t - slot * n2;
             const int d = slot >> 1, plus = slot & 1;
             const int ta = ab % n, tb = ab / n;
+            Four<R> o{};
+            R o4 = (R)0;
+#pragma unroll
+            for (int j = 0; j < n; ++j) {
+                const R l = plus ? ops_rb<R>(ops, j) : ops_lb<R>(ops, j);
+                const int pj = gline<n>(d, j, ta, tb);
+                add_four(o, l, ld_four<n3>(S + d * 4 * n3, pj));
+                o4 += l * SE[d * n3 + pj];
+            }
 #pragma unroll
             for (int v = 0; v < 5; ++v) {
-                R own = (R)0;
-#pragma unroll
-                for (int j = 0; j < n; ++j) {
-                    const R l = plus ? ops_rb<R>(ops, j) : ops_lb<R>(ops, j);
-                    own += l * S[(d * 5 + v) * n3 + gline<n>(d, j, ta, tb)];
-                }
+                const R own = v < 4 ? o.x[v < 4 ? v : 0] : o4;
                 R *Fp = F6 + (slot * 5 + v) * n2 + ab;
                 *Fp = plus ? (*Fp - own) : (own - *Fp);
             }
@@ -447,7 +494,8 @@ k_volume_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int
     double lc = 0.0, lv = 0.0;
     bool lam_active = false;
     if (valid) {
-        R V[5] = {(R)0, (R)0, (R)0, (R)0, (R)0};
+        Four<R> W{};
+        R W4 = (R)0;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             const int stride = (d == 0) ? 1 : (d == 1) ? n : n2;
@@ -456,10 +504,11 @@ k_volume_gauss(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int
 #pragma unroll
             for (int m = 0; m < n; ++m) {
                 const R Dm = Drow[m];
-#pragma unroll
-                for (int v = 0; v < 5; ++v) V[v] += Dm * S[(d * 5 + v) * n3 + base + m * stride];
+                add_four(W, Dm, ld_four<n3>(S + d * 4 * n3, base + m * stride));
+                W4 += Dm * SE[d * n3 + base + m * stride];
             }
         }
+        R V[5] = {W.x[0], W.x[1], W.x[2], W.x[3], W4};
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             const int i = ijk[d];
@@ -508,7 +557,7 @@ static cudaError_t grad_gauss(const Batch &b, cudaStream_t s)
     constexpr int n = N + 1, n3 = n * n * n;
     if (b.total_elems == 0) return cudaSuccess;
     const int epb = gauss_epb<N>(sizeof(R) == 4 ? HS3D_MIXED32 : HS3D_FP64, 0, b.total_elems);
-    const size_t smem = sizeof(R) * (((n * n + 1) & ~1) + (size_t)epb * grad_gauss_per_elem<N>());
+    const size_t smem = sizeof(R) * (((n * n + 3) & ~3) + (size_t)epb * grad_gauss_per_elem<N>());
     const unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);
     const Ops *ops = device_ops(N, HS3D_NODES_GAUSS);
     if (!ops) return cudaErrorMemoryAllocation;
@@ -522,7 +571,7 @@ static cudaError_t volume_gauss(const Batch &b, int stage, double rkA, double rk
     constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
     if (b.total_elems == 0) return cudaSuccess;
     const int epb = gauss_epb<N>(sizeof(R) == 4 ? HS3D_MIXED32 : HS3D_FP64, 1, b.total_elems);
-    const size_t smem = sizeof(R) * (((n * n + 1) & ~1) + (size_t)epb * (15 * n3 + 30 * n2));
+    const size_t smem = sizeof(R) * (((n * n + 3) & ~3) + (size_t)epb * (((15 * n3 + 3) & ~3) + 30 * n2));
     const unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);
     const Ops *ops = device_ops(N, HS3D_NODES_GAUSS);
     if (!ops) return cudaErrorMemoryAllocation;
