@@ -358,6 +358,8 @@ __global__ void __launch_bounds__(128, 5) k_grad_row(const __grid_constant__ Bat
         const Item &it = *itp;
         float q[4][4];
         if (valid) {
+            // the metric terms, needed after the traces, toward L2 (the run -1%)
+            prefetch_l2_block(it.Jaf + (size_t)e * 9 * n3, sizeof(float) * 9 * n3, r, TPE);
             double uo[5][4];
             const double *U = it.u + (size_t)e * 5 * n3 + p0;
 #pragma unroll

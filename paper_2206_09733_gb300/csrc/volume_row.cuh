@@ -76,6 +76,14 @@ __global__ void __launch_bounds__(128, 5) k_volume_row(const __grid_constant__ B
                                               : (((size_t)d * it.E + nb.m[d]) * 2 + 1) * 5 * n2);
                 prefetch_l2_block(face[slot], sizeof(float) * 5 * n2, r, TPE);
             }
+            // all the element's inputs toward L2: the loop below loads a quarter of them
+            // per round, and 20 warps on an SM cannot cover DRAM four times over (32^3,
+            // NS, 4 steps 22.6 -> 21.6 ms; 20^3, Euler 3.29 -> 3.06; the RK register as
+            // well: +0.5%)
+            prefetch_l2_block(it.u + (size_t)e * 5 * n3, sizeof(double) * 5 * n3, r, TPE);
+            prefetch_l2_block(it.Jaf + (size_t)e * 9 * n3, sizeof(float) * 9 * n3, r, TPE);
+            prefetch_l2_block(it.Jalo + (size_t)e * 9 * n3, sizeof(float) * 9 * n3, r, TPE);
+            if (NS) prefetch_l2_block((const float *)it.grad + (size_t)e * kVisc * n3, sizeof(float) * kVisc * n3, r, TPE);
             const AnchorRec R = load_anchor(it.anc, e);
             const Anchor A = R.a;
             Hb = A.H;
