@@ -30,6 +30,7 @@
 #include <mutex>
 #include <vector>
 
+#include "fours.cuh"
 #include "internal.cuh"
 #include "mortar.cuh"
 #include "physics.cuh"
@@ -196,8 +197,14 @@ struct MortarShape {
     static constexpr int TARGET = 128;                             // threads per CTA aimed at
     static constexpr int FPC = TARGET / P >= 1 ? TARGET / P : 1;  // faces per CTA
     static constexpr int THREADS = FPC * P;
-    // shared values per face: two sides' traces, the first-pass buffer, the mortar result
-    static constexpr int PER_FACE = 2 * NV * P + NV * P + 5 * P;
+    // shared values per face: two sides' traces, the first-pass buffer, the mortar
+    // result; first all groups of four (fours.cuh), then the NR values left over
+    // (single values cost a load per value and term of the interpolation, 17 of them
+    // with viscosity; 32^3, degrees 2..5, NS, two steps, with the element kernel's own
+    // viscous flux taken from its staging: 6.94 -> 6.64 ms)
+    static constexpr int NQ = NV / 4, NR = NV % 4;
+    static constexpr int QUADS = 4 * P * (3 * NQ + 1);
+    static constexpr int PER_FACE = (QUADS + P * (3 * NR + 1) + 3) & ~3;
     // resident CTAs per SM asked of the register allocator (FP32): 8 (64
     // registers) where that spills nothing, 6 for the viscous flux, whose
     // two sides' state and gradients (34 values) are live at once
@@ -218,9 +225,13 @@ k_mortar(const MortarFace *__restrict__ faces, int nfaces, const MortarSide *__r
     const int q = threadIdx.x / P, p = threadIdx.x - q * P;
     const int f = blockIdx.x * S::FPC + q;
     const bool live = f < nfaces;
-    R *tr = (R *)smem_raw + (size_t)q * S::PER_FACE;   // [2][NV][P]
-    R *T = tr + 2 * NV * P;                            // [NV][P]
-    R *fm = T + NV * P;                                // [5][P]
+    constexpr int NQ = S::NQ, NR = S::NR;
+    R *tr = (R *)smem_raw + (size_t)q * S::PER_FACE;   // [2][NQ][P] fours
+    R *T = tr + 2 * NQ * 4 * P;                        // [NQ][P] fours
+    R *fm = T + NQ * 4 * P;                            // [P] fours
+    R *tr1 = fm + 4 * P;                               // [2][NR][P]
+    R *T1 = tr1 + 2 * NR * P;                          // [NR][P]
+    R *fm1 = T1 + NR * P;                              // [P]
     const int a = p % nM, b = p / nM;
     MortarFace F{};
     int Nside[2] = {NM, NM};
@@ -240,21 +251,26 @@ k_mortar(const MortarFace *__restrict__ faces, int nfaces, const MortarSide *__r
             const int le = s ? F.lR : F.lL;
             if (p < ns * ns) {
                 const int node = mortar_face_node(ns, d, s ? 0 : SD.N, p % ns, p / ns);
-                R *dst = tr + s * NV * P + p;
+                R in[NV];
                 if constexpr (sizeof(R) == 8) {
                     const double *src = u + SD.base + (size_t)le * 5 * n3 + node;
 #pragma unroll
-                    for (int v = 0; v < 5; ++v) dst[v * P] = src[(size_t)v * n3];
+                    for (int v = 0; v < 5; ++v) in[v] = src[(size_t)v * n3];
                 } else {
                     const float *src = SD.uf + (size_t)le * 5 * n3 + node;
 #pragma unroll
-                    for (int v = 0; v < 5; ++v) dst[v * P] = src[(size_t)v * n3];
+                    for (int v = 0; v < 5; ++v) in[v] = src[(size_t)v * n3];
                 }
                 if constexpr (MODE == 1 && NS) {
                     const R *G = (const R *)SD.grad + (size_t)le * mortar_grads<R>() * n3 + node;
 #pragma unroll
-                    for (int k = 0; k < mortar_grads<R>(); ++k) dst[(5 + k) * P] = G[(size_t)k * n3];
+                    for (int k = 0; k < mortar_grads<R>(); ++k) in[5 + k] = G[(size_t)k * n3];
                 }
+#pragma unroll
+                for (int g = 0; g < NQ; ++g)
+                    st_four<P>(tr + (s * NQ + g) * 4 * P, p, in[4 * g], in[4 * g + 1], in[4 * g + 2], in[4 * g + 3]);
+#pragma unroll
+                for (int v = 0; v < NR; ++v) tr1[(s * NR + v) * P + p] = in[4 * NQ + v];
             }
         }
     }
@@ -265,7 +281,7 @@ k_mortar(const MortarFace *__restrict__ faces, int nfaces, const MortarSide *__r
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
         const int Ns = Nside[s], ns = Ns + 1;
-        const R *src = tr + s * NV * P;
+        const R *src = tr + s * NQ * 4 * P, *src1 = tr1 + s * NR * P;
         // (nM ns <= P entries: at most one per thread; loops unrolled to nM with
         // the side's ns as a predicate)
         if (Ns < NM && p < nM * ns) {
@@ -276,12 +292,20 @@ k_mortar(const MortarFace *__restrict__ faces, int nfaces, const MortarSide *__r
 #pragma unroll
             for (int i = 0; i < nM; ++i) row[i] = i < ns ? I[ap * ns + i] : (R)0;
 #pragma unroll
-            for (int v = 0; v < NV; ++v) {
+            for (int g = 0; g < NQ; ++g) {
+                Four<R> acc{};
+#pragma unroll
+                for (int i = 0; i < nM; ++i)
+                    if (i < ns) add_four(acc, row[i], ld_four<P>(src + g * 4 * P, i + ns * j));
+                st_four<P>(T + g * 4 * P, p, acc.x[0], acc.x[1], acc.x[2], acc.x[3]);
+            }
+#pragma unroll
+            for (int v = 0; v < NR; ++v) {
                 R acc = (R)0;
 #pragma unroll
                 for (int i = 0; i < nM; ++i)
-                    if (i < ns) acc += row[i] * src[v * P + i + ns * j];
-                T[v * P + p] = acc;
+                    if (i < ns) acc += row[i] * src1[v * P + i + ns * j];
+                T1[v * P + p] = acc;
             }
         }
         __syncthreads();   // (uniform: every thread of the CTA reaches it for both sides)
@@ -291,16 +315,31 @@ k_mortar(const MortarFace *__restrict__ faces, int nfaces, const MortarSide *__r
 #pragma unroll
             for (int j = 0; j < nM; ++j) col[j] = j < ns ? I[b * ns + j] : (R)0;
 #pragma unroll
-            for (int v = 0; v < NV; ++v) {
+            for (int g = 0; g < NQ; ++g) {
+                Four<R> acc{};
+#pragma unroll
+                for (int j = 0; j < nM; ++j)
+                    if (j < ns) add_four(acc, col[j], ld_four<P>(T + g * 4 * P, a + nM * j));
+#pragma unroll
+                for (int v = 0; v < 4; ++v) w[s][4 * g + v] = acc.x[v];
+            }
+#pragma unroll
+            for (int v = 0; v < NR; ++v) {
                 R acc = (R)0;
 #pragma unroll
                 for (int j = 0; j < nM; ++j)
-                    if (j < ns) acc += col[j] * T[v * P + a + nM * j];
-                w[s][v] = acc;
+                    if (j < ns) acc += col[j] * T1[v * P + a + nM * j];
+                w[s][4 * NQ + v] = acc;
             }
         } else {
 #pragma unroll
-            for (int v = 0; v < NV; ++v) w[s][v] = src[v * P + p];
+            for (int g = 0; g < NQ; ++g) {
+                const Four<R> f = ld_four<P>(src + g * 4 * P, p);
+#pragma unroll
+                for (int v = 0; v < 4; ++v) w[s][4 * g + v] = f.x[v];
+            }
+#pragma unroll
+            for (int v = 0; v < NR; ++v) w[s][4 * NQ + v] = src1[v * P + p];
         }
         __syncthreads();   // T is reused by the other side
     }
@@ -311,8 +350,8 @@ k_mortar(const MortarFace *__restrict__ faces, int nfaces, const MortarSide *__r
             R qL[4], qR[4];
             mortar_q(w[0], Ph.gm1, qL);
             mortar_q(w[1], Ph.gm1, qR);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) fm[v * P + p] = (R)0.5 * (qL[v] + qR[v]);
+            st_four<P>(fm, p, (R)0.5 * (qL[0] + qR[0]), (R)0.5 * (qL[1] + qR[1]), (R)0.5 * (qL[2] + qR[2]),
+                       (R)0.5 * (qL[3] + qR[3]));
         } else {
             // face metric of the side of degree NM (L on a tie), at its own face point (a, b)
             const bool useL = Nside[0] >= Nside[1];
@@ -332,14 +371,14 @@ k_mortar(const MortarFace *__restrict__ faces, int nfaces, const MortarSide *__r
 #pragma unroll
                 for (int v = 1; v < 5; ++v) fs[v] -= (R)0.5 * (fl[v] + fr[v]);
             }
-#pragma unroll
-            for (int v = 0; v < 5; ++v) fm[v * P + p] = fs[v];
+            st_four<P>(fm, p, fs[0], fs[1], fs[2], fs[3]);
+            fm1[p] = fs[4];
         }
     }
     __syncthreads();
 
     // 4. projection onto each side and the write to its own face block
-    constexpr int NOUT = MODE == 0 ? 4 : 5;
+    constexpr bool FIVE = MODE == 1;
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
         const int Ns = Nside[s], ns = Ns + 1, n2 = ns * ns;
@@ -350,47 +389,51 @@ k_mortar(const MortarFace *__restrict__ faces, int nfaces, const MortarSide *__r
             R row[nM];
 #pragma unroll
             for (int i = 0; i < nM; ++i) row[i] = Pr[ap * nM + i];
+            Four<R> acc{};
+            R acc1 = (R)0;
 #pragma unroll
-            for (int v = 0; v < NOUT; ++v) {
-                R acc = (R)0;
-#pragma unroll
-                for (int i = 0; i < nM; ++i) acc += row[i] * fm[v * P + i + nM * j];
-                T[v * P + p] = acc;
+            for (int i = 0; i < nM; ++i) {
+                add_four(acc, row[i], ld_four<P>(fm, i + nM * j));
+                if (FIVE) acc1 += row[i] * fm1[i + nM * j];
             }
+            st_four<P>(T, p, acc.x[0], acc.x[1], acc.x[2], acc.x[3]);
+            if (FIVE) T1[p] = acc1;
         }
         __syncthreads();
         if (live && p < n2) {
             const int ap = p % ns, bp = p / ns;
-            R val[5];
+            Four<R> val{};
+            R val1 = (R)0;
             if (Ns < NM) {
                 const R *Pr = mo_proj<R>(mo, Ns, NM);
                 R col[nM];
 #pragma unroll
                 for (int j = 0; j < nM; ++j) col[j] = Pr[bp * nM + j];
 #pragma unroll
-                for (int v = 0; v < NOUT; ++v) {
-                    R acc = (R)0;
-#pragma unroll
-                    for (int j = 0; j < nM; ++j) acc += col[j] * T[v * P + ap + ns * j];
-                    val[v] = acc;
+                for (int j = 0; j < nM; ++j) {
+                    add_four(val, col[j], ld_four<P>(T, ap + ns * j));
+                    if (FIVE) val1 += col[j] * T1[ap + ns * j];
                 }
             } else {
-#pragma unroll
-                for (int v = 0; v < NOUT; ++v) val[v] = fm[v * P + p];
+                val = ld_four<P>(fm, p);
+                if (FIVE) val1 = fm1[p];
             }
             const MortarSide &SD = sides[s ? F.bR : F.bL];
             const int slot = s ? 2 * d : 2 * d + 1;
             const int le = s ? F.lR : F.lL;
             if constexpr (MODE == 0) {
+                const Four<R> t = ld_four<P>(tr + s * NQ * 4 * P, p);
+                const R own[5] = {t.x[0], t.x[1], t.x[2], t.x[3], tr1[s * NR * P + p]};
                 R qin[4];
-                mortar_q(tr + s * NV * P + p, Ph.gm1, qin, P);
+                mortar_q(own, Ph.gm1, qin);
                 R *dst = (R *)SD.qhat6 + ((size_t)slot * SD.E + le) * 4 * n2 + p;
 #pragma unroll
-                for (int v = 0; v < 4; ++v) dst[v * n2] = (R)2 * val[v] - qin[v];
+                for (int v = 0; v < 4; ++v) dst[v * n2] = (R)2 * val.x[v] - qin[v];
             } else {
                 R *dst = (R *)SD.fstar6 + ((size_t)slot * SD.E + le) * 5 * n2 + p;
 #pragma unroll
-                for (int v = 0; v < 5; ++v) dst[v * n2] = val[v];
+                for (int v = 0; v < 4; ++v) dst[v * n2] = val.x[v];
+                dst[4 * n2] = val1;
             }
         }
         __syncthreads();   // T is reused by the other side

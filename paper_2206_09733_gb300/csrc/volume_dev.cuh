@@ -727,7 +727,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
             for (int v = 0; v < 5; ++v) ad[v] = AD[v];
             const Prim<float> q = dev_prim(make_dev(u, ad, A, it.gm1f), A);
             float G[NG];
-            if (NS) {
+            if (NS && STD) {
                 const float *Gp = (const float *)it.grad + (size_t)e * NG * n3 + p;
 #pragma unroll
                 for (int k = 0; k < NG; ++k) G[k] = Gp[k * n3];
@@ -738,11 +738,18 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                 if (ijk[d] != 0 && ijk[d] != N) continue;
                 const float a1 = JA[(d * 3) * n3], a2 = JA[(d * 3 + 1) * n3], a3 = JA[(d * 3 + 2) * n3];
                 euler_flux(q, q.E, a1, a2, a3, own[d]);
-                if (NS) {
+                if (NS && STD) {
                     float fv[5];
                     dev_visc<MORT>(q, G, it, a1, a2, a3, fv);
 #pragma unroll
                     for (int v = 1; v < 5; ++v) own[d][v] -= fv[v];
+                } else if (NS) {
+                    // (split forms: the viscous flux is the staged one)
+                    const float4 f = S4[(VOFF / 4 + d) * n3 + p];
+                    own[d][1] += f.x;
+                    own[d][2] += f.y;
+                    own[d][3] += f.z;
+                    own[d][4] += f.w;
                 }
             }
         }
