@@ -232,7 +232,7 @@ __device__ __forceinline__ void ec_load(const float4 *S4, const float4 *DA, int 
 // thread that initialised its element's bulk-copy barrier.  MORT: the items
 // take their face fluxes from the mortar kernels (Item::face6).
 template <int N, bool NS, int FORM, bool MORT>
-__device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__restrict__ ops, int stage, double rkA,
+__device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__restrict__ ops, int stage, float rkA,
                                                 double rkB, int lam_slot, int epb, long long tile,
                                                 unsigned long long *bulk_bar)
 {
@@ -779,15 +779,17 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
     } else {
         // the register g holds FP32 increments (dt R is an FP32 quantity here);
         // the state accumulates in FP64: u <- u + B g, one FP64 FMA a variable
-        const float sdt = d2f_rn(dtv) * ijf;
-        const float rkAf = d2f_rn(rkA);
+        // (one conversion in hardware: the FP64 pipe is a third busy, the integer one of
+        // d2f_rn costs 18 issue slots; more of them on the FP64 pipe, 64^3 Euler N = 3:
+        // the two dev_round +0.5%, the three momentum ones +9%)
+        const float sdt = __double2float_rn(dtv) * ijf;
         double *Up = it.u + (size_t)e * 5 * n3 + p;
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
             const float inc = -V[v] * sdt;
             float gv;
             if (stage == 0) gv = inc;
-            else gv = fmaf(rkAf, STD ? sG[(size_t)le * 5 * n3 + v * n3 + p] : gprev[v], inc);
+            else gv = fmaf(rkA, STD ? sG[(size_t)le * 5 * n3 + v * n3 + p] : gprev[v], inc);
             Gp[v * n3] = gv;
             u[v] = fma(rkB, f2d_exact(gv), u[v]);
             Up[v * n3] = u[v];
@@ -834,7 +836,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
 // The tile as a separate function for the persistent loop (inlined into a
 // loop, its values were hoisted across iterations and spilled).
 template <int N, bool NS, int FORM>
-__device__ __noinline__ bool volume_dev_tile_call(const Batch &b, const Ops *__restrict__ ops, int stage, double rkA,
+__device__ __noinline__ bool volume_dev_tile_call(const Batch &b, const Ops *__restrict__ ops, int stage, float rkA,
                                                   double rkB, int lam_slot, int epb, long long tile,
                                                   unsigned long long *bulk_bar)
 {
@@ -847,7 +849,7 @@ __device__ __noinline__ bool volume_dev_tile_call(const Batch &b, const Ops *__r
 // before the next tile initialises them again.
 template <int N, bool NS, int FORM, bool PERSIST, bool MORT = false>
 __global__ void __launch_bounds__(dev_threads<N, FORM>(), dev_min_blocks<N, NS, FORM>())
-k_volume_dev(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int stage, double rkA, double rkB,
+k_volume_dev(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int stage, float rkA, double rkB,
              int lam_slot, int epb, long long ntiles)
 {
     pdl_wait();
@@ -876,12 +878,12 @@ constexpr bool has_row_kernel()
     return is_standard(FORM) && N == 7;
 }
 template <int N, bool NS>
-static cudaError_t vol_row_launch(const Batch &b, int stage, double rkA, double rkB, int lam_slot, cudaStream_t s);
+static cudaError_t vol_row_launch(const Batch &b, int stage, float rkA, double rkB, int lam_slot, cudaStream_t s);
 template <int N>
 static cudaError_t vol_row_prep();
 
 template <int N, bool NS, int FORM>
-static cudaError_t vol_dev_launch2(const Batch &b, int stage, double rkA, double rkB, int lam_slot, cudaStream_t s)
+static cudaError_t vol_dev_launch2(const Batch &b, int stage, float rkA, double rkB, int lam_slot, cudaStream_t s)
 {
     if constexpr (has_row_kernel<N, FORM>()) {
         if (!b.mortar) return vol_row_launch<N, NS>(b, stage, rkA, rkB, lam_slot, s);
@@ -918,8 +920,8 @@ cudaError_t launch_volume_dev_form(int N, int physics, const Batch &b, int stage
     if (b.total_elems == 0) return cudaSuccess;
 #define HS3D_VDN(K)                                                                                       \
     case K:                                                                                               \
-        return physics == HS3D_NS ? vol_dev_launch2<K, true, FORM>(b, stage, rkA, rkB, lam_slot, s)       \
-                                  : vol_dev_launch2<K, false, FORM>(b, stage, rkA, rkB, lam_slot, s);
+        return physics == HS3D_NS ? vol_dev_launch2<K, true, FORM>(b, stage, (float)rkA, rkB, lam_slot, s)  \
+                                  : vol_dev_launch2<K, false, FORM>(b, stage, (float)rkA, rkB, lam_slot, s);
     switch (N) {
         HS3D_VDN(1) HS3D_VDN(2) HS3D_VDN(3) HS3D_VDN(4) HS3D_VDN(5) HS3D_VDN(6) HS3D_VDN(7)
     }

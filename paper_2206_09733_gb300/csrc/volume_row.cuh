@@ -35,7 +35,7 @@ struct VolRow {
 
 template <int N, bool NS, bool PERSIST>
 __global__ void __launch_bounds__(128, 5) k_volume_row(const __grid_constant__ Batch b, const Ops *__restrict__ ops,
-                                                       int stage, double rkA, double rkB, int lam_slot,
+                                                       int stage, float rkA, double rkB, int lam_slot,
                                                        long long ntiles)
 {
     using S = VolRow<N>;
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(128, 5) k_volume_row(const __grid_constant__ B
                 }
             } else {
                 // FP32 register, FP64 state (as volume_dev_tile)
-                const float dtf = d2f_rn(dtv), rkAf = d2f_rn(rkA);
+                const float dtf = __double2float_rn(dtv);
                 double *Up = it.u + (size_t)e * 5 * n3 + p0;
                 float nf[4][5];
                 double uc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // the centre node's new state
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(128, 5) k_volume_row(const __grid_constant__ B
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const float inc = -V[i][v] * (dtf * ijf[i]);
-                        gv[i] = (stage == 0) ? inc : fmaf(rkAf, gp[i], inc);
+                        gv[i] = (stage == 0) ? inc : fmaf(rkA, gp[i], inc);
                         u[i] = fma(rkB, f2d_exact(gv[i]), u[i]);
                         if (lam_slot >= 0) nf[i][v] = d2f_rn(u[i]);
                     }
@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(128, 5) k_volume_row(const __grid_constant__ B
 }
 
 template <int N, bool NS>
-static cudaError_t vol_row_launch(const Batch &b, int stage, double rkA, double rkB, int lam_slot, cudaStream_t s)
+static cudaError_t vol_row_launch(const Batch &b, int stage, float rkA, double rkB, int lam_slot, cudaStream_t s)
 {
     using S = VolRow<N>;
     const unsigned tiles = (unsigned)b.total_elems;
