@@ -282,9 +282,10 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
 
     double u[5];
     if (valid) {
-        if constexpr (n3 > 256) {
-            // N = 7: the element's metric terms and gradients toward L2 ahead of
-            // their per-thread loads (-3% at 24^3; at N = 3 it measured +1-2%)
+        if constexpr (n3 > 200) {
+            // from N = 5: the element's metric terms and gradients toward L2 ahead of
+            // their per-thread loads (N = 7, 24^3 -3%; N = 5, 24^3: standard form Euler
+            // 2.74 -> 2.62 ms, Chandrashekar NS 7.91 -> 7.76; at N = 3 it measured +1-2%)
             prefetch_l2_block(itp->Jaf + (size_t)e * 9 * n3, sizeof(float) * 9 * n3, p, n3);
             if (LM) prefetch_l2_block(itp->Jalo + (size_t)e * 9 * n3, sizeof(float) * 9 * n3, p, n3);
             if (NS) prefetch_l2_block((const float *)itp->grad + (size_t)e * NG * n3, sizeof(float) * NG * n3, p, n3);
