@@ -234,7 +234,7 @@ def measured_volume_traffic():
 
 # ------------------------------------------------------------------ algorithmic cost model (per launch)
 
-def kernel_bytes(kernel, prec, E=None, n=N + 1):
+def kernel_bytes(kernel, prec, E=None, n=N + 1, visc=9):
     """Compulsory DRAM bytes of one launch of each kernel.  FP64 path: state,
     metric terms, 1/J and scratch in FP64.  Mixed path: every kernel reads
     the FP64 state (it forms the deviations from it) and FP32 copies of Ja,
@@ -242,7 +242,9 @@ def kernel_bytes(kernel, prec, E=None, n=N + 1):
     part of Ja (the float-float mass divergence), keeps the RK register in
     FP32 and reads and rewrites each element's 112-byte reference state,
     which the gradient kernel reads too; the face kernel writes one flux
-    block per side of each face; scratch in FP32."""
+    block per side of each face; scratch in FP32.  `visc`: values per node
+    that the gradient kernel leaves (stress and heat flux; the FP32 mortar
+    path keeps the twelve gradients)."""
     E = EX * EY * EZ if E is None else E
     n2, n3 = n * n, n ** 3
     if prec == "fp64":
@@ -251,12 +253,12 @@ def kernel_bytes(kernel, prec, E=None, n=N + 1):
         s, geo, jal, sides, reg, anc = 4, 36 + 4, 36, 2, 4, 112
     if kernel == "volume":     # u, metrics (+ low part), 1/J, grads, this element's 6 face blocks, reference
         #                        state in and out; g in/out, u out
-        return E * (40 * n3 + (geo + jal) * n3 + 12 * n3 * s + 6 * 5 * n2 * s + 2 * anc + 2 * 5 * reg * n3 + 40 * n3)
-    if kernel == "face":       # two FP64 traces, face normal, two gradient traces in; flux (per side) out
-        return 3 * E * (2 * 40 * n2 + 3 * n2 * s + 2 * 12 * n2 * s + sides * 5 * n2 * s)
+        return E * (40 * n3 + (geo + jal) * n3 + visc * n3 * s + 6 * 5 * n2 * s + 2 * anc + 2 * 5 * reg * n3 + 40 * n3)
+    if kernel == "face":       # two FP64 traces, face normal, two stress traces in; flux (per side) out
+        return 3 * E * (2 * 40 * n2 + 3 * n2 * s + 2 * visc * n2 * s + sides * 5 * n2 * s)
     if kernel == "grad":       # own FP64 state, metrics, 1/J, 6 neighbour FP64 traces, reference state in;
-        #                        gradients out
-        return E * (40 * n3 + geo * n3 + 6 * 40 * n2 + anc + 12 * n3 * s)
+        #                        stress and heat flux out
+        return E * (40 * n3 + geo * n3 + 6 * 40 * n2 + anc + visc * n3 * s)
     return 0
 
 
@@ -531,7 +533,7 @@ def step_bytes(prec, physics, E, n, stages=3):
         per_stage += kernel_bytes("grad", prec, E, n)
     else:   # no gradients are read by the face and element kernels
         s = 8 if prec == "fp64" else 4
-        per_stage -= E * 12 * n ** 3 * s + 3 * E * 24 * n * n * s
+        per_stage -= E * 9 * n ** 3 * s + 3 * E * 18 * n * n * s
     return stages * per_stage
 
 
@@ -591,19 +593,19 @@ def pstep_bytes(prec, physics, deg, ex, ey, ez, stages=3):
     viscous flux, + the face metric of the side of the larger degree) and
     write each side's projected block."""
     import numpy as np
-    s, st = (8, 40) if prec == "fp64" else (4, 20)
+    s, st, visc = (8, 40, 9) if prec == "fp64" else (4, 20, 12)
     ns = physics == "ns"
     deg = np.asarray(deg)
     n = deg + 1
     per_stage = 0
     for N in np.unique(deg):
         E = int((deg == N).sum())
-        per_stage += kernel_bytes("volume", prec, E, int(N) + 1)
+        per_stage += kernel_bytes("volume", prec, E, int(N) + 1, visc)
         if ns:
             nn = int(N) + 1
-            per_stage += kernel_bytes("grad", prec, E, nn) - E * 6 * st * nn * nn + E * 6 * 4 * nn * nn * s
+            per_stage += kernel_bytes("grad", prec, E, nn, visc) - E * 6 * st * nn * nn + E * 6 * 4 * nn * nn * s
     if not ns:
-        per_stage -= int(((12 * n ** 3 * s) * 1).sum())
+        per_stage -= int((visc * n ** 3 * s).sum())
     e = np.arange(deg.size)
     a, b, c = e % ex, (e // ex) % ey, e // (ex * ey)
     for d in range(3):
@@ -612,7 +614,7 @@ def pstep_bytes(prec, physics, deg, ex, ey, ez, stages=3):
         r = ab[0] + ex * (ab[1] + ey * ab[2])
         nL2, nR2 = n ** 2, n[r] ** 2
         nH2 = np.maximum(nL2, nR2)
-        flux = (nL2 + nR2) * (st + 5 * s + (12 * s if ns else 0)) + 3 * nH2 * s
+        flux = (nL2 + nR2) * (st + 5 * s + (visc * s if ns else 0)) + 3 * nH2 * s
         per_stage += int(flux.sum())
         if ns:
             per_stage += int(((nL2 + nR2) * (st + 4 * s)).sum())
