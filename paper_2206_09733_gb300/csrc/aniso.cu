@@ -949,10 +949,10 @@ cudaError_t allow_smem(K kernel, size_t bytes)
                              : cudaSuccess;
 }
 
-// (set once at mesh set-up: not a stream operation, but kept out of captured launches)
 template <int T, bool NS>
-cudaError_t allow_avol_smem(int kp)
+cudaError_t allow_avol_smem()
 {
+    constexpr int kp = kMaxn / 2;
     cudaError_t e = cudaSuccess;
 #define HS3D_ALLOW(FORM) \
     if (e == cudaSuccess) e = allow_smem(k_avol<T, NS, FORM>, sizeof(double) * avol_smem_per<FORM, NS>(kp) * T);
@@ -967,13 +967,26 @@ cudaError_t allow_avol_smem(int kp)
     return e;
 }
 
+// The stage kernels' shared-memory limits, for the largest degree whatever the
+// mesh's: a limit belongs to the function, so one set from a mesh's own degrees
+// would lower it under every live mesh of higher ones.  Once per device, at the
+// set-up of its first mesh with packs of T slots (not a stream operation, but
+// kept out of captured launches).
 template <int T>
-cudaError_t allow_stage_smem(const AnisoMesh *a)
+cudaError_t allow_stage_smem()
 {
-    const int kp = (a->Pmax + 1) / 2;
-    cudaError_t e = allow_avol_smem<T, false>(kp);
-    if (e == cudaSuccess) e = allow_avol_smem<T, true>(kp);
+    static std::mutex mu;
+    static std::vector<char> done;   // per device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    if ((int)done.size() <= dev) done.resize(dev + 1, 0);
+    if (done[dev]) return cudaSuccess;
+    e = allow_avol_smem<T, false>();
+    if (e == cudaSuccess) e = allow_avol_smem<T, true>();
     if (e == cudaSuccess) e = allow_smem(k_agrad<T>, sizeof(double) * kAGradSmemPer * T);
+    if (e == cudaSuccess) done[dev] = 1;
     return e;
 }
 
@@ -1224,7 +1237,7 @@ hs3d_status aniso_build(const hs3d_mesh_desc *desc, const int *degree3, AnisoMes
             return cudaGetLastError();
         });
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    if (e == cudaSuccess) e = a->T == 256 ? allow_stage_smem<256>(a) : allow_stage_smem<512>(a);
+    if (e == cudaSuccess) e = a->T == 256 ? allow_stage_smem<256>() : allow_stage_smem<512>();
     if (e != cudaSuccess) {
         cudaGetLastError();
         aniso_free(a);
