@@ -26,6 +26,7 @@ hs3d_status fail(hs3d_status st, const char *fmt, ...)
 
 hs3d_status cuda_fail(cudaError_t e, const char *what)
 {
+    cudaGetLastError();   // reported here: the next call's launch checks must not meet it again
     return fail(e == cudaErrorMemoryAllocation ? HS3D_ERR_NOMEM : HS3D_ERR_CUDA, "%s: %s (%s)", what,
                 cudaGetErrorString(e), cudaGetErrorName(e));
 }
