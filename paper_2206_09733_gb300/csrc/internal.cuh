@@ -336,6 +336,10 @@ inline int spread_elems(int epb, long long elems)
     return fit >= epb ? epb : fit < 1 ? 1 : (int)fit;
 }
 
+// Launches over at most this many elements (two per SM) take the N = 7 kernels
+// written for few elements (volume_dev.cuh, grad_dev.cu).
+constexpr long long kFewElems = 2 * kSMs;
+
 // CTA size for `total` independent threads: 256, or 64 while fewer than 256 per SM.
 inline int spread_threads(long long total) { return total < 256LL * kSMs ? 64 : 256; }
 

@@ -171,6 +171,22 @@ constexpr int dev_min_blocks()
     return (FORM == HS3D_VOL_STANDARD && (!NS || n3 > 125)) ? 5 : 4;
 }
 
+// The standard form at N = 7 without mortars has a kernel with four nodes per
+// thread (volume_row.cuh) beside this one, for launches over more than
+// kFewElems elements and persistent ones.  Up to two elements an SM, the four
+// warps of an element's CTA are too few to cover their own latencies, and one
+// thread per node is the faster: per launch 15.6 -> 12.8 us (150 elements,
+// Euler), 18.0 -> 15.3 (294), while at 343 it is 22.4 against the rows' 19.0;
+// a run of 4 steps, 150 elements, Euler 212 -> 175 us, NS 312 -> 266.  A solve
+// may run alone or in a larger batch, so the two kernels agree bit for bit: the
+// mass pairs are summed node by node here too, and the surface term is a
+// multiply-add.
+template <int N, int FORM>
+constexpr bool has_row_kernel()
+{
+    return is_standard(FORM) && N == 7;
+}
+
 // Viscous flux from the gradient kernel's values: stress and heat flux, or the
 // twelve gradients on the mortar path.
 template <bool MORT>
@@ -183,7 +199,8 @@ __device__ __forceinline__ void dev_visc(const Prim<float> &q, const float *G, c
 
 // One line of the float-float mass divergence, two nodes at a time (even and odd
 // ones summed apart); `first`: nothing summed before.  SEQ: node by node in
-// Ch.x + Cl.x (the mortar path, where the order of the sum is kept).
+// Ch.x + Cl.x (the mortar path and beside the row kernel, where the order of the
+// sum is kept).
 template <int n, bool SEQ>
 __device__ __forceinline__ void mass_line(bool first, const float *D, const float *Dl, const float *wh, const float *wl,
                                           int stride, float2 &Ch, float2 &Cl)
@@ -244,6 +261,8 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
     constexpr int VOFF = dev_visc_off<FORM, NS>(), WOFF = dev_mass_off<FORM, NS>();
     constexpr int KP = n / 2;
     constexpr int NG = MORT ? 12 : kVisc;
+    constexpr bool ROW = has_row_kernel<N, FORM>() && !MORT;   // (agrees with k_volume_row)
+    constexpr bool SEQ = MORT || ROW;
     constexpr bool BULK = (n % 2 == 0);
     constexpr int D2 = (n2 + 3) & ~3;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -484,7 +503,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
 #pragma unroll
                 for (int m = 0; m < n; ++m) add4(Drow[m], S4[d * n3 + base + m * stride]);
                 const float *wh = S + (WOFF + 2 * d) * n3 + base;
-                mass_line<n, MORT>(d == 0, Drow, Dlrow, wh, wh + n3, stride, Ch, Cl);
+                mass_line<n, SEQ>(d == 0, Drow, Dlrow, wh, wh + n3, stride, Ch, Cl);
             }
         }
     } else {
@@ -578,7 +597,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                         if (NS) add4(Drow[m], S4[(VOFF / 4 + d) * n3 + base + m * sd]);
                     if constexpr (EC) {
                         const float *wh = S + (WOFF + 2 * d) * n3 + base;
-                        mass_line<n, MORT>(d == 0, Drow, Dlrow, wh, wh + n3, sd, Ch, Cl);
+                        mass_line<n, SEQ>(d == 0, Drow, Dlrow, wh, wh + n3, sd, Ch, Cl);
                     }
                 }
                 continue;
@@ -666,7 +685,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
                 }
                 if constexpr (EC) {
                     const float *wh = S + (WOFF + 2 * d) * n3 + base;
-                    mass_line<n, MORT>(d == 0, Drow, Dlrow, wh, wh + n3, sd, Ch, Cl);
+                    mass_line<n, SEQ>(d == 0, Drow, Dlrow, wh, wh + n3, sd, Ch, Cl);
                 }
             }
             // (after the last direction the pair buffer is not written again)
@@ -704,7 +723,7 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
     // volume rows: mass = C (+ the split form's remainder), energy = Hbar mass + rest
     float Vr = V[0];
     if constexpr (LM) {
-        if constexpr (MORT) {
+        if constexpr (SEQ) {
             Vr = (Ch.x + Cl.x) + V[0];
         } else {
             float c, ce;
@@ -766,6 +785,10 @@ __device__ __forceinline__ bool volume_dev_tile(const Batch &b, const Ops *__res
         if constexpr (MORT) {
 #pragma unroll
             for (int v = 0; v < 5; ++v) V[v] += plus ? iw * (F[v * n2] - own[d][v]) : iw * (own[d][v] - F[v * n2]);
+        } else if constexpr (ROW) {
+            const float sw = plus ? iw : -iw;
+#pragma unroll
+            for (int v = 0; v < 5; ++v) V[v] += sw * F[v * n2];
         } else {
 #pragma unroll
             for (int v = 0; v < 5; ++v) V[v] += plus ? iw * F[v * n2] : -iw * F[v * n2];
@@ -872,12 +895,6 @@ k_volume_dev(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int s
 
 // ------------------------------------------------------------------ launch (one volume form)
 
-// The standard form at N = 7 without mortars has its own kernel (volume_row.cuh).
-template <int N, int FORM>
-constexpr bool has_row_kernel()
-{
-    return is_standard(FORM) && N == 7;
-}
 template <int N, bool NS>
 static cudaError_t vol_row_launch(const Batch &b, int stage, float rkA, double rkB, int lam_slot, cudaStream_t s);
 template <int N>
@@ -887,7 +904,8 @@ template <int N, bool NS, int FORM>
 static cudaError_t vol_dev_launch2(const Batch &b, int stage, float rkA, double rkB, int lam_slot, cudaStream_t s)
 {
     if constexpr (has_row_kernel<N, FORM>()) {
-        if (!b.mortar) return vol_row_launch<N, NS>(b, stage, rkA, rkB, lam_slot, s);
+        if (!b.mortar && (b.persistent || b.total_elems > kFewElems))
+            return vol_row_launch<N, NS>(b, stage, rkA, rkB, lam_slot, s);
     }
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
     int epb = spread_elems(elems_per_block_p(N, HS3D_MIXED32, 1, (is_standard(FORM) || FORM == HS3D_VOL_EC) ? kSmallCta : 256), b.total_elems);
@@ -901,17 +919,15 @@ static cudaError_t vol_dev_launch2(const Batch &b, int stage, float rkA, double 
     if (b.mortar)
         return launch_pdl(k_volume_dev<N, NS, FORM, false, true>, blocks, threads, smem, s, b, ops, stage, rkA, rkB,
                           stage >= 0 ? lam_slot : -1, epb, (long long)blocks);
-    if constexpr (has_row_kernel<N, FORM>()) {
-        return cudaErrorInvalidValue;   // (taken above)
-    } else {
+    if constexpr (!has_row_kernel<N, FORM>()) {
         if (b.persistent) {
             const unsigned grid = persistent_grid(k_volume_dev<N, NS, FORM, true>, threads, smem, blocks);
             return launch_pdl(k_volume_dev<N, NS, FORM, true>, grid, threads, smem, s, b, ops, stage, rkA, rkB,
                               stage >= 0 ? lam_slot : -1, epb, (long long)blocks);
         }
-        return launch_pdl(k_volume_dev<N, NS, FORM, false>, blocks, threads, smem, s, b, ops, stage, rkA, rkB,
-                          stage >= 0 ? lam_slot : -1, epb, (long long)blocks);
     }
+    return launch_pdl(k_volume_dev<N, NS, FORM, false>, blocks, threads, smem, s, b, ops, stage, rkA, rkB,
+                      stage >= 0 ? lam_slot : -1, epb, (long long)blocks);
 }
 
 template <int FORM>
@@ -942,12 +958,11 @@ static cudaError_t prep_vol_dev_kernel(K kernel)
 template <int N, int FORM>
 static cudaError_t prep_vol_dev_n()
 {
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = prep_vol_dev_kernel(k_volume_dev<N, false, FORM, false>);
+    if (e == cudaSuccess) e = prep_vol_dev_kernel(k_volume_dev<N, true, FORM, false>);
     if constexpr (has_row_kernel<N, FORM>()) {
-        e = vol_row_prep<N>();
+        if (e == cudaSuccess) e = vol_row_prep<N>();
     } else {
-        e = prep_vol_dev_kernel(k_volume_dev<N, false, FORM, false>);
-        if (e == cudaSuccess) e = prep_vol_dev_kernel(k_volume_dev<N, true, FORM, false>);
         if (e == cudaSuccess) e = prep_vol_dev_kernel(k_volume_dev<N, false, FORM, true>);
         if (e == cudaSuccess) e = prep_vol_dev_kernel(k_volume_dev<N, true, FORM, true>);
     }
