@@ -895,6 +895,17 @@ k_volume_dev(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int s
 
 // ------------------------------------------------------------------ launch (one volume form)
 
+// CTA size aimed at (untuned): kSmallCta for the standard and Chandrashekar forms,
+// 256 for the others.  The Chandrashekar form at N = 2 fills 108 of 128 lanes but
+// 243 of 256: from 80 elements per SM on, where the finer grid no longer pays for
+// that, it takes 256 (Euler, 4 steps: 11,000 elements 649 us against 677,
+// 15,000 916 against 876, 150,000 7430 against 7361).
+template <int N, int FORM>
+inline int dev_cta_target(long long elems)
+{
+    if (FORM == HS3D_VOL_EC && N == 2 && elems > 80LL * kSMs) return 256;
+    return (is_standard(FORM) || FORM == HS3D_VOL_EC) ? kSmallCta : 256;
+}
 template <int N, bool NS>
 static cudaError_t vol_row_launch(const Batch &b, int stage, float rkA, double rkB, int lam_slot, cudaStream_t s);
 template <int N>
@@ -908,7 +919,7 @@ static cudaError_t vol_dev_launch2(const Batch &b, int stage, float rkA, double 
             return vol_row_launch<N, NS>(b, stage, rkA, rkB, lam_slot, s);
     }
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
-    int epb = spread_elems(elems_per_block_p(N, HS3D_MIXED32, 1, (is_standard(FORM) || FORM == HS3D_VOL_EC) ? kSmallCta : 256), b.total_elems);
+    int epb = spread_elems(elems_per_block_p(N, HS3D_MIXED32, 1, dev_cta_target<N, FORM>(b.total_elems)), b.total_elems);
     if (epb * n3 > dev_threads<N, FORM>()) epb = dev_threads<N, FORM>() / n3;
     if (epb < 1) epb = 1;
     const int threads = ((epb * n3) + 31) & ~31;
