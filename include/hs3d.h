@@ -269,14 +269,18 @@ hs3d_status hs3d_diagnostics(const hs3d_mesh *mesh, const hs3d_solver_cfg *cfg, 
 hs3d_status hs3d_diagnostics_noalloc(int N, int64_t E, double gamma, int nodes, const double *J, const double *u,
                                      const double *dudt, double *out, void *stream);
 
-/* Autotuner: times every admissible launch shape (elements per CTA) of the
- * BR1-gradient and element kernels for this mesh and configuration on a
- * scratch state, keeps the fastest for (N, precision, kernel) for the rest of
- * the process, and writes the choices to the JSON file named by the
- * environment variable HS3D_TUNE_CACHE if set (read back at the next mesh
- * creation).  choice_out (HOST, 2 ints, may be NULL) receives [gradient,
- * element] elements per CTA.  Synchronous; allocates two scratch states.
- * Call it outside any stream capture. */
+/* Autotuner: times the launch shapes (elements per CTA) of the BR1-gradient
+ * and element kernels for this mesh and configuration on a scratch state, keeps
+ * the fastest for (N, precision, kernel; the element kernel of the standard and
+ * Chandrashekar forms and that of the other split forms apart) for the rest of
+ * the process, and writes the choices to the JSON file named by the environment
+ * variable HS3D_TUNE_CACHE if set (read back at the next mesh creation).  A mesh
+ * too small for its shapes to differ (its elements are spread over the GPU) has
+ * them timed on a larger scratch mesh of its degree (about 0.1 GB; without the
+ * memory nothing is timed and the choices stay as they were).
+ * choice_out (HOST, 2 ints, may be NULL) receives [gradient, element]: the
+ * elements per CTA of this mesh's launches.  Synchronous; allocates two scratch
+ * states.  Call it outside any stream capture. */
 hs3d_status hs3d_autotune(const hs3d_mesh *mesh, const hs3d_solver_cfg *cfg, int *choice_out, void *stream);
 
 /* ---------------------------------------------------------------- per-element degree (Sec. 3.6) */

@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(kFaceThreads) k_face(const __grid_constant__ B
 template <int N>
 constexpr int grad_threads()
 {
-    return ((N + 1) * (N + 1) * (N + 1) > 256) ? (N + 1) * (N + 1) * (N + 1) : 256;
+    return max_cta_threads(N, HS3D_FP64, kShapeGrad, HS3D_VOL_STANDARD, false);
 }
 
 // (v, T) of a conserved state.
@@ -296,8 +296,7 @@ static cudaError_t grad_launch(const Batch &b, cudaStream_t s)
 {
     constexpr int n = N + 1, n3 = n * n * n;
     if (b.total_elems == 0) return cudaSuccess;
-    int epb = spread_elems(elems_per_block_p(N, HS3D_FP64, 0), b.total_elems);
-    if (epb * n3 > grad_threads<N>()) epb = grad_threads<N>() / n3;
+    const int epb = elems_per_cta(N, HS3D_FP64, kShapeGrad, HS3D_VOL_STANDARD, false, b.total_elems);
     int threads = epb * n3;
     size_t smem = sizeof(double) * (((n * n + 1) & ~1) + (size_t)epb * grad_per_elem<N>());
     unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);

@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(256) k_face_gauss(const __grid_constant__ Batc
 template <int N>
 constexpr int gauss_threads()
 {
-    return ((N + 1) * (N + 1) * (N + 1) > 256) ? (N + 1) * (N + 1) * (N + 1) : 256;
+    return max_cta_threads(N, HS3D_FP64, kShapeElem, HS3D_VOL_STANDARD, true);
 }
 
 template <int N>
@@ -496,21 +496,13 @@ static cudaError_t face_gauss(int physics, int flux, const Batch &b, cudaStream_
     return cudaGetLastError();
 }
 
-template <int N>
-static int gauss_epb(int prec, int which, long long elems)
-{
-    constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
-    int epb = spread_elems(elems_per_block_p(N, prec, which, kSmallCta), elems);
-    if (epb * n3 > gauss_threads<N>()) epb = gauss_threads<N>() / n3;
-    return epb < 1 ? 1 : epb;
-}
-
 template <int N, typename R>
 static cudaError_t grad_gauss(const Batch &b, cudaStream_t s)
 {
     constexpr int n = N + 1, n3 = n * n * n;
     if (b.total_elems == 0) return cudaSuccess;
-    const int epb = gauss_epb<N>(sizeof(R) == 4 ? HS3D_MIXED32 : HS3D_FP64, 0, b.total_elems);
+    const int epb = elems_per_cta(N, sizeof(R) == 4 ? HS3D_MIXED32 : HS3D_FP64, kShapeGrad, HS3D_VOL_STANDARD, true,
+                                  b.total_elems);
     const size_t smem = sizeof(R) * (((n * n + 3) & ~3) + (size_t)epb * grad_gauss_per_elem<N>());
     const unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);
     const Ops *ops = device_ops(N, HS3D_NODES_GAUSS);
@@ -524,7 +516,8 @@ static cudaError_t volume_gauss(const Batch &b, int stage, double rkA, double rk
 {
     constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
     if (b.total_elems == 0) return cudaSuccess;
-    const int epb = gauss_epb<N>(sizeof(R) == 4 ? HS3D_MIXED32 : HS3D_FP64, 1, b.total_elems);
+    const int epb = elems_per_cta(N, sizeof(R) == 4 ? HS3D_MIXED32 : HS3D_FP64, kShapeElem, HS3D_VOL_STANDARD, true,
+                                  b.total_elems);
     const size_t smem = sizeof(R) * (((n * n + 3) & ~3) + (size_t)epb * (((15 * n3 + 3) & ~3) + 30 * n2));
     const unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);
     const Ops *ops = device_ops(N, HS3D_NODES_GAUSS);

@@ -26,7 +26,7 @@ namespace hs3d {
 template <int N>
 constexpr int grad_dev_threads()
 {
-    return ((N + 1) * (N + 1) * (N + 1) > 256) ? (N + 1) * (N + 1) * (N + 1) : 256;
+    return max_cta_threads(N, HS3D_MIXED32, kShapeGrad, HS3D_VOL_STANDARD, false);
 }
 
 // Shared-memory floats per element: q' [n3] and neighbour-trace deviations [6][n2]
@@ -548,8 +548,7 @@ static cudaError_t grad_dev_launch(const Batch &b, cudaStream_t s)
             return e != cudaSuccess ? e : cudaGetLastError();
         }
     }
-    int epb = spread_elems(elems_per_block_p(N, HS3D_MIXED32, 0), b.total_elems);
-    if (epb * n3 > grad_dev_threads<N>()) epb = grad_dev_threads<N>() / n3;
+    const int epb = elems_per_cta(N, HS3D_MIXED32, kShapeGrad, HS3D_VOL_STANDARD, false, b.total_elems);
     const int threads = epb * n3;
     const size_t smem = sizeof(float) * (((n * n + 3) & ~3) + (size_t)epb * grad_dev_per_elem<N>());
     const unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);

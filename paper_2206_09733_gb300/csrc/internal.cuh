@@ -557,19 +557,54 @@ cudaError_t prepare_kernels(int N);
 cudaError_t prepare_volume(int N);
 cudaError_t prepare_grad(int N);
 
-// Elements per block for the element kernels (threads = epb * n^3), per
-// (N, precision 0 = FP64 / 1 = mixed, kernel: 0 = BR1 gradient, 1 = volume);
-// the autotuner's choice if one was made, else `threads` threads' worth.
-int elems_per_block_p(int N, int prec, int which, int threads = 256);
+// Launch shapes of the BR1-gradient and element kernels: epb elements per CTA,
+// threads = epb * n^3 (rounded up to warps in the mixed element kernel).
+enum ShapeKernel { kShapeGrad, kShapeElem };
+// Threads of the largest CTA a kernel is compiled for (one element where that is
+// more): 128 for the mixed Chandrashekar form at N = 3 and 4 (dev_min_blocks), one
+// element (216 threads, seven warps) at N = 5 of the mixed element kernel, else 256.
+constexpr int max_cta_threads(int N, int prec, ShapeKernel k, int form, bool gauss)
+{
+    const int n3 = (N + 1) * (N + 1) * (N + 1);
+    if (prec != HS3D_FP64 && k == kShapeElem && !gauss) {
+        if (form == HS3D_VOL_EC && (N == 3 || N == 4)) return 128;
+        if (N == 5) return 224;
+    }
+    return n3 > 256 ? n3 : 256;
+}
 // CTA size of the kernels whose warps spend their time at barriers or on loads:
 // as many warps are resident as with 256 threads, but a barrier or a late load
 // stalls half as many at once.  Measured, 256 -> 128: FP64 element kernel (EC,
 // 16^3, N = 3) -8% per step; standard form, mixed: 64^3 N = 3 14.71 -> 13.74 ms,
 // 53x52x51 N = 4 17.95 -> 16.93; Gauss-Legendre 32^3 N = 3 4.76 -> 4.47; mixed
-// Chandrashekar form 24^3 N = 4 -1%.  The BR1 gradients of Lobatto meshes do not gain.
+// Chandrashekar form 24^3 N = 4 -1%.  The BR1 gradients of Lobatto meshes and the
+// other mixed split forms do not gain.
 constexpr int kSmallCta = 128;
-int tuned_elems_per_block(int N, int prec, int which);   // 0 if untuned
-void set_elems_per_block_p(int N, int prec, int which, int epb);
+// CTA size aimed at when untuned.  The mixed Chandrashekar form at N = 2 fills 108
+// of 128 lanes but 243 of 256: from 80 elements per SM on, where the finer grid no
+// longer pays for that, it takes 256 (Euler, 4 steps: 11,000 elements 649 us against
+// 677, 15,000 916 against 876, 150,000 7430 against 7361).
+constexpr int cta_target(int N, int prec, ShapeKernel k, int form, bool gauss, long long elems)
+{
+    if (gauss) return kSmallCta;
+    if (k == kShapeGrad) return 256;
+    if (prec == HS3D_FP64 || is_standard(form)) return kSmallCta;
+    if (form == HS3D_VOL_EC) return N == 2 && elems > 80LL * kSMs ? 256 : kSmallCta;
+    return 256;
+}
+// Elements per CTA of a launch over `elems` elements: the autotuner's choice if one
+// was made, else cta_target's, within the largest CTA, spread over the SMs.
+int elems_per_cta(int N, int prec, ShapeKernel k, int form, bool gauss, long long elems);
+// The tuned choices, by degree, precision (FP64 / mixed) and slot: the gradient
+// kernel, the element kernel of the standard and Chandrashekar forms, that of the
+// other split forms (their best shapes differ).  0: none.
+constexpr int kShapeSlots = 3;
+constexpr int shape_slot(ShapeKernel k, int form)
+{
+    return k == kShapeGrad ? 0 : is_standard(form) || form == HS3D_VOL_EC ? 1 : 2;
+}
+int tuned_elems(int N, int prec, int slot);
+void set_tuned_elems(int N, int prec, int slot, int epb);
 void tune_cache_load();
 
 }  // namespace hs3d

@@ -1,20 +1,29 @@
 // Autotuner for the element kernels' launch shape.
 //
 // The BR1-gradient and element (volume) kernels run one thread per node with
-// `epb` elements per CTA.  hs3d_autotune times every admissible epb (the CTA
-// must stay within the kernel's thread bound and shared-memory limit) for
-// the given mesh and configuration on scratch copies of a smooth state (the
-// element kernel as a middle RK stage, with its own clock and a tiny dt, so
-// that the timed launches move the bytes of a real step), and keeps the
-// fastest per (N, precision, kernel).  Choices
-// persist across processes in a small JSON file when HS3D_TUNE_CACHE names
+// `epb` elements per CTA.  hs3d_autotune times every epb that gives a launch of
+// its own (up to the kernel's largest CTA, max_cta_threads) on scratch copies of a
+// smooth state (the element kernel as a middle RK stage, with its own clock and a
+// tiny dt, so that the timed launches move the bytes of a real step), and keeps
+// the fastest per (N, precision, kernel slot): the default, unless another is
+// faster by more than kMargin.
+// A mesh of fewer than kSMs elements per element of the largest CTA is spread over
+// the SMs whatever epb is (spread_elems): there every epb would be the same launch
+// and the choice noise, so the shapes are timed on a cube of the same degree that
+// is large enough; the choice is for such meshes, and a small mesh's launches
+// stay spread.
+// Choices persist across processes in a small JSON file when HS3D_TUNE_CACHE names
 // one: it is read on first use and rewritten after each tuning.
+#include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
+#include <cmath>
 #include <mutex>
 #include <string>
+#include <vector>
 
 #include "api_internal.h"
 
@@ -29,7 +38,7 @@ static std::string cache_path()
     return p ? std::string(p) : std::string();
 }
 
-// Cache format: {"N<N>_p<prec>_k<which>": epb, ...}
+// Cache format: {"N<N>_p<prec>_k<slot>": epb, ...} (shape_slot)
 static void load_cache_locked()
 {
     if (g_cache_loaded) return;
@@ -44,10 +53,10 @@ static void load_cache_locked()
     buf[len] = 0;
     const char *s = buf;
     while ((s = strchr(s, '"')) != nullptr) {
-        int N = 0, prec = 0, which = 0, epb = 0;
-        if (sscanf(s, "\"N%d_p%d_k%d\": %d", &N, &prec, &which, &epb) == 4 && N >= 1 && N <= kMaxN && epb >= 1 &&
-            epb <= 64 && prec >= 0 && prec <= 2 && (which == 0 || which == 1))
-            set_elems_per_block_p(N, prec, which, epb);
+        int N = 0, prec = 0, slot = 0, epb = 0;
+        if (sscanf(s, "\"N%d_p%d_k%d\": %d", &N, &prec, &slot, &epb) == 4 && N >= 1 && N <= kMaxN && epb >= 1 &&
+            epb <= 64 && prec >= 0 && prec <= 2 && slot >= 0 && slot < kShapeSlots)
+            set_tuned_elems(N, prec, slot, epb);
         s = strchr(s + 1, '"');
         if (s) ++s;
     }
@@ -64,10 +73,10 @@ static void save_cache_locked()
     bool first = true;
     for (int N = 1; N <= kMaxN; ++N)
         for (int prec = 0; prec < 2; ++prec)
-            for (int which = 0; which < 2; ++which) {
-                int v = tuned_elems_per_block(N, prec, which);
+            for (int slot = 0; slot < kShapeSlots; ++slot) {
+                int v = tuned_elems(N, prec, slot);
                 if (v <= 0) continue;
-                fprintf(f, "%s\"N%d_p%d_k%d\": %d", first ? "" : ", ", N, prec, which, v);
+                fprintf(f, "%s\"N%d_p%d_k%d\": %d", first ? "" : ", ", N, prec, slot, v);
                 first = false;
             }
     fprintf(f, "}\n");
@@ -81,46 +90,41 @@ void tune_cache_load()
     load_cache_locked();
 }
 
-// Time `reps` launches of the gradient kernel, or of the element kernel as
-// RK stage 1 (reads and writes u and g), with a given epb.
-static float time_kernels(hs3d_mesh *m, const hs3d_solver_cfg *c, const Batch &b, int which, int reps, cudaStream_t s,
-                          cudaError_t &err)
+// Time per launch (the least of three runs of `reps`) of the gradient kernel, or
+// of the element kernel as RK stage 1 (reads and writes u and g).
+static float time_kernels(const hs3d_mesh *m, const hs3d_solver_cfg *c, const Batch &b, ShapeKernel k, int reps,
+                          cudaStream_t s, cudaError_t &err)
 {
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    err = cudaSuccess;
-    // one untimed launch (also surfaces launch errors for this shape)
-    if (which == 0) err = launch_grad(m->N, c->precision, b, s);
-    else err = launch_volume(m->N, c->precision, c->physics, c->volume_form, c->time_scheme, b, 1, -1, s);
-    if (err == cudaSuccess) err = cudaEventRecord(e0, s);
-    for (int r = 0; r < reps && err == cudaSuccess; ++r) {
-        if (which == 0) err = launch_grad(m->N, c->precision, b, s);
-        else err = launch_volume(m->N, c->precision, c->physics, c->volume_form, c->time_scheme, b, 1, -1, s);
+    auto launch = [&] {
+        return k == kShapeGrad ? launch_grad(m->N, c->precision, b, s)
+                               : launch_volume(m->N, c->precision, c->physics, c->volume_form, c->time_scheme, b, 1, -1, s);
+    };
+    err = launch();   // untimed (also surfaces launch errors for this shape)
+    float best = 1e30f;
+    for (int run = 0; run < 3 && err == cudaSuccess; ++run) {
+        err = cudaEventRecord(e0, s);
+        for (int r = 0; r < reps && err == cudaSuccess; ++r) err = launch();
+        if (err == cudaSuccess) err = cudaEventRecord(e1, s);
+        if (err == cudaSuccess) err = cudaEventSynchronize(e1);
+        float ms = 0.f;
+        if (err == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
+        best = ms < best ? ms : best;
     }
-    if (err == cudaSuccess) err = cudaEventRecord(e1, s);
-    if (err == cudaSuccess) err = cudaEventSynchronize(e1);
-    float ms = 0.f;
-    if (err == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    return ms / reps;
+    return best / reps;
 }
 
-}  // namespace hs3d
+// A shape replaces the default only where it is faster by more than this (the runs
+// of one shape differ by about 1%).
+constexpr float kMargin = 0.98f;
 
-using namespace hs3d;
-
-extern "C" hs3d_status hs3d_autotune(const hs3d_mesh *mc, const hs3d_solver_cfg *c, int *choice_out, void *stream)
+// Time the shapes of cfg's kernels on mesh m and set the choices.
+static hs3d_status tune_on(hs3d_mesh *m, const hs3d_solver_cfg *c, cudaStream_t s)
 {
-    hs3d_mesh *m = const_cast<hs3d_mesh *>(mc);
-    if (!m) return fail(HS3D_ERR_INVALID, "mesh is NULL");
-    hs3d_status st = validate_cfg(c);
-    if (st == HS3D_OK) st = check_mesh_cfg(m, c);
-    if (st != HS3D_OK) return st;
-    std::lock_guard<std::mutex> lock(g_tune_mu);
-    load_cache_locked();
-    cudaStream_t s = (cudaStream_t)stream;
     size_t sz = sizeof(double) * (size_t)m->E * 5 * m->n3;
     double *u = nullptr, *g = nullptr;
     Clock *clk = nullptr;
@@ -149,41 +153,91 @@ extern "C" hs3d_status hs3d_autotune(const hs3d_mesh *mc, const hs3d_solver_cfg 
     if (e == cudaSuccess && c->precision != HS3D_FP64) e = launch_shadow(m->N, b, s);
     if (e == cudaSuccess && c->physics == HS3D_NS) e = launch_grad(m->N, c->precision, b, s);
     if (e == cudaSuccess) e = launch_face(m->N, c->precision, c->physics, c->surface_flux, b, s);
-    int best[2] = {0, 0};
     const int n3 = m->n3;
-    const int maxthreads = n3 > 256 ? n3 : 256;
+    const bool gauss = m->nodes == HS3D_NODES_GAUSS;
     const int reps = m->E >= 4096 ? 5 : 20;
-    for (int which = 0; which < 2 && e == cudaSuccess; ++which) {
-        if (which == 0 && c->physics != HS3D_NS) continue;
-        float best_ms = 1e30f;
-        const int keep = tuned_elems_per_block(m->N, c->precision, which);
-        for (int epb = 1; epb * n3 <= maxthreads && e == cudaSuccess; epb *= 2) {
-            set_elems_per_block_p(m->N, c->precision, which, epb);
-            float ms = time_kernels(m, c, b, which, reps, s, e);
-            if (e != cudaSuccess) {
+    for (const ShapeKernel k : {kShapeGrad, kShapeElem}) {
+        if (e != cudaSuccess || (k == kShapeGrad && c->physics != HS3D_NS)) continue;
+        const int slot = shape_slot(k, c->volume_form), keep = tuned_elems(m->N, c->precision, slot);
+        const int most = max_cta_threads(m->N, c->precision, k, c->volume_form, gauss) / n3;
+        int deflt = cta_target(m->N, c->precision, k, c->volume_form, gauss, m->E) / n3;
+        deflt = deflt < 1 ? 1 : deflt > most ? most : deflt;
+        std::vector<int> shapes;   // the default first, then the powers of two; one shape only: nothing to time
+        if (most > 1) {
+            shapes.push_back(deflt);
+            for (int t = 1; t <= most; t *= 2)
+                if (t != deflt) shapes.push_back(t);
+        }
+        int best = most > 1 ? 0 : 1;
+        float best_ms = 0.f;
+        for (const int t : shapes) {
+            set_tuned_elems(m->N, c->precision, slot, t);
+            const float ms = time_kernels(m, c, b, k, reps, s, e);
+            if (e == cudaErrorInvalidValue || e == cudaErrorInvalidConfiguration) {
                 // a shape the device cannot launch (shared memory): not a candidate
-                if (e == cudaErrorInvalidValue || e == cudaErrorInvalidConfiguration) {
-                    cudaGetLastError();
-                    e = cudaSuccess;
-                }
-                continue;
-            }
-            if (ms < best_ms) {
+                cudaGetLastError();
+                e = cudaSuccess;
+            } else if (e != cudaSuccess) {
+                break;
+            } else if (best == 0 || ms < best_ms * (best == deflt ? kMargin : 1.0f)) {
                 best_ms = ms;
-                best[which] = epb;
+                best = t;
             }
         }
-        set_elems_per_block_p(m->N, c->precision, which, best[which] ? best[which] : keep);
+        set_tuned_elems(m->N, c->precision, slot, best ? best : keep);
     }
     cudaStreamSynchronize(s);
     cudaFree(u);
     cudaFree(g);
     cudaFree(clk);
-    if (e != cudaSuccess) return cuda_fail(e, "autotune");
-    save_cache_locked();
+    return e == cudaSuccess ? HS3D_OK : cuda_fail(e, "autotune");
+}
+
+}  // namespace hs3d
+
+using namespace hs3d;
+
+extern "C" hs3d_status hs3d_autotune(const hs3d_mesh *mc, const hs3d_solver_cfg *c, int *choice_out, void *stream)
+{
+    hs3d_mesh *m = const_cast<hs3d_mesh *>(mc);
+    if (!m) return fail(HS3D_ERR_INVALID, "mesh is NULL");
+    hs3d_status st = validate_cfg(c);
+    if (st == HS3D_OK) st = check_mesh_cfg(m, c);
+    if (st != HS3D_OK) return st;
+    const bool gauss = m->nodes == HS3D_NODES_GAUSS;
+    int most = max_cta_threads(m->N, c->precision, kShapeElem, c->volume_form, gauss);
+    if (c->physics == HS3D_NS) most = std::max(most, max_cta_threads(m->N, c->precision, kShapeGrad, c->volume_form, gauss));
+    most /= m->n3;
+    hs3d_mesh *big = nullptr;
+    if (most > 1 && m->E < (long long)kSMs * most) {
+        // a cube of the same degree with four of the largest CTAs per SM (built before
+        // the lock is taken: creating a mesh reads the cache under it)
+        hs3d_mesh_desc d{};
+        d.N = m->N;
+        d.nodes = m->nodes;
+        d.perturb_amp = 0.05;
+        for (int k = 0; k < 3; ++k) {
+            d.lo[k] = -M_PI;
+            d.hi[k] = M_PI;
+            d.periodic[k] = 1;
+        }
+        d.ex = d.ey = d.ez = (int)std::ceil(std::cbrt(4.0 * kSMs * most));
+        st = mesh_build(&d, &big);
+    }
+    {
+        std::lock_guard<std::mutex> lock(g_tune_mu);
+        load_cache_locked();
+        if (st == HS3D_OK) st = tune_on(big ? big : m, c, (cudaStream_t)stream);
+        if (st == HS3D_OK) save_cache_locked();
+    }
+    // no memory for the larger mesh: nothing is timed, the choices stay as they were
+    if (st == HS3D_ERR_NOMEM && most > 1 && m->E < (long long)kSMs * most) st = HS3D_OK;
+    mesh_free(big);
+    if (st != HS3D_OK) return st;
     if (choice_out) {
-        choice_out[0] = elems_per_block_p(m->N, c->precision, 0);
-        choice_out[1] = elems_per_block_p(m->N, c->precision, 1);
+        // what this mesh's launches use
+        choice_out[0] = elems_per_cta(m->N, c->precision, kShapeGrad, c->volume_form, gauss, m->E);
+        choice_out[1] = elems_per_cta(m->N, c->precision, kShapeElem, c->volume_form, gauss, m->E);
     }
     return HS3D_OK;
 }

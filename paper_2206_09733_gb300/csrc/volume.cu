@@ -37,24 +37,25 @@ void rk_coeffs(int scheme, int k, double *A, double *B)
     *B = four ? kRK4B[k] : kRK3B[k];
 }
 
-// Tuned elements per CTA by (N, precision FP64 / mixed, kernel).
-static int g_epb[kMaxn + 1][2][2] = {};
+// Tuned elements per CTA by (N, precision FP64 / mixed, slot).
+static int g_epb[kMaxn + 1][2][kShapeSlots] = {};
 
 // (HS3D_MIXED_TC runs the MIXED32 kernels and shares their slot)
 static int prec_slot(int prec) { return prec == HS3D_FP64 ? 0 : 1; }
 
-int tuned_elems_per_block(int N, int prec, int which) { return g_epb[N][prec_slot(prec)][which]; }
+int tuned_elems(int N, int prec, int slot) { return g_epb[N][prec_slot(prec)][slot]; }
 
-int elems_per_block_p(int N, int prec, int which, int threads)
+void set_tuned_elems(int N, int prec, int slot, int epb) { g_epb[N][prec_slot(prec)][slot] = epb; }
+
+int elems_per_cta(int N, int prec, ShapeKernel k, int form, bool gauss, long long elems)
 {
-    const int v = g_epb[N][prec_slot(prec)][which];
-    if (v > 0) return v;
     const int n3 = (N + 1) * (N + 1) * (N + 1);
-    const int e = threads / n3;
-    return e < 1 ? 1 : e;
+    const int most = max_cta_threads(N, prec, k, form, gauss) / n3;
+    int epb = tuned_elems(N, prec, shape_slot(k, form));
+    if (epb <= 0) epb = cta_target(N, prec, k, form, gauss, elems) / n3;
+    if (epb > most) epb = most;
+    return spread_elems(epb < 1 ? 1 : epb, elems);
 }
-
-void set_elems_per_block_p(int N, int prec, int which, int epb) { g_epb[N][prec_slot(prec)][which] = epb; }
 
 cudaError_t prepare_volume(int N)
 {

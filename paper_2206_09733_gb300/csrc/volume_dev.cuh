@@ -45,16 +45,11 @@ constexpr bool dev_lowmach()
     return FORM == HS3D_VOL_STANDARD || FORM == HS3D_VOL_EC;
 }
 
-// Largest CTA: 128 threads for the Chandrashekar form at N = 3 and 4
-// (dev_min_blocks), one element (216 threads, seven warps) at N = 5 and where an
-// element has more than 256 nodes, else 256.
+// Largest CTA, in whole warps.
 template <int N, int FORM>
 constexpr int dev_threads()
 {
-    if (FORM == HS3D_VOL_EC && (N == 3 || N == 4)) return 128;
-    if (N == 5) return 224;
-    constexpr int t = ((N + 1) * (N + 1) * (N + 1) > 256) ? (N + 1) * (N + 1) * (N + 1) : 256;
-    return (t + 31) & ~31;
+    return (max_cta_threads(N, HS3D_MIXED32, kShapeElem, FORM, false) + 31) & ~31;
 }
 
 // Staged floats per node, in groups of four that one 16-byte load brings (the
@@ -898,17 +893,6 @@ k_volume_dev(const __grid_constant__ Batch b, const Ops *__restrict__ ops, int s
 
 // ------------------------------------------------------------------ launch (one volume form)
 
-// CTA size aimed at (untuned): kSmallCta for the standard and Chandrashekar forms,
-// 256 for the others.  The Chandrashekar form at N = 2 fills 108 of 128 lanes but
-// 243 of 256: from 80 elements per SM on, where the finer grid no longer pays for
-// that, it takes 256 (Euler, 4 steps: 11,000 elements 649 us against 677,
-// 15,000 916 against 876, 150,000 7430 against 7361).
-template <int N, int FORM>
-inline int dev_cta_target(long long elems)
-{
-    if (FORM == HS3D_VOL_EC && N == 2 && elems > 80LL * kSMs) return 256;
-    return (is_standard(FORM) || FORM == HS3D_VOL_EC) ? kSmallCta : 256;
-}
 template <int N, bool NS>
 static cudaError_t vol_row_launch(const Batch &b, int stage, float rkA, double rkB, int lam_slot, cudaStream_t s);
 template <int N>
@@ -922,9 +906,7 @@ static cudaError_t vol_dev_launch2(const Batch &b, int stage, float rkA, double 
             return vol_row_launch<N, NS>(b, stage, rkA, rkB, lam_slot, s);
     }
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
-    int epb = spread_elems(elems_per_block_p(N, HS3D_MIXED32, 1, dev_cta_target<N, FORM>(b.total_elems)), b.total_elems);
-    if (epb * n3 > dev_threads<N, FORM>()) epb = dev_threads<N, FORM>() / n3;
-    if (epb < 1) epb = 1;
+    const int epb = elems_per_cta(N, HS3D_MIXED32, kShapeElem, FORM, false, b.total_elems);
     const int threads = ((epb * n3) + 31) & ~31;
     const size_t smem = dev_smem_bytes<N, NS, FORM>(epb);
     const unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);

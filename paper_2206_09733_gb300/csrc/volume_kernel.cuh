@@ -45,13 +45,11 @@
 namespace hs3d {
 
 // Largest CTA of the element kernel: 256 threads, or one element when it has
-// more nodes, rounded up to whole warps (the tensor-core contraction needs
-// complete warps; threads beyond the CTA's elements only join it).
+// more nodes, in whole warps.
 template <int N>
 constexpr int vol_threads()
 {
-    constexpr int t = ((N + 1) * (N + 1) * (N + 1) > 256) ? (N + 1) * (N + 1) * (N + 1) : 256;
-    return (t + 31) & ~31;
+    return (max_cta_threads(N, HS3D_FP64, kShapeElem, HS3D_VOL_STANDARD, false) + 31) & ~31;
 }
 
 // Minimum resident CTAs per SM asked of the compiler: the mixed path is
@@ -431,12 +429,8 @@ template <int N, bool NS, int FORM>
 static cudaError_t vol_launch2(const Batch &b, int stage, double rkA, double rkB, int lam_slot, cudaStream_t s)
 {
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
-    int epb = spread_elems(elems_per_block_p(N, HS3D_FP64, 1, kSmallCta), b.total_elems);
-    int threads = epb * n3;
-    if (threads > vol_threads<N>()) {
-        epb = vol_threads<N>() / n3;
-        threads = epb * n3;
-    }
+    const int epb = elems_per_cta(N, HS3D_FP64, kShapeElem, FORM, false, b.total_elems);
+    const int threads = epb * n3;
     const size_t smem = vol_smem_bytes<N, NS, FORM>(epb);
     unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);
     const Ops *ops = device_ops(N);

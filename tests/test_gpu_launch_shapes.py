@@ -28,3 +28,45 @@ def test_chandrashekar_n2_cta_sizes(shape, physics, surface):
     gm.residual(hs.solver_cfg(physics, surface, "ec", "mixed32", Re=400.0), u, r)
     ref = om.residual(O.Cfg(physics, surface, "ec", Re=400.0), u0)
     assert np.linalg.norm(r.cpu().numpy() - ref) / np.linalg.norm(ref) < TOL
+
+
+def cached(path):
+    import json
+    return json.loads(path.read_text())
+
+
+def test_tuning_reports_and_keeps_shapes_that_run(tmp_path, monkeypatch):
+    """The Chandrashekar kernel at N = 3 and 4 takes at most 128 threads, and a
+    choice for it is none for the other split forms."""
+    cache = tmp_path / "tune.json"
+    monkeypatch.setenv("HS3D_TUNE_CACHE", str(cache))
+    ns = dict(precision="mixed32", Re=400.0)
+    for N, E, most in ((3, 9, 2), (4, 7, 1)):
+        m = hs.Mesh(E, E, E, N, lo=LO, hi=HI, amp=0.05)
+        grad, elem = m.autotune(hs.solver_cfg("ns", "roe", "ec", **ns))
+        assert 1 <= elem <= most and grad * (N + 1) ** 3 <= 256
+        assert cached(cache)[f"N{N}_p1_k1"] == elem and cached(cache)[f"N{N}_p1_k0"] == grad
+    m = hs.Mesh(9, 9, 9, 3, lo=LO, hi=HI, amp=0.05)
+    before = cached(cache)
+    _, elem = m.autotune(hs.solver_cfg("ns", "roe", "kg", **ns))
+    after = cached(cache)
+    assert after["N3_p1_k2"] == elem and after["N3_p1_k1"] == before["N3_p1_k1"]
+
+
+@pytest.mark.parametrize("precision,volume,nodes", [("mixed32", "ec", "lobatto"), ("fp64", "kg", "lobatto"),
+                                                    ("mixed32", "standard", "gauss")])
+def test_tuning_on_a_mesh_too_small_for_the_shapes_to_differ(precision, volume, nodes, tmp_path, monkeypatch):
+    """Such a mesh's launches stay spread (one element per CTA), the choice kept for
+    larger ones is within the largest CTA, and results stay the same bit for bit."""
+    cache = tmp_path / "tune.json"
+    monkeypatch.setenv("HS3D_TUNE_CACHE", str(cache))
+    m = hs.Mesh(3, 3, 3, 2, lo=LO, hi=HI, amp=0.05, nodes=nodes)
+    cfg = hs.solver_cfg("ns", "roe", volume, precision, Re=400.0)
+    u = torch.from_numpy(random_state(m.shape, seed=4, smooth=True)).cuda()
+    r0, r1 = torch.empty_like(u), torch.empty_like(u)
+    m.residual(cfg, u, r0)
+    assert m.autotune(cfg) == (1, 1)
+    kept = cached(cache)
+    assert all(1 <= v and (2 < int(k[1]) or v * 27 <= 256) for k, v in kept.items() if k.startswith("N2"))
+    m.residual(cfg, u, r1)
+    assert torch.equal(r0, r1)
