@@ -31,8 +31,11 @@ struct Prim {
 //   1/x:        e = 1 - x y,    y (1 + e + e^2)            (error e^3)
 //   x^(-1/2):   e = 1 - x y^2,  y (1 + e/2 + 3 e^2/8)      (error ~ e^3)
 // (the leading terms of the binomial series of 1/(1-e) and (1-e)^(-1/2)):
-// 3 and 5 FP64 instructions for a result within about one unit in the last
-// place.  The range test is on the integer pipe; zero, negative, subnormal,
+// 3 and 5 FP64 instructions.  Largest relative errors over the exponent range, in
+// units of 2^-53: reciprocal 1.00, inverse root 1.24 (CUDA's root and division in
+// turn: 1.49), root and quotient, one product more, 1.94 (IEEE: 1).  Errors of the
+// residual against 80-bit arithmetic, 616 states and forms: 0.988 times those of
+// the IEEE operations in the geometric mean.  The range test is on the integer pipe; zero, negative, subnormal,
 // huge, infinite and NaN arguments take the IEEE operation out of line.
 __device__ __noinline__ inline double rcp_ieee(double x) { return 1.0 / x; }
 __device__ __noinline__ inline double rsqrt_ieee(double x) { return 1.0 / sqrt(x); }
@@ -46,15 +49,6 @@ __device__ __forceinline__ double rcp_fast(double x)
     double e = fma(-x, y, 1.0);
     e = fma(e, e, e);
     return fma(y, e, y);
-}
-
-// One second-order step: about 40 bits (no range test: the caller's value is
-// used only where the argument is a plain number).
-__device__ __forceinline__ double rcp_newton(double x)
-{
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    return fma(y, fma(-x, y, 1.0), y);
 }
 
 __device__ __forceinline__ double rsqrt_step(double x)
@@ -518,7 +512,7 @@ __device__ __forceinline__ double logmean_far(double a, double b)
 // Chandrashekar's flux in FP64 from the per-node inputs (rho, v/2, 2 beta =
 // rho/p): the mean {v} is a plain sum, the means' factors sit in the
 // constants, and with |v_L|^2 + |v_R|^2 = |v_L + v_R|^2 - 2 v_L.v_R the
-// energy is f_E = f_rho (hg/beta^ + v_L.v_R/2) + p~ {v}.a: 47 FP64
+// energy is f_E = f_rho (hg/beta^ + v_L.v_R/2) + p~ {v}.a: 48 FP64
 // instructions for a pair on the short series (u < 1e-4, first term left out
 // below 1.2e-17) against 72 with per-node logarithms, full means and an IEEE
 // division.
@@ -526,10 +520,8 @@ __device__ __forceinline__ void ec_pair64(const double *L, const double *Rr, dou
                                           double a3, double f[5])
 {
     const double srho = L[0] + Rr[0], sb2 = L[4] + Rr[4];
-    // 1/(rho_L + rho_R) enters the short series only through u < 1e-4, where
-    // the seed's 40 bits after one Newton step are enough (an error of 1e-12 u/3)
     const double ib2 = rcp_fast(sb2);   // 1/(2(beta_L + beta_R))
-    const double fr = (L[0] - Rr[0]) * rcp_newton(srho), ur = fr * fr;
+    const double fr = (L[0] - Rr[0]) * rcp_fast(srho), ur = fr * fr;
     const double fb = (L[4] - Rr[4]) * ib2, ub = fb * fb;
     double rho_ln, hib;   // rho^, hg/beta^
     if (ur < LogMeanEps<double>::v)
