@@ -12,6 +12,9 @@ of a step has 20 significant bits, so its relative error d is below 2^-19.
               relative to 1, halved by e/2), the first term left out is 5 e^3/16
               with e = 2 d: 2^-54 5/16, and the final fma: 1/2 + 0.16 + 1
   root        that and one product: 2.66
+  corrected   root and quotient by their residuals, which are exact to 2^-53 of
+              themselves: the square of the error corrected (2^-104) and one
+              rounding, 1 + 2^-20, where the residual is a normal number
 """
 import ctypes as C
 import subprocess
@@ -35,9 +38,9 @@ __global__ void k_steps(const double *a, const double *x, long long n, double *o
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double v = x[i];
-    const double r[8] = {rcp_fast(v), rsqrt_fast(v), sqrt_fast(v), div_(a[i], v),
-                         1.0 / v, 1.0 / sqrt(v), sqrt(v), a[i] * (1.0 / v)};
-    for (int k = 0; k < 8; ++k) out[k * n + i] = r[k];
+    const double r[10] = {rcp_fast(v), rsqrt_fast(v), sqrt_fast(v), div_(a[i], v),
+                          1.0 / v, 1.0 / sqrt(v), sqrt(v), a[i] * (1.0 / v), root(v), quotient(a[i], v)};
+    for (int k = 0; k < 10; ++k) out[k * n + i] = r[k];
 }
 extern "C" int run_steps(const double *a, const double *x, long long n, double *out)
 {
@@ -59,7 +62,7 @@ def steps(tmp_path_factory):
 
     def run(a, x):
         ad, xd = torch.from_numpy(a).cuda(), torch.from_numpy(x).cuda()
-        out = torch.empty((8, x.size), dtype=torch.float64, device="cuda")
+        out = torch.empty((10, x.size), dtype=torch.float64, device="cuda")
         torch.cuda.synchronize()
         assert f(ad.data_ptr(), xd.data_ptr(), x.size, out.data_ptr()) == 0
         return out.cpu().numpy()
@@ -92,6 +95,17 @@ def test_steps_against_exact_values(steps):
         assert err <= bound, (name, float(err))
 
 
+def test_corrected_root_and_quotient(steps):
+    rng = np.random.default_rng(19)
+    n = 1 << 20
+    x = np.ldexp(rng.uniform(1.0, 2.0, size=n), rng.integers(-400, 400, size=n))
+    a = np.ldexp(rng.uniform(1.0, 2.0, size=n), rng.integers(-400, 400, size=n))
+    got = steps(a, x)
+    xl, al = x.astype(np.longdouble), a.astype(np.longdouble)
+    for v, exact in ((got[8], np.sqrt(xl)), (got[9], al / xl)):
+        assert np.abs((v - exact) / exact).max() * 2.0 ** 53 <= 1 + 2.0 ** -20
+
+
 def test_arguments_outside_the_steps_take_the_ieee_operations(steps):
     rng = np.random.default_rng(18)
     x = np.concatenate([[0.0, -0.0, np.inf, -np.inf, np.nan, 5e-324, -5e-324, 2.0 ** -1022, np.nextafter(2.0 ** -1021, 0),
@@ -105,6 +119,11 @@ def test_arguments_outside_the_steps_take_the_ieee_operations(steps):
     assert same(got[0], got[4])[~step].all() and same(got[3], got[7])[~step].all()
     step = plain(x) & (x > 0)
     assert same(got[1], got[5])[~step].all() and same(got[2], got[6])[~step].all()
+    assert same(got[8], got[6])[~step].all()
+    # a quotient by an infinite value is zero, by zero or one that overflows infinite
+    assert (got[9][np.isinf(x)] == 0).all() and np.isinf(got[9][x == 0]).all()
+    big, small = np.full(1, 1e300), np.full(1, 1e-300)
+    assert np.isposinf(steps(big, small)[9]).all()
 
 
 def test_logarithmic_mean_of_densities_whose_sum_is_near_the_largest_double():
