@@ -73,3 +73,15 @@ def test_both_sides_of_the_line_match_the_oracle(shape, physics, surface, volume
     uo = u0.copy()
     om.rk3_step(oc, uo, np.zeros_like(uo))
     assert np.linalg.norm((u.cpu().numpy() - u0) - (uo - u0)) / np.linalg.norm(uo - u0) < TOL
+
+
+@pytest.mark.parametrize("physics,surface,volume", FORMS)
+def test_persistent_grids_equal_cta_grids(physics, surface, volume):
+    """More elements (1,190) than CTAs fit on the GPU at once, in a batch of three:
+    the persistent CTAs walk several tiles.  The kernels are instantiations of
+    their own, in which the compiler may fuse the FP32 multiply-adds differently:
+    equal to the FP32 rounding of the residual, as for the other degrees."""
+    shapes = [(9, 9, 9), (5, 5, 5), (6, 7, 8)]
+    cfg = hs.solver_cfg(physics, surface, volume, "mixed32", Re=400.0, Ma=0.1, cfl=0.5)
+    for a, b in zip(serve(shapes, cfg, 0.05, 3), serve(shapes, cfg, 0.05, 3, "persistent")):
+        assert np.abs(a - b).max() <= 1e-7 * np.abs(a).max()
