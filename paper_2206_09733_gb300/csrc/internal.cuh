@@ -209,23 +209,31 @@ __device__ __forceinline__ void raise_max(unsigned long long *dst, unsigned long
     if (v > cur) atomicMax(dst, v);
 }
 
+// The lanes of this thread's warp that the CTA has (its last warp may be partly
+// filled: FP64 and Gauss-Legendre CTAs hold whole elements).
+__device__ __forceinline__ unsigned cta_warp_mask()
+{
+    const int left = (int)blockDim.x - (int)(threadIdx.x & ~31u);
+    return left >= 32 ? 0xffffffffu : (1u << left) - 1u;
+}
+
 // Max-reduce non-negative rates over the lanes of a warp that share the same
 // clock (threads map to consecutive nodes and an item's elements are
 // consecutive, so each group is a contiguous run of lanes).  The bits of
-// non-negative doubles order as integers.  All 32 lanes must call this.
+// non-negative doubles order as integers.  Every thread of the CTA must call this.
 __device__ __forceinline__ void warp_max_to_clock(unsigned long long *dst_c, unsigned long long *dst_v, double lc,
                                                   double lv, bool active)
 {
-    const unsigned full = 0xffffffffu;
+    const unsigned warp = cta_warp_mask();
     const int lane = threadIdx.x & 31;
     unsigned long long key = active ? (unsigned long long)dst_c : 0ull;
-    unsigned peers = __match_any_sync(full, key);
+    unsigned peers = __match_any_sync(warp, key);
     const int first = __ffs(peers) - 1;
     const int last = 31 - __clz(peers);
     unsigned long long bc = (unsigned long long)__double_as_longlong(lc), bv = (unsigned long long)__double_as_longlong(lv);
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-        const unsigned long long oc = __shfl_down_sync(full, bc, off), ov = __shfl_down_sync(full, bv, off);
+        const unsigned long long oc = __shfl_down_sync(warp, bc, off), ov = __shfl_down_sync(warp, bv, off);
         if (lane + off <= last) {
             bc = oc > bc ? oc : bc;
             bv = ov > bv ? ov : bv;
@@ -261,8 +269,7 @@ __device__ __forceinline__ void cta_max_to_clock(unsigned long long *lam, bool n
 {
     __shared__ unsigned long long part[2][16];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = (int)(blockDim.x + 31) >> 5;
-    const int left = (int)blockDim.x - (warp << 5);
-    const unsigned mask = left >= 32 ? 0xffffffffu : (1u << left) - 1u;
+    const unsigned mask = cta_warp_mask();
     const unsigned long long wc = warp_max_bits(mask, lc), wv = ns ? warp_max_bits(mask, lv) : 0ull;
     if (lane == 0) {
         part[0][warp] = wc;
