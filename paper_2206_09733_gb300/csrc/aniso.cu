@@ -39,7 +39,7 @@
 #include <algorithm>
 #include <mutex>
 #include <new>
-#include <utility>
+#include <tuple>
 #include <vector>
 
 #include "aniso.cuh"
@@ -1048,6 +1048,7 @@ void pack_elements(const AnisoMesh *a, int T, std::vector<int> &slot_elem, std::
     std::vector<std::vector<int>> by_n3(T + 1), open(T + 1);   // elements by node count, packs by free slots
     for (int e = 0; e < a->E; ++e) by_n3[a->noff[e + 1] - a->noff[e]].push_back(e);
     slot0.assign(a->E, 0);
+    slot_elem.reserve((size_t)a->noff[a->E] * 9 / 8 + T);
     int packs = 0;
     for (int n3 = T; n3 > 0; --n3)
         for (int e : by_n3[n3]) {
@@ -1069,32 +1070,66 @@ void pack_elements(const AnisoMesh *a, int T, std::vector<int> &slot_elem, std::
 }
 
 // The face table sorted by mortar degrees, then by the sides' degrees, and its CTAs.
+// A face's kind is the two sides' points (2 .. 8) in both tangential directions:
+// 7^4 kinds, ranked once, and one counting pass (a comparison sort was a tenth of
+// the set-up of 4352 elements).
 void pack_faces(const AnisoMesh *a, std::vector<AFace> &faces, std::vector<AFaceCta> &ctas)
 {
-    auto side = [&](const AFace &f, int k, int t) {   // points of side k (0: L) in tangential direction t
-        const int d0 = f.d == 0 ? 1 : 0, d1 = f.d == 2 ? 1 : 2;
-        return a->P3[3 * (size_t)(k ? f.eR : f.eL) + (t ? d1 : d0)] + 1;
+    constexpr int kKinds = kMaxN * kMaxN * kMaxN * kMaxN;
+    struct Kind {
+        int l0, r0, l1, r1, m0, m1;
     };
-    std::vector<std::pair<unsigned, int>> key(faces.size());
+    static const std::vector<Kind> kinds = [] {   // in the order of the table
+        std::vector<Kind> k;
+        for (int l0 = 2; l0 <= kMaxn; ++l0)
+            for (int r0 = 2; r0 <= kMaxn; ++r0)
+                for (int l1 = 2; l1 <= kMaxn; ++l1)
+                    for (int r1 = 2; r1 <= kMaxn; ++r1)
+                        k.push_back(Kind{l0, r0, l1, r1, std::max(l0, r0), std::max(l1, r1)});
+        std::sort(k.begin(), k.end(), [](const Kind &x, const Kind &y) {
+            return std::tie(x.m0, x.m1, x.l0, x.r0, x.l1, x.r1) < std::tie(y.m0, y.m1, y.l0, y.r0, y.l1, y.r1);
+        });
+        return k;
+    }();
+    auto index = [](int l0, int r0, int l1, int r1) { return (((l0 - 2) * kMaxN + r0 - 2) * kMaxN + l1 - 2) * kMaxN + r1 - 2; };
+    static const std::vector<int> rank = [&] {
+        std::vector<int> r(kKinds);
+        for (int k = 0; k < kKinds; ++k) r[index(kinds[k].l0, kinds[k].r0, kinds[k].l1, kinds[k].r1)] = k;
+        return r;
+    }();
+    std::vector<int> kind(faces.size()), at(kKinds + 1, 0);
     for (size_t i = 0; i < faces.size(); ++i) {
         const AFace &f = faces[i];
-        const unsigned l0 = side(f, 0, 0), r0 = side(f, 1, 0), l1 = side(f, 0, 1), r1 = side(f, 1, 1);
-        const unsigned m0 = l0 > r0 ? l0 : r0, m1 = l1 > r1 ? l1 : r1;
-        key[i] = {(((((m0 * 16 + m1) * 16 + l0) * 16 + r0) * 16 + l1) * 16 + r1), (int)i};
+        const int *L = &a->P3[3 * (size_t)f.eL], *R = &a->P3[3 * (size_t)f.eR];
+        const int d0 = f.d == 0 ? 1 : 0, d1 = f.d == 2 ? 1 : 2;
+        kind[i] = rank[index(L[d0] + 1, R[d0] + 1, L[d1] + 1, R[d1] + 1)];
+        ++at[kind[i] + 1];
     }
-    std::sort(key.begin(), key.end());
+    for (int k = 0; k < kKinds; ++k) at[k + 1] += at[k];
     std::vector<AFace> sorted(faces.size());
-    for (size_t i = 0; i < faces.size(); ++i) sorted[i] = faces[key[i].second];
-    faces.swap(sorted);
-    for (size_t i = 0; i < faces.size();) {
-        const unsigned m = key[i].first >> 16;
-        AFaceCta c{(int)i, 0, (int)(m >> 4), (int)(m & 15), 0};
-        const int most = kAFaceThreads / (c.nm0 * c.nm1);
-        for (; i < faces.size() && c.count < most && key[i].first >> 16 == m; ++i, ++c.count)
-            for (int k = 0; k < 2; ++k)
-                if (side(faces[i], k, 0) < c.nm0) c.passes |= 1 << k;
-        ctas.push_back(c);
+    {
+        std::vector<int> next(at.begin(), at.end() - 1);
+        for (size_t i = 0; i < faces.size(); ++i) sorted[next[kind[i]]++] = faces[i];
     }
+    faces.swap(sorted);
+    // CTAs of faces of equal mortar degrees, kind by kind
+    AFaceCta c{0, 0, 0, 0, 0};
+    for (int k = 0; k < kKinds; ++k) {
+        const Kind &K = kinds[k];
+        const int most = kAFaceThreads / (K.m0 * K.m1);
+        for (int i = at[k]; i < at[k + 1];) {
+            if (c.count > 0 && (c.nm0 != K.m0 || c.nm1 != K.m1 || c.count == most)) {
+                ctas.push_back(c);
+                c.count = 0;
+            }
+            if (c.count == 0) c = AFaceCta{i, 0, K.m0, K.m1, 0};
+            const int take = std::min(most - c.count, at[k + 1] - i);
+            c.count += take;
+            c.passes |= (K.l0 < K.m0 ? 1 : 0) | (K.r0 < K.m0 ? 2 : 0);
+            i += take;
+        }
+    }
+    if (c.count > 0) ctas.push_back(c);
 }
 
 }  // namespace
@@ -1104,10 +1139,7 @@ void pack_faces(const AnisoMesh *a, std::vector<AFace> &faces, std::vector<AFace
 void aniso_free(AnisoMesh *a)
 {
     if (!a) return;
-    void *ptrs[] = {a->dP3, a->dnoff, a->doff, a->dfnoff, a->cls_elems, a->slot_elem, a->slot0, a->faces, a->fctas, a->X, a->Ja, a->J, a->invJ,
-                    a->grad, a->fstar, a->qhat, a->diag_part, a->clk, a->clkp, a->one};
-    for (void *p : ptrs)
-        if (p) cudaFree(p);
+    if (a->slab) cudaFree(a->slab);
     delete a;
 }
 
@@ -1206,10 +1238,15 @@ hs3d_status aniso_build(const hs3d_mesh_desc *desc, const int *degree3, AnisoMes
         {(void **)&a->clkp, sizeof(Clock *)},
         {(void **)&a->one, sizeof(int)},
     };
-    cudaError_t e = cudaSuccess;
+    // one allocation for all of them (as api.cu's mesh_alloc), every array on a
+    // 256-byte boundary
+    for (auto &al : allocs) a->bytes += (al.bytes + 255) & ~(size_t)255;
+    cudaError_t e = cudaMalloc(&a->slab, a->bytes);
+    if (e != cudaSuccess) a->slab = nullptr;
+    char *at = (char *)a->slab;
     for (auto &al : allocs) {
-        if (e == cudaSuccess) e = cudaMalloc(al.p, al.bytes);
-        if (e == cudaSuccess) a->bytes += al.bytes;
+        *al.p = a->slab ? at : nullptr;
+        at += (al.bytes + 255) & ~(size_t)255;
     }
     const int one = 1;
     static_assert(sizeof(long long) == sizeof(int64_t), "offset layout");

@@ -49,6 +49,7 @@ struct AnisoMesh {
     std::vector<int64_t> fnoff;       // [6E+1] face-node offsets, face slot s = 2d (-d) or 2d+1 (+d)
     int cls_begin[kAnisoClasses + 1] = {0};
     // device
+    void *slab = nullptr;             // the one allocation behind the arrays below
     int *dP3 = nullptr;
     long long *dnoff = nullptr, *doff = nullptr, *dfnoff = nullptr;
     int *cls_elems = nullptr;         // element ids, class by class
