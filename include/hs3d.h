@@ -256,10 +256,10 @@ hs3d_status hs3d_diagnostics(const hs3d_mesh *mesh, const hs3d_solver_cfg *cfg, 
  * [E][n3] e.g. copied out by hs3d_mesh_geometry, the state u and optionally
  * dudt, all DEVICE FP64) and the DEVICE output out[7] (same meaning as
  * hs3d_diagnostics; the two give the same result on the same mesh).  The
- * per-block partial sums live in one fixed device array of 4096 slots, each
- * covering 2048 nodes, so E*(N+1)^3 may not exceed 8,388,608 nodes
+ * per-block partial sums live in one fixed device array, 7 doubles for each of
+ * at most 1216 blocks.  E*(N+1)^3 may not exceed 8,388,608 nodes
  * (HS3D_ERR_INVALID beyond).  The array is compiled into the library: every
- * GPU that loads it holds the array (256 KB) until the process exits.  The
+ * GPU that loads it holds the array (67 KB) until the process exits.  The
  * first call on a device looks up the array's device address
  * (cudaGetSymbolAddress); make that first call before any stream capture.
  * Every call reuses the same array and leaves its partial sums in it; each

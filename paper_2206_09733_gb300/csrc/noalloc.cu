@@ -18,13 +18,11 @@
 
 namespace hs3d {
 
-// Capacity: one partial-sum slot (7 doubles, padded to 8) per 2048 nodes.
-constexpr int kStaticSlots = 4096;
-constexpr int kStaticNodesPerSlot = 2048;
-constexpr long long kStaticMaxNodes = (long long)kStaticSlots * kStaticNodesPerSlot;   // 8,388,608
+// Capacity stated in the interface.  (The grid stops growing at kDiagMaxBlocks, so
+// the array holds the sums of any number of nodes; what was refused stays refused.)
+constexpr long long kStaticMaxNodes = 8388608;
 
-static __device__ __align__(256) double g_static_partials[kStaticSlots * 8];
-static_assert(7 * kDiagMaxBlocks <= kStaticSlots * 8, "the fixed array holds the largest grid's partial sums");
+static __device__ __align__(256) double g_static_partials[7 * kDiagMaxBlocks];
 
 // Device address of g_static_partials, looked up once per device.
 static double *static_partials_ptr(int dev, cudaError_t &err)
@@ -62,9 +60,8 @@ extern "C" hs3d_status hs3d_diagnostics_noalloc(int N, int64_t E, double gamma, 
     const long long total = (long long)E * n3;
     if (total > kStaticMaxNodes)
         return fail(HS3D_ERR_INVALID,
-                    "E*(N+1)^3 = %lld nodes exceeds the static scratch capacity of %lld nodes "
-                    "(%d partial-sum slots of %d nodes); use hs3d_diagnostics",
-                    total, kStaticMaxNodes, kStaticSlots, kStaticNodesPerSlot);
+                    "E*(N+1)^3 = %lld nodes exceeds this entry point's capacity of %lld nodes; use hs3d_diagnostics",
+                    total, kStaticMaxNodes);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e, "no CUDA device");
