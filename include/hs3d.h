@@ -457,7 +457,8 @@ void hs3d_server_destroy(hs3d_server *server);
  *     group, uploaded when the set of running requests changes) and a
  *     persistent grid per kernel (as many CTAs as are resident at once), whose
  *     CTAs walk the tiles with a stride of the grid size.
- * Both compute the same results bit for bit. */
+ * Both compute the same results: bit for bit in FP64, to the FP32 rounding of
+ * the residual in mixed precision. */
 enum { HS3D_LAUNCH_GRID = 0, HS3D_LAUNCH_PERSISTENT = 1 };
 hs3d_status hs3d_server_set_launch_mode(hs3d_server *server, int mode);
 /* Copies the request and queues it; never blocks on the GPU.  HS3D_ERR_NOMEM

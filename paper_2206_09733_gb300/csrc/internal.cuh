@@ -421,9 +421,6 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned by
                  "l"(src), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
 }
-// Wait for phase `parity` of the barrier, at most `limit` polls (each poll
-// may suspend the thread for a hardware-defined interval).  Returns false
-// when the limit ran out.
 // Invalidate a barrier whose copies have all completed, so that the same
 // shared-memory word can be initialised again (the next tile of a
 // persistent CTA).
@@ -432,6 +429,9 @@ __device__ __forceinline__ void mbar_inval(unsigned long long *bar)
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// Wait for phase `parity` of the barrier, at most `limit` polls (each poll
+// may suspend the thread for a hardware-defined interval).  Returns false
+// when the limit ran out.
 __device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned parity, long long limit)
 {
     const unsigned a = smem_u32(bar);

@@ -135,14 +135,6 @@ __device__ __forceinline__ double reload_state(const double *ptr)
     return x;
 }
 
-template <int n>
-__device__ __forceinline__ int dev_line_node(int d, int idx, int ta, int tb)
-{
-    if (d == 0) return idx + n * (ta + n * tb);
-    if (d == 1) return ta + n * (idx + n * tb);
-    return ta + n * (tb + n * idx);
-}
-
 // Minimum resident CTAs asked of the compiler (its register budget), in CTAs
 // of 256 threads: the split forms 4 (64 registers; ~56 bytes of spills per
 // thread, and still 8-12% faster than 3 CTAs at 80 registers, 16^3 and 32^3

@@ -52,10 +52,10 @@ constexpr int vol_threads()
     return (max_cta_threads(N, HS3D_FP64, kShapeElem, HS3D_VOL_STANDARD, false) + 31) & ~31;
 }
 
-// Minimum resident CTAs per SM asked of the compiler: the mixed path is
-// latency bound, so its register budget is capped (64 per thread with
-// 256- or 512-thread CTAs) to keep more warps resident; the FP64 path is
-// bound by the FP64 pipe and keeps its registers.
+// Minimum resident CTAs per SM asked of the compiler (Gauss-Legendre element
+// kernel): the mixed path is latency bound, so its register budget is capped (64
+// per thread with 256- or 512-thread CTAs) to keep more warps resident; the FP64
+// path is bound by the FP64 pipe and keeps its registers.
 template <int N, typename R>
 constexpr int vol_min_blocks()
 {
@@ -70,15 +70,6 @@ __device__ __forceinline__ size_t face_block(const Item &it, int slot, int d, in
     return it.face6 ? (size_t)slot * it.E + e : (size_t)d * it.E + owner;
 }
 
-// Node with index `idx` along direction d on the line with tangential indices (ta, tb).
-template <int n>
-__device__ __forceinline__ int line_node(int d, int idx, int ta, int tb)
-{
-    if (d == 0) return idx + n * (ta + n * tb);
-    if (d == 1) return ta + n * (idx + n * tb);
-    return ta + n * (tb + n * idx);
-}
-
 template <typename R>
 __device__ __forceinline__ const R *metric_ptr(const Item &it);
 template <>
@@ -89,20 +80,16 @@ __device__ __forceinline__ const float *metric_ptr<float>(const Item &it) { retu
 // Residual store or RK stage of one node from V (volume + surface sum), then,
 // after the last stage (lam_slot >= 0), the dt maxima of the updated state.
 // u holds the FP64 state on the FP64 path (loaded here on the mixed path).
-// Mixed path: sU and sG, when given, are the element's FP64 u and g
-// blocks (5 n3 each) and sIJ its 1/J (FP32), staged in shared memory by
-// asynchronous copies at the start of the kernel (g only for stage > 0).
 template <typename R, bool NS>
 __device__ __forceinline__ void node_update(const Item &it, int e, int p, int n3, const R V[5], double u[5],
                                             int stage, double rkA, double rkB, int lam_slot, double &lc, double &lv,
-                                            bool &lam_active, const double *sU = nullptr, const double *sG = nullptr,
-                                            const float *sIJ = nullptr)
+                                            bool &lam_active)
 {
     if constexpr (sizeof(R) == 4) {
         // the FP64 state is needed only for the RK accumulation
         if (stage >= 0) {
 #pragma unroll
-            for (int v = 0; v < 5; ++v) u[v] = sU ? sU[v * n3 + p] : it.u[(size_t)e * 5 * n3 + p + v * n3];
+            for (int v = 0; v < 5; ++v) u[v] = it.u[(size_t)e * 5 * n3 + p + v * n3];
         }
     }
 
@@ -131,7 +118,7 @@ __device__ __forceinline__ void node_update(const Item &it, int e, int p, int n3
         // register g holds FP32 increments ([E][5][n3] floats in the first half
         // of the caller's buffer) and the state accumulates in FP64 (one FP64
         // FMA per variable).
-        const float ijf = sIJ ? sIJ[p] : it.invJf[(size_t)e * n3 + p];
+        const float ijf = it.invJf[(size_t)e * n3 + p];
         if (stage < 0) {
             double *O = it.out + (size_t)e * 5 * n3 + p;
 #pragma unroll
@@ -168,7 +155,7 @@ __device__ __forceinline__ void node_update(const Item &it, int e, int p, int n3
                 const R c = sound_speed(qn, P.gamma);
                 R iJ;
                 if constexpr (sizeof(R) == 8) iJ = it.invJ[(size_t)e * n3 + p];
-                else iJ = sIJ ? sIJ[p] : it.invJf[(size_t)e * n3 + p];
+                else iJ = it.invJf[(size_t)e * n3 + p];
                 R sc = (R)0, sv = (R)0;
                 const R *JA = metric_ptr<R>(it) + (size_t)e * 9 * n3 + p;
 #pragma unroll

@@ -1,6 +1,6 @@
-// Element kernel of the mixed path's standard form at N = 7 (volume_dev.cuh
-// states the method): four consecutive nodes along xi per thread in the
-// contraction.
+// Element kernel of the mixed path's standard form at N = 7 for launches over more
+// than kFewElems elements (volume_dev.cuh states the method and why the line lies
+// there): four consecutive nodes along xi per thread in the contraction.
 //
 // With one thread per node an element is a CTA of 512 threads, two of which
 // fill an SM's registers: each of its barriers stalls half the SM, and every
