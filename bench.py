@@ -263,15 +263,19 @@ def kernel_bytes(kernel, prec, E=None, n=N + 1, visc=9):
 
 
 def volume_flops(E=None, n=N + 1):
-    """Algorithmic flops of one launch of the split-form NS element kernel
-    (an FMA counts 2, a divide / sqrt / log 1 each), counted from the
-    formulas the kernel evaluates:
-      primitives 14, three Euler fluxes 3*13, three viscous fluxes 3*40,
-      two-point fluxes 3*(n-1) * 63 (two log means 2*14, averages 14,
-      flux 21) plus the 5-term axpy 10 each, diagonal 3*10,
-      viscous D-contraction 3*n*8, surface lift <= 3*10, scale + RK 5*5."""
+    """Flops of one launch of the split-form NS element kernel (an FMA counts 2,
+    a divide or root 1), counted from the formulas that the FP64 kernel
+    evaluates; the mixed one evaluates the same method in deviations, with more
+    operations, and is charged the same.  Per node:
+      primitives 13, pair inputs 4, three viscous fluxes from the stored stress
+      3*26, two-point fluxes 3*(n-1)/2 pairs of 57 (each pair of a line once:
+      sums of inputs and metrics 8, two reciprocals and their ratios 7, the two
+      logarithmic means by the short series 15, velocity sums and pressure 4,
+      the flux 23), their sums over the line 3*(n-1)*10, the viscous part of
+      them 3*(n-1)*8, surface term 19 per face node (6/n of the nodes), scale
+      and RK 26.  No own Euler flux, no diagonal pair, no logarithm per node."""
     E = EX * EY * EZ if E is None else E
-    per_node = 14 + 3 * 13 + 3 * 40 + 3 * (n - 1) * (63 + 10) + 3 * 10 + 3 * n * 8 + 30 + 25
+    per_node = 13 + 4 + 3 * 26 + 3 * (n - 1) * (57 / 2 + 10 + 8) + 19 * 6 / n + 26
     return E * n ** 3 * per_node
 
 
