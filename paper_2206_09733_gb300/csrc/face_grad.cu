@@ -296,7 +296,7 @@ static cudaError_t grad_launch(const Batch &b, cudaStream_t s)
 {
     constexpr int n = N + 1, n3 = n * n * n;
     if (b.total_elems == 0) return cudaSuccess;
-    const int epb = elems_per_cta(N, HS3D_FP64, kShapeGrad, HS3D_VOL_STANDARD, false, b.total_elems);
+    const int epb = elems_per_cta(N, HS3D_FP64, kShapeGrad, HS3D_VOL_STANDARD, false, b.total_elems, b.beside);
     int threads = epb * n3;
     size_t smem = sizeof(double) * (((n * n + 1) & ~1) + (size_t)epb * grad_per_elem<N>());
     unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);

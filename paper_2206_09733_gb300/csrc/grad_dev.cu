@@ -548,7 +548,7 @@ static cudaError_t grad_dev_launch(const Batch &b, cudaStream_t s)
             return e != cudaSuccess ? e : cudaGetLastError();
         }
     }
-    const int epb = elems_per_cta(N, HS3D_MIXED32, kShapeGrad, HS3D_VOL_STANDARD, false, b.total_elems);
+    const int epb = elems_per_cta(N, HS3D_MIXED32, kShapeGrad, HS3D_VOL_STANDARD, false, b.total_elems, b.beside);
     const int threads = epb * n3;
     const size_t smem = sizeof(float) * (((n * n + 3) & ~3) + (size_t)epb * grad_dev_per_elem<N>());
     const unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);

@@ -115,6 +115,9 @@ struct Batch {
     int nitems;
     long long total_elems;
     long long total_faces;
+    // elements of this launch and of those that run beside it on parallel branches (the
+    // degree buckets of one mesh); 0: this launch runs alone
+    long long beside;
     double dt_fixed;        // > 0: every item steps with this dt
     int gauss;              // every item on Gauss-Legendre nodes (items of a batch share the node family)
     // work table (nitems > 1, optional): item of every element of the batch, items[elem_item[ge]],
@@ -600,8 +603,11 @@ constexpr int cta_target(int N, int prec, ShapeKernel k, int form, bool gauss, l
     return 256;
 }
 // Elements per CTA of a launch over `elems` elements: the autotuner's choice if one
-// was made, else cta_target's, within the largest CTA, spread over the SMs.
-int elems_per_cta(int N, int prec, ShapeKernel k, int form, bool gauss, long long elems);
+// was made, else cta_target's, within the largest CTA, spread over the SMs.  beside
+// (Batch::beside): launches side by side share the SMs, so the elements of all count
+// in the spreading: degrees 2..5 on 576 elements, four buckets of 144, each spread by
+// itself, took 5-12% longer than not spread.
+int elems_per_cta(int N, int prec, ShapeKernel k, int form, bool gauss, long long elems, long long beside = 0);
 // The tuned choices, by degree, precision (FP64 / mixed) and slot: the gradient
 // kernel, the element kernel of the standard and Chandrashekar forms, that of the
 // other split forms (their best shapes differ).  0: none.

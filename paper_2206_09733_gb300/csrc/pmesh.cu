@@ -319,6 +319,7 @@ std::vector<Batch> bucket_batches(const hs3d_pmesh *pm, const hs3d_solver_cfg *c
         it.qhat6 = bk.qhat6;
         if (!with_clock) it.clk = nullptr;
         v.push_back(single_batch(it));
+        v.back().beside = pm->E;
     }
     return v;
 }

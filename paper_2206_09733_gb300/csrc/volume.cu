@@ -47,14 +47,14 @@ int tuned_elems(int N, int prec, int slot) { return g_epb[N][prec_slot(prec)][sl
 
 void set_tuned_elems(int N, int prec, int slot, int epb) { g_epb[N][prec_slot(prec)][slot] = epb; }
 
-int elems_per_cta(int N, int prec, ShapeKernel k, int form, bool gauss, long long elems)
+int elems_per_cta(int N, int prec, ShapeKernel k, int form, bool gauss, long long elems, long long beside)
 {
     const int n3 = (N + 1) * (N + 1) * (N + 1);
     const int most = max_cta_threads(N, prec, k, form, gauss) / n3;
     int epb = tuned_elems(N, prec, shape_slot(k, form));
     if (epb <= 0) epb = cta_target(N, prec, k, form, gauss, elems) / n3;
     if (epb > most) epb = most;
-    return spread_elems(epb < 1 ? 1 : epb, elems);
+    return spread_elems(epb < 1 ? 1 : epb, beside > elems ? beside : elems);
 }
 
 cudaError_t prepare_volume(int N)

@@ -898,7 +898,7 @@ static cudaError_t vol_dev_launch2(const Batch &b, int stage, float rkA, double 
             return vol_row_launch<N, NS>(b, stage, rkA, rkB, lam_slot, s);
     }
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
-    const int epb = elems_per_cta(N, HS3D_MIXED32, kShapeElem, FORM, false, b.total_elems);
+    const int epb = elems_per_cta(N, HS3D_MIXED32, kShapeElem, FORM, false, b.total_elems, b.beside);
     const int threads = ((epb * n3) + 31) & ~31;
     const size_t smem = dev_smem_bytes<N, NS, FORM>(epb);
     const unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);

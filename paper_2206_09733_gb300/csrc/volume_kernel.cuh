@@ -416,7 +416,7 @@ template <int N, bool NS, int FORM>
 static cudaError_t vol_launch2(const Batch &b, int stage, double rkA, double rkB, int lam_slot, cudaStream_t s)
 {
     constexpr int n3 = (N + 1) * (N + 1) * (N + 1);
-    const int epb = elems_per_cta(N, HS3D_FP64, kShapeElem, FORM, false, b.total_elems);
+    const int epb = elems_per_cta(N, HS3D_FP64, kShapeElem, FORM, false, b.total_elems, b.beside);
     const int threads = epb * n3;
     const size_t smem = vol_smem_bytes<N, NS, FORM>(epb);
     unsigned blocks = (unsigned)((b.total_elems + epb - 1) / epb);

@@ -70,3 +70,20 @@ def test_tuning_on_a_mesh_too_small_for_the_shapes_to_differ(precision, volume, 
     assert all(1 <= v and (2 < int(k[1]) or v * 27 <= 256) for k, v in kept.items() if k.startswith("N2"))
     m.residual(cfg, u, r1)
     assert torch.equal(r0, r1)
+
+
+# buckets of about 144 elements, three to a CTA (576 elements share the SMs), and of a few
+@pytest.mark.parametrize("shape", [(8, 8, 9), (3, 2, 2)])
+@pytest.mark.parametrize("precision,volume", [("mixed32", "ec"), ("mixed32", "standard"), ("fp64", "ec")])
+def test_degree_buckets_side_by_side(shape, precision, volume):
+    # (mixed: the bar of the mixed path's other mortar tests)
+    from tests import inputs as I
+    from tests.test_gpu_pmesh import TOLMIX, pair, rel, to_dev, to_host
+    deg = I.random_degrees(int(np.prod(shape)), seed=11, lo=2, hi=5)
+    om, gm = pair(*shape, deg, amp=0.05)
+    u0 = I.random_state_blocks(deg, seed=43, smooth=True)
+    ref = om.residual(O.Cfg("ns", "roe", volume, Re=400.0), u0)
+    ud = to_dev(om, gm, u0)
+    r = torch.zeros_like(ud)
+    gm.residual(hs.solver_cfg("ns", "roe", volume, precision, Re=400.0), ud, r)
+    assert rel(to_host(om, gm, r), ref) <= (TOLMIX if precision == "mixed32" else 1e-12)
